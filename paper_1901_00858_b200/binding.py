@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libhgc.so: argument marshalling only.
+"""Thin binding of libhgc.so: argument marshalling only (ctypes; the calls that a forward pass
+repeats go through the CPython module _calls, csrc/py_calls.c).
 
 Every step of the path runs inside the CUDA library; torch is used for device memory and
 streams.  The names mirror the C ABI (include/hgc.h).  If the compiled library is missing
@@ -45,11 +46,33 @@ class hgc_conv_params(ctypes.Structure):
 
 
 _lib = None
+_calls = None   # the CPython module with the calls of a forward pass, once the library is loaded
+
+
+def _first_stream() -> int:
+    """torch's current stream; from then on _calls asks torch for it directly."""
+    import torch
+    handle = torch.cuda.current_stream().cuda_stream
+    device, raw = getattr(torch._C, "_cuda_getDevice", None), getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if device is not None and raw is not None:
+        _calls.stream_hooks(device, raw)
+    return handle
+
+
+def _bind_calls(L: ctypes.CDLL):
+    try:
+        from . import _calls as calls
+    except ImportError as e:
+        raise RuntimeError("the module _calls is missing: build it with `python -m paper_1901_00858_b200.build`") from e
+    calls.bind(_first_stream, *(ctypes.cast(f, ctypes.c_void_p).value for f in (
+        L.hgc_conv_forward, L.hgc_conv_forward_host, L.hgc_dwpw_forward, L.hgc_conv_set_weights, L.hgc_dwpw_set_weights,
+        L.hgc_cast_f32_to_f16, L.hgc_bn_fold)))
+    return calls
 
 
 def lib() -> ctypes.CDLL:
     """Loads libhgc.so (built in-tree by `python -m paper_1901_00858_b200.build`)."""
-    global _lib
+    global _lib, _calls
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -102,8 +125,15 @@ def lib() -> ctypes.CDLL:
                      "hgc_dwpw_set_weights", "hgc_dwpw_forward", "hgc_debug_checked_build", "hgc_debug_violations",
                      "hgc_debug_shrink_ranges"):
             getattr(L, name).restype = ctypes.c_int
+        _calls = _bind_calls(L)
         _lib = L
     return _lib
+
+
+def _load():
+    """The module _calls, for calls that may come before any descriptor has loaded the library."""
+    lib()
+    return _calls
 
 
 def status_string(status: int) -> str:
@@ -220,7 +250,7 @@ class ConvDesc:
             self.set_workspace(torch.empty(need, dtype=torch.uint8, device="cuda"))
 
     def set_weights(self, w, stream=None):
-        _check(lib().hgc_conv_set_weights(self._h, _ptr(w), _stream(stream)), "hgc_conv_set_weights")
+        _check(_calls.set_weights(self, w, stream), "hgc_conv_set_weights")
 
     def last_device_status(self) -> int:
         v = ctypes.c_int32()
@@ -242,27 +272,30 @@ class DwPwDesc(ConvDesc):
                "hgc_dwpw_desc_create")
 
     def set_weights(self, w_dw, w_pw, stream=None):
-        _check(lib().hgc_dwpw_set_weights(self._h, _ptr(w_dw), _ptr(w_pw), _stream(stream)), "hgc_dwpw_set_weights")
+        _check(_calls.set_weights(self, w_dw, w_pw, stream), "hgc_dwpw_set_weights")
 
 
 def dwpw_forward(desc: DwPwDesc, x, w_dw, bias_dw, w_pw, bias_pw, y, relu_dw: bool, relu_pw: bool, stream=None):
     """hgc_dwpw_forward: x [N,H,W,C] channels-last, w_dw [C,1,3,3], w_pw [K,C,1,1], y [N,K,P,Q] (or
     [N,P,Q,K] with HGC_FLAG_Y_NHWC): CUDA fp16 tensors; biases may be None."""
-    _check(lib().hgc_dwpw_forward(desc.handle, _ptr(x), _ptr(w_dw), _ptr(bias_dw), _ptr(w_pw), _ptr(bias_pw), _ptr(y),
-                                  int(bool(relu_dw)), int(bool(relu_pw)), _stream(stream)), "hgc_dwpw_forward")
+    status = _calls.dwpw_forward(desc, x, w_dw, bias_dw, w_pw, bias_pw, y, relu_dw, relu_pw, stream)
+    if status:
+        raise HgcError(status, "hgc_dwpw_forward")
 
 
 def conv_forward(desc: ConvDesc, x, w, bias, y, relu: bool, stream=None):
     """hgc_conv_forward: x, w, bias (or None), y are CUDA fp16 tensors (or raw addresses)."""
-    _check(lib().hgc_conv_forward(desc.handle, _ptr(x), _ptr(w), _ptr(bias), _ptr(y), int(bool(relu)),
-                                  _stream(stream)), "hgc_conv_forward")
+    status = _calls.conv_forward(desc, x, w, bias, y, relu, stream)
+    if status:
+        raise HgcError(status, "hgc_conv_forward")
 
 
 def conv_forward_host(desc: ConvDesc, x, w, bias, y, relu: bool, stream=None):
     """hgc_conv_forward_host: x, w, bias (or None), y are HOST fp16 buffers (pinned torch
     tensors or numpy arrays); copies are queued on the stream."""
-    _check(lib().hgc_conv_forward_host(desc.handle, _ptr(x), _ptr(w), _ptr(bias), _ptr(y),
-                                       int(bool(relu)), _stream(stream)), "hgc_conv_forward_host")
+    status = _calls.conv_forward_host(desc, x, w, bias, y, relu, stream)
+    if status:
+        raise HgcError(status, "hgc_conv_forward_host")
 
 
 def conv_forward_static(params: hgc_conv_params, x, w, bias, y, relu: bool, stream=None):
@@ -276,9 +309,9 @@ def conv_forward_static(params: hgc_conv_params, x, w, bias, y, relu: bool, stre
 def cast_f32_to_f16(src, dst, count=None, overflow_count=None, stream=None):
     """hgc_cast_f32_to_f16: src float32 -> dst float16 CUDA tensors (round to nearest even);
     overflow_count: a 1-element int64 CUDA tensor that the kernel adds to, or None."""
-    n = src.numel() if count is None else count
-    _check(lib().hgc_cast_f32_to_f16(_ptr(src), _ptr(dst), n, _ptr(overflow_count), _stream(stream)),
-           "hgc_cast_f32_to_f16")
+    status = (_calls or _load()).cast_f32_to_f16(src, dst, count, overflow_count, stream)
+    if status:
+        raise HgcError(status, "hgc_cast_f32_to_f16")
 
 
 def batchnorm_workspace_bytes(n: int, c: int, hw: int) -> int:
@@ -299,10 +332,9 @@ def batchnorm_forward(x, y, eps, mean, var, workspace=None, shift_log2=0, use_st
 def bn_fold(w, bias, mean, var, eps, w_out, b_out, gamma=None, beta=None, stream=None):
     """hgc_bn_fold: stored statistics (float32 [K]) and optional gamma/beta folded into conv
     weights w [K,...] and bias [K] (or None); results in w_out, b_out (float16)."""
-    k = int(w.shape[0])
-    per_k = w.numel() // k
-    _check(lib().hgc_bn_fold(_ptr(w), _ptr(bias), _ptr(mean), _ptr(var), _ptr(gamma), _ptr(beta), float(eps), k,
-                             per_k, _ptr(w_out), _ptr(b_out), _stream(stream)), "hgc_bn_fold")
+    status = (_calls or _load()).bn_fold(w, bias, mean, var, eps, w_out, b_out, gamma, beta, stream)
+    if status:
+        raise HgcError(status, "hgc_bn_fold")
 
 
 def layout_nchw_to_nhwc(src, dst, n, c, h, w, c_pad, stream=None):

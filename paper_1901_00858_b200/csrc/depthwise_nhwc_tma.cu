@@ -308,12 +308,12 @@ cudaError_t launch_depthwise3x3_nhwc_tma(const ConvGeom& g, const __half* x, con
   uint16_t* ys = reinterpret_cast<uint16_t*>(y);
   cudaError_t err;
   if (cb == 64) {
-    err = cudaFuncSetAttribute(depthwise3x3_nhwc_tma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    err = allow_dynamic_smem<depthwise3x3_nhwc_tma_kernel<64>>();
     if (err != cudaSuccess) return err;
     err = launch_kernel(depthwise3x3_nhwc_tma_kernel<64>, dim3((unsigned)blocks), dim3(256), smem, stream, tm, a, ws, bs,
                         ys, relu);
   } else {
-    err = cudaFuncSetAttribute(depthwise3x3_nhwc_tma_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    err = allow_dynamic_smem<depthwise3x3_nhwc_tma_kernel<32>>();
     if (err != cudaSuccess) return err;
     err = launch_kernel(depthwise3x3_nhwc_tma_kernel<32>, dim3((unsigned)blocks), dim3(256), smem, stream, tm, a, ws, bs,
                         ys, relu);

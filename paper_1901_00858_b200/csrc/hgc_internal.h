@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "hgc.h"
 
 namespace hgc {
@@ -99,6 +101,24 @@ inline cudaError_t launch_kernel_coop(bool cooperative, void (*kernel)(KArgs...)
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Lets a kernel take all of an SM's shared memory: once per kernel and device, not per launch (the
+// attribute call costs the host about as much as a quarter of a launch).
+template <auto* Kernel>
+cudaError_t allow_dynamic_smem() {
+  static std::atomic<uint64_t> done{0};  // bit per device ordinal
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (dev < 64 && (done.load(std::memory_order_acquire) & bit)) return cudaSuccess;
+  cudaFuncAttributes fa;
+  err = cudaFuncGetAttributes(&fa, Kernel);
+  if (err == cudaSuccess)
+    err = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(232448u - fa.sharedSizeBytes));
+  if (err == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return err;
 }
 
 #ifdef __CUDACC__

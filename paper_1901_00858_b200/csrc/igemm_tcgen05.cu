@@ -31,7 +31,6 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
-
 #include "hgc_internal.h"
 
 namespace hgc {
@@ -3115,8 +3114,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   // the size of the code around them)
 #define HGC_LAUNCH_IGEMM_EW(KBV, HALOV, EWV, EPIV, SPLITV)                                                 \
   do {                                                                                                     \
-    err = cudaFuncSetAttribute(igemm_kernel<KBV, HALOV, EWV, EPIV, SPLITV>,                                \
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);            \
+    err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, EWV, EPIV, SPLITV>>();            \
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_overlapped(igemm_kernel<KBV, HALOV, EWV, EPIV, SPLITV>, grid, dim3(64 + 32 * EWV), \
                           p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \
@@ -3124,8 +3122,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   // depthwise + pointwise block: its own instantiations (8 epilogue + 8 depthwise warps)
 #define HGC_LAUNCH_DWPW_EPI(KBV, EPIV)                                                                     \
   do {                                                                                                     \
-    err = cudaFuncSetAttribute(igemm_kernel<KBV, true, 8, EPIV, false, false, false, false, true>,         \
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);            \
+    err = allow_dynamic_smem<igemm_kernel<KBV, true, 8, EPIV, false, false, false, false, true>>();            \
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_overlapped(igemm_kernel<KBV, true, 8, EPIV, false, false, false, false, true>, grid, \
                           dim3(64 + 32 * 8 + 32 * kDwWarps), p.smem_bytes, stream, p.tmA, p.tmB, p.tmY,    \
@@ -3142,8 +3139,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   // (a tile waits for segments that other CTAs' layout warps convert)
 #define HGC_LAUNCH_FUSED_EPI(KBV, HALOV, EPIV)                                                             \
   do {                                                                                                     \
-    err = cudaFuncSetAttribute(igemm_kernel<KBV, HALOV, 8, EPIV, false, false, false, true>,               \
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);            \
+    err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, false, false, false, true>>();            \
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_coop(true, igemm_kernel<KBV, HALOV, 8, EPIV, false, false, false, true>, grid,   \
                                dim3(64 + 32 * 8 + 32 * kLayoutWarps), p.smem_bytes, stream, p.tmA, p.tmB,  \
@@ -3153,8 +3149,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   // tiles shared between CTAs: their own instantiations (8 epilogue warps), launched cooperatively
 #define HGC_LAUNCH_SHARED_EPI(KBV, HALOV, EPIV)                                                            \
   do {                                                                                                     \
-    err = cudaFuncSetAttribute(igemm_kernel<KBV, HALOV, 8, EPIV, false, false, true>,                      \
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);            \
+    err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, false, false, true>>();            \
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_coop(true, igemm_kernel<KBV, HALOV, 8, EPIV, false, false, true>, grid,          \
                                dim3(64 + 32 * 8), p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a,    \
@@ -3179,14 +3174,12 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
 #define HGC_LAUNCH_PAIR_EPI(KBV, HALOV, EPIV)                                                                  \
   do {                                                                                                       \
     if (cooperative) {                                                                                       \
-      err = cudaFuncSetAttribute(igemm_kernel<KBV, HALOV, 8, EPIV, false, true, true>,                       \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);            \
+      err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, false, true, true>>();            \
       if (err == cudaSuccess)                                                                                \
         err = launch_pair(igemm_kernel<KBV, HALOV, 8, EPIV, false, true, true>, p, sms, true,                \
                           dim3(64 + 32 * 8), stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \
     } else {                                                                                                 \
-      err = cudaFuncSetAttribute(igemm_kernel<KBV, HALOV, 8, EPIV, false, true, false>,                      \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem_bytes);            \
+      err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, false, true, false>>();            \
       if (err == cudaSuccess)                                                                                \
         err = launch_pair(igemm_kernel<KBV, HALOV, 8, EPIV, false, true, false>, p, sms, false,              \
                           dim3(64 + 32 * 8), stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \

@@ -646,8 +646,7 @@ cudaError_t launch_nchw_to_nhwc(const __half* src, __half* dst, int32_t n, int32
   if ((hw % 8) != 0 && hw <= 640 && ((int64_t)c * hw) % 8 == 0 && (kTileC * hw) % 8 == 0) {
     // small odd plane: contiguous 64-channel spans (at most 80 KB of shared memory)
     const size_t smem = (size_t)kTileC * hw * sizeof(uint16_t);
-    cudaError_t err = cudaFuncSetAttribute(nchw_to_nhwc_smallplane_kernel,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_dynamic_smem<nchw_to_nhwc_smallplane_kernel>();
     if (err != cudaSuccess) return err;
     dim3 grid2((unsigned)c_tiles, (unsigned)n);
     launch_kernel(nchw_to_nhwc_smallplane_kernel, dim3(grid2), dim3(kThreads), smem, stream, reinterpret_cast<const uint16_t*>(src),
