@@ -123,7 +123,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return mbar_wait_slow(bar, parity, abort_flag, sleep_ns);
 }
 
-// One lane of a converged warp.
+// One lane of a converged warp (the same one every time).  Copies are issued under this predicate, not
+// under `lane == 0`: the copy instructions take their operands from uniform registers, and only for
+// an elected lane does the compiler know that one thread is left; for any other condition it walks
+// through the lanes, which costs the issuing warp about 500 clocks per copy (a stand-alone loop of
+// copies: 640 clocks per copy against 142, whatever the copy's size).
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred;
   asm volatile(
@@ -1211,7 +1215,7 @@ __device__ __noinline__ uint32_t epilogue_planes(uint32_t t_addr, uint32_t qstag
   const uint32_t tile = shared_tile ? qstage : qstage + (uint32_t)half * tile_bytes;
   const uint32_t row = tile + (uint32_t)lane * (uint32_t)(pq * 2);
   const bool wide = (pq & 3) == 0;
-  const bool sender = lane == 0 && (half == 0 || !shared_tile);
+  const bool sender = elect_one() && (half == 0 || !shared_tile);
   for (int img = shared_tile ? 0 : half; img < tn; img += shared_tile ? 1 : 2) {
     if (n0 + img >= N) break;
     // the staging tile's previous copy must have read it
@@ -1307,6 +1311,10 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   uint32_t rank = 0;
   if constexpr (PAIR) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
 
+  if (warp == 0 && lane < 4) {  // the descriptors' first fetch, beside the set-up
+    const CUtensorMap* tm = lane == 0 ? &tmA : lane == 1 ? &tmB : lane == 2 ? &tmY : &tmYr;
+    asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
+  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.stages; ++s) {
       // (the weight copy + one arrival per depthwise / gathering warp)
@@ -1346,10 +1354,14 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   // the previous kernel in the stream; from here on global memory is read and written
   grid_dependency_wait();
   grid_launch_dependents();
-  // an earlier CTA gave up: do not start new work on a path that is not progressing
-  const bool skip = status != nullptr && *reinterpret_cast<volatile int*>(status) != 0;
+  // An earlier CTA gave up: do not start new work on a path that is not progressing.  The warps that
+  // write global memory look at the status word; the producer and the MMA issuer do not wait for
+  // that read (it is the first access of the kernel and would delay the first copy by a trip to
+  // L2): they fill the ring and the accumulators once and leave through abort_flag.
+  const bool skip = warp >= 2 && status != nullptr && *reinterpret_cast<volatile int*>(status) != 0;
 
   if (skip) {
+    abort_flag = 1;
     // fall through to the release of the tensor memory
   } else if (warp == 0) {
     // ---------------- TMA producer ----------------
@@ -1410,16 +1422,17 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           // (with its one-pixel border) that is fetched here, beside the pointwise weights
           const uint32_t fb = smem_u32(&full_bar[ring.idx]);
           // the weight tiles of the item's channel tiles (one per accumulator), behind one another
-          if (lane == 0) mbar_expect_tx(fb, (uint32_t)(a.nacc * a.taps) * a.a_bytes);
-          __syncwarp();
-          if (lane < a.nacc)
-            tma_load_4d(sbase + a.b_alloc + (uint32_t)(lane * a.taps) * a.a_bytes, &tmA, fb, cb * KB, m0 + lane * 128, tap0, grp);
+          if (elect_one()) {
+            mbar_expect_tx(fb, (uint32_t)(a.nacc * a.taps) * a.a_bytes);
+            for (int i = 0; i < a.nacc; ++i)
+              tma_load_4d(sbase + a.b_alloc + (uint32_t)(i * a.taps) * a.a_bytes, &tmA, fb, cb * KB, m0 + i * 128, tap0, grp);
+          }
           const uint32_t ib = issued & 1u;
           if (!a.gather && !mbar_wait(smem_u32(&in_empty[ib]), ((issued >> 1) & 1u) ^ 1u, &abort_flag, 64)) {
             ok = false;
             break;
           }
-          if (lane == 0 && !a.gather) {
+          if (!a.gather && elect_one()) {
             const uint32_t in_base = ring_base + (uint32_t)a.stages * a.stage_bytes + (uint32_t)(EW * a.nbuf) * kWarpStageBytes;
             mbar_expect_tx(smem_u32(&in_full[ib]), a.dw_in_bytes);
             tma_load_5d(in_base + ib * a.dw_in_alloc, &tmB, smem_u32(&in_full[ib]), cb * KB, 0, -1, p0 * a.dw_stride - 1, n0);
@@ -1427,27 +1440,26 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         } else if constexpr (PAIR) {
           // both CTAs' copies are counted on the first CTA's barrier, which expects the bytes of both
           const uint32_t fb = cluster_addr(smem_u32(&full_bar[ring.idx]), 0);
-          if (lane == 0 && rank == 0)
-            mbar_expect_tx(smem_u32(&full_bar[ring.idx]), 2u * (a.b_bytes + (uint32_t)a.taps * a.a_bytes));
-          if (lane == 0)
+          if (elect_one()) {
+            if (rank == 0) mbar_expect_tx(smem_u32(&full_bar[ring.idx]), 2u * (a.b_bytes + (uint32_t)a.taps * a.a_bytes));
             tma_load_5d_pair(sbase, &tmB, fb, cb * KB, grp, (HALO ? 0 : sg * a.dil_w) - a.pad_w, h_base + r * a.dil_h, n0);
-          if (lane == 8) tma_load_4d_pair(sbase + a.b_alloc, &tmA, fb, cb * KB, m0, tap0, grp);
+            tma_load_4d_pair(sbase + a.b_alloc, &tmA, fb, cb * KB, m0, tap0, grp);
+          }
         } else {
         const uint32_t fb = smem_u32(&full_bar[ring.idx]);
-        // A thread gets a bulk-tensor copy under way only every few hundred clocks, whatever its
-        // size (measured), so a stage is few, large copies issued by different lanes at once:
-        // lane 0 announces the bytes and fetches the activation tile, lane 8 fetches the weight
-        // tiles of all taps of the stage as one box (the 1x1 mode's 64-pixel blocks: one lane each).
-        if (lane == 0) mbar_expect_tx(fb, a.b_bytes + (uint32_t)a.taps * a.a_bytes);
-        if (a.nchw) {
-          // x itself, (pixel, channel, image): blocks of 64 pixels x KB channels, pixels contiguous
-          if (lane < a.nblk)
-            tma_load_3d(sbase + (uint32_t)lane * (uint32_t)(KB * 128), &tmB, fb, p0 * a.Q + 64 * lane,
-                        grp * a.cg + cb * KB, n0);
-        } else if (lane == 0) {
-          tma_load_5d(sbase, &tmB, fb, cb * KB, grp, (HALO ? 0 : sg * a.dil_w) - a.pad_w, h_base + r * a.dil_h, n0);
+        // the activation tile and the weight tiles of all taps of the stage as one box each (the 1x1
+        // mode's 64-pixel blocks: one copy per block)
+        if (elect_one()) {
+          mbar_expect_tx(fb, a.b_bytes + (uint32_t)a.taps * a.a_bytes);
+          if (a.nchw) {
+            // x itself, (pixel, channel, image): blocks of 64 pixels x KB channels, pixels contiguous
+            for (int b = 0; b < a.nblk; ++b)
+              tma_load_3d(sbase + (uint32_t)b * (uint32_t)(KB * 128), &tmB, fb, p0 * a.Q + 64 * b, grp * a.cg + cb * KB, n0);
+          } else {
+            tma_load_5d(sbase, &tmB, fb, cb * KB, grp, (HALO ? 0 : sg * a.dil_w) - a.pad_w, h_base + r * a.dil_h, n0);
+          }
+          tma_load_4d(sbase + a.b_alloc, &tmA, fb, cb * KB, m0, tap0, grp);
         }
-        if (lane == 8) tma_load_4d(sbase + a.b_alloc, &tmA, fb, cb * KB, m0, tap0, grp);
         }
         __syncwarp();
         tap0 += a.taps;
@@ -1759,6 +1771,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     uint16_t* yb = reinterpret_cast<uint16_t*>(y);
     const uint32_t stage_base = ring_base + (uint32_t)a.stages * a.stage_bytes;
     const bool relu = a.relu != 0;
+    const bool leader = elect_one();  // issues this warp's bulk stores and waits for them (their groups are per thread)
     // this warp's own staging tiles: 32 channel rows of 128 bytes each, 128-byte swizzled
     const uint32_t my_stage = stage_base + (uint32_t)ew * (uint32_t)a.nbuf * kWarpStageBytes;
     const uint32_t row_off = (uint32_t)lane * 128u + (((uint32_t)lane & 7u) << 4);
@@ -1954,7 +1967,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
               }
               if (g == 0) {
                 // this buffer's previous store must have been read out of shared memory
-                if (lane == 0) {
+                if (leader) {
                   if (a.nbuf == 1) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                   else asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                 }
@@ -1966,7 +1979,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
-            if (lane == 0) {
+            if (leader) {
               // past P*Q the store is clipped (row pairs: the next row of y belongs to other warps)
               const bool full_box = !a.fine_units && ((e_hi - e_lo == kPassElems) || (last_row_tile && !a.rowpair));
               tma_store_4d(full_box ? &tmY : &tmYr, sbuf, (a.rowpair ? 2 * p0 + odd_row : p0) * a.Q + e_lo, m0 + cq * 32, grp, n0);
@@ -2020,7 +2033,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                         }
                         if (first) {
                           // this buffer's previous store must have been read out of shared memory
-                          if (lane == 0) {
+                          if (leader) {
                             if (a.nbuf == 1) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                             else asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                           }
@@ -2035,7 +2048,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) {
+                    if (leader) {
                       // a short unit at the end of the image takes the full box: the rest is clipped
                       const bool image_end = p0 + hr0 + nrows == a.P && wc0 + ncol == a.Q;
                       tma_store_4d((nrows * ncol == a.y_full_w || image_end) ? &tmY : &tmYr, sbuf, m0 + quarter * 32, grp,
@@ -2091,9 +2104,9 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         else mbar_arrive(acc_empty_bar);
       }
     }
-    // the shared-memory tiles of outstanding stores must stay intact until they have been read,
-    // and the stores themselves must be complete before the kernel ends
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    // the shared-memory tiles of outstanding stores must stay intact until they have been read (the
+    // end of the grid completes the writes)
+    if (leader) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   }
 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
