@@ -18,7 +18,8 @@
 //       - for few-channel stems, overlapping windows of a zero-bordered 8-channel copy, or an
 //         expanded copy holding the values under the kernel per output pixel.
 //
-// One persistent CTA per SM walks its tiles:  warp 0 = TMA producer (a ring stage = one
+// One persistent CTA per SM walks its tiles:  warp 0 and the warp after the epilogue's = TMA
+// producers of activations and weights (a ring stage = one
 // activation tile + the weight tiles of its taps, one mbarrier), warp 1 = TMEM allocator and MMA
 // issuer (one elected lane issues tcgen05.mma; tcgen05.commit releases ring stages and hands
 // accumulators over through mbarriers; two 256-column accumulators alternate), warps 2.. =
@@ -121,6 +122,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
                                           uint32_t sleep_ns = 0) {
   if (mbar_test_wait(bar, parity)) return true;
   return mbar_wait_slow(bar, parity, abort_flag, sleep_ns);
+}
+
+// The same for a converged warp, with an answer that the compiler knows to be warp-uniform (a vote):
+// the loops of the MMA issuer then keep their addresses and descriptors in uniform registers.
+__device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_test_wait(bar, parity) != 0) != 0;
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  if (mbar_test_warp(bar, parity)) return true;
+  return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, 0)) != 0;
 }
 
 // One lane of a converged warp (the same one every time).  Copies are issued under this predicate, not
@@ -484,114 +495,26 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap* tm, uint32_t src
                : "memory");
 }
 
-// Polls barrier `next_bar` (non-blocking), issues KSTEPS MMAs of one shared-memory stage from one
-// elected lane (16 channels per step: +32 bytes = +2 in the descriptors' address field), commits
-// them to `a_bar` (and to `b_bar` if release_b), and returns the poll's result.  Warp-collective.
-// The poll is issued first and its answer read last, so its latency hides behind the MMA issue.
+// KSTEPS MMAs of one weight tile against one activation tile (16 channels per step: +32 bytes = +2 in
+// the descriptors' address field, `b_step` for pixel-major activation tiles).  Called by ONE thread.
+// The descriptors' upper words do not change; only the address field is advanced.
 // PAIR: the MMAs are those of a CTA pair (cta_group::2: 256 output channels, each CTA's tensor
-// core reads its own 128 weight rows and both halves of the activation tile) and the commits
-// arrive on the barriers at the same offsets in both CTAs.
-#define HGC_MMA_FIRST(CG) "@p_mma tcgen05.mma.cta_group::" CG ".kind::f16 [%3], %4, %5, %6, p_acc;\n"
-#define HGC_MMA_NEXT(CG)      \
-  "add.u64 da, da, 2;\n"      \
-  "add.u64 db, db, %12;\n"    \
-  "@p_mma tcgen05.mma.cta_group::" CG ".kind::f16 [%3], da, db, %6, p_one;\n"
-#define HGC_COMMITS_1                                                                      \
-  "@p_el tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%8];\n"    \
-  "@p_rel tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%9];\n"
-#define HGC_COMMITS_2                                                                                            \
-  "@p_el tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%8], cm;\n"   \
-  "@p_rel tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%9], cm;\n"
-#define HGC_STAGE_HEAD                                                  \
-  "{\n"                                                                 \
-  ".reg .pred p_next, p_el, p_mma, p_acc, p_one, p_rel;\n"              \
-  ".reg .b64 da, db;\n"                                                 \
-  ".reg .b16 cm;\n"                                                     \
-  "mov.b16 cm, 3;\n"                                                    \
-  "mov.b64 da, %4;\n"                                                   \
-  "mov.b64 db, %5;\n"                                                   \
-  "mbarrier.test_wait.parity.shared::cta.b64 p_next, [%1], %2;\n"       \
-  "elect.sync _|p_el, 0xffffffff;\n"                                    \
-  "setp.ne.b32 p_mma, %11, 0;\n"                                        \
-  "and.pred p_mma, p_mma, p_el;\n"                                      \
-  "setp.ne.b32 p_acc, %7, 0;\n"                                         \
-  "setp.eq.b32 p_one, 0, 0;\n"                                          \
-  "setp.ne.b32 p_rel, %10, 0;\n"                                        \
-  "and.pred p_rel, p_rel, p_el;\n"
-#define HGC_STAGE_TAIL "selp.u32 %0, 1, 0, p_next;\n}\n"
+// core reads its own 128 weight rows and both halves of the activation tile).
 template <int KSTEPS, bool PAIR>
-__device__ __forceinline__ uint32_t issue_stage(uint32_t next_bar, uint32_t next_parity, uint32_t d_tmem,
-                                                uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc,
-                                                uint32_t a_bar, uint32_t b_bar, uint32_t release_b,
-                                                uint32_t do_mma, uint64_t b_step) {
-  uint32_t ready;
-#define HGC_STAGE_OPERANDS                                                                                   \
-  : "=r"(ready)                                                                                              \
-  : "r"(next_bar), "r"(next_parity), "r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "r"(a_bar), \
-    "r"(b_bar), "r"(release_b), "r"(do_mma), "l"(b_step)                                                     \
-  : "memory"
-  if constexpr (!PAIR) {
-    if (KSTEPS == 4) {
-      asm volatile(HGC_STAGE_HEAD HGC_MMA_FIRST("1") HGC_MMA_NEXT("1") HGC_MMA_NEXT("1") HGC_MMA_NEXT("1") HGC_COMMITS_1
-                       HGC_STAGE_TAIL HGC_STAGE_OPERANDS);
-    } else if (KSTEPS == 2) {
-      asm volatile(HGC_STAGE_HEAD HGC_MMA_FIRST("1") HGC_MMA_NEXT("1") HGC_COMMITS_1 HGC_STAGE_TAIL HGC_STAGE_OPERANDS);
-    } else {
-      asm volatile(HGC_STAGE_HEAD HGC_MMA_FIRST("1") HGC_COMMITS_1 HGC_STAGE_TAIL HGC_STAGE_OPERANDS);
-    }
-  } else {
-    if (KSTEPS == 4) {
-      asm volatile(HGC_STAGE_HEAD HGC_MMA_FIRST("2") HGC_MMA_NEXT("2") HGC_MMA_NEXT("2") HGC_MMA_NEXT("2") HGC_COMMITS_2
-                       HGC_STAGE_TAIL HGC_STAGE_OPERANDS);
-    } else if (KSTEPS == 2) {
-      asm volatile(HGC_STAGE_HEAD HGC_MMA_FIRST("2") HGC_MMA_NEXT("2") HGC_COMMITS_2 HGC_STAGE_TAIL HGC_STAGE_OPERANDS);
-    } else {
-      asm volatile(HGC_STAGE_HEAD HGC_MMA_FIRST("2") HGC_COMMITS_2 HGC_STAGE_TAIL HGC_STAGE_OPERANDS);
-    }
+__device__ __forceinline__ void issue_mmas(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
+                                           uint32_t acc, uint32_t b_step) {
+#define HGC_MMA(CG)                                                                                        \
+  asm volatile(                                                                                            \
+      "{\n.reg .pred p;\n.reg .b64 da, db;\nmov.b64 da, {%1, %2};\nmov.b64 db, {%3, %4};\n"               \
+      "setp.ne.b32 p, %6, 0;\ntcgen05.mma.cta_group::" CG ".kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d_tmem), \
+      "r"(a_lo + 2u * i), "r"(a_hi), "r"(b_lo + b_step * i), "r"(b_hi), "r"(idesc), "r"(i == 0 ? acc : 1u)  \
+      : "memory")
+#pragma unroll
+  for (uint32_t i = 0; i < (uint32_t)KSTEPS; ++i) {
+    if constexpr (PAIR) HGC_MMA("2");
+    else HGC_MMA("1");
   }
-#undef HGC_STAGE_OPERANDS
-  return ready;
-}
-
-// KSTEPS MMAs of one weight tile against one activation tile, issued by one elected lane.
-#define HGC_MMAS_HEAD                             \
-  "{\n"                                           \
-  ".reg .pred p_el, p_mma, p_acc, p_one;\n"       \
-  ".reg .b64 da, db;\n"                           \
-  "mov.b64 da, %1;\n"                             \
-  "mov.b64 db, %2;\n"                             \
-  "elect.sync _|p_el, 0xffffffff;\n"              \
-  "setp.ne.b32 p_mma, %5, 0;\n"                   \
-  "and.pred p_mma, p_mma, p_el;\n"                \
-  "setp.ne.b32 p_acc, %4, 0;\n"                   \
-  "setp.eq.b32 p_one, 0, 0;\n"
-#define HGC_MMAS_FIRST(CG) "@p_mma tcgen05.mma.cta_group::" CG ".kind::f16 [%0], %1, %2, %3, p_acc;\n"
-#define HGC_MMAS_NEXT(CG)    \
-  "add.u64 da, da, 2;\n"     \
-  "add.u64 db, db, %6;\n"    \
-  "@p_mma tcgen05.mma.cta_group::" CG ".kind::f16 [%0], da, db, %3, p_one;\n"
-template <int KSTEPS, bool PAIR>
-__device__ __forceinline__ void issue_mmas(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                           uint32_t acc, uint32_t do_mma, uint64_t b_step) {
-#define HGC_MMA_OPERANDS ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "r"(do_mma), "l"(b_step) : "memory"
-  if constexpr (!PAIR) {
-    if (KSTEPS == 4) {
-      asm volatile(HGC_MMAS_HEAD HGC_MMAS_FIRST("1") HGC_MMAS_NEXT("1") HGC_MMAS_NEXT("1") HGC_MMAS_NEXT("1") "}\n" HGC_MMA_OPERANDS);
-    } else if (KSTEPS == 2) {
-      asm volatile(HGC_MMAS_HEAD HGC_MMAS_FIRST("1") HGC_MMAS_NEXT("1") "}\n" HGC_MMA_OPERANDS);
-    } else {
-      asm volatile(HGC_MMAS_HEAD HGC_MMAS_FIRST("1") "}\n" HGC_MMA_OPERANDS);
-    }
-  } else {
-    if (KSTEPS == 4) {
-      asm volatile(HGC_MMAS_HEAD HGC_MMAS_FIRST("2") HGC_MMAS_NEXT("2") HGC_MMAS_NEXT("2") HGC_MMAS_NEXT("2") "}\n" HGC_MMA_OPERANDS);
-    } else if (KSTEPS == 2) {
-      asm volatile(HGC_MMAS_HEAD HGC_MMAS_FIRST("2") HGC_MMAS_NEXT("2") "}\n" HGC_MMA_OPERANDS);
-    } else {
-      asm volatile(HGC_MMAS_HEAD HGC_MMAS_FIRST("2") "}\n" HGC_MMA_OPERANDS);
-    }
-  }
-#undef HGC_MMA_OPERANDS
+#undef HGC_MMA
 }
 
 // Copy epilogue (every shape the TMA-store epilogue does not take: planes whose size is not a
@@ -1285,7 +1208,7 @@ constexpr int kDwWarps = 8;      // extra warps of the depthwise + pointwise ins
 
 template <int KB, bool HALO, int EW, int EPI, bool SPLIT, bool PAIR = false, bool SHARED = false, bool FUSEL = false,
           bool DWPW = false>
-__global__ void __launch_bounds__(64 + 32 * EW + (FUSEL ? 32 * kLayoutWarps : 0) + (DWPW ? 32 * kDwWarps : 0), 1)
+__global__ void __launch_bounds__(96 + 32 * EW + (FUSEL ? 32 * kLayoutWarps : 0) + (DWPW ? 32 * kDwWarps : 0), 1)
 igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
              const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmYr,
              const IgemmArgs a, const __half* __restrict__ bias, __half* __restrict__ y, float* __restrict__ partials,
@@ -1295,6 +1218,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
+  __shared__ volatile int produced_stages[2];  // stages that each producer has announced, once it has left its loop
   __shared__ __align__(8) uint64_t sk_bar;    // shared tiles: the partial sums of the unit's last tile are in its accumulator
   __shared__ __align__(8) uint64_t meet_bar;  // shared tiles: meeting point of all epilogue warps,
   __shared__ __align__(8) uint64_t ho_bar;    //   of the warps that hand accumulators over (the first of each lane quarter),
@@ -1302,7 +1226,8 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __shared__ __align__(8) uint64_t in_full[2], in_empty[2];  // depthwise input tiles (depthwise + pointwise blocks)
   __shared__ __align__(8) uint64_t q_bar[4];  // whole-plane epilogue: meeting point of the two warps of a lane quarter
 
-  const int warp = threadIdx.x >> 5;
+  // (through a shuffle: the compiler then knows that the roles' branches are taken by whole warps)
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const int lane = threadIdx.x & 31;
   // ring of stages; a stage holds one activation tile followed by `taps` weight tiles
   const uint32_t ring_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -1317,8 +1242,8 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   }
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.stages; ++s) {
-      // (the weight copy + one arrival per depthwise / gathering warp)
-      mbar_init(smem_u32(&full_bar[s]), DWPW ? 1 + kDwWarps : 1);
+      // (one announcement per producer; blocks: the weights' + one arrival per depthwise / gathering warp)
+      mbar_init(smem_u32(&full_bar[s]), DWPW ? 1 + kDwWarps : 2);
       mbar_init(smem_u32(&empty_bar[s]), 1);
     }
     for (int s = 0; s < 2; ++s) {
@@ -1335,6 +1260,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     mbar_init(smem_u32(&ho_bar), EW / 2);
     mbar_init(smem_u32(&pl_bar), EW / 2);
     abort_flag = 0;
+    produced_stages[0] = produced_stages[1] = -1;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -1358,26 +1284,28 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   // write global memory look at the status word; the producer and the MMA issuer do not wait for
   // that read (it is the first access of the kernel and would delay the first copy by a trip to
   // L2): they fill the ring and the accumulators once and leave through abort_flag.
-  const bool skip = warp >= 2 && status != nullptr && *reinterpret_cast<volatile int*>(status) != 0;
+  const bool skip = warp >= 2 && warp != 2 + EW && status != nullptr && *reinterpret_cast<volatile int*>(status) != 0;
 
   if (skip) {
     abort_flag = 1;
     // fall through to the release of the tensor memory
-  } else if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    // The whole warp walks the loop (warp-uniform control flow keeps addresses, coordinates and
-    // barrier operands in uniform registers); one elected lane issues the copies.  A stage is
-    // the activation tile of one kernel row (or one tap when taps cannot share it) plus the
-    // weight tiles of its `taps` taps, all completing on one barrier: the MMA warp then pays the
-    // barrier handshake once per taps*KB/16 MMAs.
+  } else if (warp == 0 || warp == 2 + EW) {
+    // ---------------- TMA producers: warp 0 the activation tiles, the warp after the epilogue's the weights ----
+    // A stage is the activation tile of one kernel row (or one tap when taps cannot share it) plus
+    // the weight tiles of its `taps` taps, all completing on one barrier (each producer announces
+    // its own bytes): the MMA warp then pays the barrier handshake once per taps*KB/16 MMAs.  Waiting
+    // for a stage and getting one copy under way takes a warp about 200 clocks, so the two kinds of
+    // copies have a warp each: with one warp for both, stages of four short MMAs waited for it.
+    const bool weights = warp != 0;
     Ring ring;
     uint32_t issued = 0;
     bool ok = true;
+    const bool leader = elect_one();
     const uint32_t depth = (uint32_t)a.stages;
     const int groups_per_row = a.S / a.taps;  // 1 in halo mode (taps == S), S otherwise (taps == 1)
     typename WorkIterOf<SPLIT, SHARED>::type it;
     const int stages_per_block = a.R * groups_per_row;
-    for (it.init(a); it.valid(a) && ok; it.next(a)) {
+    for (it.init(a); it.valid(a) && ok && !(DWPW && a.gather && !weights); it.next(a)) {
       int grp, m0;
       it.channel_tile(a, grp, m0);
       int n0 = it.pt * a.tn;
@@ -1391,9 +1319,9 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       it.stage_range(a, s0, s1);
       if constexpr (FUSEL) {
         // the tile reads input rows h_base .. h_base + (th-1)*stride + (R-1)*dil of tn images
-        if (!layout_wait(a.lay_flags, a.N, a.lay_hw / a.lay_w, a.lay_w, a.lay_seg_units * (32 / a.lay_ch) * a.lay_px,
-                         a.lay_seg_units, a.lay_segs, a.lay_units_p, a.lay_units_c, n0, a.tn, h_base,
-                         h_base + (a.th - 1) * a.stride_h + (a.R - 1) * a.dil_h + 1, &abort_flag)) {
+        if (!weights && !layout_wait(a.lay_flags, a.N, a.lay_hw / a.lay_w, a.lay_w, a.lay_seg_units * (32 / a.lay_ch) * a.lay_px,
+                                     a.lay_seg_units, a.lay_segs, a.lay_units_p, a.lay_units_c, n0, a.tn, h_base,
+                                     h_base + (a.th - 1) * a.stride_h + (a.R - 1) * a.dil_h + 1, &abort_flag)) {
           ok = false;
           break;
         }
@@ -1407,59 +1335,59 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       }
       int tap0 = (r * groups_per_row + sg) * a.taps;  // first tap (r*S + s) of the stage
       for (int st = s0; st < s1; ++st) {
-        if (!mbar_wait(smem_u32(&empty_bar[ring.idx]), ring.phase ^ 1u, &abort_flag, 64)) {
-          ok = false;
-          break;
-        }
-        const uint32_t sbase = ring_base + ring.idx * a.stage_bytes;
         // test hook: the first CTA announces the bytes of its `dbg_drop`-th stage but never fetches
         // them, so that the wait for that stage runs out (hgc_debug_drop_copies)
-        const bool drop = a.dbg_drop >= 0 && blockIdx.x == 0 && issued == (uint32_t)a.dbg_drop;
-        if (drop) {
-          if (lane == 0) mbar_expect_tx(smem_u32(&full_bar[ring.idx]), (PAIR ? 2u : 1u) * (a.b_bytes + (uint32_t)((DWPW ? a.nacc : 1) * a.taps) * a.a_bytes));
-        } else if constexpr (DWPW) {
+        const bool drop = weights == DWPW && a.dbg_drop >= 0 && blockIdx.x == 0 && issued == (uint32_t)a.dbg_drop;
+        if (DWPW && !weights) {
           // the activation tile of the stage is computed by the depthwise warps from an input tile
-          // (with its one-pixel border) that is fetched here, beside the pointwise weights
-          const uint32_t fb = smem_u32(&full_bar[ring.idx]);
-          // the weight tiles of the item's channel tiles (one per accumulator), behind one another
-          if (elect_one()) {
-            mbar_expect_tx(fb, (uint32_t)(a.nacc * a.taps) * a.a_bytes);
-            for (int i = 0; i < a.nacc; ++i)
-              tma_load_4d(sbase + a.b_alloc + (uint32_t)(i * a.taps) * a.a_bytes, &tmA, fb, cb * KB, m0 + i * 128, tap0, grp);
-          }
+          // (with its one-pixel border) that is fetched here
           const uint32_t ib = issued & 1u;
-          if (!a.gather && !mbar_wait(smem_u32(&in_empty[ib]), ((issued >> 1) & 1u) ^ 1u, &abort_flag, 64)) {
+          if (!mbar_wait(smem_u32(&in_empty[ib]), ((issued >> 1) & 1u) ^ 1u, &abort_flag, 64)) {
             ok = false;
             break;
           }
-          if (!a.gather && elect_one()) {
+          if (leader) {
             const uint32_t in_base = ring_base + (uint32_t)a.stages * a.stage_bytes + (uint32_t)(EW * a.nbuf) * kWarpStageBytes;
             mbar_expect_tx(smem_u32(&in_full[ib]), a.dw_in_bytes);
             tma_load_5d(in_base + ib * a.dw_in_alloc, &tmB, smem_u32(&in_full[ib]), cb * KB, 0, -1, p0 * a.dw_stride - 1, n0);
           }
-        } else if constexpr (PAIR) {
-          // both CTAs' copies are counted on the first CTA's barrier, which expects the bytes of both
-          const uint32_t fb = cluster_addr(smem_u32(&full_bar[ring.idx]), 0);
-          if (elect_one()) {
-            if (rank == 0) mbar_expect_tx(smem_u32(&full_bar[ring.idx]), 2u * (a.b_bytes + (uint32_t)a.taps * a.a_bytes));
-            tma_load_5d_pair(sbase, &tmB, fb, cb * KB, grp, (HALO ? 0 : sg * a.dil_w) - a.pad_w, h_base + r * a.dil_h, n0);
-            tma_load_4d_pair(sbase + a.b_alloc, &tmA, fb, cb * KB, m0, tap0, grp);
-          }
         } else {
-        const uint32_t fb = smem_u32(&full_bar[ring.idx]);
-        // the activation tile and the weight tiles of all taps of the stage as one box each (the 1x1
-        // mode's 64-pixel blocks: one copy per block)
-        if (elect_one()) {
-          mbar_expect_tx(fb, a.b_bytes + (uint32_t)a.taps * a.a_bytes);
-          if (a.nchw) {
-            // x itself, (pixel, channel, image): blocks of 64 pixels x KB channels, pixels contiguous
-            for (int b = 0; b < a.nblk; ++b)
-              tma_load_3d(sbase + (uint32_t)b * (uint32_t)(KB * 128), &tmB, fb, p0 * a.Q + 64 * b, grp * a.cg + cb * KB, n0);
-          } else {
-            tma_load_5d(sbase, &tmB, fb, cb * KB, grp, (HALO ? 0 : sg * a.dil_w) - a.pad_w, h_base + r * a.dil_h, n0);
+          if (!mbar_wait(smem_u32(&empty_bar[ring.idx]), ring.phase ^ 1u, &abort_flag, 64)) {
+            ok = false;
+            break;
           }
-          tma_load_4d(sbase + a.b_alloc, &tmA, fb, cb * KB, m0, tap0, grp);
-        }
+          const uint32_t sbase = ring_base + ring.idx * a.stage_bytes;
+          const uint32_t own_fb = smem_u32(&full_bar[ring.idx]);
+          // a pair: both CTAs' copies are counted on the first CTA's barrier, which expects the bytes of both
+          const uint32_t fb = PAIR ? cluster_addr(own_fb, 0) : own_fb;
+          if (weights) {
+            // the weight tiles of all taps of the stage as one box (blocks: of the item's channel
+            // tiles, one per accumulator, behind one another)
+            if (leader) {
+              const uint32_t bytes = (uint32_t)((DWPW ? a.nacc : 1) * a.taps) * a.a_bytes;
+              if (!PAIR || rank == 0) mbar_expect_tx(own_fb, (PAIR ? 2u : 1u) * bytes);
+              if (!drop) {
+                if constexpr (PAIR) {
+                  tma_load_4d_pair(sbase + a.b_alloc, &tmA, fb, cb * KB, m0, tap0, grp);
+                } else {
+                  for (int i = 0; i < (DWPW ? a.nacc : 1); ++i)
+                    tma_load_4d(sbase + a.b_alloc + (uint32_t)(i * a.taps) * a.a_bytes, &tmA, fb, cb * KB, m0 + i * 128, tap0, grp);
+                }
+              }
+            }
+          } else if (leader) {
+            if (!PAIR || rank == 0) mbar_expect_tx(own_fb, (PAIR ? 2u : 1u) * a.b_bytes);
+            if (drop) {
+            } else if (PAIR) {
+              tma_load_5d_pair(sbase, &tmB, fb, cb * KB, grp, (HALO ? 0 : sg * a.dil_w) - a.pad_w, h_base + r * a.dil_h, n0);
+            } else if (a.nchw) {
+              // x itself, (pixel, channel, image): blocks of 64 pixels x KB channels, pixels contiguous
+              for (int b = 0; b < a.nblk; ++b)
+                tma_load_3d(sbase + (uint32_t)b * (uint32_t)(KB * 128), &tmB, fb, p0 * a.Q + 64 * b, grp * a.cg + cb * KB, n0);
+            } else {
+              tma_load_5d(sbase, &tmB, fb, cb * KB, grp, (HALO ? 0 : sg * a.dil_w) - a.pad_w, h_base + r * a.dil_h, n0);
+            }
+          }
         }
         __syncwarp();
         tap0 += a.taps;
@@ -1475,15 +1403,31 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         ++issued;
       }
     }
+    if (lane == 0) produced_stages[weights ? 1 : 0] = (int)issued;
     if (PAIR && rank != 0) {
       // (its copies are counted on the partner's barriers: after giving up it just waits a while)
       if (abort_flag && lane == 0) {
         const uint64_t t0 = global_timer_ns();
         while (global_timer_ns() - t0 < 2000000ull) __nanosleep(1000);
       }
+    } else if (abort_flag && lane == 0 && DWPW && !weights) {
+      for (uint32_t it = issued > 2 ? issued - 2 : 0; it < issued; ++it) {
+        const uint64_t t0 = global_timer_ns();
+        while (!mbar_try_wait(smem_u32(&in_full[it & 1u]), (it >> 1) & 1u)) {
+          if (global_timer_ns() - t0 > g_wait_limit_ns) break;
+        }
+      }
     } else if (abort_flag && lane == 0) {
-      // let the copies that were issued land before the CTA's shared memory goes away
+      // let the copies that were issued land before the CTA's shared memory goes away.  The other
+      // producer may have given up some stages earlier: its arrivals on those are made up for
+      // (otherwise their barriers would never complete).
       const uint32_t first = issued > depth ? issued - depth : 0;
+      if (!DWPW) {
+        const uint64_t t0 = global_timer_ns();
+        int other;
+        while ((other = produced_stages[weights ? 0 : 1]) < 0 && global_timer_ns() - t0 < g_wait_limit_ns) __nanosleep(200);
+        for (uint32_t it = other > (int)first ? (uint32_t)other : first; other >= 0 && it < issued; ++it) mbar_arrive(smem_u32(&full_bar[it % depth]));
+      }
       for (uint32_t it = first; it < issued; ++it) {
         const uint32_t bar = smem_u32(&full_bar[it % depth]);
         const uint64_t t0 = global_timer_ns();
@@ -1504,10 +1448,11 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     constexpr uint32_t row_bytes = (uint32_t)KB * 2u;
     const uint32_t depth = (uint32_t)a.stages;
     const uint32_t tap_step = (uint32_t)a.dil_w * row_bytes;  // halo mode: tap s starts s*dil pixels in
-    const uint64_t desc_hi = a.desc_hi;
+    const uint32_t a_hi = (uint32_t)(a.desc_hi >> 32), b_hi = (uint32_t)(a.desc_hi_b >> 32);
+    const uint32_t a_fix = (uint32_t)a.desc_hi, b_fix = (uint32_t)a.desc_hi_b;  // (bits 16..29: leading offset)
+    const uint32_t b_step = (uint32_t)a.b_kstep;
     const uint32_t idesc = a.idesc;
-    const uint32_t do_mma = 1u;
-    uint32_t ready = mbar_test_wait(smem_u32(&full_bar[0]), 0u);
+    bool ready = mbar_test_warp(smem_u32(&full_bar[0]), 0u);
     typename WorkIterOf<SPLIT, SHARED>::type it;
     for (it.init(a); it.valid(a) && ok; it.next(a), ++lt) {  // only the number of stages of an item matters here
       int s0, s1;
@@ -1518,10 +1463,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       const bool one_set = DWPW && a.nacc > 1;
       const uint32_t buf = one_set ? 0u : (lt & 1u);
       // the epilogue must have drained this accumulator (two tiles ago)
-      if (!mbar_wait(smem_u32(&acc_empty[buf]), ((one_set ? lt : (lt >> 1)) & 1u) ^ 1u, &abort_flag, 64)) {
-        ok = false;
-        break;
-      }
+      if (!mbar_wait_warp(smem_u32(&acc_empty[buf]), ((one_set ? lt : (lt >> 1)) & 1u) ^ 1u, &abort_flag)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t d_tmem = tmem_base + buf * 256u;
       uint32_t acc = 0;
@@ -1529,55 +1471,53 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         if (it.kind(a) == 2) {
           // the first part of a tile whose later parts other units computed: the epilogue warps
           // have put the sum of those parts into the accumulator (see there); add to it
-          if (!mbar_wait(smem_u32(&sk_bar), 0u, &abort_flag, 64)) {
-            ok = false;
-            break;
-          }
+          if (!mbar_wait_warp(smem_u32(&sk_bar), 0u, &abort_flag)) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           acc = 1;
         }
       }
       for (int gi = 0; gi < groups_per_tile; ++gi) {
-        if (!ready && !mbar_wait(smem_u32(&full_bar[ring.idx]), ring.phase, &abort_flag)) {
+        if (!ready && !mbar_wait_warp(smem_u32(&full_bar[ring.idx]), ring.phase, &abort_flag)) {
           ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t sbase = ring_base + ring.idx * a.stage_bytes;
         const uint32_t e_bar = smem_u32(&empty_bar[ring.idx]);
-        uint64_t bdesc = a.desc_hi_b | (uint64_t)((sbase & 0x3FFFFu) >> 4);
-        uint64_t adesc = desc_hi | (uint64_t)(((sbase + a.b_alloc) & 0x3FFFFu) >> 4);
+        uint32_t b_lo = b_fix | ((sbase & 0x3FFFFu) >> 4);
+        uint32_t a_lo = a_fix | (((sbase + a.b_alloc) & 0x3FFFFu) >> 4);
         ring.advance(depth);
-        if constexpr (DWPW) {
-          // further channel tiles of the item: the same activation tile against their weight tiles
-          for (int ci = 0; ci + 1 < a.nacc; ++ci) {
-            issue_mmas<ksteps, PAIR>(d_tmem + (uint32_t)(ci * a.acc_stride), adesc, bdesc, idesc, acc, do_mma, a.b_kstep);
-            adesc += (uint64_t)(((uint32_t)a.taps * a.a_bytes) >> 4);
+        if (elect_one()) {
+          if constexpr (DWPW) {
+            // the channel tiles of the item: the same activation tile against their weight tiles
+            for (int ci = 0; ci < a.nacc; ++ci) {
+              issue_mmas<ksteps, PAIR>(d_tmem + (uint32_t)(ci * a.acc_stride), a_lo, a_hi, b_lo, b_hi, idesc, acc, b_step);
+              a_lo += ((uint32_t)a.taps * a.a_bytes) >> 4;
+            }
+          } else {
+            issue_mmas<ksteps, PAIR>(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, acc, b_step);
+            for (int t = 1; t < a.taps; ++t) {
+              a_lo += a.a_bytes >> 4;
+              b_lo += tap_step >> 4;
+              issue_mmas<ksteps, PAIR>(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, 1u, b_step);
+            }
           }
+          if constexpr (PAIR) umma_commit_pair(e_bar);
+          else umma_commit(e_bar);
         }
-        const uint32_t d_last = DWPW ? d_tmem + (uint32_t)((a.nacc - 1) * a.acc_stride) : d_tmem;
-        // all taps but the last: MMAs only
-        for (int t = 0; t + 1 < a.taps; ++t) {
-          issue_mmas<ksteps, PAIR>(d_last, adesc, bdesc, idesc, acc, do_mma, a.b_kstep);
-          acc = 1;
-          adesc += (uint64_t)(a.a_bytes >> 4);
-          bdesc += (uint64_t)(tap_step >> 4);
-        }
-        // last tap: poll the NEXT stage's barrier first and read the answer after the MMAs and the
-        // commit have been issued, so that the poll's latency hides behind them
-        ready = issue_stage<ksteps, PAIR>(smem_u32(&full_bar[ring.idx]), ring.phase, d_last, adesc, bdesc, idesc, acc, e_bar,
-                                    e_bar, 0u, do_mma, a.b_kstep);
+        __syncwarp();
         acc = 1;
+        ready = mbar_test_warp(smem_u32(&full_bar[ring.idx]), ring.phase);
       }
-      if (ok) {
-        if (elect_one()) {  // accumulator complete
+      if (ok) {  // accumulator complete
+        if (elect_one()) {
           if constexpr (PAIR) umma_commit_pair(smem_u32(&acc_full[buf]));
           else umma_commit(smem_u32(&acc_full[buf]));
         }
         __syncwarp();
       }
     }
-  } else if (DWPW && warp >= 2 + EW) {
+  } else if (DWPW && warp >= 3 + EW) {
     // ---------------- depthwise warps: compute the activation tiles of the 1x1 layer ----------------
     // A stage holds [pixel of the tile][KB channels], 16-byte chunks of 8 channels swizzled by the
     // pixel row as the copy engine would have written them.  The input tile of the stage lies in
@@ -1587,7 +1527,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     // threads of a warp read consecutive chunks: no bank conflicts.
     constexpr int CPR = KB / 8;                     // chunks per pixel
     constexpr int PASS = kDwWarps * 32 / CPR;       // pairs per pass of the 256 threads
-    const int dt = (warp - 2 - EW) * 32 + lane;
+    const int dt = (warp - 3 - EW) * 32 + lane;
     const int chunk = dt % CPR;
     const int slot = dt / CPR;
     Ring ring;
@@ -1729,9 +1669,9 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         ring.advance(depth);
       }
     }
-  } else if (FUSEL && warp >= 2 + EW) {
+  } else if (FUSEL && warp >= 3 + EW) {
     // ---------------- fused layout pass (warps past the epilogue's) ----------------
-    const int64_t gw = (int64_t)blockIdx.x * kLayoutWarps + (warp - 2 - EW);
+    const int64_t gw = (int64_t)blockIdx.x * kLayoutWarps + (warp - 3 - EW);
     const int64_t nw = (int64_t)gridDim.x * kLayoutWarps;
     if (a.lay_ch == 8 && a.lay_px == 8)
       layout_warp_loop<8, 8>(a.lay_x, a.lay_xp, a.lay_c, a.lay_hw, a.lay_cpad, a.lay_units_p, a.lay_units_c, a.lay_seg_units,
@@ -3129,7 +3069,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   do {                                                                                                     \
     err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, EWV, EPIV, SPLITV>>();            \
     if (err == cudaSuccess)                                                                                \
-      err = launch_kernel_overlapped(igemm_kernel<KBV, HALOV, EWV, EPIV, SPLITV>, grid, dim3(64 + 32 * EWV), \
+      err = launch_kernel_overlapped(igemm_kernel<KBV, HALOV, EWV, EPIV, SPLITV>, grid, dim3(96 + 32 * EWV), \
                           p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \
   } while (0)
   // depthwise + pointwise block: its own instantiations (8 epilogue + 8 depthwise warps)
@@ -3138,7 +3078,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     err = allow_dynamic_smem<igemm_kernel<KBV, true, 8, EPIV, false, false, false, false, true>>();            \
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_overlapped(igemm_kernel<KBV, true, 8, EPIV, false, false, false, false, true>, grid, \
-                          dim3(64 + 32 * 8 + 32 * kDwWarps), p.smem_bytes, stream, p.tmA, p.tmB, p.tmY,    \
+                          dim3(96 + 32 * 8 + 32 * kDwWarps), p.smem_bytes, stream, p.tmA, p.tmB, p.tmY,    \
                           p.tmYr, a, bias, y, partials, status);                                           \
   } while (0)
 #define HGC_LAUNCH_DWPW(KBV)                                   \
@@ -3155,7 +3095,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, false, false, false, true>>();            \
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_coop(true, igemm_kernel<KBV, HALOV, 8, EPIV, false, false, false, true>, grid,   \
-                               dim3(64 + 32 * 8 + 32 * kLayoutWarps), p.smem_bytes, stream, p.tmA, p.tmB,  \
+                               dim3(96 + 32 * 8 + 32 * kLayoutWarps), p.smem_bytes, stream, p.tmA, p.tmB,  \
                                p.tmY, p.tmYr, a, bias, y, partials, status);                               \
   } while (0)
 #define HGC_LAUNCH_FUSED(KBV, HALOV) HGC_LAUNCH_FUSED_EPI(KBV, HALOV, 0)
@@ -3165,7 +3105,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, false, false, true>>();            \
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_coop(true, igemm_kernel<KBV, HALOV, 8, EPIV, false, false, true>, grid,          \
-                               dim3(64 + 32 * 8), p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a,    \
+                               dim3(96 + 32 * 8), p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a,    \
                                bias, y, partials, status);                                                 \
   } while (0)
 #define HGC_LAUNCH_SHARED(KBV, HALOV)                                \
@@ -3190,12 +3130,12 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
       err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, false, true, true>>();            \
       if (err == cudaSuccess)                                                                                \
         err = launch_pair(igemm_kernel<KBV, HALOV, 8, EPIV, false, true, true>, p, sms, true,                \
-                          dim3(64 + 32 * 8), stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \
+                          dim3(96 + 32 * 8), stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \
     } else {                                                                                                 \
       err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, false, true, false>>();            \
       if (err == cudaSuccess)                                                                                \
         err = launch_pair(igemm_kernel<KBV, HALOV, 8, EPIV, false, true, false>, p, sms, false,              \
-                          dim3(64 + 32 * 8), stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \
+                          dim3(96 + 32 * 8), stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \
     }                                                                                                        \
   } while (0)
 #define HGC_LAUNCH_PAIR(KBV, HALOV)                                \
