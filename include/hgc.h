@@ -327,7 +327,7 @@ int hgc_cast_f32_to_f16(const void* src, void* dst, int64_t count, uint64_t* ove
  * irrelevant before, undefined after).  use_stored != 0: mean and var are READ (stored
  * statistics, e.g. a trained model's), workspace may be NULL.  No scale/shift parameters: Caffe
  * keeps them in a separate layer (see hgc_bn_fold for inference).
- * x, y: device pointers, 16-byte aligned, not overlapping.  Queued on `stream` (three kernels, or
+ * x, y: device pointers, 16-byte aligned, not overlapping.  Queued on `stream` (two kernels, or
  * one with stored statistics); nothing is allocated, nothing synchronises.
  * Errors: HGC_INVALID_ARG (NULL pointers, n/c/hw < 1, eps < 0, shift out of range),
  * HGC_UNSUPPORTED (c > 65535 or more than 2^31-1 groups), HGC_BAD_ALIGNMENT, HGC_NO_WORKSPACE
