@@ -42,13 +42,20 @@ int debug_drop_copies();
 cudaError_t igemm_set_wait_limit_ns(uint64_t ns);
 cudaError_t depthwise_nhwc_tma_set_wait_limit_ns(uint64_t ns);
 
-// Programmatic dependent launch: a kernel launched with this helper may be scheduled while the
+// Programmatic dependent launch: a kernel launched with the attribute may be scheduled while the
 // kernel before it in the stream is still draining; every kernel of this library therefore
 // executes grid_dependency_wait() before its first access to global memory (it returns when the
 // preceding kernel has completed and its writes are visible; a no-op for a kernel launched
-// without the attribute), so only launch latency and on-chip set-up overlap.  Off by default
-// (hgc_set_launch_overlap): it helps eager launches by a few per cent and slows a step replayed
-// as a CUDA graph down.
+// without the attribute), so only launch latency and on-chip set-up overlap.
+// Which kernels: the tensor-core kernels always (below), the copy, depthwise and element-wise
+// kernels when their grid is at most two blocks of 256 threads per SM.  Such a short kernel is mostly
+// launch latency, and the launch itself costs the host less (1.7 against 2.0 us).  Larger ones lose:
+// blocks that move in beside a tensor-core CTA find its carve-out of shared memory and a small
+// L1, and keep the SM in it.  Measured, limit in threads 0 / 38k / 76k / 152k / none: MobileNet at batch
+// 32 as a graph 272 / 272 / 264 / 292 / 294 us, ResNet-50 at batch 64 1039 / 1041 / 1038 / 1072 / 1115,
+// VGG-16 at batch 1, eager, 195 / 187 / 188 / 184 / 184, preparing 49 layers' weights 658 / 503 / 483 / 497.
+// hgc_set_launch_overlap lifts the limit.
+constexpr int64_t kOverlapThreads = 148 * 512;
 bool launch_overlap_enabled();
 void set_launch_overlap(bool on);
 
@@ -70,7 +77,8 @@ inline cudaError_t launch_kernel_attr(bool overlap, void (*kernel)(KArgs...), di
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                  Args... args) {
-  return launch_kernel_attr(launch_overlap_enabled(), kernel, grid, block, smem, stream, args...);
+  const bool small = (int64_t)grid.x * grid.y * grid.z * block.x <= kOverlapThreads;
+  return launch_kernel_attr(small || launch_overlap_enabled(), kernel, grid, block, smem, stream, args...);
 }
 // The persistent tensor-core kernel is always launched with the attribute: its set-up (barriers,
 // tensor memory) then overlaps the tail of the kernel before it, and where one tensor-core kernel
@@ -126,12 +134,13 @@ cudaError_t allow_dynamic_smem() {
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the stream, if it was launched with the attribute (the tensor-core
 // kernels always are), be scheduled as soon as EVERY CTA of this grid has called this or exited.
-// The persistent tensor-core kernel calls it at its start: its CTAs hold a whole SM, so the next
-// kernel's CTAs start exactly where one of them has finished.  The many-block copy and depthwise
-// kernels call it at their start too: the condition is met only when their last blocks are
+// The persistent tensor-core kernel calls it when a CTA's last copy is under way: blocks of a short
+// copy kernel then move in at its tail, not at its start, and the CTAs of a following tensor-core
+// kernel, which need a whole SM, start where one has finished (ResNet-50 at batch 64 as a graph:
+// 1040 us with the call at the start, 1021 with it here).  The copy and depthwise kernels call it at
+// their start: the condition is met only when their last blocks are
 // running, so the CTAs of a following tensor-core kernel take SMs that have no more blocks to
-// wait for and set themselves up (barriers, tensor memory) beside the last wave.  Measured, NCHW
-// steps as CUDA graphs: VGG-16 0.596 -> 0.589 ms, ResNet-50 1.287 -> 1.263, MobileNet 0.327 -> 0.321.
+// wait for and set themselves up (barriers, tensor memory) beside the last wave.
 __device__ __forceinline__ void grid_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

@@ -1279,7 +1279,6 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   // everything above touched only this CTA's shared and tensor memory and may overlap the tail of
   // the previous kernel in the stream; from here on global memory is read and written
   grid_dependency_wait();
-  grid_launch_dependents();
   // An earlier CTA gave up: do not start new work on a path that is not progressing.  The warps that
   // write global memory look at the status word; the producer and the MMA issuer do not wait for
   // that read (it is the first access of the kernel and would delay the first copy by a trip to
@@ -1403,6 +1402,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         ++issued;
       }
     }
+    if (!weights) grid_launch_dependents();  // this CTA's last copy is under way: the next kernel may set itself up
     if (lane == 0) produced_stages[weights ? 1 : 0] = (int)issued;
     if (PAIR && rank != 0) {
       // (its copies are counted on the partner's barriers: after giving up it just waits a while)
