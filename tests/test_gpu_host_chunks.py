@@ -1,0 +1,63 @@
+"""hgc_conv_forward_host with enough images to be cut into chunks (copies in, kernels and copies out on
+streams of their own): results against the oracle for chunks that do and do not divide the batch,
+for planes whose bytes are not a multiple of the staging alignment, on the paths that read x in
+place, through a layout pass and without tensor cores."""
+import numpy as np
+import pytest
+
+from paper_1901_00858_b200 import workloads
+from gpu_util import check_close, params_dict, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def hgc():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_1901_00858_b200 import binding
+    binding.lib()
+    return binding
+
+
+# (name, layer): 2 MB of x and of y per chunk at least
+CASES = [
+    ("3x3, five images in chunks of two and a last one of one", params_dict(5, 32, 149, 151, 32, 3, 3, 1, 1)),
+    ("1x1 read in place, chunks of one", params_dict(3, 128, 96, 96, 128, 1, 1)),
+    ("depthwise, four chunks", params_dict(10, 24, 160, 160, 24, 3, 3, 1, 1, 1, 1, 1, 1, 24)),
+    ("grouped, generic kernel", params_dict(4, 63, 131, 127, 63, 3, 3, 1, 1, 1, 1, 1, 1, 3)),
+    ("below two chunks: one piece", params_dict(3, 16, 100, 100, 16, 3, 3, 1, 1)),
+]
+
+
+@pytest.mark.parametrize("name,a", CASES, ids=[c[0] for c in CASES])
+def test_host_forward_in_chunks(hgc, oracle, name, a):
+    import torch
+    d = hgc.ConvDesc(**a)
+    d.ensure_workspace(host=True)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    shape = d.output_dims()
+    calls = []
+    for i in range(4):   # new tensors on every call, alternating streams; nothing waits in between
+        rng = np.random.default_rng(70 + i)
+        x, w, b = workloads.random_layer_tensors(rng, a["n"], a["c"], a["h"], a["w"], a["k"], a["r"], a["s"], a["group"])
+        bias = b if i % 2 == 0 else None
+        pin = lambda t: None if t is None else torch.from_numpy(t.view(np.int16)).pin_memory()
+        xh, wh, bh = pin(x), pin(w), pin(bias)
+        yh = torch.full(shape, 0x7e00, dtype=torch.int16).pin_memory()   # binary16 NaN
+        if i > 0:
+            streams[i % 2].wait_stream(streams[(i - 1) % 2])
+        hgc.conv_forward_host(d, xh, wh, bh, yh, True, streams[i % 2])
+        calls.append((x, w, bias, xh, wh, bh, yh))
+    streams[1].synchronize()
+    assert d.last_device_status() == hgc.HGC_OK
+    for x, w, bias, _, _, _, yh in calls:
+        ref = oracle.conv_fast(oracle.ConvParams(**a), x, w, bias, True)
+        check_close(yh.numpy().view(np.float16), ref, what=name)
+    # the descriptor still serves device tensors from the same workspace
+    x, w, bias = calls[0][:3]
+    y = torch.empty(shape, dtype=torch.float16, device="cuda")
+    hgc.conv_forward(d, to_dev(x), to_dev(w), to_dev(bias), y, True)
+    torch.cuda.synchronize()
+    check_close(to_host(y), oracle.conv_fast(oracle.ConvParams(**a), x, w, bias, True), what=name + " (device)")
+    d.close()
