@@ -429,12 +429,11 @@ int hgc_debug_shrink_ranges(int64_t bytes);
  * tensor-core kernel follows another its CTAs start as the previous kernel's leave.  Results are
  * the same either way.  Measured on B200, steps replayed as CUDA graphs: ResNet-50 channels-last
  * 1.065 -> 1.018 ms, MobileNet channels-last 0.332 -> 0.321 ms, NCHW steps unchanged.
- * So are the other kernels when their grid is small (at most two blocks of 256 threads per SM).
- * With enabled != 0 EVERY kernel of the library is launched that way (off by default): with
- * eager launches the gap between dependent kernels shrinks (a VGG-16 step 0.776 -> 0.757 ms,
- * ResNet-50 1.76 -> 1.69 ms), but a step replayed as a CUDA graph gets slower when layout passes
- * sit between the tensor-core kernels (NCHW VGG-16 layers: 0.605 -> 0.696 ms), which is why it
- * is off unless asked for (`python bench.py --launch-overlap` repeats the measurement).
+ * So are the other kernels of eager launches, and in captured graphs those of a small grid (at most two
+ * blocks of 256 threads per SM).
+ * With enabled != 0 the others are launched that way in graphs too (off by default: a captured step
+ * gets slower when large layout passes sit between the tensor-core kernels, MobileNet at batch 32
+ * 272 -> 281 us; `python bench.py --launch-overlap` repeats the measurement).
  * Applies to all later launches of this process.
  * Always returns HGC_OK.
  */

@@ -281,7 +281,7 @@ cudaError_t launch_batchnorm(const __half* x, __half* y, int32_t n, int32_t c, i
     if (err != cudaSuccess) return err;
     count_launch();
   }
-  err = launch_kernel_attr(!use_stored || launch_overlap_enabled(), small ? bn_apply_kernel<8> : bn_apply_kernel<32>, grid,
+  err = launch_kernel_attr(true, kCopyKernelCarveout, small ? bn_apply_kernel<8> : bn_apply_kernel<32>, grid,
                            dim3(kBnThreads), 0, stream, x16, reinterpret_cast<uint16_t*>(y), (const float2*)stats, mean, var,
                            (int)use_stored, (int)n, (int)c, hw, chunks, eps, shift);
   if (err != cudaSuccess) return err;

@@ -47,38 +47,54 @@ cudaError_t depthwise_nhwc_tma_set_wait_limit_ns(uint64_t ns);
 // executes grid_dependency_wait() before its first access to global memory (it returns when the
 // preceding kernel has completed and its writes are visible; a no-op for a kernel launched
 // without the attribute), so only launch latency and on-chip set-up overlap.
-// Which kernels: the tensor-core kernels always (below), the copy, depthwise and element-wise
-// kernels when their grid is at most two blocks of 256 threads per SM.  Such a short kernel is mostly
-// launch latency, and the launch itself costs the host less (1.7 against 2.0 us).  Larger ones lose:
-// blocks that move in beside a tensor-core CTA find its carve-out of shared memory and a small
-// L1, and keep the SM in it.  Measured, limit in threads 0 / 38k / 76k / 152k / none: MobileNet at batch
-// 32 as a graph 272 / 272 / 264 / 292 / 294 us, ResNet-50 at batch 64 1039 / 1041 / 1038 / 1072 / 1115,
-// VGG-16 at batch 1, eager, 195 / 187 / 188 / 184 / 184, preparing 49 layers' weights 658 / 503 / 483 / 497.
-// hgc_set_launch_overlap lifts the limit.
+// Which kernels: the tensor-core kernels always (below); the copy, depthwise and element-wise kernels
+// when the launch is not being captured or their grid is at most two blocks of 256 threads per SM (or
+// hgc_set_launch_overlap asks for all).  In a graph, launches follow one another closely without it.
+// These kernels also ask for a quarter of the SM's memory as shared memory, although few of them use
+// any: an SM can only change its split while it is idle, so blocks that move in beside a
+// tensor-core CTA find its split and the little L1 that is left, and with their default (all L1) the
+// SMs change over between every two kernels.  Measured, limit of two blocks per SM or none x
+// split as it comes or a quarter, eager: MobileNet at batch 32 304 / 302 / 305 / 293 us, ResNet-50 at
+// batch 64 1111 / 1115 / 1144 / 1075, VGG-16 at batch 16 628 / 629 / 636 / 620, at batch 1 188 / 188 / 184 / 183;
+// as graphs MobileNet 272 / 271 / 294 / 281, ResNet-50 1036 / 1040 / 1112 / 1042.  (All shared memory or
+// none: 3 to 6 % slower.)
 constexpr int64_t kOverlapThreads = 148 * 512;
+constexpr unsigned kCopyKernelCarveout = 25;  // per cent
 bool launch_overlap_enabled();
 void set_launch_overlap(bool on);
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_kernel_attr(bool overlap, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+inline cudaError_t launch_kernel_attr(bool overlap, unsigned carveout, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                       cudaStream_t stream, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  unsigned n = 0;
+  if (overlap) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (carveout != 0) {
+    attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[n++].val.sharedMemCarveout = carveout;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = overlap ? 1 : 0;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                  Args... args) {
   const bool small = (int64_t)grid.x * grid.y * grid.z * block.x <= kOverlapThreads;
-  return launch_kernel_attr(small || launch_overlap_enabled(), kernel, grid, block, smem, stream, args...);
+  bool overlap = small || launch_overlap_enabled();
+  if (!overlap) {
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    overlap = cudaStreamIsCapturing(stream, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone;
+  }
+  return launch_kernel_attr(overlap, kCopyKernelCarveout, kernel, grid, block, smem, stream, args...);
 }
 // The persistent tensor-core kernel is always launched with the attribute: its set-up (barriers,
 // tensor memory) then overlaps the tail of the kernel before it, and where one tensor-core kernel
@@ -89,7 +105,7 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                             cudaStream_t stream, Args... args) {
-  return launch_kernel_attr(true, kernel, grid, block, smem, stream, args...);
+  return launch_kernel_attr(true, 0, kernel, grid, block, smem, stream, args...);
 }
 
 // The same with the cooperative attribute when `cooperative` is set: the launch waits until every
