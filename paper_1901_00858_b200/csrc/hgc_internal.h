@@ -349,6 +349,7 @@ struct IgemmPlan {
   // depthwise + pointwise block: the depthwise layer's input tile in shared memory
   int32_t dw_in_h, dw_in_w;
   uint32_t dw_in_bytes, dw_in_alloc;
+  int32_t dw_teams_log2;   // depthwise warps form 1, 2 or 4 teams
   int32_t pair, ncols_sub, pair_fit;
   double est_clk;  // the cost model's estimate for the launch, in SM clocks
   size_t ws_status_off, ws_w_off, ws_x_off, ws_part_off, ws_sk_off, ws_total;

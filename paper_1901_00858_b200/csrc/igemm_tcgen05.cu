@@ -874,6 +874,7 @@ struct IgemmArgs {
   // out-of-bounds fill) alternate between two buffers behind the epilogue's staging tiles
   int32_t dw_in_h, dw_in_w;
   uint32_t dw_in_bytes, dw_in_alloc;
+  int32_t dw_teams_log2;  // log2 of the teams that the depthwise warps form: team t computes every stage s with s % teams == t
   int32_t dbg_drop;     // test hook: stage of the first CTA whose copies are left out (-1: none)
   int32_t ts;           // ring stages per tile: cblocks * R * (S / taps)
   // CTA pairs (clusters of two, tcgen05 cta_group::2): a tile is 256 output channels x two pixel
@@ -1205,6 +1206,7 @@ __device__ __noinline__ uint32_t epilogue_planes(uint32_t t_addr, uint32_t qstag
 
 constexpr int kLayoutWarps = 8;  // extra warps of the instantiations with the fused layout pass
 constexpr int kDwWarps = 8;      // extra warps of the depthwise + pointwise instantiations
+constexpr int kMaxDwTeams = 4;   // (and two input tiles per team)
 
 template <int KB, bool HALO, int EW, int EPI, bool SPLIT, bool PAIR = false, bool SHARED = false, bool FUSEL = false,
           bool DWPW = false>
@@ -1223,7 +1225,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __shared__ __align__(8) uint64_t meet_bar;  // shared tiles: meeting point of all epilogue warps,
   __shared__ __align__(8) uint64_t ho_bar;    //   of the warps that hand accumulators over (the first of each lane quarter),
   __shared__ __align__(8) uint64_t pl_bar;    //   of the warps that fetch partial sums (the second of each lane quarter)
-  __shared__ __align__(8) uint64_t in_full[2], in_empty[2];  // depthwise input tiles (depthwise + pointwise blocks)
+  __shared__ __align__(8) uint64_t in_full[2 * kMaxDwTeams], in_empty[2 * kMaxDwTeams];  // depthwise input tiles (depthwise + pointwise blocks)
   __shared__ __align__(8) uint64_t q_bar[4];  // whole-plane epilogue: meeting point of the two warps of a lane quarter
 
   // (through a shuffle: the compiler then knows that the roles' branches are taken by whole warps)
@@ -1243,16 +1245,16 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.stages; ++s) {
       // (one announcement per producer; blocks: the weights' + one arrival per depthwise / gathering warp)
-      mbar_init(smem_u32(&full_bar[s]), DWPW ? 1 + kDwWarps : 2);
+      mbar_init(smem_u32(&full_bar[s]), DWPW ? 1 + (kDwWarps >> a.dw_teams_log2) : 2);
       mbar_init(smem_u32(&empty_bar[s]), 1);
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(smem_u32(&acc_full[s]), 1);
       mbar_init(smem_u32(&acc_empty[s]), PAIR ? 2 * EW : EW);  // one arrival per epilogue warp (of both CTAs)
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < 2 * kMaxDwTeams; ++b) {
       mbar_init(smem_u32(&in_full[b]), 1);
-      mbar_init(smem_u32(&in_empty[b]), kDwWarps);
+      mbar_init(smem_u32(&in_empty[b]), kDwWarps >> a.dw_teams_log2);
     }
     mbar_init(smem_u32(&sk_bar), PAIR ? EW : EW / 2);  // one arrival per fetching warp (of both CTAs)
     for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&q_bar[q]), EW / 4);
@@ -1340,8 +1342,8 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         if (DWPW && !weights) {
           // the activation tile of the stage is computed by the depthwise warps from an input tile
           // (with its one-pixel border) that is fetched here
-          const uint32_t ib = issued & 1u;
-          if (!mbar_wait(smem_u32(&in_empty[ib]), ((issued >> 1) & 1u) ^ 1u, &abort_flag, 64)) {
+          const uint32_t ib = issued & ((2u << a.dw_teams_log2) - 1u);  // two input tiles per team
+          if (!mbar_wait(smem_u32(&in_empty[ib]), ((issued >> (1 + a.dw_teams_log2)) & 1u) ^ 1u, &abort_flag, 64)) {
             ok = false;
             break;
           }
@@ -1411,9 +1413,10 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         while (global_timer_ns() - t0 < 2000000ull) __nanosleep(1000);
       }
     } else if (abort_flag && lane == 0 && DWPW && !weights) {
-      for (uint32_t it = issued > 2 ? issued - 2 : 0; it < issued; ++it) {
+      const uint32_t bufs = 2u << a.dw_teams_log2;
+      for (uint32_t it = issued > bufs ? issued - bufs : 0; it < issued; ++it) {
         const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(smem_u32(&in_full[it & 1u]), (it >> 1) & 1u)) {
+        while (!mbar_try_wait(smem_u32(&in_full[it & (bufs - 1u)]), (it >> (1 + a.dw_teams_log2)) & 1u)) {
           if (global_timer_ns() - t0 > g_wait_limit_ns) break;
         }
       }
@@ -1524,10 +1527,15 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     // shared memory as [image][row][column][KB] with a zero border.  Thread dt owns chunk
     // dt % (KB/8) of every (256 / (KB/8))-th pair of horizontally adjacent output pixels: the pair
     // shares its input columns (3 rows x 4 or 5 columns of 16 bytes for two outputs), and the
-    // threads of a warp read consecutive chunks: no bank conflicts.
+    // threads of a warp read consecutive chunks: no bank conflicts.  A stage of a small tile has
+    // fewer pairs than the 256 threads could take and is one trip through the latencies of
+    // its waits, loads and stores: there the warps form two or four teams that take the stages in turn.
     constexpr int CPR = KB / 8;                     // chunks per pixel
-    constexpr int PASS = kDwWarps * 32 / CPR;       // pairs per pass of the 256 threads
-    const int dt = (warp - 3 - EW) * 32 + lane;
+    const int team_warps = kDwWarps >> a.dw_teams_log2;
+    const uint32_t team = (uint32_t)(warp - 3 - EW) / (uint32_t)team_warps;
+    const uint32_t other_teams = (1u << a.dw_teams_log2) - 1u;
+    const int PASS = team_warps * 32 / CPR;         // pairs per pass of the team's threads
+    const int dt = ((warp - 3 - EW) & (team_warps - 1)) * 32 + lane;
     const int chunk = dt % CPR;
     const int slot = dt / CPR;
     Ring ring;
@@ -1604,6 +1612,10 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     } else
     for (it.init(a); it.valid(a) && ok; it.next(a)) {
       for (int cb = 0; cb < a.cblocks && ok; ++cb, ++produced) {
+        if ((produced & other_teams) != team) {
+          ring.advance(depth);
+          continue;
+        }
         const int c0 = cb * KB + chunk * 8;
         const bool cvalid = c0 < a.dw_c;            // (dw_c is a multiple of 8)
         // this thread's 8 channels: the nine taps' weights (packed pairs) and the bias
@@ -1623,8 +1635,8 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             bv[2 * j + 1] = __half2float(__ushort_as_half((uint16_t)(u[j] >> 16)));
           }
         }
-        const uint32_t ib = produced & 1u;
-        if (!mbar_wait(smem_u32(&in_full[ib]), (produced >> 1) & 1u, &abort_flag, 32) ||
+        const uint32_t ib = produced & ((2u << a.dw_teams_log2) - 1u);
+        if (!mbar_wait(smem_u32(&in_full[ib]), (produced >> (1 + a.dw_teams_log2)) & 1u, &abort_flag, 32) ||
             !mbar_wait(smem_u32(&empty_bar[ring.idx]), ring.phase ^ 1u, &abort_flag, 32)) {
           ok = false;
           break;
@@ -1945,7 +1957,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                                         (((uint32_t)lane & 7u) >> 1) * 16u;
               const int rows_valid = (a.P - p0) < a.th ? (a.P - p0) : a.th;
               const int cpu = a.Q > kPassElems ? kPassElems : a.Q;  // columns per unit
-              int unit = 0;
+              int unit = DWPW ? ci : 0;  // (a channel tile of one unit: the warps of a quarter take the tiles in turn)
               for (int img = 0; img < a.tn; ++img) {
                 if (n0 + img >= a.N) break;
                 for (int hr0 = 0; hr0 < rows_valid; hr0 += a.y_rpu) {
@@ -2558,10 +2570,12 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
           }
           const int64_t tiles = (int64_t)((g.n + tn - 1) / tn) * ((g.p + th - 1) / th) * ((p.mtiles + na - 1) / na);
           const double waves = (double)((tiles + sms - 1) / sms);
-          const double t_dw = 33.0 * (double)px * (p.kb / 64.0);
-          const double t_mma = (double)na * (p.kb / 16.0) * ((double)px / 2.0 > 58.0 ? (double)px / 2.0 : 58.0);
+          const double t_dw = 22.0 * (double)px * (p.kb / 64.0);
+          double t_mma = (double)na * (p.kb / 16.0) * ((double)px / 2.0 > 58.0 ? (double)px / 2.0 : 58.0);
           const double units = (double)((px + 63) / 64);
-          const double t_epi = 2000.0 * units * (na > 1 ? 2.0 * na : 1.0);  // (one set of accumulators: not hidden)
+          const double t_epi = 1200.0 * ((units * na + 1) / 2) + 800.0;
+          const double t_l2 = ((double)na * 128 * p.kb * 2 + (double)tn * in_h * in_w * p.kb * 2) / 60.0;
+          if (t_l2 > t_mma) t_mma = t_l2;
           const double cost = waves * ((double)p.cblocks * (t_dw > t_mma ? t_dw : t_mma) + t_epi + 4000.0);
           if (cost < best_blk) {
             best_blk = cost;
@@ -2684,13 +2698,22 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   size_t budget_all = 232448u - 1024u - 512u;
   p.dw_in_h = p.dw_in_w = 0;
   p.dw_in_bytes = p.dw_in_alloc = 0;
+  p.dw_teams_log2 = 0;
   if (g.dw_stride > 0) {
     p.dw_in_h = (p.th - 1) * g.dw_stride + 3;
     p.dw_in_w = (g.q - 1) * g.dw_stride + 3;
     p.dw_in_bytes = (uint32_t)((size_t)p.tn * p.dw_in_h * p.dw_in_w * p.kb * 2);
     // (a pair of outputs at the end of a row reads up to two pixels past the tile)
     p.dw_in_alloc = (uint32_t)round_up_sz((size_t)p.dw_in_bytes + 2u * p.kb * 2u, 1024);
-    budget_all -= 2u * p.dw_in_alloc;
+    // teams of depthwise warps: as many as a stage's pairs of pixels leave threads for, while the input
+    // tiles (two per team) stay small beside the ring
+    const size_t stage_est = round_up_sz((size_t)p.ncols * p.kb * 2u, 1024) + (size_t)p.nacc * 128u * p.kb * 2u;  // (four must fit)
+    const int64_t pair_threads = (int64_t)p.tn * p.th * ((g.q + 1) / 2) * (p.kb / 8);
+    while ((1 << p.dw_teams_log2) < kMaxDwTeams && (pair_threads << (p.dw_teams_log2 + 1)) <= kDwWarps * 32 &&
+           (p.dw_in_alloc << (p.dw_teams_log2 + 2)) <= 48u * 1024u &&
+           (p.dw_in_alloc << (p.dw_teams_log2 + 2)) + 4u * stage_est + stage_buf_bytes <= budget_all)
+      ++p.dw_teams_log2;
+    budget_all -= p.dw_in_alloc << (1 + p.dw_teams_log2);
   }
   const size_t budget = budget_all - stage_buf_bytes;
   // ring of stages: one activation tile + `taps` weight tiles each, at least two deep; if the
@@ -2734,7 +2757,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   }
   // a second staging tile per epilogue warp (its store overlaps the next unit) if memory is left
   p.nbuf = (!p.plane_store && (size_t)p.stages * p.stage_bytes + 2u * stage_buf_bytes <= budget_all) ? 2 : 1;
-  p.smem_bytes = (size_t)p.stages * p.stage_bytes + (size_t)p.nbuf * stage_buf_bytes + 2u * p.dw_in_alloc + 1024;
+  p.smem_bytes = (size_t)p.stages * p.stage_bytes + (size_t)p.nbuf * stage_buf_bytes + (p.dw_in_alloc << (1 + p.dw_teams_log2)) + 1024;
   // more than half of an SM's shared memory: at most one CTA per SM, so that the kernel can take
   // all 512 TMEM columns without ever waiting for another CTA to free them
   if (p.smem_bytes < 120u * 1024u) p.smem_bytes = 120u * 1024u;
@@ -3035,6 +3058,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     a.dw_b = reinterpret_cast<const uint16_t*>(dw->bias);
     a.dw_h = dw->h; a.dw_wd = dw->w; a.dw_c = dw->c; a.dw_stride = dw->stride; a.dw_relu = dw->relu;
     a.dw_in_h = p.dw_in_h; a.dw_in_w = p.dw_in_w; a.dw_in_bytes = p.dw_in_bytes; a.dw_in_alloc = p.dw_in_alloc;
+    a.dw_teams_log2 = p.dw_teams_log2;
   }
   a.gather = p.gather;
   a.g_x = reinterpret_cast<const uint16_t*>(x);
