@@ -109,6 +109,27 @@ inline cudaError_t launch_kernel_overlapped(void (*kernel)(KArgs...), dim3 grid,
   return launch_kernel_attr(true, 0, kernel, grid, block, smem, stream, args...);
 }
 
+// The same for a kernel of clusters of `cluster` CTAs.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_kernel_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                         cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // The same with the cooperative attribute when `cooperative` is set: the launch waits until every
 // CTA of the grid can be resident at once (kernels whose CTAs wait for one another).
 template <typename... KArgs, typename... Args>
@@ -336,6 +357,7 @@ struct IgemmPlan {
   int32_t dup_log2;  // log2 of the number of copies of the layer's weight rows in w' and in a weight tile (0, 1, 2)
   size_t smem_bytes;
   int32_t ks_log2;  // log2 of the number of reduction slices a tile is split into (0 = none)
+  bool recv;        // split reduction: the parts have shared memory of their own (else they go into the ring)
   // work distribution of the kernels without reduction slices: `grid` CTAs take contiguous ranges
   // of the ring stages of all tiles; sk_split = 1: equal ranges, a tile that straddles a boundary
   // is reduced by several CTAs (fp32 hand-over through the workspace, sk_cols32 * 32 columns)
@@ -352,7 +374,7 @@ struct IgemmPlan {
   int32_t dw_teams_log2;   // depthwise warps form 1, 2 or 4 teams
   int32_t pair, ncols_sub, pair_fit;
   double est_clk;  // the cost model's estimate for the launch, in SM clocks
-  size_t ws_status_off, ws_w_off, ws_x_off, ws_part_off, ws_sk_off, ws_total;
+  size_t ws_status_off, ws_w_off, ws_x_off, ws_sk_off, ws_total;
   bool maps_ready;
   alignas(64) CUtensorMap tmA;
   alignas(64) CUtensorMap tmB;

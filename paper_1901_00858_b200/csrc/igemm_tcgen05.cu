@@ -134,6 +134,34 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
   return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, 0)) != 0;
 }
 
+// The same for a barrier that other CTAs of the cluster arrive on: what they wrote before is visible.
+__device__ __noinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  uint64_t t0 = 0;
+  for (uint32_t i = 0;; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if ((i & 1023u) == 1023u) {
+      if (*abort_flag) return false;
+      const uint64_t t = global_timer_ns();
+      if (t0 == 0) {
+        t0 = t;
+      } else if (t - t0 > g_wait_limit_ns) {
+        *abort_flag = 1;
+        return false;
+      }
+    }
+  }
+}
+
 // One lane of a converged warp (the same one every time).  Copies are issued under this predicate, not
 // under `lane == 0`: the copy instructions take their operands from uniform registers, and only for
 // an elected lane does the compiler know that one thread is left; for any other condition it walks
@@ -219,6 +247,10 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+
+// the two halves of cluster_sync_all
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
   asm volatile(
@@ -517,6 +549,37 @@ __device__ __forceinline__ void issue_mmas(uint32_t d_tmem, uint32_t a_lo, uint3
 #undef HGC_MMA
 }
 
+// Where an epilogue reads its fp32 sums: the accumulator in tensor memory (lane = output channel), or,
+// for a tile whose reduction a cluster of CTAs shared (SPLIT), the parts that the CTAs put into this
+// one's shared memory as [part][column][lanes], added up in the order of the parts.
+struct AccSource {
+  uint32_t addr;        // tensor-memory address of column 0, or shared-memory address of this lane's column 0
+  uint32_t col_bytes;   // SPLIT: bytes from column to column and from part to part, and the number of parts
+  uint32_t part_bytes;
+  int parts;
+};
+template <bool SPLIT, int N>
+__device__ __forceinline__ void acc_load(const AccSource& s, uint32_t col, uint32_t* v) {
+  if constexpr (!SPLIT) {
+    if constexpr (N == 32) tmem_ld32(s.addr + col, *reinterpret_cast<uint32_t(*)[32]>(v));
+    else tmem_ld8(s.addr + col, v);
+  } else {
+    float f[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) f[j] = 0.f;
+    for (int p = 0; p < s.parts; ++p) {
+      const uint32_t src = s.addr + (uint32_t)p * s.part_bytes + col * s.col_bytes;
+      float t[N];  // (all of a part's loads are under way before the first sum waits for one)
+#pragma unroll
+      for (int j = 0; j < N; ++j) asm volatile("ld.shared.f32 %0, [%1];" : "=f"(t[j]) : "r"(src + (uint32_t)j * s.col_bytes));
+#pragma unroll
+      for (int j = 0; j < N; ++j) f[j] += t[j];
+    }
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = __float_as_uint(f[j]);
+  }
+}
+
 // Copy epilogue (every shape the TMA-store epilogue does not take: planes whose size is not a
 // multiple of 8 pixels, tiles with junk columns between their rows, several images per tile).
 // A unit of work is this warp's 32 channels (its TMEM lanes) x up to 64 accumulator columns of
@@ -527,7 +590,8 @@ __device__ __forceinline__ void issue_mmas(uint32_t d_tmem, uint32_t a_lo, uint3
 // writes consecutive pixels of one channel plane (64 or 128 contiguous bytes).  The two warps
 // of a lane quarter take alternate units.  Kept out of line: the hot loops of the kernel should
 // stay compact in the instruction cache.
-__device__ __noinline__ void epilogue_copy(uint32_t t_addr, uint32_t sbuf, int first_unit, int unit_step, int tn, int th,
+template <bool SPLIT>
+__device__ __noinline__ void epilogue_copy(AccSource acc, uint32_t sbuf, int first_unit, int unit_step, int tn, int th,
                                            int pitch, int N, int K, int P, int Q, int n0, int p0, int k0,
                                            int kvalid_rows, float bv, bool relu, uint16_t* yb) {
   const int lane = threadIdx.x & 31;
@@ -544,10 +608,11 @@ __device__ __noinline__ void epilogue_copy(uint32_t t_addr, uint32_t sbuf, int f
   for (int img = 0; img < tn; ++img) {
     if (n0 + img >= N) break;
     uint16_t* yimg = yb + ((int64_t)(n0 + img) * K + k0) * pq;  // this warp's first channel plane
-    for (int c0 = 0; c0 < cols_need; c0 += 64, ++unit) {
+    constexpr int kCols = SPLIT ? 32 : 64;  // (more warps share the units of a split tile)
+    for (int c0 = 0; c0 < cols_need; c0 += kCols, ++unit) {
       if (unit % unit_step != first_unit) continue;
-      const int ncol = cols_need - c0 < 64 ? cols_need - c0 : 64;
-      const uint32_t tcol = t_addr + (uint32_t)(img * img_cols + c0);
+      const int ncol = cols_need - c0 < kCols ? cols_need - c0 : kCols;
+      const uint32_t tcol = (uint32_t)(img * img_cols + c0);
       // ---- accumulators -> fp16 staging tile (lane = channel) ----
       __syncwarp();  // the previous unit has been copied out
 #pragma unroll 1
@@ -555,11 +620,11 @@ __device__ __noinline__ void epilogue_copy(uint32_t t_addr, uint32_t sbuf, int f
         if (g * 32 >= ncol) break;
         uint32_t v[32];
         if (g * 32 + 32 <= ncol) {
-          tmem_ld32(tcol + (uint32_t)(g * 32), v);
+          acc_load<SPLIT, 32>(acc, tcol + (uint32_t)(g * 32), v);
         } else {
 #pragma unroll
           for (int c = 0; c < 4; ++c)
-            if (g * 32 + c * 8 < ncol) tmem_ld8(tcol + (uint32_t)(g * 32 + c * 8), &v[8 * c]);
+            if (g * 32 + c * 8 < ncol) acc_load<SPLIT, 8>(acc, tcol + (uint32_t)(g * 32 + c * 8), &v[8 * c]);
         }
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         {
@@ -613,12 +678,13 @@ __device__ __noinline__ void epilogue_copy(uint32_t t_addr, uint32_t sbuf, int f
 // Epilogue of the inner-product layer (1x1 output plane: a column is an image).  y[n][k] has the
 // channels of one image contiguous, so the lanes (channels) of a warp write 64 contiguous bytes
 // per column straight from registers.
-__device__ __noinline__ void epilogue_columns(uint32_t t_addr, int first_unit, int unit_step, int nimg, int K, int n0,
+template <bool SPLIT>
+__device__ __noinline__ void epilogue_columns(AccSource acc, int first_unit, int unit_step, int nimg, int K, int n0,
                                               int k0, int kvalid_rows, float bv, bool relu, uint16_t* yb) {
   const int lane = threadIdx.x & 31;
   for (int c0 = first_unit * 32; c0 < nimg; c0 += unit_step * 32) {
     uint32_t v[32];
-    tmem_ld32(t_addr + (uint32_t)c0, v);  // columns past the tile's last image are read and dropped
+    acc_load<SPLIT, 32>(acc, (uint32_t)c0, v);  // columns past the tile's last image are read and dropped
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
     if (lane < kvalid_rows) {
 #pragma unroll
@@ -634,104 +700,11 @@ __device__ __noinline__ void epilogue_columns(uint32_t t_addr, int first_unit, i
   __syncwarp();
 }
 
-// Epilogue of a reduction slice: the fp32 accumulators go, unrounded, to this slice's copy of
-// the output (same [n][k][p][q] order as y).  Same two-phase scheme as epilogue_copy with 4-byte
-// elements: a unit is 32 channels x 32 columns; lane = channel stages its row of 32 floats
-// (128 bytes, swizzled), then lane = column walks the 32 rows, so a store instruction writes 32
-// consecutive floats of one channel plane.  On a 1x1 plane (inner product) a column is an image
-// and the lanes' channels are contiguous: straight from registers.
-__device__ __noinline__ void epilogue_partial(uint32_t t_addr, uint32_t sbuf, int first_unit, int unit_step, int tn,
-                                              int th, int pitch, int N, int K, int P, int Q, int n0, int p0, int k0,
-                                              int kvalid_rows, float* part) {
-  const int lane = threadIdx.x & 31;
-  const int64_t pq = (int64_t)P * Q;
-  if (pq == 1) {
-    const int nimg = N - n0 < tn ? N - n0 : tn;
-    for (int c0 = first_unit * 32; c0 < nimg; c0 += unit_step * 32) {
-      uint32_t v[32];
-      tmem_ld32(t_addr + (uint32_t)c0, v);  // columns past the tile's last image are read and dropped
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (lane < kvalid_rows) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (c0 + j < nimg) HGC_CHECKED_STORE(part + (int64_t)(n0 + c0 + j) * K + k0 + lane, part[(int64_t)(n0 + c0 + j) * K + k0 + lane] = __uint_as_float(v[j]));
-      }
-    }
-    __syncwarp();
-    return;
-  }
-  const int rows_valid = (P - p0) < th ? (P - p0) : th;
-  const int cols_need = (rows_valid - 1) * pitch + Q;
-  const int img_cols = th * pitch;
-  const uint32_t row_off = (uint32_t)lane * 128u;
-  int unit = 0;
-  for (int img = 0; img < tn; ++img) {
-    if (n0 + img >= N) break;
-    float* pimg = part + ((int64_t)(n0 + img) * K + k0) * pq;
-    for (int c0 = 0; c0 < cols_need; c0 += 32, ++unit) {
-      if (unit % unit_step != first_unit) continue;
-      const int ncol = cols_need - c0 < 32 ? cols_need - c0 : 32;
-      const uint32_t tcol = t_addr + (uint32_t)(img * img_cols + c0);
-      __syncwarp();  // the previous unit has been copied out
-      uint32_t v[32];
-      if (ncol == 32) {
-        tmem_ld32(tcol, v);
-      } else {
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (c * 8 < ncol) tmem_ld8(tcol + (uint32_t)(c * 8), &v[8 * c]);
-      }
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        if (c * 4 < ncol) {
-          const uint32_t dst = sbuf + row_off + ((uint32_t)(c ^ (lane & 7)) << 4);
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(v[4 * c]), "r"(v[4 * c + 1]),
-                       "r"(v[4 * c + 2]), "r"(v[4 * c + 3])
-                       : "memory");
-        }
-      }
-      __syncwarp();
-      const int cabs = c0 + lane;
-      const int hr = cabs / pitch;
-      const int wc = cabs - hr * pitch;
-      if (lane < ncol && wc < Q) {
-        float* dst = pimg + (int64_t)(p0 + hr) * Q + wc;
-        const uint32_t chunk = (uint32_t)lane >> 2, within = ((uint32_t)lane & 3u) * 4u;
-#pragma unroll 4
-        for (int r = 0; r < kvalid_rows; ++r) {
-          uint32_t w;
-          asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(sbuf + (uint32_t)r * 128u + ((chunk ^ ((uint32_t)r & 7u)) << 4) + within));
-          HGC_CHECKED_STORE(dst + (int64_t)r * pq, dst[(int64_t)r * pq] = __uint_as_float(w));
-        }
-      }
-    }
-  }
-  __syncwarp();
-}
-
-// y = round( relu?( bias[k] + partial[0] + partial[1] + ... ) ): the slices are added in a fixed
-// order, so the result does not depend on which CTA finished first
-__global__ void __launch_bounds__(256)
-splitk_finish_kernel(const float* __restrict__ part, int slices, int64_t stride, const __half* __restrict__ bias,
-                     uint16_t* __restrict__ y, int K, int64_t pq, int64_t total, int relu) {
-  grid_dependency_wait();
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    float acc = bias != nullptr ? __half2float(__ldg(bias + (int)((i / pq) % K))) : 0.f;
-    for (int sidx = 0; sidx < slices; ++sidx) {
-      float pv;
-      HGC_CHECKED_LOAD(pv, part + sidx * stride + i, __ldcs(part + sidx * stride + i));
-      acc += pv;
-    }
-    if (relu) acc = fmaxf(acc, 0.f);
-    HGC_CHECKED_STORE(y + i, y[i] = __half_as_ushort(__float2half_rn(acc)));
-  }
-}
-
 // Channels-last epilogue (y[N][P][Q][K]): a lane owns a channel, so for every output pixel the 32
 // lanes of a warp write 32 consecutive channels (64 contiguous bytes) straight from registers.
 // A unit of work is one tile row x up to 32 pixels; the warps of a lane quarter take units in turn.
-__device__ __noinline__ void epilogue_nhwc(uint32_t t_addr, int first_unit, int unit_step, int tn, int th, int pitch,
+template <bool SPLIT>
+__device__ __noinline__ void epilogue_nhwc(AccSource acc, int first_unit, int unit_step, int tn, int th, int pitch,
                                            int N, int K, int P, int Q, int n0, int p0, int k, bool kvalid, float bv,
                                            bool relu, uint16_t* yb) {
   const int rows_valid = (P - p0) < th ? (P - p0) : th;
@@ -742,14 +715,14 @@ __device__ __noinline__ void epilogue_nhwc(uint32_t t_addr, int first_unit, int 
       for (int wc0 = 0; wc0 < Q; wc0 += 32, ++unit) {
         if (unit % unit_step != first_unit) continue;
         const int ncol = Q - wc0 < 32 ? Q - wc0 : 32;
-        const uint32_t tcol = t_addr + (uint32_t)((img * th + hr) * pitch + wc0);
+        const uint32_t tcol = (uint32_t)((img * th + hr) * pitch + wc0);
         uint32_t v[32];
         if (ncol == 32) {
-          tmem_ld32(tcol, v);
+          acc_load<SPLIT, 32>(acc, tcol, v);
         } else {
 #pragma unroll
           for (int c = 0; c < 4; ++c)
-            if (c * 8 < ncol) tmem_ld8(tcol + (uint32_t)(c * 8), &v[8 * c]);
+            if (c * 8 < ncol) acc_load<SPLIT, 8>(acc, tcol + (uint32_t)(c * 8), &v[8 * c]);
         }
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         uint16_t* dst = yb + (((int64_t)(n0 + img) * P + (p0 + hr)) * Q + wc0) * K + k;
@@ -835,11 +808,10 @@ struct IgemmArgs {
   const uint16_t* g_x;
   int32_t mshift;     // log2 of the channel tiles that one work item covers (pairs: 1; nacc: 0, 1, 2)
   int32_t acc_stride; // accumulator columns between the channel tiles of an item (nacc > 1: 512 / nacc)
-  // split reduction (its own kernel instantiation): the channel blocks of a tile are dealt out to
-  // 2^ks_log2 CTAs, each of which writes its fp32 partial sums to its own slice of `partials`; a
-  // second kernel adds the slices in a fixed order (+ bias, ReLU, rounding)
+  // split reduction (its own kernel instantiations): the ring stages of a tile are dealt out to the
+  // 2^ks_log2 CTAs of a cluster; CTA i of it then finishes the i-th part of the tile's channels
   int32_t ks_log2;
-  int64_t part_stride;  // elements between two slices: N * K * P * Q
+  uint32_t recv_bytes;  // room for the parts behind the ring (0: they go into the ring, when nobody reads it any more)
   int32_t y_tma;        // channels-last output staged for TMA stores (else plain stores)
   int32_t y_full_w;     // pixels of a full channels-last store
   int32_t y_rpu;        // tile rows per channels-last store (rows of at most 32 pixels are batched)
@@ -938,25 +910,12 @@ struct TileIter {
       m0 = (mgc - grp * a.mtiles) * 128;
     }
   }
-  // reduction slice of this unit and its range of channel blocks
+  // reduction slice of this unit (its rank in the cluster) and its range of the tile's ring stages
   __device__ __forceinline__ int slice(const IgemmArgs& a) const { return SPLIT ? (mg & ((1 << a.ks_log2) - 1)) : 0; }
-  __device__ __forceinline__ void block_range(const IgemmArgs& a, int& cb0, int& cb1) const {
-    if (SPLIT) {
-      const int sl = slice(a);
-      cb0 = (sl * a.cblocks) >> a.ks_log2;
-      cb1 = ((sl + 1) * a.cblocks) >> a.ks_log2;
-    } else {
-      cb0 = 0;
-      cb1 = a.cblocks;
-    }
-  }
-  // the same as a range of ring stages of the tile
   __device__ __forceinline__ void stage_range(const IgemmArgs& a, int& s0, int& s1) const {
-    int cb0, cb1;
-    block_range(a, cb0, cb1);
-    const int per_block = a.ts / a.cblocks;
-    s0 = cb0 * per_block;
-    s1 = cb1 * per_block;
+    const int sl = slice(a);
+    s0 = SPLIT ? (sl * a.ts) >> a.ks_log2 : 0;
+    s1 = SPLIT ? ((sl + 1) * a.ts) >> a.ks_log2 : a.ts;
   }
   __device__ __forceinline__ int kind(const IgemmArgs&) const { return 0; }
   __device__ __forceinline__ bool sub_tile(const IgemmArgs&, int, int&, int&) const { return true; }  // (no CTA pairs here)
@@ -1213,8 +1172,7 @@ template <int KB, bool HALO, int EW, int EPI, bool SPLIT, bool PAIR = false, boo
 __global__ void __launch_bounds__(96 + 32 * EW + (FUSEL ? 32 * kLayoutWarps : 0) + (DWPW ? 32 * kDwWarps : 0), 1)
 igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
              const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmYr,
-             const IgemmArgs a, const __half* __restrict__ bias, __half* __restrict__ y, float* __restrict__ partials,
-             int* status) {
+             const IgemmArgs a, const __half* __restrict__ bias, __half* __restrict__ y, int* status) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages];
   __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
@@ -1226,6 +1184,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __shared__ __align__(8) uint64_t ho_bar;    //   of the warps that hand accumulators over (the first of each lane quarter),
   __shared__ __align__(8) uint64_t pl_bar;    //   of the warps that fetch partial sums (the second of each lane quarter)
   __shared__ __align__(8) uint64_t in_full[2 * kMaxDwTeams], in_empty[2 * kMaxDwTeams];  // depthwise input tiles (depthwise + pointwise blocks)
+  __shared__ __align__(8) uint64_t peers_done, parts_in;  // split reduction: the cluster's MMAs are complete; the parts have arrived
   __shared__ __align__(8) uint64_t q_bar[4];  // whole-plane epilogue: meeting point of the two warps of a lane quarter
 
   // (through a shuffle: the compiler then knows that the roles' branches are taken by whole warps)
@@ -1259,6 +1218,8 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     mbar_init(smem_u32(&sk_bar), PAIR ? EW : EW / 2);  // one arrival per fetching warp (of both CTAs)
     for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&q_bar[q]), EW / 4);
     mbar_init(smem_u32(&meet_bar), EW);
+    mbar_init(smem_u32(&peers_done), 1u << a.ks_log2);
+    mbar_init(smem_u32(&parts_in), EW);
     mbar_init(smem_u32(&ho_bar), EW / 2);
     mbar_init(smem_u32(&pl_bar), EW / 2);
     abort_flag = 0;
@@ -1273,7 +1234,11 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  if constexpr (PAIR) cluster_sync_all();  // the partner's barriers must exist before anything arrives on them
+  // the partners' barriers must exist before anything arrives on them (a split reduction waits for that
+  // when it first does)
+  if constexpr (SPLIT) cluster_arrive();
+  [[maybe_unused]] bool met = false;
+  if constexpr (PAIR) cluster_sync_all();
   else __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = tmem_slot;
@@ -1713,15 +1678,18 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     // that every epilogue warp has work although the layer fills only part of the MMA's 128 rows.
     // Row pairs: quarters 2 and 3 hold the same channels too, but of the odd output rows; the
     // two halves do not share pixels, they store to rows 2 * p0 and 2 * p0 + 1.
-    const int rep_q = EPI == 0 ? (a.rowpair ? 2 : (4 >> a.dup_log2)) : 4;  // lane quarters per replica
-    const int cq = quarter & (rep_q - 1);                                  // the quarter's place among the channels
-    const bool split_px = EPI == 0 && !a.rowpair;
+    // Split reduction: this CTA finishes the part-th share of the tile's channels from shared memory,
+    // so here too the warps of all lane quarters share the pixels of those channels.
+    const int rep_q = SPLIT ? 4 >> a.ks_log2 : (EPI == 0 ? (a.rowpair ? 2 : (4 >> a.dup_log2)) : 4);  // lane quarters per replica
+    const int part = SPLIT ? (int)blockIdx.x & ((1 << a.ks_log2) - 1) : 0;
+    const int cq = part * rep_q + (quarter & (rep_q - 1));                   // the quarter's place among the channels
+    const bool split_px = SPLIT || (EPI == 0 && !a.rowpair);
     const int half_eff = split_px ? (quarter / rep_q) * kPerQuarter + half : half;  // which of the warps that share the pixels
-    const int per_eff = split_px ? (kPerQuarter << a.dup_log2) : kPerQuarter;
+    const int per_eff = split_px ? (kPerQuarter << (SPLIT ? a.ks_log2 : a.dup_log2)) : kPerQuarter;
     const int odd_row = (EPI == 0 && a.rowpair) ? (quarter >> 1) : 0;
     const int row = cq * 32 + ((EPI == 2 && a.y_tma) ? ((lane & 3) << 3) + (lane >> 2) : lane);
     uint16_t* yb = reinterpret_cast<uint16_t*>(y);
-    const uint32_t stage_base = ring_base + (uint32_t)a.stages * a.stage_bytes;
+    const uint32_t stage_base = ring_base + (uint32_t)a.stages * a.stage_bytes + (SPLIT ? a.recv_bytes : 0u);
     const bool relu = a.relu != 0;
     const bool leader = elect_one();  // issues this warp's bulk stores and waits for them (their groups are per thread)
     // this warp's own staging tiles: 32 channel rows of 128 bytes each, 128-byte swizzled
@@ -1866,7 +1834,51 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       if constexpr (PAIR) {
         if (!it.sub_tile(a, sub, n0, p0)) break;  // (only the last pair tile can lack its second sub-tile)
       }
-      const uint32_t t_addr = t_tile + (uint32_t)(sub * a.ncols_sub);
+      AccSource acc_src{t_tile + (uint32_t)(sub * a.ncols_sub), 0u, 0u, 0};
+      if constexpr (SPLIT) {
+        // Every CTA of the cluster has the sums of its ring stages for all 128 channels in its tensor
+        // memory and sends every CTA those of the channels that one finishes, as [part][column][lanes],
+        // 128 bytes per column and warp; the receiver adds the parts in order.  They go behind the
+        // ring where the plan found room (three ring stages are left), else into the ring
+        // once all MMAs of the cluster are complete.  The transfer runs at about 27 bytes per clock and
+        // SM, 1.2 us for 128 columns over four CTAs; waiting for the partners first costs 0.7 us.
+        // (The first form of this wrote the parts to global memory for a second kernel to add.)
+        const uint32_t col_bytes = (uint32_t)(128 * 4) >> a.ks_log2;
+        const uint32_t part_bytes = (uint32_t)a.ncols * col_bytes;
+        // (reads of whole vectors may run up to 31 columns past the last part: into the staging tiles)
+        const uint32_t recv_base = ring_base + (a.recv_bytes != 0 ? (uint32_t)a.stages * a.stage_bytes : 0u);
+        cluster_wait();
+        met = true;
+        if (a.recv_bytes == 0) {
+          if (ew == 0 && lane < (1 << a.ks_log2)) mbar_arrive_cluster(cluster_addr(smem_u32(&peers_done), (uint32_t)lane));
+          __syncwarp();
+          if (!mbar_wait_cluster(smem_u32(&peers_done), 0u, &abort_flag)) {
+            gave_up = true;
+            break;
+          }
+        }
+        const uint32_t dest = (uint32_t)(quarter / rep_q);
+        const uint32_t dst = cluster_addr(recv_base, dest) + (uint32_t)part * part_bytes +
+                             (uint32_t)((quarter & (rep_q - 1)) * 32 + lane) * 4u;
+        if (m0 + quarter * 32 < a.kg) {
+          for (int c = half * 32; c < a.ncols; c += kPerQuarter * 32) {
+            uint32_t v[32];
+            tmem_ld32(t_tile + (uint32_t)c, v);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (c + j < a.ncols)
+                asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(dst + (uint32_t)(c + j) * col_bytes), "r"(v[j]) : "memory");
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(cluster_addr(smem_u32(&parts_in), dest));
+        if (!mbar_wait_cluster(smem_u32(&parts_in), 0u, &abort_flag)) {
+          gave_up = true;
+          break;
+        }
+        acc_src = AccSource{recv_base + (uint32_t)((quarter & (rep_q - 1)) * 32 + lane) * 4u, col_bytes, part_bytes, 1 << a.ks_log2};
+      }
       if constexpr (EPI == 0) {
         // ---- staged epilogue: TMEM -> registers -> swizzled fp16 tile in smem -> TMA store ----
         // (taken when Q % 8 == 0, hence P*Q % 8 == 0, and a tile holds one image: every staged run
@@ -1898,7 +1910,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
               // 32 pixels: one wide accumulator load when they are 32 consecutive columns (always
               // when columns are pixels; else when the row does not end inside them)
               if (nchunks == 4 && (linear || uw + 32 <= a.Q)) {
-                tmem_ld32(t_addr + (uint32_t)(linear ? e0 : uh * a.pitch + uw), v);
+                acc_load<SPLIT, 32>(acc_src, (uint32_t)(linear ? e0 : uh * a.pitch + uw), v);
                 if (!linear) {
                   uw += 32;
                   if (uw == a.Q) { uw = 0; ++uh; }
@@ -1914,7 +1926,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     uw += 8;
                     if (uw == a.Q) { uw = 0; ++uh; }  // next output row: the junk columns of the pitch are skipped
                   }
-                  if (c < nchunks) tmem_ld8(t_addr + col, &v[8 * c]);
+                  if (c < nchunks) acc_load<SPLIT, 8>(acc_src, col, &v[8 * c]);
                 }
               }
               if (g == 0) {
@@ -1962,7 +1974,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 if (n0 + img >= a.N) break;
                 for (int hr0 = 0; hr0 < rows_valid; hr0 += a.y_rpu) {
                   for (int wc0 = 0; wc0 < a.Q; wc0 += cpu, ++unit) {
-                    if (unit % kPerQuarter != half) continue;
+                    if (unit % per_eff != half_eff) continue;
                     const int nrows = rows_valid - hr0 < a.y_rpu ? rows_valid - hr0 : a.y_rpu;
                     const int ncol = a.Q - wc0 < cpu ? a.Q - wc0 : cpu;
                     const uint32_t sbuf = my_stage + stage_sel * kWarpStageBytes;
@@ -1974,14 +1986,14 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                       for (int g = 0; g < 2; ++g) {
                         const int rem = ncol - g * 32;
                         if (rem <= 0) break;
-                        const uint32_t tcol = t_addr + (uint32_t)((img * a.th + hr0 + r) * a.pitch + wc0 + g * 32);
+                        const uint32_t tcol = (uint32_t)((img * a.th + hr0 + r) * a.pitch + wc0 + g * 32);
                         uint32_t v[32];
                         if (rem >= 32) {
-                          tmem_ld32(tcol, v);
+                          acc_load<SPLIT, 32>(acc_src, tcol, v);
                         } else {
 #pragma unroll
                           for (int c = 0; c < 4; ++c)
-                            if (c * 8 < rem) tmem_ld8(tcol + (uint32_t)(c * 8), &v[8 * c]);
+                            if (c * 8 < rem) acc_load<SPLIT, 8>(acc_src, tcol + (uint32_t)(c * 8), &v[8 * c]);
                         }
                         if (first) {
                           // this buffer's previous store must have been read out of shared memory
@@ -2003,7 +2015,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     if (leader) {
                       // a short unit at the end of the image takes the full box: the rest is clipped
                       const bool image_end = p0 + hr0 + nrows == a.P && wc0 + ncol == a.Q;
-                      tma_store_4d((nrows * ncol == a.y_full_w || image_end) ? &tmY : &tmYr, sbuf, m0 + quarter * 32, grp,
+                      tma_store_4d((nrows * ncol == a.y_full_w || image_end) ? &tmY : &tmYr, sbuf, m0 + cq * 32, grp,
                                    (p0 + hr0) * a.Q + wc0, n0 + img);
                       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
@@ -2012,33 +2024,26 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
               }
             }
             else if (EW == 8 && quarter_live)  // (16 epilogue warps only ever run the staged form)
-              epilogue_nhwc(t_addr, half, kPerQuarter, a.tn, a.th, a.pitch, a.N, a.K, a.P, a.Q, n0, p0, k, kvalid, bv,
+              epilogue_nhwc<SPLIT>(acc_src, half_eff, per_eff, a.tn, a.th, a.pitch, a.N, a.K, a.P, a.Q, n0, p0, k, kvalid, bv,
                             relu, yb);
-          } else if constexpr (SPLIT) {
-            if (quarter_live) {
-              const int kleft = a.kg - (m0 + quarter * 32);
-              epilogue_partial(t_addr, my_stage, half, kPerQuarter, a.tn, a.th, a.pitch, a.N, a.K, a.P, a.Q, n0, p0,
-                               grp * a.kg + m0 + quarter * 32, kleft < 32 ? kleft : 32,
-                               partials + (int64_t)it.slice(a) * a.part_stride);
-            }
           } else {
             if (quarter_live && a.P * a.Q == 1) {
-              const int kleft = a.kg - (m0 + quarter * 32);
+              const int kleft = a.kg - (m0 + cq * 32);
               const int nimg = a.N - n0 < a.tn ? a.N - n0 : a.tn;
-              epilogue_columns(t_addr, half, kPerQuarter, nimg, a.K, n0, grp * a.kg + m0 + quarter * 32,
+              epilogue_columns<SPLIT>(acc_src, half_eff, per_eff, nimg, a.K, n0, grp * a.kg + m0 + cq * 32,
                                kleft < 32 ? kleft : 32, bv, relu, yb);
             } else if constexpr (EPI == 3) {
               // whole-plane tiles (instantiations of their own: the other kernels' code stays as it is)
               if (quarter_live) {
-                q_phase = epilogue_planes(t_addr, stage_base + (uint32_t)quarter * a.plane_bytes, half, a.plane_store, a.tn, a.N, a.K,
-                                          a.P * a.Q, n0, grp * a.kg + m0 + quarter * 32, bv, relu, yb, smem_u32(&q_bar[quarter]),
+                q_phase = epilogue_planes(acc_src.addr, stage_base + (uint32_t)quarter * a.plane_bytes, half, a.plane_store, a.tn, a.N, a.K,
+                                          a.P * a.Q, n0, grp * a.kg + m0 + cq * 32, bv, relu, yb, smem_u32(&q_bar[quarter]),
                                           q_phase, &abort_flag);
                 if (q_phase == ~0u) gave_up = true;
               }
             } else if (quarter_live) {
-              const int kleft = a.kg - (m0 + quarter * 32);
-              epilogue_copy(t_addr, my_stage, half, kPerQuarter, a.tn, a.th, a.pitch, a.N, a.K, a.P, a.Q, n0, p0,
-                            grp * a.kg + m0 + quarter * 32, kleft < 32 ? kleft : 32, bv, relu, yb);
+              const int kleft = a.kg - (m0 + cq * 32);
+              epilogue_copy<SPLIT>(acc_src, my_stage, half_eff, per_eff, a.tn, a.th, a.pitch, a.N, a.K, a.P, a.Q, n0, p0,
+                            grp * a.kg + m0 + cq * 32, kleft < 32 ? kleft : 32, bv, relu, yb);
             }
           }
         }
@@ -2065,6 +2070,13 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   // (a pair leaves together: the first CTA's MMAs read the partner's shared memory and write its tensor memory)
   if constexpr (PAIR) cluster_sync_all();
   else __syncthreads();
+  if constexpr (SPLIT) {
+    // The CTAs of a split reduction write into one another's shared memory: one that has received
+    // every part gets no more, and its own parts go to CTAs that cannot leave before they have them.
+    // After giving up that need not hold: then it stays until the others have given up or left.
+    if (!met) cluster_wait();
+    if (abort_flag) cluster_sync_all();
+  }
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
@@ -2357,8 +2369,6 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   const double mps = (double)taps_est * (p.kb / 16.0);                       // MMAs per stage
   const double mpt = (double)p.cblocks * p.eff_r * p.eff_s * (p.kb / 16.0);  // MMAs per tile
   const double a_bytes_mma = 32.0 * (g.kg < 128 ? g.kg : 128);
-  // ks: log2 of the number of CTAs that share the reduction of a tile (each then writes fp32
-  // partial sums, added by a second kernel): main loop / 2^ks, an epilogue of twice the bytes
   // clocks of one MMA step in the main loop of a tile of `cols` accumulator columns
   auto mma_clk = [&](int64_t brow, int64_t cols) {
     const double ncols = (double)((cols + 15) / 16 * 16);
@@ -2373,9 +2383,9 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     return t;
   };
   auto epilogue_clk = [&](int64_t cols) { return 600.0 + 10.0 * (double)((cols + 15) / 16 * 16); };
-  auto tile_clk = [&](int64_t brow, int64_t cols, int ks) {
-    const double main_loop = mpt / (double)(1 << ks) * mma_clk(brow, cols);
-    const double epilogue = epilogue_clk(cols) * (ks > 0 ? 2.0 : 1.0);
+  auto tile_clk = [&](int64_t brow, int64_t cols) {
+    const double main_loop = mpt * mma_clk(brow, cols);
+    const double epilogue = epilogue_clk(cols);
     return (main_loop > epilogue ? main_loop : epilogue) + 300.0;
   };
   // Contiguous ranges of ring stages per CTA (kernels without reduction slices).  Whole tiles per
@@ -2403,14 +2413,6 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     *grid_out = (int)grid;
     *cost_out = (main_loop > epi ? main_loop : epi) + 300.0 * (tiles_per_cta > 1.0 ? tiles_per_cta : 1.0) + hand_over;
   };
-  // the second kernel of a split reduction: a launch plus reading the slices and writing y
-  auto finish_clk = [&](int ks) {
-    if (ks == 0) return 0.0;
-    const double elems = (double)g.n * g.k * g.p * g.q;
-    return 8000.0 + elems * (4.0 * (1 << ks) + 2.0) / 3000.0;
-  };
-  // the split kernel exists for 64-channel stages of stride-1 layers without the direct-x mode
-  const bool can_split = p.kb == 64 && p.halo && !p.nchw && !p.y_nhwc;
   double best = 1e300;
   int best_th = 0, best_tn = 0, best_ks = 0, best_shared = 0, best_grid = 0;
   // shared tiles: asked for (no_split == 0: taken wherever tiles do not fill whole waves), or left
@@ -2436,22 +2438,14 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
         if (in_h > 256 || in_w > 256 || tn * in_h * in_w * p.kb * 2 > 48 * 1024) break;
       }
       const int64_t tiles = (int64_t)((g.n + tn - 1) / tn) * ((g.p + th - 1) / th) * mg;
-      for (int ks = 0; ks <= 3; ++ks) {
-        // a slice keeps at least two channel blocks and a main loop of 24 MMAs; only layers whose
-        // tiles leave three quarters of the SMs idle are split (inner products, tiny planes): on
-        // a 14x14 layer of 128 tiles the second pass costs what the split gains (measured)
-        if (ks > 0 && (!can_split || (p.cblocks >> ks) < 2 || mpt / (1 << ks) < 24.0 || 4 * tiles > sms)) break;
-        const int64_t units = tiles << ks;
-        const int64_t waves = (units + sms - 1) / sms;
-        double cost = (double)waves * tile_clk((int64_t)tn * th * p.pitch, cols, ks) + finish_clk(ks) +
-                      1e-3 * (double)units;
+      {
+        const int64_t waves = (tiles + sms - 1) / sms;
+        double cost = (double)waves * tile_clk((int64_t)tn * th * p.pitch, cols) + 1e-3 * (double)tiles;
         if (force_share && can_share && tiles % sms != 0) cost *= 1e3;  // shared tiles were asked for (HGC_FLAG_SHARED_TILES)
-        if (cost < best - 1e-9 ||
-            (cost < best + 1e-9 && ks == best_ks && !best_shared && (int64_t)tn * th > (int64_t)best_tn * best_th)) {
+        if (cost < best - 1e-9 || (cost < best + 1e-9 && !best_shared && (int64_t)tn * th > (int64_t)best_tn * best_th)) {
           best = cost;
           best_th = th;
           best_tn = tn;
-          best_ks = ks;
           best_shared = 0;
           best_grid = (int)(tiles < sms ? tiles : sms);
         }
@@ -2466,14 +2460,13 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
           // whole tiles in between (at least 2.5 tiles per unit); the contiguous ranges cost some
           // locality in L2 and the hand-overs some time, together about 10k clocks per launch
           // (conv3_2: 3.03 waves of 11 us tiles, 61.3 -> 55.6 us; conv2_2, conv4_x: slower).
-          cost_s = (double)tiles / (double)sms * tile_clk((int64_t)tn * th * p.pitch, cols, 0) + 10000.0;
+          cost_s = (double)tiles / (double)sms * tile_clk((int64_t)tn * th * p.pitch, cols) + 10000.0;
           if (2 * tiles < 5 * (int64_t)sms || grid_s != sms || ts_est < 16) grid_s = 0;
         }
         if (grid_s > 1 && cost_s < best - 1e-9) {
           best = cost_s;
           best_th = th;
           best_tn = tn;
-          best_ks = 0;
           best_shared = 1;
           best_grid = grid_s;
         }
@@ -2481,6 +2474,65 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     }
   }
   if (best_th == 0) return false;
+  // Split reductions: the ring stages of a tile dealt out to a cluster of 2 or 4 CTAs, each of which
+  // sends the others their channels' sums through distributed shared memory and finishes its own.
+  // A layer with few pixels and a long reduction then runs with wide tiles (few bytes per MMA) on all
+  // SMs.  Estimated with what bounds a stage of the kernel, measured on B200:
+  //   the tensor pipe:     N/2 clocks per MMA of N columns, never less than its shared-memory reads at
+  //                        128 bytes per clock (4 KB of weights + 32 N of activations) or 48,
+  //   the issuing warp:    about 200 clocks per stage and 45 per MMA,
+  //   L2 -> shared memory: about 78 bytes per clock and SM;
+  // and of a split tile's end, 512 bytes per column leave at 27 bytes per clock, the waits and the
+  // first run of the epilogue take about 5000 clocks (9000 with channels-last output).  Taken only where
+  // that is well below the best whole tiles.  Measured: 512 -> 512 3x3 on 28x28, one image, 18.9 -> 15.0 us;
+  // stride 2 on 14x14, 16 images channels-last, 19.8 -> 14.1; inner products of 64 x 25088 and 64 x 4096
+  // to 4096 41.5 -> 39.0 and 12.3 -> 10.9 (both with partial sums in global memory and a second kernel
+  // before); 256 -> 256 3x3 on 14x14, 16 images, would go from 9.1 to 11.7.
+  auto stage_clk = [&](int64_t brow, int64_t cols) {
+    const double ncols = (double)((cols + 15) / 16 * 16);
+    const double brows = p.nchw ? (double)((cols + 63) / 64 * 64) : (double)brow;
+    double t_mma = ncols / 2.0;
+    if (32.0 + ncols / 4.0 > t_mma) t_mma = 32.0 + ncols / 4.0;
+    if (t_mma < 48.0) t_mma = 48.0;
+    double t = mps * t_mma;
+    const double t_issue = 200.0 + 45.0 * mps;
+    const double t_l2 = (taps_est * p.kb * 2.0 * (g.kg <= 64 ? 64 : 128) + brows * p.kb * 2.0) / 78.0;
+    if (t_issue > t) t = t_issue;
+    return t_l2 > t ? t_l2 : t;
+  };
+  if (p.kb >= 32 && !p.window && !p.patch && !p.gather && !g.rowpair && g.dw_stride == 0 && !want_pair && !best_shared && g.no_fuse &&
+      !force_share) {
+    const int64_t cols0 = (int64_t)best_tn * best_th * p.pitch - junk;
+    const int64_t tiles0 = (int64_t)((g.n + best_tn - 1) / best_tn) * ((g.p + best_th - 1) / best_th) * mg;
+    const double main0 = ts_est * stage_clk((int64_t)best_tn * best_th * p.pitch, cols0);
+    const double epi0 = epilogue_clk(cols0);
+    double best_split = ((double)((tiles0 + sms - 1) / sms) * (main0 > epi0 ? main0 : epi0) + epi0) * 0.85;
+    for (int th = 1; th <= g.p; ++th) {
+      if ((int64_t)th * p.pitch - junk > 256 || (int64_t)th * g.stride_h > 256) break;
+      if (p.nchw && th != g.p && ((int64_t)th * g.q) % 8 != 0) continue;
+      const int tn_hi = (th == g.p && !p.nchw) ? g.n : 1;
+      for (int tn = 1; tn <= tn_hi; ++tn) {
+        const int64_t cols = (int64_t)tn * th * p.pitch - junk;
+        if (cols > (tn > 1 ? 248 : 256) || tn > 256) break;
+        const int64_t tiles = (int64_t)((g.n + tn - 1) / tn) * ((g.p + th - 1) / th) * mg;
+        for (int ks = 1; ks <= 2 && (ts_est >> ks) >= 2; ++ks) {
+          // (clusters of four do not fill every SM: the GPCs' SM counts are not multiples of four)
+          const int64_t units = tiles << ks, room = ks == 2 ? (int64_t)sms * 8 / 9 : sms;
+          if (units > room) break;  // a cluster per tile, all at once
+          const double ncols = (double)((cols + 15) / 16 * 16);
+          const int stages = (ts_est + (1 << ks) - 1) >> ks;
+          const double cost = stages * stage_clk((int64_t)tn * th * p.pitch, cols) + (p.y_nhwc ? 9000.0 : 5000.0) +
+                              512.0 * ncols * (1.0 - 1.0 / (1 << ks)) / 27.0 + epilogue_clk(cols) / (1 << ks) + 1e-3 * (double)units;
+          if (cost < best_split) {
+            best_split = cost;
+            best_th = th;
+            best_tn = tn;
+            best_ks = ks;
+          }
+        }
+      }
+    }
+  }
   p.est_clk = best;
   // CTA pairs (tcgen05 cta_group::2) for layers with more than 128 output channels per group: a
   // tile is 256 channels x two pixel sub-tiles of at most 128 accumulator columns each.  Every
@@ -2642,7 +2694,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     // transposing staging stores), else plain stores (any shape)
     p.tma_store = (g.kg % 32) == 0 ? 1 : 0;
     p.y_perm = p.tma_store;
-    p.y_rpu = g.q > 32 ? 1 : (kPassElems / g.q < p.th ? kPassElems / g.q : p.th);
+    p.y_rpu = (g.q > 32 || best_ks > 0) ? 1 : (kPassElems / g.q < p.th ? kPassElems / g.q : p.th);  // (split tiles: more warps share them)
     p.y_full_w = g.q > kPassElems ? kPassElems : p.y_rpu * g.q;
     p.rem = g.q > kPassElems ? g.q % kPassElems : (p.th % p.y_rpu) * g.q;
     p.epi_warps = kEpilogueWarps;
@@ -2669,11 +2721,11 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   p.a_bytes = (uint32_t)p.a_rows * p.kb * 2u;
   p.sk_cols32 = (p.ncols + 31) / 32;
   if (p.pair || p.sk_split || g.dw_stride > 0 || p.gather) p.epi_warps = kEpilogueWarps;
-  // split reduction (chosen with the tile shape above): fp32 partials, copy-style epilogue
+  // split reduction (chosen with the tile shape above)
   p.ks_log2 = best_ks;
   if (p.ks_log2 > 0) {
     p.epi_warps = kEpilogueWarps;
-    p.tma_store = 0;
+    if (!p.y_nhwc && p.tma_store && (p.th * g.q) % 32 == 0) p.fine_units = 1;
   }
   // Whole-plane tiles whose 32-channel blocks are contiguous, 16-byte aligned runs in y: one bulk
   // copy per block (epilogue_planes)
@@ -2738,7 +2790,10 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
       p.b_alloc = p.b_bytes;
     }
     p.stage_bytes = p.b_alloc + (uint32_t)(p.nacc > 1 ? p.nacc : 1) * (uint32_t)p.taps * p.a_bytes;
-    p.stages = (int)(budget / p.stage_bytes);
+    // split reductions: room for the parts that the other CTAs send, if three stages still fit
+    const size_t recv = best_ks > 0 ? (size_t)512 * p.ncols : 0;
+    p.recv = best_ks > 0 && recv + 3 * (size_t)p.stage_bytes <= budget;
+    p.stages = (int)((budget - (p.recv ? recv : 0)) / p.stage_bytes);
     if (p.stages > 8) p.stages = 8;
     if (p.stages >= 2) break;
     if (!p.halo) return false;
@@ -2756,8 +2811,9 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     }
   }
   // a second staging tile per epilogue warp (its store overlaps the next unit) if memory is left
-  p.nbuf = (!p.plane_store && (size_t)p.stages * p.stage_bytes + 2u * stage_buf_bytes <= budget_all) ? 2 : 1;
-  p.smem_bytes = (size_t)p.stages * p.stage_bytes + (size_t)p.nbuf * stage_buf_bytes + (p.dw_in_alloc << (1 + p.dw_teams_log2)) + 1024;
+  p.nbuf = (!p.plane_store && !p.recv && (size_t)p.stages * p.stage_bytes + 2u * stage_buf_bytes <= budget_all) ? 2 : 1;
+  p.smem_bytes = (size_t)p.stages * p.stage_bytes + (size_t)p.nbuf * stage_buf_bytes + (p.dw_in_alloc << (1 + p.dw_teams_log2)) + 1024 +
+                 (p.recv ? (size_t)512 * p.ncols : 0);
   // more than half of an SM's shared memory: at most one CTA per SM, so that the kernel can take
   // all 512 TMEM columns without ever waiting for another CTA to free them
   if (p.smem_bytes < 120u * 1024u) p.smem_bytes = 120u * 1024u;
@@ -2773,15 +2829,10 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   p.ws_status_off = 0;
   p.ws_w_off = kWsHeaderBytes;
   p.ws_x_off = p.ws_w_off + round_up_sz(((size_t)g.k << p.dup_log2) * p.eff_r * p.eff_s * p.cw * 2, 256);
-  p.ws_part_off = 0;
   p.ws_total = p.ws_x_off + ((p.nchw || p.x_nhwc) ? 0
                                     : round_up_sz(p.patch    ? (size_t)g.n * g.p * g.q * p.cw * 2
                                                   : p.window ? (size_t)g.n * p.hp * p.wp * p.px_ch * 2 + 256
                                                            : (size_t)g.n * g.h * g.w * p.c_pad * 2, 256));
-  if (p.ks_log2 > 0) {
-    p.ws_part_off = p.ws_total;
-    p.ws_total += round_up_sz(((size_t)g.n * g.k * g.p * g.q * 4) << p.ks_log2, 256);
-  }
   // Layout pass inside the tensor-core kernel (extra warps convert x while the MMAs run; a tile
   // waits for the segments it reads): layers that take the plain NHWC copy of x, planes of a
   // multiple of 4 pixels, whole 8-channel chunks, 8 epilogue warps, NCHW output.
@@ -3047,7 +3098,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   a.acc_stride = a.nacc > 1 ? 512 / a.nacc : 0;
   a.mshift = p.pair + (a.nacc == 4 ? 2 : (a.nacc == 2 ? 1 : 0));
   a.ks_log2 = p.ks_log2;
-  a.part_stride = (int64_t)g.n * g.k * g.p * g.q;
+  a.recv_bytes = p.recv ? 512u * (uint32_t)p.ncols : 0u;
   a.y_tma = (p.y_nhwc && p.tma_store) ? 1 : 0;
   a.y_full_w = p.y_full_w;
   a.y_rpu = p.y_rpu > 0 ? p.y_rpu : 1;
@@ -3078,10 +3129,9 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   a.sk_cols32 = p.sk_cols32;
   a.sk_part = p.sk_split ? reinterpret_cast<float*>(static_cast<char*>(ws) + p.ws_sk_off) : nullptr;
   a.sk_flags = reinterpret_cast<int*>(static_cast<char*>(ws) + p.ws_status_off + kWsFlagsOff);
-  float* partials = p.ks_log2 > 0 ? reinterpret_cast<float*>(static_cast<char*>(ws) + p.ws_part_off) : nullptr;
   const int sms = sm_count();
-  const int64_t units = (int64_t)p.total_tiles << p.ks_log2;
-  dim3 grid((unsigned)(p.ks_log2 > 0 ? (units < sms ? units : sms) : p.grid));
+  // (split reductions: a cluster per tile, which leaves when its tile is done)
+  dim3 grid((unsigned)(p.ks_log2 > 0 ? p.total_tiles << p.ks_log2 : p.grid));
   // CTAs that share a tile wait for one another: all of them must be resident together
   const bool cooperative = p.sk_split != 0;
   int* status = reinterpret_cast<int*>(static_cast<char*>(ws) + p.ws_status_off);
@@ -3094,7 +3144,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, EWV, EPIV, SPLITV>>();            \
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_overlapped(igemm_kernel<KBV, HALOV, EWV, EPIV, SPLITV>, grid, dim3(96 + 32 * EWV), \
-                          p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \
+                          p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, status); \
   } while (0)
   // depthwise + pointwise block: its own instantiations (8 epilogue + 8 depthwise warps)
 #define HGC_LAUNCH_DWPW_EPI(KBV, EPIV)                                                                     \
@@ -3103,7 +3153,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_overlapped(igemm_kernel<KBV, true, 8, EPIV, false, false, false, false, true>, grid, \
                           dim3(96 + 32 * 8 + 32 * kDwWarps), p.smem_bytes, stream, p.tmA, p.tmB, p.tmY,    \
-                          p.tmYr, a, bias, y, partials, status);                                           \
+                          p.tmYr, a, bias, y, status);                                           \
   } while (0)
 #define HGC_LAUNCH_DWPW(KBV)                                   \
   do {                                                         \
@@ -3120,7 +3170,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_coop(true, igemm_kernel<KBV, HALOV, 8, EPIV, false, false, false, true>, grid,   \
                                dim3(96 + 32 * 8 + 32 * kLayoutWarps), p.smem_bytes, stream, p.tmA, p.tmB,  \
-                               p.tmY, p.tmYr, a, bias, y, partials, status);                               \
+                               p.tmY, p.tmYr, a, bias, y, status);                               \
   } while (0)
 #define HGC_LAUNCH_FUSED(KBV, HALOV) HGC_LAUNCH_FUSED_EPI(KBV, HALOV, 0)
   // tiles shared between CTAs: their own instantiations (8 epilogue warps), launched cooperatively
@@ -3130,7 +3180,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     if (err == cudaSuccess)                                                                                \
       err = launch_kernel_coop(true, igemm_kernel<KBV, HALOV, 8, EPIV, false, false, true>, grid,          \
                                dim3(96 + 32 * 8), p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a,    \
-                               bias, y, partials, status);                                                 \
+                               bias, y, status);                                                 \
   } while (0)
 #define HGC_LAUNCH_SHARED(KBV, HALOV)                                \
   do {                                                               \
@@ -3147,6 +3197,20 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     else if (p.epi_warps == kEpilogueWarpsWide) HGC_LAUNCH_IGEMM_EW(KBV, HALOV, 16, 0, false);    \
     else HGC_LAUNCH_IGEMM_EW(KBV, HALOV, 8, 0, false);                                            \
   } while (0)
+  // split reductions: a cluster per tile
+#define HGC_LAUNCH_SPLIT_EPI(KBV, HALOV, EPIV)                                                             \
+  do {                                                                                                     \
+    err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, true>>();                                   \
+    if (err == cudaSuccess)                                                                                \
+      err = launch_kernel_cluster(1u << p.ks_log2, igemm_kernel<KBV, HALOV, 8, EPIV, true>, grid, dim3(96 + 32 * 8), p.smem_bytes, \
+                                  stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, status);                \
+  } while (0)
+#define HGC_LAUNCH_SPLIT(KBV, HALOV)                                \
+  do {                                                              \
+    if (p.y_nhwc) HGC_LAUNCH_SPLIT_EPI(KBV, HALOV, 2);              \
+    else if (!p.tma_store) HGC_LAUNCH_SPLIT_EPI(KBV, HALOV, 1);     \
+    else HGC_LAUNCH_SPLIT_EPI(KBV, HALOV, 0);                       \
+  } while (0)
   // CTA pairs: launched as clusters of two, 8 epilogue warps, the three epilogue kinds
 #define HGC_LAUNCH_PAIR_EPI(KBV, HALOV, EPIV)                                                                  \
   do {                                                                                                       \
@@ -3154,12 +3218,12 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
       err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, false, true, true>>();            \
       if (err == cudaSuccess)                                                                                \
         err = launch_pair(igemm_kernel<KBV, HALOV, 8, EPIV, false, true, true>, p, sms, true,                \
-                          dim3(96 + 32 * 8), stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \
+                          dim3(96 + 32 * 8), stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, status); \
     } else {                                                                                                 \
       err = allow_dynamic_smem<igemm_kernel<KBV, HALOV, 8, EPIV, false, true, false>>();            \
       if (err == cudaSuccess)                                                                                \
         err = launch_pair(igemm_kernel<KBV, HALOV, 8, EPIV, false, true, false>, p, sms, false,              \
-                          dim3(96 + 32 * 8), stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, partials, status); \
+                          dim3(96 + 32 * 8), stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, status); \
     }                                                                                                        \
   } while (0)
 #define HGC_LAUNCH_PAIR(KBV, HALOV)                                \
@@ -3196,7 +3260,13 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     }
   } else
   if (p.ks_log2 > 0) {
-    HGC_LAUNCH_IGEMM_EW(64, true, 8, 1, true);  // the one instantiation with a split reduction
+    if (p.kb == 64) {
+      if (p.halo) HGC_LAUNCH_SPLIT(64, true); else HGC_LAUNCH_SPLIT(64, false);
+    } else if (p.kb == 32) {
+      if (p.halo) HGC_LAUNCH_SPLIT(32, true); else HGC_LAUNCH_SPLIT(32, false);
+    } else {
+      err = cudaErrorInvalidValue;  // (the planner splits only with 32- or 64-channel stages)
+    }
   } else
   if (p.kb == 64) {
     if (p.halo) HGC_LAUNCH_IGEMM(64, true); else HGC_LAUNCH_IGEMM(64, false);
@@ -3206,6 +3276,8 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     if (p.halo) HGC_LAUNCH_IGEMM(16, true); else HGC_LAUNCH_IGEMM(16, false);
   }
 #undef HGC_LAUNCH_IGEMM_EW
+#undef HGC_LAUNCH_SPLIT_EPI
+#undef HGC_LAUNCH_SPLIT
 #undef HGC_LAUNCH_IGEMM
 #undef HGC_LAUNCH_PAIR_EPI
 #undef HGC_LAUNCH_PAIR
@@ -3217,16 +3289,6 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
 #undef HGC_LAUNCH_DWPW
   if (err != cudaSuccess) return err;
   count_launch();
-  if (p.ks_log2 > 0) {
-    const int64_t total = a.part_stride;
-    int64_t blocks = (total + 255) / 256;
-    if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
-    err = launch_kernel(splitk_finish_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, (const float*)partials,
-                        1 << p.ks_log2, a.part_stride, bias, reinterpret_cast<uint16_t*>(y), g.k,
-                        (int64_t)g.p * g.q, total, relu);
-    if (err != cudaSuccess) return err;
-    count_launch();
-  }
   return cudaGetLastError();
 }
 
