@@ -490,6 +490,13 @@ __device__ __noinline__ void sk_preload(uint32_t t_addr, int quarter, int cols32
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
+// (a + b, c + b) in one instruction
+__device__ __forceinline__ void add2(uint32_t a, uint32_t c, float b, float& lo, float& hi) {
+  asm("{\n.reg .b64 x, y;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %4};\nadd.rn.f32x2 x, x, y;\nmov.b64 {%0, %1}, x;\n}\n"
+      : "=f"(lo), "=f"(hi)
+      : "r"(a), "r"(c), "f"(b));
+}
+
 // two fp32 -> packed fp16x2 (round to nearest even), lo = first value; optional ReLU in the convert
 template <bool RELU>
 __device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) {
@@ -512,8 +519,11 @@ __device__ __forceinline__ void convert_store(const uint32_t (&v)[32], int nchun
     if (c < nchunks) {
       uint32_t o[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        o[i] = pack_f16x2<RELU>(__uint_as_float(v[8 * c + 2 * i]) + bv, __uint_as_float(v[8 * c + 2 * i + 1]) + bv);
+      for (int i = 0; i < 4; ++i) {
+        float lo, hi;
+        add2(v[8 * c + 2 * i], v[8 * c + 2 * i + 1], bv, lo, hi);
+        o[i] = pack_f16x2<RELU>(lo, hi);
+      }
       const uint32_t dst = dst0 ^ ((chunk0 + (uint32_t)c) << 4);
       asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3])
                    : "memory");
@@ -755,12 +765,15 @@ __device__ __forceinline__ void convert_store_pixels(const uint32_t (&v)[32], in
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     if (c * 8 < npix) {
-      const uint32_t o0 = pack_f16x2<RELU>(__uint_as_float(v[8 * c + 0]) + bv, __uint_as_float(v[8 * c + 1]) + bv);
-      const uint32_t o1 = pack_f16x2<RELU>(__uint_as_float(v[8 * c + 2]) + bv, __uint_as_float(v[8 * c + 3]) + bv);
-      const uint32_t o2 = pack_f16x2<RELU>(__uint_as_float(v[8 * c + 4]) + bv, __uint_as_float(v[8 * c + 5]) + bv);
-      const uint32_t o3 = pack_f16x2<RELU>(__uint_as_float(v[8 * c + 6]) + bv, __uint_as_float(v[8 * c + 7]) + bv);
+      uint32_t o[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float lo, hi;
+        add2(v[8 * c + 2 * i], v[8 * c + 2 * i + 1], bv, lo, hi);
+        o[i] = pack_f16x2<RELU>(lo, hi);
+      }
       asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)c * 512u),
-                   "r"(o0), "r"(o1), "r"(o2), "r"(o3)
+                   "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3])
                    : "memory");
     }
   }
@@ -1716,6 +1729,96 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       fin_tile = (int)(g_end / a.ts);
       if (g_end > g_beg && g_end % a.ts != 0 && (int64_t)fin_tile * a.ts >= g_beg) fin_item = fin_tile - (int)(g_beg / a.ts);
     }
+    if constexpr (EPI == 0 && !SPLIT && !PAIR && !SHARED && !DWPW) {
+      // The staged TMA-store epilogue on its own loop (see the general one below for what it does): in
+      // layers of short main loops an epilogue warp has one or two units per tile, and the
+      // general loop's bookkeeping was 700 of the 1800 clocks that a tile took it.
+      const bool linear = a.pitch == a.Q;  // no junk columns: accumulator columns are consecutive pixels
+      const int upx = a.fine_units ? 32 : kPassElems;
+      const int e_first = half_eff * upx, e_step = per_eff * upx;
+      int hr_first = 0, wc_first = e_first;  // (row, column) of the warp's first pixel in a tile
+      while (!linear && wc_first >= a.Q) { wc_first -= a.Q; ++hr_first; }
+      const int live_k = a.rowpair ? 64 : a.kg;
+      const bool one_channel_tile = a.mtiles * a.group == 1;
+      const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
+      int grp = 0, m0 = 0;
+      bool live = false;
+      SegIter<false> it;
+      for (it.init(a); it.valid(a); it.next(a), ++lt) {
+        if (lt == 0 || !one_channel_tile) {
+          it.channel_tile(a, grp, m0);
+          live = m0 + cq * 32 < live_k;  // any real output channel in this warp's lanes?
+          const int k = m0 + row < live_k ? grp * a.kg + m0 + row : -2;
+          if (k != bias_k) {
+            bv = 0.f;
+            if (bias != nullptr && k >= 0) {
+              if (HGC_ADDR_OK(bias + k, sizeof(__half))) bv = __half2float(__ldg(bias + k));
+            }
+            bias_k = k;
+          }
+        }
+        const uint32_t buf = lt & 1u;
+        if (!mbar_wait(smem_u32(&acc_full[buf]), (lt >> 1) & 1u, &abort_flag, 256)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (live) {
+          const uint32_t t_addr = t_lane + buf * 256u;
+          const int p0 = it.ph * a.th;
+          const int e_valid = (a.P - p0 < a.th ? a.P - p0 : a.th) * a.Q;  // output pixels of one channel in this tile
+          int hr = hr_first, wc = wc_first;
+          for (int e_lo = e_first; e_lo < e_valid; e_lo += e_step) {
+            const int npx = e_valid - e_lo < upx ? e_valid - e_lo : upx;
+            const uint32_t sbuf = my_stage + stage_sel * kWarpStageBytes;
+            stage_sel = a.nbuf == 2 ? stage_sel ^ 1u : 0u;
+            int uh = hr, uw = wc;  // walks through this unit
+#pragma unroll 1
+            for (int g = 0; g * 32 < npx; ++g) {
+              const int nchunks = npx - g * 32 >= 32 ? 4 : (npx - g * 32) >> 3;
+              uint32_t v[32];
+              // 32 pixels: one wide accumulator load when they are 32 consecutive columns
+              if (nchunks == 4 && (linear || uw + 32 <= a.Q)) {
+                tmem_ld32(t_addr + (uint32_t)(linear ? e_lo + g * 32 : uh * a.pitch + uw), v);
+                uw += 32;
+                if (!linear && uw == a.Q) { uw = 0; ++uh; }
+              } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                  const uint32_t col = (uint32_t)(linear ? e_lo + g * 32 + 8 * c : uh * a.pitch + uw);
+                  uw += 8;
+                  if (!linear && uw == a.Q) { uw = 0; ++uh; }  // next output row: the junk columns of the pitch are skipped
+                  if (c < nchunks) tmem_ld8(t_addr + col, &v[8 * c]);
+                }
+              }
+              if (g == 0) {
+                // this buffer's previous store must have been read out of shared memory
+                if (leader) {
+                  if (a.nbuf == 1) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                  else asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                }
+                __syncwarp();
+              }
+              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+              if (relu) convert_store<true>(v, nchunks, bv, sbuf + row_off, (uint32_t)(g * 4));
+              else convert_store<false>(v, nchunks, bv, sbuf + row_off, (uint32_t)(g * 4));
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (leader) {
+              // past P*Q the store is clipped (row pairs: the next row of y belongs to other warps)
+              const bool full_box = !a.fine_units && (npx == kPassElems || (p0 + a.th >= a.P && !a.rowpair));
+              tma_store_4d(full_box ? &tmY : &tmYr, sbuf, (a.rowpair ? 2 * p0 + odd_row : p0) * a.Q + e_lo, m0 + cq * 32, grp, it.pt * a.tn);
+              asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
+            // first pixel of this warp's next unit
+            wc += e_step;
+            while (!linear && wc >= a.Q) { wc -= a.Q; ++hr; }
+          }
+        }
+        // this warp has read its lanes of the accumulator: hand the buffer back to the MMA issuer
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (leader) mbar_arrive(smem_u32(&acc_empty[buf]));
+      }
+    } else {
     typename WorkIterOf<SPLIT, SHARED>::type it;
     for (it.init(a); it.valid(a); it.next(a), ++lt) {
       if constexpr (!SPLIT && SHARED) {
@@ -2060,6 +2163,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         if constexpr (PAIR) mbar_arrive_cluster(acc_empty_bar);
         else mbar_arrive(acc_empty_bar);
       }
+    }
     }
     // the shared-memory tiles of outstanding stores must stay intact until they have been read (the
     // end of the grid completes the writes)
