@@ -343,7 +343,8 @@ struct IgemmPlan {
   void* y_mapped;  // output pointer tmY/tmYr were encoded for
   uint32_t a_bytes, b_bytes, b_alloc;
   int32_t a_rows;  // rows of a weight tile in shared memory (128, or 64 for layers of <= 64 channels per group)
-  int32_t fine_units;  // TMA-store epilogue works in units of 32 pixels (else 64)
+  int32_t resident;    // weight tiles stay in their ring stages from the first lap on
+  int32_t fine_units;  // TMA-store epilogue works in units of 32 or 16 pixels (0: 64)
   int32_t plane_store; // whole-plane tiles leave as one bulk copy per 32-channel block
   uint32_t plane_bytes;  //   bytes of a lane quarter's staging tile
   int32_t gather;      // 1x1 layer on planes of a multiple of 4 pixels read from x (NCHW) by the kernel's extra warps (a form of nchw)

@@ -812,7 +812,8 @@ struct IgemmArgs {
   int32_t rem;        // (th*Q) % 64: width of the last staged pass of a full tile (0 = none)
   int32_t nbuf;       // staging tiles per epilogue warp (1 or 2)
   int32_t dup_log2;   // log2 of the number of copies of the layer's rows in a weight tile (0, 1, 2)
-  int32_t fine_units; // TMA-store epilogue: units of 32 pixels instead of 64
+  int32_t resident;   // 1: a ring stage holds the same weight tiles on every lap, so they are fetched once (see the planner)
+  int32_t fine_units; // TMA-store epilogue: units of 32 or 16 pixels instead of 64 (0)
   int32_t rowpair;    // lanes 64..127 hold the odd output rows of the layer's 64 channels (IgemmPlan::rowpair)
   int32_t nacc;       // depthwise + pointwise blocks: channel tiles (accumulators) per pixel tile: 1, 2 or 4
   // 1x1 layers on planes that start on 8-byte boundaries only: the extra warps gather the
@@ -1342,7 +1343,10 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           if (weights) {
             // the weight tiles of all taps of the stage as one box (blocks: of the item's channel
             // tiles, one per accumulator, behind one another)
-            if (leader) {
+            if (!PAIR && a.resident && issued >= depth) {
+              // resident weights: this stage has held the same tiles since the first lap of the ring
+              if (leader) mbar_arrive(own_fb);
+            } else if (leader) {
               const uint32_t bytes = (uint32_t)((DWPW ? a.nacc : 1) * a.taps) * a.a_bytes;
               if (!PAIR || rank == 0) mbar_expect_tx(own_fb, (PAIR ? 2u : 1u) * bytes);
               if (!drop) {
@@ -1734,7 +1738,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       // layers of short main loops an epilogue warp has one or two units per tile, and the
       // general loop's bookkeeping was 700 of the 1800 clocks that a tile took it.
       const bool linear = a.pitch == a.Q;  // no junk columns: accumulator columns are consecutive pixels
-      const int upx = a.fine_units ? 32 : kPassElems;
+      const int upx = a.fine_units ? a.fine_units : kPassElems;
       const int e_first = half_eff * upx, e_step = per_eff * upx;
       int hr_first = 0, wc_first = e_first;  // (row, column) of the warp's first pixel in a tile
       while (!linear && wc_first >= a.Q) { wc_first -= a.Q; ++hr_first; }
@@ -1996,7 +2000,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           // (row, column) of the unit's first pixel, kept up to date without divisions
           const bool linear = a.pitch == a.Q;  // no junk columns: accumulator columns are consecutive pixels
           // pixels per unit: 64, or 32 where the replicas would otherwise leave warps without a unit
-          const int upx = a.fine_units ? 32 : kPassElems;
+          const int upx = a.fine_units ? a.fine_units : kPassElems;
           int hr = 0, wc = half_eff * upx;
           while (!linear && wc >= a.Q) { wc -= a.Q; ++hr; }
           for (int e_lo = half_eff * upx; e_lo < e_valid; e_lo += per_eff * upx, ++unit_ctr) {
@@ -2807,20 +2811,27 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   }
   p.sk_split = best_shared;
   p.grid = best_grid;
-  // Layers of exactly 64 output channels and a short reduction whose tiles are bound by the
-  // epilogue (the wide epilogue was chosen): the weight tensor is laid out twice, one copy after the
-  // other, the weight tile is 128 rows again, and all lane quarters hold real channels (see the kernel).
-  if (p.epi_warps == kEpilogueWarpsWide && !p.y_nhwc && p.tma_store && g.group == 1 && best_ks == 0 && !best_shared &&
-      !want_pair && g.dw_stride == 0 && g.kg == 64 && mpt <= 8.0) {
-    // (measured: VGG conv1_1 47.5 -> 41.1 us, 1x1 layers 32 -> 64 and 64 -> 64 channels 7 % faster;
-    //  with a longer reduction the doubled weight traffic costs more than the epilogue gains, and
-    //  four copies of a 32-channel layer were slower than one)
-    p.dup_log2 = 1;
-    p.a_rows = 128;
-    // a tile's units of 64 pixels x 32 channels are fewer than the warps that can now take them:
-    // units of 32 pixels (stored through the remainder map, whose box is then 32 pixels)
-    const int px = p.th * g.q;
-    if (px % 32 == 0 && ((px + 63) / 64) * (g.kg / 32) < p.epi_warps) p.fine_units = 1;
+  // Layers of exactly 64 or 32 output channels and a short reduction whose tiles are bound by the
+  // epilogue: the weight tensor is laid out two or four times, one copy after the other, the weight
+  // tile is 128 rows again, all lane quarters hold real channels (see the kernel) and 16
+  // epilogue warps share the tile's pixels.
+  {
+    const bool resident_ok = ts_est == 1;  // (a layer of one channel tile: its weights are fetched once, see below)
+    const int px = p.th * g.q, copies_log2 = g.kg == 64 ? 1 : 2;
+    if (!p.y_nhwc && p.tma_store && g.group == 1 && best_ks == 0 && !best_shared && !want_pair && g.dw_stride == 0 && !g.rowpair &&
+        !p.gather && g.no_fuse && (g.kg == 64 || g.kg == 32) && mpt <= (resident_ok ? 16.0 : 8.0) && px >= 96) {
+      // (measured: VGG conv1_1 47.5 -> 41.1 us, 1x1 layers 32 -> 64 and 64 -> 64 channels 7 % faster,
+      //  MobileNet's 32-channel stem 30.0 -> 26.6; with a longer reduction the doubled weight traffic costs
+      //  more than the epilogue gains, ResNet-50's stem 76 -> 97, unless the weights stay resident: 60)
+      p.dup_log2 = copies_log2;
+      p.a_rows = 128;
+      p.epi_warps = kEpilogueWarpsWide;
+      // units that 16 warps take in one go, sent through the remainder map, whose box is then a unit
+      // (16 pixels only where 32 do not divide: MobileNet's stem 26.6 us in units of 32, 27.5 of 16)
+      const int quarters = g.kg / 32;
+      if (px % 16 == 0 && (px / 16) * quarters <= kEpilogueWarpsWide) p.fine_units = px % 32 == 0 ? 32 : 16;
+      else if (px % 32 == 0 && (px / 32) * quarters <= kEpilogueWarpsWide) p.fine_units = 32;
+    }
   }
   p.a_bytes = (uint32_t)p.a_rows * p.kb * 2u;
   p.sk_cols32 = (p.ncols + 31) / 32;
@@ -2829,7 +2840,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   p.ks_log2 = best_ks;
   if (p.ks_log2 > 0) {
     p.epi_warps = kEpilogueWarps;
-    if (!p.y_nhwc && p.tma_store && (p.th * g.q) % 32 == 0) p.fine_units = 1;
+    if (!p.y_nhwc && p.tma_store && (p.th * g.q) % 32 == 0) p.fine_units = 32;
   }
   // Whole-plane tiles whose 32-channel blocks are contiguous, 16-byte aligned runs in y: one bulk
   // copy per block (epilogue_planes)
@@ -2912,6 +2923,21 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
       p.ncols = 2 * p.ncols_sub;
     } else {
       p.ncols = (p.tn * p.th * g.q + 15) / 16 * 16;
+    }
+  }
+  // Resident weights: where every tile of a CTA has the same channel tile (the grid is a multiple of
+  // their number) and the ring holds a whole number of tiles' stages, a stage finds the weights it
+  // needs in place after the first lap; only activations are fetched from then on.  The ring is
+  // cut to such a number when at least three stages are left.  (ResNet-50's 7x7 stem fetched 28 KB of
+  // weights for every output row of 13 KB.)
+  p.resident = 0;
+  {
+    const int64_t mgn = (int64_t)p.mtiles * g.group;
+    const int ts = p.cblocks * p.eff_r * (p.eff_s / p.taps), st = p.stages / ts * ts;
+    if (!p.pair && !p.sk_split && best_ks == 0 && p.grid % mgn == 0 && p.total_tiles > p.grid && st > 0 &&
+        (st == p.stages || st >= 3)) {
+      p.resident = 1;
+      p.stages = st;
     }
   }
   // a second staging tile per epilogue warp (its store overlaps the next unit) if memory is left
@@ -3125,7 +3151,7 @@ bool igemm_encode_y_maps(const ConvGeom& g, IgemmPlan* p, void* y) {
   cuuint64_t strides[3] = {pq * 2, pq * 2 * (cuuint64_t)g.kg, pq * 2 * (cuuint64_t)g.k};
   cuuint32_t es[4] = {1, 1, 1, 1};
   for (int i = 0; i < 2; ++i) {
-    cuuint32_t box[4] = {(cuuint32_t)(i == 0 ? kPassElems : (p->fine_units ? 32 : (p->rem == 0 ? kPassElems : p->rem))), 32, 1, 1};
+    cuuint32_t box[4] = {(cuuint32_t)(i == 0 ? kPassElems : (p->fine_units ? p->fine_units : (p->rem == 0 ? kPassElems : p->rem))), 32, 1, 1};
     if (enc(i == 0 ? &p->tmY : &p->tmYr, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, y, dims, strides, box, es,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -3197,6 +3223,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   a.nbuf = p.nbuf;
   a.dup_log2 = p.dup_log2;
   a.fine_units = p.fine_units;
+  a.resident = p.resident;
   a.rowpair = p.rowpair;
   a.nacc = p.nacc > 0 ? p.nacc : 1;
   a.acc_stride = a.nacc > 1 ? 512 / a.nacc : 0;
