@@ -343,6 +343,7 @@ struct IgemmPlan {
   void* y_mapped;  // output pointer tmY/tmYr were encoded for
   uint32_t a_bytes, b_bytes, b_alloc;
   int32_t a_rows;  // rows of a weight tile in shared memory (128, or 64 for layers of <= 64 channels per group)
+  int32_t slabs;       // row pairs: bytes of the weight slabs that stay in shared memory (0: weights in the ring)
   int32_t resident;    // weight tiles stay in their ring stages from the first lap on
   int32_t fine_units;  // TMA-store epilogue works in units of 32 or 16 pixels (0: 64)
   int32_t plane_store; // whole-plane tiles leave as one bulk copy per 32-channel block

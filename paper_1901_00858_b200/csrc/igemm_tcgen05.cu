@@ -812,6 +812,7 @@ struct IgemmArgs {
   int32_t rem;        // (th*Q) % 64: width of the last staged pass of a full tile (0 = none)
   int32_t nbuf;       // staging tiles per epilogue warp (1 or 2)
   int32_t dup_log2;   // log2 of the number of copies of the layer's rows in a weight tile (0, 1, 2)
+  uint32_t slab_off;  // row pairs with all weights in shared memory: where their 64-row slabs lie, bytes from the ring's start (0: none)
   int32_t resident;   // 1: a ring stage holds the same weight tiles on every lap, so they are fetched once (see the planner)
   int32_t fine_units; // TMA-store epilogue: units of 32 or 16 pixels instead of 64 (0)
   int32_t rowpair;    // lanes 64..127 hold the odd output rows of the layer's 64 channels (IgemmPlan::rowpair)
@@ -1198,6 +1199,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __shared__ __align__(8) uint64_t ho_bar;    //   of the warps that hand accumulators over (the first of each lane quarter),
   __shared__ __align__(8) uint64_t pl_bar;    //   of the warps that fetch partial sums (the second of each lane quarter)
   __shared__ __align__(8) uint64_t in_full[2 * kMaxDwTeams], in_empty[2 * kMaxDwTeams];  // depthwise input tiles (depthwise + pointwise blocks)
+  __shared__ __align__(8) uint64_t slabs_full;  // row pairs: the weight slabs have arrived
   __shared__ __align__(8) uint64_t peers_done, parts_in;  // split reduction: the cluster's MMAs are complete; the parts have arrived
   __shared__ __align__(8) uint64_t q_bar[4];  // whole-plane epilogue: meeting point of the two warps of a lane quarter
 
@@ -1218,7 +1220,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.stages; ++s) {
       // (one announcement per producer; blocks: the weights' + one arrival per depthwise / gathering warp)
-      mbar_init(smem_u32(&full_bar[s]), DWPW ? 1 + (kDwWarps >> a.dw_teams_log2) : 2);
+      mbar_init(smem_u32(&full_bar[s]), DWPW ? 1 + (kDwWarps >> a.dw_teams_log2) : (a.slab_off != 0 ? 1 : 2));
       mbar_init(smem_u32(&empty_bar[s]), 1);
     }
     for (int s = 0; s < 2; ++s) {
@@ -1233,6 +1235,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&q_bar[q]), EW / 4);
     mbar_init(smem_u32(&meet_bar), EW);
     mbar_init(smem_u32(&peers_done), 1u << a.ks_log2);
+    mbar_init(smem_u32(&slabs_full), 1);
     mbar_init(smem_u32(&parts_in), EW);
     mbar_init(smem_u32(&ho_bar), EW / 2);
     mbar_init(smem_u32(&pl_bar), EW / 2);
@@ -1285,7 +1288,22 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     const int groups_per_row = a.S / a.taps;  // 1 in halo mode (taps == S), S otherwise (taps == 1)
     typename WorkIterOf<SPLIT, SHARED>::type it;
     const int stages_per_block = a.R * groups_per_row;
-    for (it.init(a); it.valid(a) && ok && !(DWPW && a.gather && !weights); it.next(a)) {
+    // Row pairs with all weights in shared memory: the slabs are fetched once, and the ring carries
+    // activations only.  Weight tile (kernel row r, tap s) is rows [half * 64 + k] = w[r - half][s], so
+    // with the taps' slabs laid out as 0, w[R-2], ..., w[0], 0, w[R-2], ... (a.R = the layer's rows + 1)
+    // it is two neighbouring slabs, starting at slab s * a.R + (a.R - 1 - r).
+    const bool slabs = EPI == 0 && a.slab_off != 0;
+    if (slabs && weights && leader) {
+      const uint32_t bar = smem_u32(&slabs_full);
+      const int n_slabs = a.S * a.R + 1;
+      mbar_expect_tx(bar, (uint32_t)n_slabs * (64u * KB * 2u));
+      for (int i = 0; i < n_slabs; ++i) {
+        // (kernel row a.R - 1 of w' is zero in its first 64 rows)
+        const int r = i % a.R == 0 ? a.R - 1 : a.R - 1 - i % a.R, tap = i / a.R < a.S ? i / a.R : 0;
+        tma_load_4d(ring_base + a.slab_off + (uint32_t)i * (64u * KB * 2u), &tmA, bar, 0, 0, r * a.S + tap, 0);
+      }
+    }
+    for (it.init(a); it.valid(a) && ok && !(DWPW && a.gather && !weights) && !(slabs && weights); it.next(a)) {
       int grp, m0;
       it.channel_tile(a, grp, m0);
       int n0 = it.pt * a.tn;
@@ -1407,7 +1425,11 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       // producer may have given up some stages earlier: its arrivals on those are made up for
       // (otherwise their barriers would never complete).
       const uint32_t first = issued > depth ? issued - depth : 0;
-      if (!DWPW) {
+      if (slabs && weights) {
+        const uint64_t t0 = global_timer_ns();
+        while (!mbar_try_wait(smem_u32(&slabs_full), 0u) && global_timer_ns() - t0 < g_wait_limit_ns) {}
+      }
+      if (!DWPW && !slabs) {
         const uint64_t t0 = global_timer_ns();
         int other;
         while ((other = produced_stages[weights ? 0 : 1]) < 0 && global_timer_ns() - t0 < g_wait_limit_ns) __nanosleep(200);
@@ -1438,8 +1460,12 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     const uint32_t b_step = (uint32_t)a.b_kstep;
     const uint32_t idesc = a.idesc;
     bool ready = mbar_test_warp(smem_u32(&full_bar[0]), 0u);
+    const bool slabs = EPI == 0 && a.slab_off != 0;
+    const uint32_t a_tap = (slabs ? (uint32_t)a.R * (64u * KB * 2u) : a.a_bytes) >> 4;
+    bool ok_slabs = true;
+    if (slabs) ok_slabs = mbar_wait_warp(smem_u32(&slabs_full), 0u, &abort_flag);
     typename WorkIterOf<SPLIT, SHARED>::type it;
-    for (it.init(a); it.valid(a) && ok; it.next(a), ++lt) {  // only the number of stages of an item matters here
+    for (it.init(a); it.valid(a) && ok && ok_slabs; it.next(a), ++lt) {  // only the number of stages of an item matters here
       int s0, s1;
       it.stage_range(a, s0, s1);
       const int groups_per_tile = s1 - s0;
@@ -1470,7 +1496,9 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         const uint32_t sbase = ring_base + ring.idx * a.stage_bytes;
         const uint32_t e_bar = smem_u32(&empty_bar[ring.idx]);
         uint32_t b_lo = b_fix | ((sbase & 0x3FFFFu) >> 4);
-        uint32_t a_lo = a_fix | (((sbase + a.b_alloc) & 0x3FFFFu) >> 4);
+        // (row pairs: one stage per kernel row, its weight tiles in the slabs)
+        const uint32_t abase = slabs ? ring_base + a.slab_off + (uint32_t)(a.R - 1 - gi) * (64u * KB * 2u) : sbase + a.b_alloc;
+        uint32_t a_lo = a_fix | ((abase & 0x3FFFFu) >> 4);
         ring.advance(depth);
         if (elect_one()) {
           if constexpr (DWPW) {
@@ -1482,7 +1510,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           } else {
             issue_mmas<ksteps, PAIR>(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, acc, b_step);
             for (int t = 1; t < a.taps; ++t) {
-              a_lo += a.a_bytes >> 4;
+              a_lo += a_tap;
               b_lo += tap_step >> 4;
               issue_mmas<ksteps, PAIR>(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, 1u, b_step);
             }
@@ -2905,10 +2933,22 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
       p.b_alloc = p.b_bytes;
     }
     p.stage_bytes = p.b_alloc + (uint32_t)(p.nacc > 1 ? p.nacc : 1) * (uint32_t)p.taps * p.a_bytes;
+    // Row pairs of one channel block: the ring's stages hold 2 x 64 weight rows per tap of which half
+    // repeat those of the next kernel row or are zero; as 64-row slabs all of them fit beside a ring
+    // of activations (three 64-channel taps and rows: 104 KB), and are fetched once per CTA instead
+    // of 196 KB per tile.
+    p.slabs = 0;
+    if (g.rowpair && p.cblocks == 1 && p.kb == 64 && p.halo) {
+      const size_t slab_bytes = (size_t)(p.eff_s * p.eff_r + 1) * 64u * p.kb * 2u;
+      if (slab_bytes + 2u * p.b_alloc <= budget) {
+        p.slabs = (int32_t)slab_bytes;
+        p.stage_bytes = p.b_alloc;
+      }
+    }
     // split reductions: room for the parts that the other CTAs send, if three stages still fit
     const size_t recv = best_ks > 0 ? (size_t)512 * p.ncols : 0;
     p.recv = best_ks > 0 && recv + 3 * (size_t)p.stage_bytes <= budget;
-    p.stages = (int)((budget - (p.recv ? recv : 0)) / p.stage_bytes);
+    p.stages = (int)((budget - (p.recv ? recv : 0) - (size_t)p.slabs) / p.stage_bytes);
     if (p.stages > 8) p.stages = 8;
     if (p.stages >= 2) break;
     if (!p.halo) return false;
@@ -2934,15 +2974,15 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   {
     const int64_t mgn = (int64_t)p.mtiles * g.group;
     const int ts = p.cblocks * p.eff_r * (p.eff_s / p.taps), st = p.stages / ts * ts;
-    if (!p.pair && !p.sk_split && best_ks == 0 && p.grid % mgn == 0 && p.total_tiles > p.grid && st > 0 &&
+    if (!p.pair && !p.sk_split && best_ks == 0 && p.slabs == 0 && p.grid % mgn == 0 && p.total_tiles > p.grid && st > 0 &&
         (st == p.stages || st >= 3)) {
       p.resident = 1;
       p.stages = st;
     }
   }
   // a second staging tile per epilogue warp (its store overlaps the next unit) if memory is left
-  p.nbuf = (!p.plane_store && !p.recv && (size_t)p.stages * p.stage_bytes + 2u * stage_buf_bytes <= budget_all) ? 2 : 1;
-  p.smem_bytes = (size_t)p.stages * p.stage_bytes + (size_t)p.nbuf * stage_buf_bytes + (p.dw_in_alloc << (1 + p.dw_teams_log2)) + 1024 +
+  p.nbuf = (!p.plane_store && !p.recv && p.slabs == 0 && (size_t)p.stages * p.stage_bytes + 2u * stage_buf_bytes <= budget_all) ? 2 : 1;
+  p.smem_bytes = (size_t)p.stages * p.stage_bytes + (size_t)p.nbuf * stage_buf_bytes + (size_t)p.slabs + (p.dw_in_alloc << (1 + p.dw_teams_log2)) + 1024 +
                  (p.recv ? (size_t)512 * p.ncols : 0);
   // more than half of an SM's shared memory: at most one CTA per SM, so that the kernel can take
   // all 512 TMEM columns without ever waiting for another CTA to free them
@@ -3050,7 +3090,7 @@ bool igemm_encode_maps(const ConvGeom& g_layer, IgemmPlan* p, void* ws) {
     const cuuint64_t kred = ntaps * p->cw;
     cuuint64_t dims[4] = {(cuuint64_t)p->cw, (cuuint64_t)g.kg << p->dup_log2, ntaps, (cuuint64_t)g.group};  // (replicas: group == 1)
     cuuint64_t strides[3] = {kred * 2, (cuuint64_t)p->cw * 2, kred * 2 * (cuuint64_t)g.kg};
-    cuuint32_t box[4] = {(cuuint32_t)p->kb, (cuuint32_t)p->a_rows, (cuuint32_t)p->taps, 1};
+    cuuint32_t box[4] = {(cuuint32_t)p->kb, (cuuint32_t)(p->slabs != 0 ? 64 : p->a_rows), (cuuint32_t)(p->slabs != 0 ? 1 : p->taps), 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
     if (enc(&p->tmA, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, base + p->ws_w_off, dims, strides, box, es,
             CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -3224,6 +3264,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   a.dup_log2 = p.dup_log2;
   a.fine_units = p.fine_units;
   a.resident = p.resident;
+  a.slab_off = p.slabs != 0 ? (uint32_t)p.stages * p.stage_bytes + (uint32_t)(p.nbuf * p.epi_warps) * kWarpStageBytes : 0u;
   a.rowpair = p.rowpair;
   a.nacc = p.nacc > 0 ? p.nacc : 1;
   a.acc_stride = a.nacc > 1 ? 512 / a.nacc : 0;
