@@ -561,12 +561,13 @@ __device__ __forceinline__ void issue_mmas(uint32_t d_tmem, uint32_t a_lo, uint3
 
 // Where an epilogue reads its fp32 sums: the accumulator in tensor memory (lane = output channel), or,
 // for a tile whose reduction a cluster of CTAs shared (SPLIT), the parts that the CTAs put into this
-// one's shared memory as [part][column][lanes], added up in the order of the parts.
+// one's shared memory as [part][column][lanes], added to the bias in the order of the parts.
 struct AccSource {
   uint32_t addr;        // tensor-memory address of column 0, or shared-memory address of this lane's column 0
   uint32_t col_bytes;   // SPLIT: bytes from column to column and from part to part, and the number of parts
   uint32_t part_bytes;
   int parts;
+  float first;          // SPLIT: what the sum begins with (the bias)
 };
 template <bool SPLIT, int N>
 __device__ __forceinline__ void acc_load(const AccSource& s, uint32_t col, uint32_t* v) {
@@ -576,7 +577,7 @@ __device__ __forceinline__ void acc_load(const AccSource& s, uint32_t col, uint3
   } else {
     float f[N];
 #pragma unroll
-    for (int j = 0; j < N; ++j) f[j] = 0.f;
+    for (int j = 0; j < N; ++j) f[j] = s.first;
     for (int p = 0; p < s.parts; ++p) {
       const uint32_t src = s.addr + (uint32_t)p * s.part_bytes + col * s.col_bytes;
       float t[N];  // (all of a part's loads are under way before the first sum waits for one)
@@ -927,10 +928,11 @@ struct TileIter {
   }
   // reduction slice of this unit (its rank in the cluster) and its range of the tile's ring stages
   __device__ __forceinline__ int slice(const IgemmArgs& a) const { return SPLIT ? (mg & ((1 << a.ks_log2) - 1)) : 0; }
+  // (whole channel blocks, so that the sums do not depend on the tile's shape)
   __device__ __forceinline__ void stage_range(const IgemmArgs& a, int& s0, int& s1) const {
-    const int sl = slice(a);
-    s0 = SPLIT ? (sl * a.ts) >> a.ks_log2 : 0;
-    s1 = SPLIT ? ((sl + 1) * a.ts) >> a.ks_log2 : a.ts;
+    const int sl = slice(a), per_block = a.ts / a.cblocks;
+    s0 = SPLIT ? ((sl * a.cblocks) >> a.ks_log2) * per_block : 0;
+    s1 = SPLIT ? (((sl + 1) * a.cblocks) >> a.ks_log2) * per_block : a.ts;
   }
   __device__ __forceinline__ int kind(const IgemmArgs&) const { return 0; }
   __device__ __forceinline__ bool sub_tile(const IgemmArgs&, int, int&, int&) const { return true; }  // (no CTA pairs here)
@@ -1236,7 +1238,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     mbar_init(smem_u32(&meet_bar), EW);
     mbar_init(smem_u32(&peers_done), 1u << a.ks_log2);
     mbar_init(smem_u32(&slabs_full), 1);
-    mbar_init(smem_u32(&parts_in), EW);
+    mbar_init(smem_u32(&parts_in), a.ks_log2 > 2 ? 2 * EW : EW);
     mbar_init(smem_u32(&ho_bar), EW / 2);
     mbar_init(smem_u32(&pl_bar), EW / 2);
     abort_flag = 0;
@@ -1725,12 +1727,14 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     // two halves do not share pixels, they store to rows 2 * p0 and 2 * p0 + 1.
     // Split reduction: this CTA finishes the part-th share of the tile's channels from shared memory,
     // so here too the warps of all lane quarters share the pixels of those channels.
-    const int rep_q = SPLIT ? 4 >> a.ks_log2 : (EPI == 0 ? (a.rowpair ? 2 : (4 >> a.dup_log2)) : 4);  // lane quarters per replica
+    // (of a cluster of eight the first four finish a quarter each)
+    const int fin_log2 = SPLIT ? (a.ks_log2 < 2 ? a.ks_log2 : 2) : 0;
+    const int rep_q = SPLIT ? 4 >> fin_log2 : (EPI == 0 ? (a.rowpair ? 2 : (4 >> a.dup_log2)) : 4);  // lane quarters per replica
     const int part = SPLIT ? (int)blockIdx.x & ((1 << a.ks_log2) - 1) : 0;
-    const int cq = part * rep_q + (quarter & (rep_q - 1));                   // the quarter's place among the channels
+    const int cq = (part & ((1 << fin_log2) - 1)) * rep_q + (quarter & (rep_q - 1));  // the quarter's place among the channels
     const bool split_px = SPLIT || (EPI == 0 && !a.rowpair);
     const int half_eff = split_px ? (quarter / rep_q) * kPerQuarter + half : half;  // which of the warps that share the pixels
-    const int per_eff = split_px ? (kPerQuarter << (SPLIT ? a.ks_log2 : a.dup_log2)) : kPerQuarter;
+    const int per_eff = split_px ? (kPerQuarter << (SPLIT ? fin_log2 : a.dup_log2)) : kPerQuarter;
     const int odd_row = (EPI == 0 && a.rowpair) ? (quarter >> 1) : 0;
     const int row = cq * 32 + ((EPI == 2 && a.y_tma) ? ((lane & 3) << 3) + (lane >> 2) : lane);
     uint16_t* yb = reinterpret_cast<uint16_t*>(y);
@@ -1969,7 +1973,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       if constexpr (PAIR) {
         if (!it.sub_tile(a, sub, n0, p0)) break;  // (only the last pair tile can lack its second sub-tile)
       }
-      AccSource acc_src{t_tile + (uint32_t)(sub * a.ncols_sub), 0u, 0u, 0};
+      AccSource acc_src{t_tile + (uint32_t)(sub * a.ncols_sub), 0u, 0u, 0, 0.f};
       if constexpr (SPLIT) {
         // Every CTA of the cluster has the sums of its ring stages for all 128 channels in its tensor
         // memory and sends every CTA those of the channels that one finishes, as [part][column][lanes],
@@ -1978,7 +1982,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         // once all MMAs of the cluster are complete.  The transfer runs at about 27 bytes per clock and
         // SM, 1.2 us for 128 columns over four CTAs; waiting for the partners first costs 0.7 us.
         // (The first form of this wrote the parts to global memory for a second kernel to add.)
-        const uint32_t col_bytes = (uint32_t)(128 * 4) >> a.ks_log2;
+        const uint32_t col_bytes = (uint32_t)(128 * 4) >> fin_log2;
         const uint32_t part_bytes = (uint32_t)a.ncols * col_bytes;
         // (reads of whole vectors may run up to 31 columns past the last part: into the staging tiles)
         const uint32_t recv_base = ring_base + (a.recv_bytes != 0 ? (uint32_t)a.stages * a.stage_bytes : 0u);
@@ -2008,11 +2012,13 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         }
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(cluster_addr(smem_u32(&parts_in), dest));
+        if (part >= (1 << fin_log2)) break;  // (this CTA finishes nothing)
         if (!mbar_wait_cluster(smem_u32(&parts_in), 0u, &abort_flag)) {
           gave_up = true;
           break;
         }
-        acc_src = AccSource{recv_base + (uint32_t)((quarter & (rep_q - 1)) * 32 + lane) * 4u, col_bytes, part_bytes, 1 << a.ks_log2};
+        acc_src = AccSource{recv_base + (uint32_t)((quarter & (rep_q - 1)) * 32 + lane) * 4u, col_bytes, part_bytes, 1 << a.ks_log2, bv};
+        bv = 0.f;  // (the sum begins with the bias; one tile per CTA here)
       }
       if constexpr (EPI == 0) {
         // ---- staged epilogue: TMEM -> registers -> swizzled fp16 tile in smem -> TMA store ----
@@ -2248,6 +2254,10 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   }
   return fn;
 }
+
+// Shared memory for the parts of a split tile: fp32, all parts of the channels that a CTA finishes (a
+// quarter at least).
+inline uint32_t split_bytes(int ncols, int ks_log2) { return (ks_log2 > 2 ? 1024u : 512u) * (uint32_t)ncols; }
 
 inline size_t round_up_sz(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -2519,9 +2529,10 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     return t;
   };
   auto epilogue_clk = [&](int64_t cols) { return 600.0 + 10.0 * (double)((cols + 15) / 16 * 16); };
-  auto tile_clk = [&](int64_t brow, int64_t cols) {
-    const double main_loop = mpt * mma_clk(brow, cols);
-    const double epilogue = epilogue_clk(cols);
+  // ks: log2 of the number of CTAs that share the reduction of a tile
+  auto tile_clk = [&](int64_t brow, int64_t cols, int ks) {
+    const double main_loop = mpt / (double)(1 << ks) * mma_clk(brow, cols);
+    const double epilogue = epilogue_clk(cols) * (ks > 0 ? 2.0 : 1.0);
     return (main_loop > epilogue ? main_loop : epilogue) + 300.0;
   };
   // Contiguous ranges of ring stages per CTA (kernels without reduction slices).  Whole tiles per
@@ -2549,6 +2560,15 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     *grid_out = (int)grid;
     *cost_out = (main_loop > epi ? main_loop : epi) + 300.0 * (tiles_per_cta > 1.0 ? tiles_per_cta : 1.0) + hand_over;
   };
+  // Layers whose tiles leave three quarters of the SMs idle (inner products, tiny planes) share the
+  // reduction of a tile between 2, 4 or 8 CTAs.  (What the exchange was estimated at when it
+  // went through global memory; it decides the slices, and with them the order of the sums.)
+  auto finish_clk = [&](int ks) {
+    if (ks == 0) return 0.0;
+    const double elems = (double)g.n * g.k * g.p * g.q;
+    return 8000.0 + elems * (4.0 * (1 << ks) + 2.0) / 3000.0;
+  };
+  const bool can_split = p.kb == 64 && p.halo && !p.nchw && !p.y_nhwc;
   double best = 1e300;
   int best_th = 0, best_tn = 0, best_ks = 0, best_shared = 0, best_grid = 0;
   // shared tiles: asked for (no_split == 0: taken wherever tiles do not fill whole waves), or left
@@ -2574,14 +2594,20 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
         if (in_h > 256 || in_w > 256 || tn * in_h * in_w * p.kb * 2 > 48 * 1024) break;
       }
       const int64_t tiles = (int64_t)((g.n + tn - 1) / tn) * ((g.p + th - 1) / th) * mg;
-      {
-        const int64_t waves = (tiles + sms - 1) / sms;
-        double cost = (double)waves * tile_clk((int64_t)tn * th * p.pitch, cols) + 1e-3 * (double)tiles;
+      for (int ks = 0; ks <= 3; ++ks) {
+        // a slice keeps at least two channel blocks and a main loop of 24 MMAs
+        if (ks > 0 && (!can_split || (p.cblocks >> ks) < 2 || mpt / (1 << ks) < 24.0 || 4 * tiles > sms)) break;
+        const int64_t units = tiles << ks;
+        const int64_t waves = (units + sms - 1) / sms;
+        double cost = (double)waves * tile_clk((int64_t)tn * th * p.pitch, cols, ks) + finish_clk(ks) +
+                      1e-3 * (double)units;
         if (force_share && can_share && tiles % sms != 0) cost *= 1e3;  // shared tiles were asked for (HGC_FLAG_SHARED_TILES)
-        if (cost < best - 1e-9 || (cost < best + 1e-9 && !best_shared && (int64_t)tn * th > (int64_t)best_tn * best_th)) {
+        if (cost < best - 1e-9 ||
+            (cost < best + 1e-9 && ks == best_ks && !best_shared && (int64_t)tn * th > (int64_t)best_tn * best_th)) {
           best = cost;
           best_th = th;
           best_tn = tn;
+          best_ks = ks;
           best_shared = 0;
           best_grid = (int)(tiles < sms ? tiles : sms);
         }
@@ -2596,13 +2622,14 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
           // whole tiles in between (at least 2.5 tiles per unit); the contiguous ranges cost some
           // locality in L2 and the hand-overs some time, together about 10k clocks per launch
           // (conv3_2: 3.03 waves of 11 us tiles, 61.3 -> 55.6 us; conv2_2, conv4_x: slower).
-          cost_s = (double)tiles / (double)sms * tile_clk((int64_t)tn * th * p.pitch, cols) + 10000.0;
+          cost_s = (double)tiles / (double)sms * tile_clk((int64_t)tn * th * p.pitch, cols, 0) + 10000.0;
           if (2 * tiles < 5 * (int64_t)sms || grid_s != sms || ts_est < 16) grid_s = 0;
         }
         if (grid_s > 1 && cost_s < best - 1e-9) {
           best = cost_s;
           best_th = th;
           best_tn = tn;
+          best_ks = 0;
           best_shared = 1;
           best_grid = grid_s;
         }
@@ -2610,7 +2637,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     }
   }
   if (best_th == 0) return false;
-  // Split reductions: the ring stages of a tile dealt out to a cluster of 2 or 4 CTAs, each of which
+  // More split reductions: the channel blocks of a tile dealt out to a cluster of 2 or 4 CTAs, each of which
   // sends the others their channels' sums through distributed shared memory and finishes its own.
   // A layer with few pixels and a long reduction then runs with wide tiles (few bytes per MMA) on all
   // SMs.  Estimated with what bounds a stage of the kernel, measured on B200:
@@ -2620,10 +2647,11 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   //   L2 -> shared memory: about 78 bytes per clock and SM;
   // and of a split tile's end, 512 bytes per column leave at 27 bytes per clock, the waits and the
   // first run of the epilogue take about 5000 clocks (9000 with channels-last output).  Taken only where
-  // that is well below the best whole tiles.  Measured: 512 -> 512 3x3 on 28x28, one image, 18.9 -> 15.0 us;
-  // stride 2 on 14x14, 16 images channels-last, 19.8 -> 14.1; inner products of 64 x 25088 and 64 x 4096
-  // to 4096 41.5 -> 39.0 and 12.3 -> 10.9 (both with partial sums in global memory and a second kernel
-  // before); 256 -> 256 3x3 on 14x14, 16 images, would go from 9.1 to 11.7.
+  // that is well below the best whole tiles, and for reductions of at least 4096 terms (shorter ones gain
+  // little and keep their order of summation).  Measured: 512 -> 512 3x3 on 28x28, one image, 18.9 -> 15.0 us;
+  // stride 2 on 14x14, 16 images channels-last, 19.8 -> 14.1; 256 -> 256 3x3 on 14x14, 16 images, would go
+  // from 9.1 to 11.7.  (Inner products of 64 x 25088 and 64 x 4096 to 4096, split as before but with the
+  // exchange through global memory and a second kernel: 41.5 -> 39.0 and 12.3 -> 10.9.)
   auto stage_clk = [&](int64_t brow, int64_t cols) {
     const double ncols = (double)((cols + 15) / 16 * 16);
     const double brows = p.nchw ? (double)((cols + 63) / 64 * 64) : (double)brow;
@@ -2637,12 +2665,14 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     return t_l2 > t ? t_l2 : t;
   };
   if (p.kb >= 32 && !p.window && !p.patch && !p.gather && !g.rowpair && g.dw_stride == 0 && !want_pair && !best_shared && g.no_fuse &&
-      !force_share) {
+      !force_share && (best_ks == 0 || best_ks > 2) && (int64_t)g.cg * g.r * g.s >= 4096) {
     const int64_t cols0 = (int64_t)best_tn * best_th * p.pitch - junk;
     const int64_t tiles0 = (int64_t)((g.n + best_tn - 1) / best_tn) * ((g.p + best_th - 1) / best_th) * mg;
     const double main0 = ts_est * stage_clk((int64_t)best_tn * best_th * p.pitch, cols0);
     const double epi0 = epilogue_clk(cols0);
     double best_split = ((double)((tiles0 + sms - 1) / sms) * (main0 > epi0 ? main0 : epi0) + epi0) * 0.85;
+    // (clusters of eight are scarce: 64 x 4096 to 1000 13.8 us with them, 10.1 with four)
+    if (best_ks > 2) best_split = 1e300;
     for (int th = 1; th <= g.p; ++th) {
       if ((int64_t)th * p.pitch - junk > 256 || (int64_t)th * g.stride_h > 256) break;
       if (p.nchw && th != g.p && ((int64_t)th * g.q) % 8 != 0) continue;
@@ -2651,12 +2681,12 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
         const int64_t cols = (int64_t)tn * th * p.pitch - junk;
         if (cols > (tn > 1 ? 248 : 256) || tn > 256) break;
         const int64_t tiles = (int64_t)((g.n + tn - 1) / tn) * ((g.p + th - 1) / th) * mg;
-        for (int ks = 1; ks <= 2 && (ts_est >> ks) >= 2; ++ks) {
+        for (int ks = 1; ks <= 2 && (p.cblocks >> ks) >= 1; ++ks) {
           // (clusters of four do not fill every SM: the GPCs' SM counts are not multiples of four)
           const int64_t units = tiles << ks, room = ks == 2 ? (int64_t)sms * 8 / 9 : sms;
           if (units > room) break;  // a cluster per tile, all at once
           const double ncols = (double)((cols + 15) / 16 * 16);
-          const int stages = (ts_est + (1 << ks) - 1) >> ks;
+          const int stages = ((p.cblocks + (1 << ks) - 1) >> ks) * (ts_est / p.cblocks);
           const double cost = stages * stage_clk((int64_t)tn * th * p.pitch, cols) + (p.y_nhwc ? 9000.0 : 5000.0) +
                               512.0 * ncols * (1.0 - 1.0 / (1 << ks)) / 27.0 + epilogue_clk(cols) / (1 << ks) + 1e-3 * (double)units;
           if (cost < best_split) {
@@ -2668,6 +2698,11 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
         }
       }
     }
+  }
+  // eight parts of a tile have to fit into a CTA's shared memory: at most 128 columns
+  while (best_ks > 2 && (int64_t)best_tn * best_th * p.pitch - junk > 128) {
+    if (best_tn > 1) best_tn = (best_tn + 1) / 2;
+    else best_th = (best_th + 1) / 2;
   }
   p.est_clk = best;
   // CTA pairs (tcgen05 cta_group::2) for layers with more than 128 output channels per group: a
@@ -2946,7 +2981,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
       }
     }
     // split reductions: room for the parts that the other CTAs send, if three stages still fit
-    const size_t recv = best_ks > 0 ? (size_t)512 * p.ncols : 0;
+    const size_t recv = best_ks > 0 ? split_bytes(p.ncols, best_ks) : 0;
     p.recv = best_ks > 0 && recv + 3 * (size_t)p.stage_bytes <= budget;
     p.stages = (int)((budget - (p.recv ? recv : 0) - (size_t)p.slabs) / p.stage_bytes);
     if (p.stages > 8) p.stages = 8;
@@ -2983,7 +3018,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   // a second staging tile per epilogue warp (its store overlaps the next unit) if memory is left
   p.nbuf = (!p.plane_store && !p.recv && p.slabs == 0 && (size_t)p.stages * p.stage_bytes + 2u * stage_buf_bytes <= budget_all) ? 2 : 1;
   p.smem_bytes = (size_t)p.stages * p.stage_bytes + (size_t)p.nbuf * stage_buf_bytes + (size_t)p.slabs + (p.dw_in_alloc << (1 + p.dw_teams_log2)) + 1024 +
-                 (p.recv ? (size_t)512 * p.ncols : 0);
+                 (p.recv ? split_bytes(p.ncols, best_ks) : 0u);
   // more than half of an SM's shared memory: at most one CTA per SM, so that the kernel can take
   // all 512 TMEM columns without ever waiting for another CTA to free them
   if (p.smem_bytes < 120u * 1024u) p.smem_bytes = 120u * 1024u;
@@ -3270,7 +3305,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   a.acc_stride = a.nacc > 1 ? 512 / a.nacc : 0;
   a.mshift = p.pair + (a.nacc == 4 ? 2 : (a.nacc == 2 ? 1 : 0));
   a.ks_log2 = p.ks_log2;
-  a.recv_bytes = p.recv ? 512u * (uint32_t)p.ncols : 0u;
+  a.recv_bytes = p.recv ? split_bytes(p.ncols, p.ks_log2) : 0u;
   a.y_tma = (p.y_nhwc && p.tma_store) ? 1 : 0;
   a.y_full_w = p.y_full_w;
   a.y_rpu = p.y_rpu > 0 ? p.y_rpu : 1;

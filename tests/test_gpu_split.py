@@ -1,4 +1,4 @@
-"""Tiles whose reduction a cluster of CTAs shares (plan_info k_slices): both cluster sizes, both stage
+"""Tiles whose reduction a cluster of CTAs shares (plan_info k_slices): all cluster sizes, both stage
 widths, the three epilogues, parts behind the ring and inside it, ragged channels, rows and images.
 Against the oracle, every output; two runs give the same bits (the parts are added in a fixed order)."""
 import numpy as np
@@ -21,19 +21,21 @@ def hgc():
 
 # (n, c, h, w, k, r, stride, channels-last, CTAs per tile)
 CASES = [
-    (8, 512, 13, 13, 320, 3, 1, False, 2),    # copy epilogue, the last channel tile half empty
-    (3, 512, 24, 24, 320, 3, 1, False, 2),    # TMA-store epilogue
+    (1, 3392, 1, 1, 129, 1, 1, False, 8),
+    (8, 512, 13, 13, 320, 3, 1, False, 4),   # copy epilogue, the last channel tile half empty
+    (3, 512, 24, 24, 320, 3, 1, False, 4),   # TMA-store epilogue
     (5, 1000, 28, 28, 130, 3, 1, False, 2),   # 32-channel stages, two live channels in the second tile
-    (8, 1000, 14, 14, 320, 3, 1, True, 2),
-    (2, 520, 28, 28, 130, 3, 1, True, 4),     # channels-last, plain stores
-    (2, 520, 24, 24, 320, 3, 1, True, 4),     # channels-last, staged
+    (8, 1000, 14, 14, 320, 3, 1, True, 2),   # channels-last, staged
+    (2, 1024, 16, 16, 130, 3, 1, True, 4),   # channels-last, plain stores
     (3, 512, 24, 24, 130, 3, 1, False, 4),
-    (1, 200, 3, 3, 32, 3, 2, False, 4),       # smallest: one tap per stage, 16 columns
-    (1, 320, 3, 3, 130, 3, 2, True, 4),
-    (1, 2048, 8, 8, 32, 1, 1, False, 4),      # x read in place
+    (1, 512, 3, 3, 32, 3, 2, False, 4),   # smallest: one tap per stage, 16 columns
+    (2, 1000, 9, 9, 130, 3, 2, True, 4),
     (3, 512, 7, 7, 96, 3, 1, False, 4),
-    (1, 25088, 1, 1, 129, 1, 1, False, 4),    # inner products: one image, ragged channels
+    (1, 25088, 1, 1, 129, 1, 1, False, 4),   # inner products: one image, ragged channels
     (70, 4096, 1, 1, 200, 1, 1, False, 4),
+    (2, 8192, 3, 3, 40, 1, 1, False, 4),
+    (1, 1024, 7, 7, 64, 3, 1, False, 4),
+    (1, 2048, 16, 16, 100, 3, 1, False, 4),
 ]
 
 
