@@ -781,11 +781,11 @@ cudaError_t launch_depthwise3x3(const ConvGeom& g, const __half* x, const __half
   if (g.stride_h == 1) {
     err = allow_dynamic_smem<depthwise3x3_kernel<1>>();
     if (err != cudaSuccess) return err;
-    launch_kernel(depthwise3x3_kernel<1>, dim3((unsigned)ctas), dim3(kThreads), smem, stream, a, xs, w, bias, ys, relu);
+    launch_smem_kernel(depthwise3x3_kernel<1>, dim3((unsigned)ctas), dim3(kThreads), smem, stream, a, xs, w, bias, ys, relu);
   } else {
     err = allow_dynamic_smem<depthwise3x3_kernel<2>>();
     if (err != cudaSuccess) return err;
-    launch_kernel(depthwise3x3_kernel<2>, dim3((unsigned)ctas), dim3(kThreads), smem, stream, a, xs, w, bias, ys, relu);
+    launch_smem_kernel(depthwise3x3_kernel<2>, dim3((unsigned)ctas), dim3(kThreads), smem, stream, a, xs, w, bias, ys, relu);
   }
   count_launch();
   return cudaGetLastError();

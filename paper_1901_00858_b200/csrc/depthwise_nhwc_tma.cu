@@ -310,12 +310,12 @@ cudaError_t launch_depthwise3x3_nhwc_tma(const ConvGeom& g, const __half* x, con
   if (cb == 64) {
     err = allow_dynamic_smem<depthwise3x3_nhwc_tma_kernel<64>>();
     if (err != cudaSuccess) return err;
-    err = launch_kernel(depthwise3x3_nhwc_tma_kernel<64>, dim3((unsigned)blocks), dim3(256), smem, stream, tm, a, ws, bs,
+    err = launch_smem_kernel(depthwise3x3_nhwc_tma_kernel<64>, dim3((unsigned)blocks), dim3(256), smem, stream, tm, a, ws, bs,
                         ys, relu);
   } else {
     err = allow_dynamic_smem<depthwise3x3_nhwc_tma_kernel<32>>();
     if (err != cudaSuccess) return err;
-    err = launch_kernel(depthwise3x3_nhwc_tma_kernel<32>, dim3((unsigned)blocks), dim3(256), smem, stream, tm, a, ws, bs,
+    err = launch_smem_kernel(depthwise3x3_nhwc_tma_kernel<32>, dim3((unsigned)blocks), dim3(256), smem, stream, tm, a, ws, bs,
                         ys, relu);
   }
   if (err != cudaSuccess) return err;

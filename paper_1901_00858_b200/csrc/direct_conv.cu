@@ -111,9 +111,9 @@ cudaError_t launch_direct_conv(const ConvGeom& g, const __half* x, const __half*
   if (total > 2147483647.0) return cudaErrorInvalidConfiguration;
   dim3 grid((unsigned)(px_tiles * ktiles * g.n));
   if (kt == 8)
-    launch_kernel(direct_conv_kernel<8>, dim3(grid), dim3(kThreads), 0, stream, g, x, w, bias, y, relu);
+    launch_smem_kernel(direct_conv_kernel<8>, dim3(grid), dim3(kThreads), 0, stream, g, x, w, bias, y, relu);
   else
-    launch_kernel(direct_conv_kernel<1>, dim3(grid), dim3(kThreads), 0, stream, g, x, w, bias, y, relu);
+    launch_smem_kernel(direct_conv_kernel<1>, dim3(grid), dim3(kThreads), 0, stream, g, x, w, bias, y, relu);
   count_launch();
   return cudaGetLastError();
 }

@@ -57,8 +57,11 @@ cudaError_t depthwise_nhwc_tma_set_wait_limit_ns(uint64_t ns);
 // split as it comes or a quarter, eager: MobileNet at batch 32 304 / 302 / 305 / 293 us, ResNet-50 at
 // batch 64 1111 / 1115 / 1144 / 1075, VGG-16 at batch 16 628 / 629 / 636 / 620, at batch 1 188 / 188 / 184 / 183;
 // as graphs MobileNet 272 / 271 / 294 / 281, ResNet-50 1036 / 1040 / 1112 / 1042.  (All shared memory or
-// none: 3 to 6 % slower.  Kernels with dynamic shared memory keep the default: the preference would
-// halve the blocks of the general depthwise kernel on an SM, 1028 -> 1873 us on 17 x 1024 x 167 x 167.)
+// none: 3 to 6 % slower.)
+// Kernels that work in shared memory themselves keep the default split and overlap only with grids of
+// half a block per SM: the preference would cost them blocks per SM (the general depthwise kernel on
+// 17 x 1024 x 167 x 167 1028 -> 1873 us, the tile transpose on 22 x 80 x 133 x 133 and its layer 115 -> 129),
+// and moving in early under the tensor-core kernel's split too (58 x 192 x 15 x 15 12.5 -> 16.8).
 constexpr int64_t kOverlapThreads = 148 * 512;
 constexpr unsigned kCopyKernelCarveout = 25;  // per cent
 bool launch_overlap_enabled();
@@ -95,7 +98,14 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     overlap = cudaStreamIsCapturing(stream, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone;
   }
-  return launch_kernel_attr(overlap, smem == 0 ? kCopyKernelCarveout : 0, kernel, grid, block, smem, stream, args...);
+  return launch_kernel_attr(overlap, kCopyKernelCarveout, kernel, grid, block, smem, stream, args...);
+}
+// The same for kernels that work in shared memory.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_smem_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                      Args... args) {
+  const bool small = (int64_t)grid.x * grid.y * grid.z <= 74;
+  return launch_kernel_attr(small || launch_overlap_enabled(), 0, kernel, grid, block, smem, stream, args...);
 }
 // The persistent tensor-core kernel is always launched with the attribute: its set-up (barriers,
 // tensor memory) then overlaps the tail of the kernel before it, and where one tensor-core kernel

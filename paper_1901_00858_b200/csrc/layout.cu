@@ -649,13 +649,13 @@ cudaError_t launch_nchw_to_nhwc(const __half* src, __half* dst, int32_t n, int32
     cudaError_t err = allow_dynamic_smem<nchw_to_nhwc_smallplane_kernel>();
     if (err != cudaSuccess) return err;
     dim3 grid2((unsigned)c_tiles, (unsigned)n);
-    launch_kernel(nchw_to_nhwc_smallplane_kernel, dim3(grid2), dim3(kThreads), smem, stream, reinterpret_cast<const uint16_t*>(src),
+    launch_smem_kernel(nchw_to_nhwc_smallplane_kernel, dim3(grid2), dim3(kThreads), smem, stream, reinterpret_cast<const uint16_t*>(src),
                                                                       reinterpret_cast<uint16_t*>(dst), c, (int)hw, c_pad);
     count_launch();
     return cudaGetLastError();
   }
   dim3 grid((unsigned)px_tiles, (unsigned)c_tiles, (unsigned)n);
-  launch_kernel(nchw_to_nhwc_kernel, dim3(grid), dim3(kThreads), 0, stream, reinterpret_cast<const uint16_t*>(src),
+  launch_smem_kernel(nchw_to_nhwc_kernel, dim3(grid), dim3(kThreads), 0, stream, reinterpret_cast<const uint16_t*>(src),
                                                      reinterpret_cast<uint16_t*>(dst), c, hw, c_pad,
                                                      (hw % 8) == 0);
   count_launch();
@@ -669,7 +669,7 @@ cudaError_t launch_nhwc_to_nchw(const __half* src, __half* dst, int32_t n, int32
   const int c_tiles = (c + kTileC - 1) / kTileC;
   if (px_tiles > 0x7fffffffLL || c_tiles > 65535 || n > 65535) return cudaErrorInvalidConfiguration;
   dim3 grid((unsigned)px_tiles, (unsigned)c_tiles, (unsigned)n);
-  launch_kernel(nhwc_to_nchw_kernel, dim3(grid), dim3(kThreads), 0, stream, reinterpret_cast<const uint16_t*>(src),
+  launch_smem_kernel(nhwc_to_nchw_kernel, dim3(grid), dim3(kThreads), 0, stream, reinterpret_cast<const uint16_t*>(src),
                                                      reinterpret_cast<uint16_t*>(dst), c, hw, c_pad,
                                                      (hw % 8) == 0);
   count_launch();
