@@ -366,6 +366,8 @@ struct IgemmPlan {
   // (3x3: 12 MMA steps per two output rows instead of 18).  The plan's shapes are those of the
   // re-stated layer; w' holds the R + 1 shifted copies of the kernel rows (zero where a row has none).
   int32_t rowpair;
+  // 1x1 layers whose rows make no tile of a multiple of 8 pixels: planes taken as rows of 8
+  int32_t flat;
   int32_t dup_log2;  // log2 of the number of copies of the layer's weight rows in w' and in a weight tile (0, 1, 2)
   size_t smem_bytes;
   int32_t ks_log2;  // log2 of the number of reduction slices a tile is split into (0 = none)

@@ -2327,7 +2327,17 @@ static ConvGeom rowpair_geom(const ConvGeom& g) {
   r.rowpair = 1;
   return r;
 }
-static inline ConvGeom effective_geom(const ConvGeom& g, const IgemmPlan& p) { return p.rowpair ? rowpair_geom(g) : g; }
+// A 1x1, stride-1, unpadded layer does not see where the rows of its planes end: the same planes as rows
+// of 8 pixels (IgemmPlan::flat).
+static ConvGeom flat_geom(const ConvGeom& g) {
+  ConvGeom r = g;
+  r.w = r.q = 8;
+  r.h = r.p = (int32_t)((int64_t)g.h * g.w / 8);
+  return r;
+}
+static inline ConvGeom effective_geom(const ConvGeom& g, const IgemmPlan& p) {
+  return p.rowpair ? rowpair_geom(g) : (p.flat ? flat_geom(g) : g);
+}
 
 bool igemm_make_plan(const ConvGeom& g, IgemmPlan* out) {
   // Row pairs: stride-1 layers of exactly 64 output channels with at least two kernel rows and a
@@ -2367,6 +2377,18 @@ bool igemm_make_plan(const ConvGeom& g, IgemmPlan* out) {
       *out = pair;
       return true;
     }
+  }
+  // 1x1 layers that read x as it is need tiles of a multiple of 8 pixels.  Whole rows make none where 8
+  // is reached only beyond 256 pixels (43, 45, 65, 70, 156 a row) or a row is longer than that; rows of
+  // 8 make any.  These layers had fallen to the direct kernel: 1 x 325 -> 726 on 88 x 43 264 -> 7.5 us,
+  // 18 x 208 -> 752 on 8 x 33 265 -> 8.2, 15 x 48 -> 1136 on 60 x 158 2171 -> 86.5 (floor 51).  Layers that
+  // whole rows suit keep them, and their tiles.
+  if (!ok_single && g.r == 1 && g.s == 1 && g.stride_h == 1 && g.stride_w == 1 && g.pad_h == 0 && g.pad_w == 0 &&
+      g.group == 1 && g.cg >= 9 && !g.x_nhwc && !g.y_nhwc && g.dw_stride == 0 && ((int64_t)g.h * g.w) % 8 == 0) {
+    ConvGeom gf = flat_geom(gs);
+    gf.no_gather = 1;
+    ok_single = make_plan_impl(gf, &single, false, 64, false);
+    single.flat = ok_single ? 1 : 0;
   }
   if (ok_single) *out = single;
   return ok_single;
