@@ -150,8 +150,11 @@ int hgc_conv_forward(hgc_conv_desc* d, const void* x, const void* w, const void*
 
 /*
  * Same layer with HOST tensors: copies x, w, bias host->device into the workspace, runs
- * hgc_conv_forward, copies y device->host, all queued on `stream` (asynchronous if the host
- * memory is pinned; the caller synchronises the stream before reading y).  Needs a workspace
+ * hgc_conv_forward, copies y device->host, all ordered in `stream` (asynchronous if the host
+ * memory is pinned; the caller synchronises the stream before reading y).  Batches of a few MB and
+ * more go in chunks of images over internal streams that start behind what `stream` holds and that
+ * it waits for, so that copies in, kernels and copies out overlap; a stream that is being captured
+ * gets the plain sequence.  Needs a workspace
  * of at least hgc_conv_host_workspace_bytes.  x, w, bias, y: host pointers.
  */
 int hgc_conv_forward_host(hgc_conv_desc* d, const void* x, const void* w, const void* bias,
@@ -189,9 +192,8 @@ int hgc_conv_forward_host(hgc_conv_desc* d, const void* x, const void* w, const 
  * Limits and errors: HGC_UNSUPPORTED if the layer is not one the tensor-core path takes (fewer
  * than 9 channels per group unless it is an image stem, very wide rows ...: use hgc_conv_forward)
  * or if p->flags asks for channels-last tensors or the direct path; HGC_NO_WORKSPACE if the layer
- * needs more than the 32 MiB (1 KiB + K*R*S*c_w*2 + N*H*W*c_pad*2 bytes, channels rounded up,
- * + slices*N*K*P*Q*4 for the few layers whose reduction is split into 2, 4 or 8 slices: inner
- * products, tiny planes); HGC_INVALID_ARG / HGC_BAD_ALIGNMENT as for hgc_conv_forward;
+ * needs more than the 32 MiB (1 KiB + K*R*S*c_w*2 + N*H*W*c_pad*2 bytes, channels rounded up);
+ * HGC_INVALID_ARG / HGC_BAD_ALIGNMENT as for hgc_conv_forward;
  * HGC_CUDA_ERROR.  A device-side timeout cannot be read back through this entry point.
  *
  * All calls on a device share the one array, and it keeps the previous call's contents (the
@@ -220,7 +222,7 @@ int hgc_conv_path(const hgc_conv_desc* d, int32_t* path);
  * values under the kernel (few input channels, strided), 4 = x itself, gathered by extra warps of
  * the kernel (1x1 layers on small planes, see HGC_FLAG_GATHER_X), [11] the number of CTAs that share
  * the reduction of one tile (1, or 2 / 4 / 8 for layers with very few tiles, e.g. inner products:
- * each CTA writes fp32 partial sums and a second kernel adds them in a fixed order), [12] the
+ * a cluster whose CTAs send one another their fp32 sums and add them in a fixed order), [12] the
  * number of CTAs of the launch when the ring stages of all tiles are dealt out as contiguous
  * ranges (0 with reduction slices), [13] 1 if those ranges are equal, so that a tile straddling a
  * boundary is reduced by several CTAs inside the one launch (the CTA holding the tile's first
@@ -233,7 +235,8 @@ int hgc_conv_path(const hgc_conv_desc* d, int32_t* path);
  * hold the odd output rows ([4] then counts row pairs per tile, [7] tiles of two output rows, [9]
  * and the kernel's taps are those of a kernel with one more row), [17] the number of copies of the
  * layer's weight rows in a weight tile (2 for epilogue-bound layers of 64 output channels: lane
- * quarters 2 and 3 then hold the same channels as 0 and 1 and take other pixels; else 1), [18] how
+ * quarters 2 and 3 then hold the same channels as 0 and 1 and take other pixels; 4 for those of 32;
+ * else 1), [18] how
  * the epilogue writes y: 1 = staged tiles sent by the copy engine (tensor map over y), 2 = tiles of
  * whole planes of a 1x1 layer, one bulk copy per block of 32 channels (contiguous in y), 0 = plain
  * stores from a staging tile; zeros for the other paths.  info: host pointer; at most 19 values
@@ -318,9 +321,10 @@ int hgc_cast_f32_to_f16(const void* src, void* dst, int64_t count, uint64_t* ove
  * mean_c and var_c (the biased variance) taken per channel over its n*hw values.  The statistics
  * are computed the way the section describes: the values of a channel are partitioned into groups
  * (one image, at most 2048 consecutive pixels), the mean of each group is taken, then the mean
- * of the group means weighted by the group sizes; the centred values are multiplied by
- * 2^shift_log2 before they are squared (the section's 1/32 for large data is -5, its 32 for
- * small data is 5, 0 is no shift) and the variance is shifted back.  All sums are FP32, so the
+ * of the group means weighted by the group sizes; values centred on their group's mean, and the group
+ * means centred on the channel's, are multiplied by 2^shift_log2 before they are squared (the
+ * section's 1/32 for large data is -5, its 32 for small data is 5, 0 is no shift) and the variance
+ * is their sum shifted back.  All sums are FP32, so the
  * result does not depend on shift_log2 (|shift_log2| <= 8).
  * use_stored == 0: mean and var (device, `c` floats each) are WRITTEN; `workspace` must hold
  * hgc_batchnorm_workspace_bytes(n, c, hw) bytes of device memory (16-byte aligned; contents
