@@ -2,11 +2,9 @@
 // a whole number of 16-byte vectors) and the weight re-layout for the implicit-GEMM path.
 // Pure permutations of binary16 bit patterns; bound by HBM bandwidth.
 //
-// Transposes go through a shared-memory tile of kTileC channels x kTileP pixels.  Global
-// accesses are 16-byte vectors wherever the address allows it: always on the NHWC side
-// (c_pad % 8 == 0), and on the NCHW side when the plane size is a multiple of 8 elements (so
-// every channel row of every tile starts on a 16-byte boundary); other planes (7x7, 14x14,
-// 27x27 ...) take 2-byte accesses on the NCHW side.
+// NCHW -> NHWC transposes in registers (aligned planes; other planes with a shift), in a block's shared
+// memory (planes up to 11x11) or, for small tensors, in a shared-memory tile of kTileC channels x
+// kTileP pixels; NHWC -> NCHW in such a tile.  The NHWC side moves 16-byte vectors (c_pad % 8 == 0).
 #include <type_traits>
 
 #include "hgc_internal.h"
@@ -20,10 +18,10 @@ constexpr int kTileP = 64;
 constexpr int kRow = kTileP + 8;  // shared-memory row pitch in elements (16-byte multiple)
 constexpr int kThreads = 256;
 
-// x[n][c][hw] -> x'[n][hw][c_pad]
+// x[n][c][hw] -> x'[n][hw][c_pad] for small tensors of few channels (launch_nchw_to_nhwc)
 __global__ void __launch_bounds__(kThreads)
 nchw_to_nhwc_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst, int c, int64_t hw,
-                    int c_pad, int vec_ok) {
+                    int c_pad) {
   grid_dependency_wait();
   grid_launch_dependents();  // a tensor-core kernel that follows may set itself up beside this one
   __shared__ __align__(16) uint16_t tile[kTileC][kRow];
@@ -33,28 +31,13 @@ nchw_to_nhwc_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst
   const uint16_t* s = src + n * c * hw;
   uint16_t* d = dst + n * hw * c_pad;
 
-  if (vec_ok) {
-    // 64 rows x 8 vectors
-    for (int i = threadIdx.x; i < kTileC * (kTileP / 8); i += kThreads) {
-      const int row = i / (kTileP / 8), v = i % (kTileP / 8);
-      const int ch = c0 + row;
-      const int64_t p = p0 + v * 8;
-      uint4 val = make_uint4(0, 0, 0, 0);
-      if (ch < c && p < hw) {  // hw % 8 == 0
-        const uint4* sp = reinterpret_cast<const uint4*>(s + (int64_t)ch * hw + p);
-        HGC_CHECKED_LOAD(val, sp, *sp);
-      }
-      *reinterpret_cast<uint4*>(&tile[row][v * 8]) = val;
-    }
-  } else {
-    for (int i = threadIdx.x; i < kTileC * kTileP; i += kThreads) {
-      const int row = i / kTileP, col = i % kTileP;
-      const int ch = c0 + row;
-      const int64_t p = p0 + col;
-      uint16_t e = 0;
-      if (ch < c && p < hw) HGC_CHECKED_LOAD(e, s + (int64_t)ch * hw + p, s[(int64_t)ch * hw + p]);
-      tile[row][col] = e;
-    }
+  for (int i = threadIdx.x; i < kTileC * kTileP; i += kThreads) {
+    const int row = i / kTileP, col = i % kTileP;
+    const int ch = c0 + row;
+    const int64_t p = p0 + col;
+    uint16_t e = 0;
+    if (ch < c && p < hw) HGC_CHECKED_LOAD(e, s + (int64_t)ch * hw + p, s[(int64_t)ch * hw + p]);
+    tile[row][col] = e;
   }
   __syncthreads();
   // 64 pixels x 8 channel-vectors; a warp takes 32 consecutive pixels of one channel-vector
@@ -129,6 +112,88 @@ nchw_to_nhwc_regs_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict_
       for (int m = 0; m < 4; ++m) o[m] = __byte_perm(v[2 * m][q >> 1], v[2 * m + 1][q >> 1], sel);
       HGC_CHECKED_STORE(reinterpret_cast<uint4*>(d + (int64_t)q * c_pad),
                         *reinterpret_cast<uint4*>(d + (int64_t)q * c_pad) = make_uint4(o[0], o[1], o[2], o[3]));
+    }
+  }
+}
+
+// The same for planes of any other size, whose channel rows start on any 2-byte boundary: per channel the
+// thread loads the two aligned vectors that its 8 pixels lie in (the second is the next lane's
+// first and comes from L1) and shifts them into place, 15 instructions per 8 pixels.  Where the second
+// vector would end behind the tensor, the thread reads its elements one by one, all at once.
+// The 64 x 64 tile of 2-byte loads that these planes had taken wrote 32 scattered 16-byte pieces per
+// instruction: 22 x 80 on 133x133 67.8 -> 29.9 us (4.2 TB/s), 31 x 665 on 15x51 38.5 -> 14.7,
+// 6 x 99 on 53x67 5.6 -> 4.3.
+__device__ __forceinline__ void shift_left_elements(const uint4& lo, const uint4& hi, uint32_t sh, uint32_t (&v)[4]) {
+  const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+  uint32_t a[6], b[5];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) a[i] = (sh & 4) ? w[i + 2] : w[i];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) b[i] = (sh & 2) ? a[i + 1] : a[i];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = __funnelshift_r(b[i], b[i + 1], (sh & 1) * 16);
+}
+
+template <int CH>
+__global__ void __launch_bounds__(kThreads)
+nchw_to_nhwc_shift_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst, int c, int64_t hw,
+                          int c_pad, int64_t units_p, int units_c, int64_t total_units, int64_t elements) {
+  grid_dependency_wait();
+  grid_launch_dependents();  // a tensor-core kernel that follows may set itself up beside this one
+  constexpr int PG = 32 / CH;
+  const int lane = threadIdx.x & 31;
+  const int c8 = lane % CH, pg = lane / CH;
+  const int64_t warp0 = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
+  for (int64_t u = warp0; u < total_units; u += nwarps) {
+    const int64_t up = u % units_p;
+    const int64_t t = u / units_p;
+    const int uc = (int)(t % units_c);
+    const int64_t n = t / units_c;
+    const int ch = (uc * CH + c8) * 8;
+    const int64_t p = (up * PG + pg) * 8;
+    if (ch >= c_pad || p >= hw) continue;
+    const int live_c = c - ch < 8 ? c - ch : 8;
+    const int live_p = hw - p < 8 ? (int)(hw - p) : 8;
+    const int64_t e0 = (n * c + ch) * hw + p;  // the first pixel of the first channel
+    uint16_t* d = dst + (n * hw + p) * c_pad + ch;
+    uint32_t v[8][4];
+    if (e0 + (live_c - 1) * hw + 16 <= elements) {
+      uint4 lo[8], hi[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        lo[i] = hi[i] = make_uint4(0, 0, 0, 0);
+        if (i < live_c) {
+          const uint4* a = reinterpret_cast<const uint4*>(src + ((e0 + i * hw) & ~(int64_t)7));
+          HGC_CHECKED_LOAD(lo[i], a, __ldg(a));
+          HGC_CHECKED_LOAD(hi[i], a + 1, __ldg(a + 1));
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) shift_left_elements(lo[i], hi[i], (uint32_t)(e0 + i * hw) & 7u, v[i]);
+    } else {
+      uint16_t e[8][8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          e[i][q] = 0;
+          if (i < live_c && q < live_p) HGC_CHECKED_LOAD(e[i][q], src + e0 + i * hw + q, __ldg(src + e0 + i * hw + q));
+        }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[i][q] = (uint32_t)e[i][2 * q] | ((uint32_t)e[i][2 * q + 1] << 16);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const uint32_t sel = (q & 1) ? 0x7632u : 0x5410u;
+      uint32_t o[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) o[m] = __byte_perm(v[2 * m][q >> 1], v[2 * m + 1][q >> 1], sel);
+      if (q < live_p)
+        HGC_CHECKED_STORE(reinterpret_cast<uint4*>(d + (int64_t)q * c_pad),
+                          *reinterpret_cast<uint4*>(d + (int64_t)q * c_pad) = make_uint4(o[0], o[1], o[2], o[3]));
     }
   }
 }
@@ -643,8 +708,10 @@ cudaError_t launch_nchw_to_nhwc(const __half* src, __half* dst, int32_t n, int32
     count_launch();
     return cudaGetLastError();
   }
-  if ((hw % 8) != 0 && hw <= 640 && ((int64_t)c * hw) % 8 == 0 && (kTileC * hw) % 8 == 0) {
-    // small odd plane: contiguous 64-channel spans (at most 80 KB of shared memory)
+  if (hw <= 128 && ((int64_t)c * hw) % 8 == 0) {
+    // small odd plane: contiguous 64-channel spans (at most 16 KB of shared memory).  Up to 11x11: 16 x 512 on
+    // 7x7 2.5 us against 3.5 with the shifting kernel, 64 x 40 on 9x9 2.0 against 3.2; beyond, a block has
+    // too much to do and the other way round: 32 x 256 on 15x15 5.4 against 3.6.
     const size_t smem = (size_t)kTileC * hw * sizeof(uint16_t);
     cudaError_t err = allow_dynamic_smem<nchw_to_nhwc_smallplane_kernel>();
     if (err != cudaSuccess) return err;
@@ -654,10 +721,29 @@ cudaError_t launch_nchw_to_nhwc(const __half* src, __half* dst, int32_t n, int32
     count_launch();
     return cudaGetLastError();
   }
+  if (c_pad >= 64 || (int64_t)n * c * hw >= (1 << 20)) {
+    // (a tensor of few channels and less than a wave of blocks: the tile kernel loads only rows that
+    // exist and is the shorter program to fetch, 4 x 17 on 45x45 2.8 us against 3.3)
+    const int ch_per = c_pad >= 64 ? 8 : 4;
+    const int64_t units_p = ((hw + 7) / 8 + (32 / ch_per) - 1) / (32 / ch_per);
+    const int units_c = (c_pad / 8 + ch_per - 1) / ch_per;
+    const int64_t total_units = units_p * units_c * n;
+    int64_t blocks = (total_units + (kThreads / 32) - 1) / (kThreads / 32);
+    const int64_t cap = (int64_t)sm_count() * 8 * 4;
+    if (blocks > cap) blocks = cap;
+    const uint16_t* s16 = reinterpret_cast<const uint16_t*>(src);
+    uint16_t* d16 = reinterpret_cast<uint16_t*>(dst);
+    const int64_t elements = (int64_t)n * c * hw;
+    if (ch_per == 8)
+      launch_kernel(nchw_to_nhwc_shift_kernel<8>, dim3((unsigned)blocks), dim3(kThreads), 0, stream, s16, d16, c, hw, c_pad, units_p, units_c, total_units, elements);
+    else
+      launch_kernel(nchw_to_nhwc_shift_kernel<4>, dim3((unsigned)blocks), dim3(kThreads), 0, stream, s16, d16, c, hw, c_pad, units_p, units_c, total_units, elements);
+    count_launch();
+    return cudaGetLastError();
+  }
   dim3 grid((unsigned)px_tiles, (unsigned)c_tiles, (unsigned)n);
   launch_smem_kernel(nchw_to_nhwc_kernel, dim3(grid), dim3(kThreads), 0, stream, reinterpret_cast<const uint16_t*>(src),
-                                                     reinterpret_cast<uint16_t*>(dst), c, hw, c_pad,
-                                                     (hw % 8) == 0);
+                                                     reinterpret_cast<uint16_t*>(dst), c, hw, c_pad);
   count_launch();
   return cudaGetLastError();
 }
