@@ -2485,7 +2485,11 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     // (`wide_stages` keeps 64, for CTA pairs and for tiles small enough for three such stages: a
     // copy engine handles about one row of a box per clock whatever the row's width (measured),
     // and with 64-byte rows the rows of a stage take as long as its MMAs.)
-    if (!wide_stages && p.kb == 64 && g.stride_h == 1 && g.stride_w == 1 && g.s >= 3 && g.cg >= 128) p.kb = 32;
+    // 65 to 96 channels take them too, three blocks of 32 in place of two of 64 (a quarter of the MMAs less:
+    // 20 x 80 -> 160 on 56x56 39.0 -> 33.2 us, 4 x 96 -> 96 on 112x112 24.1 -> 20.3), except at 64 or fewer
+    // output channels, where three wide stages fit (50 x 96 -> 48 on 73x192 172 -> 183 with blocks of 32).
+    const bool narrow = g.cg >= 128 || (g.cg > 64 && g.cg <= 96 && g.kg > 64);
+    if (!wide_stages && p.kb == 64 && g.stride_h == 1 && g.stride_w == 1 && g.s >= 3 && narrow) p.kb = 32;
     if (p.kb > kb_max) p.kb = kb_max;
     p.cblocks = (g.cg + p.kb - 1) / p.kb;
     p.cw = p.cblocks * p.kb;
