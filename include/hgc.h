@@ -140,6 +140,10 @@ int hgc_conv_desc_destroy(hgc_conv_desc* d);
  * with X zero outside the image, grp(k) = k / (K/group), fp32 accumulation, bias added in
  * fp32 before the activation, act = max(.,0) if relu != 0 else identity, and one
  * round-to-nearest-even conversion to binary16 at the end.
+ * The order in which the fp32 products are added is fixed for a descriptor: the same tensors give the
+ * same bits on every call.  It depends on the whole layer, n included (how many channels a reduction
+ * block has, whether several CTAs share a tile's reduction), so an image may differ in the last
+ * bits from the same image in a batch of another size.
  * x, w, y: device pointers (required).  bias: device pointer or NULL (no bias).
  * Enqueues on `stream` and returns; results are ready when the stream reaches that point.
  * Errors: HGC_INVALID_ARG (NULL d/x/w/y), HGC_BAD_ALIGNMENT, HGC_NO_WORKSPACE,
@@ -154,7 +158,9 @@ int hgc_conv_forward(hgc_conv_desc* d, const void* x, const void* w, const void*
  * memory is pinned; the caller synchronises the stream before reading y).  Batches of a few MB and
  * more go in chunks of images over internal streams that start behind what `stream` holds and that
  * it waits for, so that copies in, kernels and copies out overlap; a stream that is being captured
- * gets the plain sequence.  Needs a workspace
+ * gets the plain sequence.  Either way y has the bits that hgc_conv_forward gives for this
+ * descriptor: chunks keep the whole layer's order of summation, and a layer whose chunks cannot (tiles
+ * shared by CTAs) goes in one piece.  Needs a workspace
  * of at least hgc_conv_host_workspace_bytes.  x, w, bias, y: host pointers.
  */
 int hgc_conv_forward_host(hgc_conv_desc* d, const void* x, const void* w, const void* bias,

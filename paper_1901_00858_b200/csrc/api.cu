@@ -100,6 +100,89 @@ HostStaging host_staging(const hgc_conv_desc* d) {
   return s;
 }
 
+// hgc_conv_desc_create; want_kb and whole_sums (no tile's reduction shared by CTAs) fix the order of the
+// sums, 0 and false leave it to the planner.
+int create_desc(hgc_conv_desc** out, const hgc_conv_params* p, int32_t want_kb, bool whole_sums) {
+  if (p->n < 1 || p->c < 1 || p->h < 1 || p->w < 1 || p->k < 1 || p->r < 1 || p->s < 1)
+    return HGC_INVALID_ARG;
+  if (p->group < 1 || p->stride_h < 1 || p->stride_w < 1 || p->dil_h < 1 || p->dil_w < 1)
+    return HGC_INVALID_ARG;
+  if (p->pad_h < 0 || p->pad_w < 0) return HGC_INVALID_ARG;
+  if (p->c % p->group != 0 || p->k % p->group != 0) return HGC_INVALID_ARG;
+  const int64_t P = out_extent(p->h, p->r, p->pad_h, p->stride_h, p->dil_h);
+  const int64_t Q = out_extent(p->w, p->s, p->pad_w, p->stride_w, p->dil_w);
+  if (P < 1 || Q < 1) return HGC_INVALID_ARG;
+  if (P > 0x7fffffffLL || Q > 0x7fffffffLL) return HGC_UNSUPPORTED;
+
+  hgc_conv_desc* d = new (std::nothrow) hgc_conv_desc();
+  if (d == nullptr) return HGC_CUDA_ERROR;
+  d->params = *p;
+  hgc::ConvGeom& g = d->geom;
+  g.n = p->n; g.c = p->c; g.h = p->h; g.w = p->w;
+  g.k = p->k; g.r = p->r; g.s = p->s;
+  g.pad_h = p->pad_h; g.pad_w = p->pad_w;
+  g.stride_h = p->stride_h; g.stride_w = p->stride_w;
+  g.dil_h = p->dil_h; g.dil_w = p->dil_w;
+  g.group = p->group;
+  g.p = (int32_t)P; g.q = (int32_t)Q;
+  g.cg = p->c / p->group; g.kg = p->k / p->group;
+  g.x_nhwc = (p->flags & HGC_FLAG_X_NHWC) ? 1 : 0;
+  g.y_nhwc = (p->flags & HGC_FLAG_Y_NHWC) ? 1 : 0;
+  g.no_pair = (p->flags & HGC_FLAG_CTA_PAIRS) ? 0 : 1;
+  g.no_split = (p->flags & HGC_FLAG_WHOLE_TILES) ? 1 : ((p->flags & HGC_FLAG_SHARED_TILES) ? 0 : 2);  // 2: the planner's cost model decides
+  g.no_fuse = (p->flags & HGC_FLAG_FUSED_LAYOUT) ? 0 : 1;
+  g.no_gather = (p->flags & HGC_FLAG_GATHER_X) ? 0 : 1;
+  g.want_kb = want_kb;
+  g.no_cluster = whole_sums ? 1 : 0;
+  if (whole_sums && g.no_split == 2) g.no_split = 1;
+  const bool channels_last = g.x_nhwc || g.y_nhwc;
+
+  d->path = HGC_PATH_DIRECT;
+  d->ws_needed = 0;
+  if (!(p->flags & HGC_FLAG_FORCE_DIRECT)) {
+    if (!channels_last && hgc::depthwise3x3_supported(g)) {
+      d->path = HGC_PATH_DEPTHWISE;
+    } else if (g.x_nhwc && g.y_nhwc && hgc::depthwise3x3_nhwc_supported(g)) {
+      d->path = HGC_PATH_DEPTHWISE;  // channels-last on both sides: its own kernel
+    } else if (hgc::igemm_make_plan(g, &d->igemm)) {
+      d->path = HGC_PATH_IGEMM;
+      d->ws_needed = d->igemm.ws_total;
+    }
+  }
+  // channels-last tensors: the tensor-core path, or a depthwise layer with both sides channels-last
+  if (channels_last && d->path != HGC_PATH_IGEMM && !(d->path == HGC_PATH_DEPTHWISE && g.x_nhwc && g.y_nhwc)) {
+    delete d;
+    return HGC_UNSUPPORTED;
+  }
+  d->ws = nullptr;
+  d->ws_bytes = 0;
+  d->registered_w = nullptr;
+  *out = d;
+  return HGC_OK;
+}
+
+// Whether two plans of one layer, for different numbers of images, add the products of an output in the same
+// order: hgc_conv_forward_host gives the bits that hgc_conv_forward gives.  (The other paths have one order.)
+bool same_sums(const hgc_conv_desc* a, const hgc_conv_desc* b) {
+  if (a->path != b->path) return false;
+  if (a->path != HGC_PATH_IGEMM) return true;
+  const hgc::IgemmPlan &p = a->igemm, &q = b->igemm;
+  return p.kb == q.kb && p.ks_log2 == q.ks_log2 && p.sk_split == 0 && q.sk_split == 0 && p.pair == q.pair &&
+         p.rowpair == q.rowpair && p.window == q.window && p.patch == q.patch;
+}
+
+// The layer of descriptor d for n images with the order of its sums kept; NULL where that cannot be had.
+hgc_conv_desc* chunk_desc(const hgc_conv_desc* d, int32_t n) {
+  hgc_conv_params p = d->params;
+  p.n = n;
+  hgc_conv_desc* sub = nullptr;
+  const bool igemm = d->path == HGC_PATH_IGEMM;
+  if (create_desc(&sub, &p, igemm && d->igemm.kb >= 32 ? d->igemm.kb : 0, igemm && d->igemm.ks_log2 == 0) != HGC_OK) return nullptr;
+  if (same_sums(d, sub)) return sub;
+  hgc_conv_desc_destroy(sub);
+  return nullptr;
+}
+
 // Plans the chunks once; host_count is 1 where the call is not cut up.
 void host_chunks(hgc_conv_desc* d) {
   if (d->host_planned) return;
@@ -115,11 +198,8 @@ void host_chunks(hgc_conv_desc* d) {
   const int32_t per = (int32_t)((d->geom.n + count - 1) / count);
   count = (d->geom.n + per - 1) / per;
   const int32_t last = d->geom.n - (int32_t)(count - 1) * per;
-  hgc_conv_params p = d->params;
-  p.n = per;
-  if (hgc_conv_desc_create(&d->host_sub[0], &p) != HGC_OK) return;
-  p.n = last;
-  if (last != per && hgc_conv_desc_create(&d->host_sub[1], &p) != HGC_OK) {
+  if ((d->host_sub[0] = chunk_desc(d, per)) == nullptr) return;
+  if (last != per && (d->host_sub[1] = chunk_desc(d, last)) == nullptr) {
     hgc_conv_desc_destroy(d->host_sub[0]);
     d->host_sub[0] = nullptr;
     return;
@@ -330,60 +410,7 @@ extern "C" {
 int hgc_conv_desc_create(hgc_conv_desc** out, const hgc_conv_params* p) {
   if (out == nullptr) return HGC_INVALID_ARG;
   *out = nullptr;
-  if (p == nullptr) return HGC_INVALID_ARG;
-  if (p->n < 1 || p->c < 1 || p->h < 1 || p->w < 1 || p->k < 1 || p->r < 1 || p->s < 1)
-    return HGC_INVALID_ARG;
-  if (p->group < 1 || p->stride_h < 1 || p->stride_w < 1 || p->dil_h < 1 || p->dil_w < 1)
-    return HGC_INVALID_ARG;
-  if (p->pad_h < 0 || p->pad_w < 0) return HGC_INVALID_ARG;
-  if (p->c % p->group != 0 || p->k % p->group != 0) return HGC_INVALID_ARG;
-  const int64_t P = out_extent(p->h, p->r, p->pad_h, p->stride_h, p->dil_h);
-  const int64_t Q = out_extent(p->w, p->s, p->pad_w, p->stride_w, p->dil_w);
-  if (P < 1 || Q < 1) return HGC_INVALID_ARG;
-  if (P > 0x7fffffffLL || Q > 0x7fffffffLL) return HGC_UNSUPPORTED;
-
-  hgc_conv_desc* d = new (std::nothrow) hgc_conv_desc();
-  if (d == nullptr) return HGC_CUDA_ERROR;
-  d->params = *p;
-  hgc::ConvGeom& g = d->geom;
-  g.n = p->n; g.c = p->c; g.h = p->h; g.w = p->w;
-  g.k = p->k; g.r = p->r; g.s = p->s;
-  g.pad_h = p->pad_h; g.pad_w = p->pad_w;
-  g.stride_h = p->stride_h; g.stride_w = p->stride_w;
-  g.dil_h = p->dil_h; g.dil_w = p->dil_w;
-  g.group = p->group;
-  g.p = (int32_t)P; g.q = (int32_t)Q;
-  g.cg = p->c / p->group; g.kg = p->k / p->group;
-  g.x_nhwc = (p->flags & HGC_FLAG_X_NHWC) ? 1 : 0;
-  g.y_nhwc = (p->flags & HGC_FLAG_Y_NHWC) ? 1 : 0;
-  g.no_pair = (p->flags & HGC_FLAG_CTA_PAIRS) ? 0 : 1;
-  g.no_split = (p->flags & HGC_FLAG_WHOLE_TILES) ? 1 : ((p->flags & HGC_FLAG_SHARED_TILES) ? 0 : 2);  // 2: the planner's cost model decides
-  g.no_fuse = (p->flags & HGC_FLAG_FUSED_LAYOUT) ? 0 : 1;
-  g.no_gather = (p->flags & HGC_FLAG_GATHER_X) ? 0 : 1;
-  const bool channels_last = g.x_nhwc || g.y_nhwc;
-
-  d->path = HGC_PATH_DIRECT;
-  d->ws_needed = 0;
-  if (!(p->flags & HGC_FLAG_FORCE_DIRECT)) {
-    if (!channels_last && hgc::depthwise3x3_supported(g)) {
-      d->path = HGC_PATH_DEPTHWISE;
-    } else if (g.x_nhwc && g.y_nhwc && hgc::depthwise3x3_nhwc_supported(g)) {
-      d->path = HGC_PATH_DEPTHWISE;  // channels-last on both sides: its own kernel
-    } else if (hgc::igemm_make_plan(g, &d->igemm)) {
-      d->path = HGC_PATH_IGEMM;
-      d->ws_needed = d->igemm.ws_total;
-    }
-  }
-  // channels-last tensors: the tensor-core path, or a depthwise layer with both sides channels-last
-  if (channels_last && d->path != HGC_PATH_IGEMM && !(d->path == HGC_PATH_DEPTHWISE && g.x_nhwc && g.y_nhwc)) {
-    delete d;
-    return HGC_UNSUPPORTED;
-  }
-  d->ws = nullptr;
-  d->ws_bytes = 0;
-  d->registered_w = nullptr;
-  *out = d;
-  return HGC_OK;
+  return p == nullptr ? HGC_INVALID_ARG : create_desc(out, p, 0, false);
 }
 
 int hgc_conv_desc_destroy(hgc_conv_desc* d) {

@@ -2361,8 +2361,8 @@ bool igemm_make_plan(const ConvGeom& g, IgemmPlan* out) {
   ConvGeom gs = g;
   gs.no_pair = 1;
   IgemmPlan single{};
-  bool ok_single = make_plan_impl(gs, &single, false, 64, false);
-  if (ok_single && single.kb == 32 && g.cg > 32) {
+  bool ok_single = make_plan_impl(gs, &single, false, g.want_kb != 0 ? g.want_kb : 64, g.want_kb == 64);
+  if (ok_single && single.kb == 32 && g.cg > 32 && g.want_kb == 0) {
     // the layer was given 32-channel stages for the sake of a deeper ring: where three 64-channel
     // stages fit as well (small pixel tiles: 14x14 and 7x7 planes) they are faster, because the
     // copies then move 128-byte rows (measured: VGG conv5 27.7 -> 22.9 us)
@@ -2622,7 +2622,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
       const int64_t tiles = (int64_t)((g.n + tn - 1) / tn) * ((g.p + th - 1) / th) * mg;
       for (int ks = 0; ks <= 3; ++ks) {
         // a slice keeps at least two channel blocks and a main loop of 24 MMAs
-        if (ks > 0 && (!can_split || (p.cblocks >> ks) < 2 || mpt / (1 << ks) < 24.0 || 4 * tiles > sms)) break;
+        if (ks > 0 && (g.no_cluster || !can_split || (p.cblocks >> ks) < 2 || mpt / (1 << ks) < 24.0 || 4 * tiles > sms)) break;
         const int64_t units = tiles << ks;
         const int64_t waves = (units + sms - 1) / sms;
         double cost = (double)waves * tile_clk((int64_t)tn * th * p.pitch, cols, ks) + finish_clk(ks) +
@@ -2691,7 +2691,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     return t_l2 > t ? t_l2 : t;
   };
   if (p.kb >= 32 && !p.window && !p.patch && !p.gather && !g.rowpair && g.dw_stride == 0 && !want_pair && !best_shared && g.no_fuse &&
-      !force_share && (best_ks == 0 || best_ks > 2) && (int64_t)g.cg * g.r * g.s >= 4096) {
+      !force_share && !g.no_cluster && (best_ks == 0 || best_ks > 2) && (int64_t)g.cg * g.r * g.s >= 4096) {
     const int64_t cols0 = (int64_t)best_tn * best_th * p.pitch - junk;
     const int64_t tiles0 = (int64_t)((g.n + best_tn - 1) / best_tn) * ((g.p + best_th - 1) / best_th) * mg;
     const double main0 = ts_est * stage_clk((int64_t)best_tn * best_th * p.pitch, cols0);

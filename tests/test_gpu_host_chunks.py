@@ -61,3 +61,42 @@ def test_host_forward_in_chunks(hgc, oracle, name, a):
     torch.cuda.synchronize()
     check_close(to_host(y), oracle.conv_fast(oracle.ConvParams(**a), x, w, bias, True), what=name + " (device)")
     d.close()
+
+
+# (name, layer, flags): layers for which the planner, asked for a chunk's few images, would take the sums in
+# another order than for the whole batch: other reduction blocks, tiles shared by CTAs or not
+SAME_BITS = [
+    ("blocks of 32 channels, a chunk alone would take 64", params_dict(4, 128, 112, 112, 128, 3, 3, 1, 1), ""),
+    ("the same, chunks of two and one", params_dict(5, 256, 56, 56, 256, 3, 3, 1, 1), ""),
+    ("a chunk alone would be split over clusters", params_dict(8, 512, 28, 28, 512, 3, 3, 1, 1), ""),
+    ("tiles shared by CTAs in the whole batch", params_dict(16, 256, 56, 56, 256, 3, 3, 1, 1), ""),
+    ("row pairs", params_dict(4, 64, 224, 224, 64, 3, 3, 1, 1), ""),
+    ("stem", params_dict(9, 3, 224, 224, 64, 7, 7, 3, 3, 2, 2), ""),
+    ("1x1 read in place", params_dict(8, 256, 56, 56, 512, 1, 1), ""),
+    ("CTA pairs", params_dict(6, 128, 56, 56, 256, 3, 3, 1, 1), "pairs"),
+    ("depthwise", params_dict(32, 32, 112, 112, 32, 3, 3, 1, 1, 1, 1, 1, 1, 32), ""),
+    ("depthwise channels-last", params_dict(32, 64, 112, 112, 64, 3, 3, 1, 1, 1, 1, 1, 1, 64), "nhwc"),
+]
+
+
+@pytest.mark.parametrize("name,a,how", SAME_BITS, ids=[c[0] for c in SAME_BITS])
+def test_host_forward_gives_the_bits_of_the_device_forward(hgc, name, a, how):
+    import torch
+    flags = {"": 0, "pairs": hgc.HGC_FLAG_CTA_PAIRS, "nhwc": hgc.HGC_FLAG_X_NHWC | hgc.HGC_FLAG_Y_NHWC}[how]
+    g = torch.Generator(device="cuda").manual_seed(a["c"] * 100 + a["n"])
+    d = hgc.ConvDesc(flags=flags, **a)
+    d.ensure_workspace(host=True)
+    n, k, p, q = d.output_dims()
+    rand = lambda *s: (torch.rand(s, generator=g, device="cuda") * 2 - 1).half()   # noqa: E731
+    x = rand(*((n, a["h"], a["w"], a["c"]) if how == "nhwc" else (n, a["c"], a["h"], a["w"])))
+    w, b = rand(k, a["c"] // a["group"], a["r"], a["s"]), rand(k)
+    y = torch.full((n, p, q, k) if how == "nhwc" else (n, k, p, q), float("nan"), dtype=torch.float16, device="cuda")
+    hgc.conv_forward(d, x, w, b, y, False)
+    yh = torch.full(tuple(y.shape), float("nan"), dtype=torch.float16).pin_memory()
+    hgc.conv_forward_host(d, *(t.cpu().pin_memory() for t in (x, w, b)), yh, False)
+    torch.cuda.synchronize()
+    assert d.last_device_status() == hgc.HGC_OK
+    assert bool(torch.isfinite(yh).all())
+    different = int((yh.view(torch.int16) != y.cpu().view(torch.int16)).sum())
+    assert different == 0, f"{name}: {different} of {yh.numel()} values differ"
+    d.close()
