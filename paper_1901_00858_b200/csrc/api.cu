@@ -47,10 +47,13 @@ struct hgc_conv_desc {
   size_t ws_dw_off;             // depthwise weights as [9][C] in the workspace
   const void* registered_w_dw;
   // hgc_conv_forward_host in chunks of images (see host_chunks): the layer for `per` images and, when
-  // that does not divide the batch, for the last chunk's; planned when the host entry points are used
-  bool host_planned, host_user;
-  int32_t host_count, host_per;       // chunks (1: none), images per chunk
-  hgc_conv_desc* host_sub[2];
+  // that does not divide the batch, for the last chunk's; planned when the host entry points are first
+  // used, which several threads may do at once (the query of the workspace's size is one of them)
+  mutable std::mutex host_lock;
+  mutable std::atomic<bool> host_planned;
+  mutable int32_t host_count, host_per;   // chunks (1: none), images per chunk
+  mutable hgc_conv_desc* host_sub[2];
+  bool host_user;
   const void* host_attached;          // the workspace that the chunk descriptors have been attached to
 };
 
@@ -183,10 +186,7 @@ hgc_conv_desc* chunk_desc(const hgc_conv_desc* d, int32_t n) {
   return nullptr;
 }
 
-// Plans the chunks once; host_count is 1 where the call is not cut up.
-void host_chunks(hgc_conv_desc* d) {
-  if (d->host_planned) return;
-  d->host_planned = true;
+void plan_host_chunks(const hgc_conv_desc* d) {
   d->host_count = 1;
   if (d->is_dwpw) return;
   const HostStaging s = host_staging(d);
@@ -206,6 +206,15 @@ void host_chunks(hgc_conv_desc* d) {
   }
   d->host_per = per;
   d->host_count = (int32_t)count;
+}
+
+// Plans the chunks once; host_count is 1 where the call is not cut up.
+void host_chunks(const hgc_conv_desc* d) {
+  if (d->host_planned.load(std::memory_order_acquire)) return;
+  std::lock_guard<std::mutex> hold(d->host_lock);
+  if (d->host_planned.load(std::memory_order_relaxed)) return;
+  plan_host_chunks(d);
+  d->host_planned.store(true, std::memory_order_release);
 }
 
 // Workspace of the chunked form: every chunk's x and y on a 256-byte boundary, then the chunk
@@ -522,8 +531,7 @@ int hgc_conv_workspace_bytes(const hgc_conv_desc* d, size_t* bytes) {
 
 int hgc_conv_host_workspace_bytes(const hgc_conv_desc* d, size_t* bytes) {
   if (d == nullptr || bytes == nullptr) return HGC_INVALID_ARG;
-  hgc_conv_desc* m = const_cast<hgc_conv_desc*>(d);  // (plans the chunks the first time)
-  host_chunks(m);
+  host_chunks(d);
   const HostStaging s = host_staging(d);
   *bytes = s.total;
   if (d->host_count > 1) {

@@ -291,3 +291,31 @@ def test_block_descriptor_validation():
         assert L.hgc_dwpw_desc_create(ctypes.byref(h), ctypes.byref(bad)) == want
     layer = hgc.ConvDesc(1, 32, 8, 8, 32, 3, 3, 1, 1)
     assert L.hgc_dwpw_forward(layer.handle, ptr, ptr, None, ptr, None, ptr, 1, 1, None) == hgc.HGC_INVALID_ARG
+
+
+def test_host_workspace_query_from_several_threads():
+    """hgc_conv_host_workspace_bytes takes a const descriptor: any number of threads may ask one
+    descriptor at once, the first time too, and all get the same answer."""
+    import threading
+    args = (8, 64, 128, 128, 96, 3, 3, 1, 1)   # cut into chunks of images, with a last one of its own
+    want = hgc.ConvDesc(*args).host_workspace_bytes()
+    L = hgc.lib()
+    descs = [hgc.ConvDesc(*args) for _ in range(1500)]
+    workers = 6
+    barrier = threading.Barrier(workers)
+    wrong = []
+
+    def ask():
+        v = ctypes.c_size_t()
+        barrier.wait()
+        for d in descs:
+            L.hgc_conv_host_workspace_bytes(d.handle, ctypes.byref(v))
+            if v.value != want:
+                wrong.append(v.value)
+
+    threads = [threading.Thread(target=ask) for _ in range(workers)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong, (len(wrong), wrong[0], want)
