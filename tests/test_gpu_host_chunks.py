@@ -100,3 +100,26 @@ def test_host_forward_gives_the_bits_of_the_device_forward(hgc, name, a, how):
     different = int((yh.view(torch.int16) != y.cpu().view(torch.int16)).sum())
     assert different == 0, f"{name}: {different} of {yh.numel()} values differ"
     d.close()
+
+
+@pytest.mark.parametrize("shift", [0, 2 * 64 * 224 * 224], ids=["y is x", "y begins two images into x"])
+def test_host_forward_in_place(hgc, shift):
+    """y may lie over x in host memory: all of x is read before any of y is written, however large the batch."""
+    import torch
+    a = params_dict(4, 64, 224, 224, 64, 3, 3, 1, 1)
+    g = torch.Generator().manual_seed(5)
+    d = hgc.ConvDesc(**a)
+    d.ensure_workspace(host=True)
+    rand = lambda *s: (torch.rand(s, generator=g) * 2 - 1).half().pin_memory()   # noqa: E731
+    x, w, b = rand(4, 64, 224, 224), rand(64, 64, 3, 3), rand(64)
+    y = torch.empty((4, 64, 224, 224), dtype=torch.float16).pin_memory()
+    hgc.conv_forward_host(d, x, w, b, y, True)
+    torch.cuda.synchronize()
+    for _ in range(3):
+        both = torch.zeros(x.numel() + shift, dtype=torch.float16).pin_memory()
+        both[:x.numel()] = x.flatten()
+        hgc.conv_forward_host(d, both.data_ptr(), w, b, both.data_ptr() + 2 * shift, True)
+        torch.cuda.synchronize()
+        got = both[shift:shift + y.numel()]
+        assert torch.equal(got.view(torch.int16), y.flatten().view(torch.int16))
+    d.close()
