@@ -161,7 +161,7 @@ int hgc_conv_forward(hgc_conv_desc* d, const void* x, const void* w, const void*
  * gets the plain sequence.  Either way y has the bits that hgc_conv_forward gives for this
  * descriptor: chunks keep the whole layer's order of summation, and a layer whose chunks cannot (tiles
  * shared by CTAs) goes in one piece, and so does one whose y overlaps x (it may: all of x is copied
- * in before any of y is copied out).  Needs a workspace
+ * in before any of y is copied out).  Device weights that were registered are forgotten.  Needs a workspace
  * of at least hgc_conv_host_workspace_bytes.  x, w, bias, y: host pointers.
  */
 int hgc_conv_forward_host(hgc_conv_desc* d, const void* x, const void* w, const void* bias,

@@ -386,6 +386,7 @@ int forward_host_chunks(hgc_conv_desc* d, const HostStaging& h, const ChunkStagi
   bool ok = cudaMemcpyAsync(wd, w, h.w_bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
   if (bias != nullptr) ok = ok && cudaMemcpyAsync(bd, bias, h.b_bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
   const size_t x_image = h.x_bytes / d->geom.n, y_image = h.y_bytes / d->geom.n;
+  d->registered_w = nullptr;  // (as the plain sequence, which overwrites their laid-out form)
   int rc = HGC_OK;
   for (int c = 0; c < d->host_count && ok && rc == HGC_OK; ++c) {
     const bool last = c == d->host_count - 1;

@@ -123,3 +123,25 @@ def test_host_forward_in_place(hgc, shift):
         got = both[shift:shift + y.numel()]
         assert torch.equal(got.view(torch.int16), y.flatten().view(torch.int16))
     d.close()
+
+
+@pytest.mark.parametrize("a", [params_dict(1, 32, 20, 20, 32, 3, 3, 1, 1), params_dict(4, 64, 112, 112, 64, 3, 3, 1, 1)],
+                         ids=["in one piece", "in chunks"])
+def test_host_forward_forgets_registered_weights(hgc, oracle, a):
+    """After a host call device weights are laid out anew on every call, however the host call went."""
+    import torch
+    rng = np.random.default_rng(21)
+    x, w, b = workloads.random_layer_tensors(rng, a["n"], a["c"], a["h"], a["w"], a["k"], 3, 3, 1)
+    w2 = workloads.random_layer_tensors(rng, a["n"], a["c"], a["h"], a["w"], a["k"], 3, 3, 1)[1]
+    d = hgc.ConvDesc(**a)
+    d.ensure_workspace(host=True)
+    xd, wd, bd = to_dev(x), to_dev(w), to_dev(b)
+    d.set_weights(wd)
+    pin = lambda t: torch.from_numpy(t.view(np.int16)).pin_memory()   # noqa: E731
+    hgc.conv_forward_host(d, pin(x), pin(w), pin(b), torch.empty(d.output_dims(), dtype=torch.float16).pin_memory(), True)
+    wd.copy_(to_dev(w2))
+    y = torch.empty(d.output_dims(), dtype=torch.float16, device="cuda")
+    hgc.conv_forward(d, xd, wd, bd, y, True)
+    torch.cuda.synchronize()
+    check_close(to_host(y), oracle.conv_fast(oracle.ConvParams(**a), x, w2, b, True), what=str(a))
+    d.close()
