@@ -156,9 +156,9 @@ int hgc_conv_forward(hgc_conv_desc* d, const void* x, const void* w, const void*
  * Same layer with HOST tensors: copies x, w, bias host->device into the workspace, runs
  * hgc_conv_forward, copies y device->host, all ordered in `stream` (asynchronous if the host
  * memory is pinned; the caller synchronises the stream before reading y).  Batches of a few MB and
- * more go in chunks of images over internal streams that start behind what `stream` holds and that
+ * more in pinned memory go in chunks of images over internal streams that start behind what `stream` holds and that
  * it waits for, so that copies in, kernels and copies out overlap; a stream that is being captured
- * gets the plain sequence.  Either way y has the bits that hgc_conv_forward gives for this
+ * gets the plain sequence, and so does a call that finds all internal streams busy with other callers' work.  Either way y has the bits that hgc_conv_forward gives for this
  * descriptor: chunks keep the whole layer's order of summation, and a layer whose chunks cannot (tiles
  * shared by CTAs) goes in one piece, and so does one whose y overlaps x (it may: all of x is copied
  * in before any of y is copied out).  Device weights that were registered are forgotten.  Needs a workspace

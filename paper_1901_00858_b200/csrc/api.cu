@@ -241,18 +241,19 @@ ChunkStaging chunk_staging(const hgc_conv_desc* d, const HostStaging& h) {
 }
 
 // The streams and events that chunked host calls run on beside the caller's stream: at most
-// kHostLanes per device, made when first needed, taken in turn and given back when the last
-// descriptor that used them is destroyed.  A call holds its lane's lock while it queues its work;
-// calls that share a lane run one after the other on it.
+// kHostLanes per device, made when first needed and given back when the last descriptor that used them is
+// destroyed.  A call takes a lane that nobody else is using: the one that its stream used last (whose work
+// the stream is behind anyway) or one whose work has completed; where there is none it goes in one
+// piece.  So no call waits for another caller's, neither on the device nor, the lock being held only while a
+// lane is looked for, on the host.
 constexpr int kHostLanes = 8;
 constexpr int kMaxHostDevices = 16;
 struct HostLane {
-  std::mutex lock;
-  bool made = false;
+  bool made = false, taken = false;
+  cudaStream_t user = nullptr;  // the stream of the last call
   cudaStream_t compute = nullptr, out = nullptr;
   cudaEvent_t in_done[kMaxHostChunks] = {}, y_done[kMaxHostChunks] = {}, done = nullptr;
   bool make() {
-    if (made) return true;
     bool ok = cudaStreamCreateWithFlags(&compute, cudaStreamNonBlocking) == cudaSuccess &&
               cudaStreamCreateWithFlags(&out, cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreateWithFlags(&done, cudaEventDisableTiming) == cudaSuccess;
@@ -268,7 +269,7 @@ struct HostLane {
     if (compute) cudaStreamDestroy(compute);
     if (out) cudaStreamDestroy(out);
     if (done) cudaEventDestroy(done);
-    compute = out = nullptr;
+    compute = out = user = nullptr;
     done = nullptr;
     for (int i = 0; i < kMaxHostChunks; ++i) {
       if (in_done[i]) cudaEventDestroy(in_done[i]);
@@ -278,19 +279,54 @@ struct HostLane {
     made = false;
   }
 };
+std::mutex g_host_lock;  // over the two below
 HostLane g_host_lanes[kMaxHostDevices][kHostLanes];
-std::atomic<unsigned> g_host_turn{0};
-std::mutex g_host_users_lock;
-int g_host_users = 0;
+int g_host_users = 0;    // descriptors that have used a lane
 
 void host_user_leaves() {
-  std::lock_guard<std::mutex> hold(g_host_users_lock);
+  std::lock_guard<std::mutex> hold(g_host_lock);
   if (--g_host_users > 0) return;
   for (auto& device : g_host_lanes)
-    for (HostLane& lane : device) {
-      std::lock_guard<std::mutex> l(lane.lock);
-      lane.give_back();
+    for (HostLane& lane : device) lane.give_back();
+}
+
+// A lane for one call of descriptor d on stream st, or NULL.
+HostLane* take_lane(hgc_conv_desc* d, int dev, cudaStream_t st) {
+  // (another thread may be capturing in global mode, which forbids this thread to ask for an event or make one)
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+  HostLane* pick = nullptr;
+  {
+    std::lock_guard<std::mutex> hold(g_host_lock);
+    for (HostLane& lane : g_host_lanes[dev])  // (the per-thread default stream is one handle for many streams)
+      if (pick == nullptr && lane.made && !lane.taken && lane.user == st && st != cudaStreamPerThread) pick = &lane;
+    for (HostLane& lane : g_host_lanes[dev])
+      if (pick == nullptr && !lane.taken && (!lane.made || cudaEventQuery(lane.done) == cudaSuccess)) pick = &lane;
+    (void)cudaGetLastError();  // ("not ready" is no error)
+    if (pick != nullptr && !pick->made && !pick->make()) pick = nullptr;
+    if (pick != nullptr) {
+      pick->taken = true;
+      pick->user = st;
+      if (!d->host_user) ++g_host_users;
+      d->host_user = true;
     }
+  }
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  return pick;
+}
+
+void leave_lane(HostLane* lane) {
+  std::lock_guard<std::mutex> hold(g_host_lock);
+  lane->taken = false;
+}
+
+// Whether copies of this host memory are asynchronous.  (Those of pageable memory block the host until they
+// are done, so that chunks could not overlap.)
+bool pinned(const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type == cudaMemoryTypeHost;
+  (void)cudaGetLastError();
+  return false;
 }
 
 // Checked build: the byte ranges that the kernels of one forward call may touch.
@@ -459,17 +495,13 @@ int hgc_conv_forward_host(hgc_conv_desc* d, const void* x, const void* w, const 
     const ChunkStaging cs = chunk_staging(d, s);
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     int dev = kMaxHostDevices;
-    if (d->ws_bytes >= cs.total && cudaStreamIsCapturing(st, &capturing) == cudaSuccess &&
-        capturing == cudaStreamCaptureStatusNone && cudaGetDevice(&dev) == cudaSuccess && dev < kMaxHostDevices) {
-      if (!d->host_user) {
-        std::lock_guard<std::mutex> hold(g_host_users_lock);
-        ++g_host_users;
-        d->host_user = true;
+    if (d->ws_bytes >= cs.total && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone &&
+        cudaGetDevice(&dev) == cudaSuccess && dev < kMaxHostDevices && pinned(x) && pinned(y)) {
+      if (HostLane* lane = take_lane(d, dev, st)) {
+        const int rc = forward_host_chunks(d, s, cs, static_cast<const char*>(x), w, bias, static_cast<char*>(y), relu, st, *lane);
+        leave_lane(lane);
+        return rc;
       }
-      HostLane& lane = g_host_lanes[dev][g_host_turn.fetch_add(1, std::memory_order_relaxed) % kHostLanes];
-      std::lock_guard<std::mutex> hold(lane.lock);
-      if (lane.make())
-        return forward_host_chunks(d, s, cs, static_cast<const char*>(x), w, bias, static_cast<char*>(y), relu, st, lane);
     }
   }
   char* base = static_cast<char*>(d->ws);

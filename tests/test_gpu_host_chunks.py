@@ -145,3 +145,58 @@ def test_host_forward_forgets_registered_weights(hgc, oracle, a):
     torch.cuda.synchronize()
     check_close(to_host(y), oracle.conv_fast(oracle.ConvParams(**a), x, w2, b, True), what=str(a))
     d.close()
+
+
+def test_host_forwards_of_other_streams_are_not_waited_for(hgc):
+    """Calls on a stream that is held up, more of them than the library has internal streams, do not hold up a
+    call on another stream.  Calls on more streams than that, all held up, come out right (they are not
+    timed: so many streams share the device's hardware queues, which make them wait for one another)."""
+    import time
+    import torch
+    a = params_dict(4, 64, 112, 112, 64, 3, 3, 1, 1)
+    tensors = lambda: tuple(torch.rand(s).half().pin_memory() for s in   # noqa: E731
+                            ((4, 64, 112, 112), (64, 64, 3, 3), (64,), (4, 64, 112, 112)))
+    descs = [hgc.ConvDesc(**a) for _ in range(10)]
+    sets = [tensors() for _ in descs]
+    for d in descs:
+        d.ensure_workspace(host=True)
+    streams = [torch.cuda.Stream() for _ in descs]
+    for d, t, s in zip(descs, sets, streams):   # (the first calls make streams)
+        hgc.conv_forward_host(d, *t, True, s)
+    torch.cuda.synchronize()
+    want = sets[-1][3].clone()
+    for held in ([streams[0]] * 9, streams[:9]):
+        sets[-1][3].zero_()
+        with torch.cuda.stream(streams[0]):
+            torch.cuda._sleep(1_500_000_000)   # most of a second
+        for s in set(held) - {streams[0]}:
+            s.wait_stream(streams[0])
+        for d, t, s in zip(descs, sets, held):
+            hgc.conv_forward_host(d, *t, True, s)
+        hgc.conv_forward_host(descs[-1], *sets[-1], True, streams[-1])
+        t0 = time.time()
+        streams[-1].synchronize()
+        took = time.time() - t0
+        if held[0] is held[1]:
+            assert not streams[0].query(), "the held stream is still held"
+            assert took < 0.2, took
+        assert torch.equal(sets[-1][3], want)
+        torch.cuda.synchronize()
+        for d in descs:
+            assert d.last_device_status() == hgc.HGC_OK
+    for d in descs:
+        d.close()
+
+
+def test_host_forward_of_pageable_memory(hgc, oracle):
+    import torch
+    a = params_dict(5, 32, 149, 151, 32, 3, 3, 1, 1)
+    rng = np.random.default_rng(12)
+    x, w, b = workloads.random_layer_tensors(rng, a["n"], a["c"], a["h"], a["w"], a["k"], 3, 3, 1)
+    d = hgc.ConvDesc(**a)
+    d.ensure_workspace(host=True)
+    y = np.full(d.output_dims(), np.nan, np.float16)
+    hgc.conv_forward_host(d, x, w, b, y, True)
+    torch.cuda.synchronize()
+    check_close(y, oracle.conv_fast(oracle.ConvParams(**a), x, w, b, True), what="pageable")
+    d.close()
