@@ -246,8 +246,13 @@ int hgc_conv_path(const hgc_conv_desc* d, int32_t* path);
  * else 1), [18] how
  * the epilogue writes y: 1 = staged tiles sent by the copy engine (tensor map over y), 2 = tiles of
  * whole planes of a 1x1 layer, one bulk copy per block of 32 channels (contiguous in y), 0 = plain
- * stores from a staging tile; zeros for the other paths.  info: host pointer; at most 19 values
- * are written.
+ * stores from a staging tile, [19] 1 if the weight tiles stay in the ring from its first lap on, [20] 1 if
+ * all weights of a row-pair layer lie in shared memory beside the ring, [21] where the parts of a
+ * shared reduction go: 1 = shared memory of their own, 2 = the ring once nobody reads it, 0 = no shared
+ * reduction, [22] the teams that the depthwise warps of a depthwise + pointwise block form (1, 2, 4), [23] 1
+ * if a 1x1 layer's planes are taken as rows of 8 pixels; zeros for the other paths.  For all
+ * paths: [24] the chunks of images that hgc_conv_forward_host works in (1: one piece).  info: host
+ * pointer; at most 25 values are written.
  */
 int hgc_conv_plan_info(const hgc_conv_desc* d, int32_t* info, int32_t count);
 

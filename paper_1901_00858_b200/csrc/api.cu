@@ -539,7 +539,8 @@ int hgc_conv_path(const hgc_conv_desc* d, int32_t* path) {
 
 int hgc_conv_plan_info(const hgc_conv_desc* d, int32_t* info, int32_t count) {
   if (d == nullptr || info == nullptr || count < 1) return HGC_INVALID_ARG;
-  int32_t v[19] = {d->path, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  constexpr int kValues = 25;
+  int32_t v[kValues] = {d->path};
   if (d->path == HGC_PATH_IGEMM) {
     const hgc::IgemmPlan& p = d->igemm;
     v[1] = p.kb; v[2] = p.halo; v[3] = p.tn; v[4] = p.th; v[5] = p.pitch; v[6] = p.ncols;
@@ -553,8 +554,17 @@ int hgc_conv_plan_info(const hgc_conv_desc* d, int32_t* info, int32_t count) {
     v[16] = p.rowpair;
     v[17] = 1 << p.dup_log2;
     v[18] = p.plane_store ? 2 : (p.tma_store ? 1 : 0);
+    v[19] = p.resident;
+    v[20] = p.slabs != 0 ? 1 : 0;
+    v[21] = p.ks_log2 > 0 ? (p.recv ? 1 : 2) : 0;
+    v[22] = d->is_dwpw ? 1 << p.dw_teams_log2 : 0;
+    v[23] = p.flat;
   }
-  for (int i = 0; i < count && i < 19; ++i) info[i] = v[i];
+  if (count >= kValues) {
+    host_chunks(d);
+    v[24] = d->host_count;
+  }
+  for (int i = 0; i < count && i < kValues; ++i) info[i] = v[i];
   return HGC_OK;
 }
 

@@ -114,7 +114,8 @@ def test_planner_paths():
 def test_plan_info_reports_tiling_and_activation_source():
     """The planner runs on the host: its choices can be checked without a GPU."""
     keys = {"path", "kb", "halo", "tn", "th", "pitch", "ncols", "tiles", "stages", "taps", "x_source", "k_slices",
-            "grid", "shared_tiles", "pair", "fused_layout", "row_pairs", "replicas", "y_store"}
+            "grid", "shared_tiles", "pair", "fused_layout", "row_pairs", "replicas", "y_store",
+            "resident", "weight_slabs", "parts", "dw_teams", "flat", "host_chunks"}
     cases = [
         # (n, c, h, w, k, r, s, pad, stride), x_source
         ((16, 256, 56, 56, 256, 3, 3, 1, 1), 0),   # NHWC copy of x
@@ -250,6 +251,8 @@ def test_64_channel_layers_fill_the_mma():
     several kernel rows run as row pairs (odd output rows in the upper lanes: tiles of two rows, one
     more kernel row); epilogue-bound ones with a short reduction hold their weight rows twice."""
     rp = hgc.ConvDesc(16, 64, 224, 224, 64, 3, 3, 1, 1).plan_info()
+    assert rp["weight_slabs"] == 1                                                  # one channel block: all weights stay
+    assert hgc.ConvDesc(2, 96, 224, 224, 64, 3, 3, 1, 1).plan_info()["weight_slabs"] == 0   # two: they stream
     assert rp["row_pairs"] == 1 and rp["th"] == 1 and rp["tiles"] == 16 * 112 and rp["replicas"] == 1
     # not: odd output height, narrow planes, strides, channels-last output, other channel counts
     for args, kw in [((16, 64, 223, 224, 64, 3, 3, 1, 1), {}), ((64, 64, 56, 56, 64, 3, 3, 1, 1), {}),

@@ -38,7 +38,7 @@ def test_flat_planes(hgc, oracle, a):
     info = d.plan_info()
     dims = d.output_dims()
     d.close()
-    assert info["path"] == hgc.HGC_PATH_IGEMM and info["x_source"] == 1 and info["pitch"] == 8, info
+    assert info["path"] == hgc.HGC_PATH_IGEMM and info["x_source"] == 1 and info["flat"] == 1, info
     assert tuple(dims) == (a["n"], a["k"], a["h"], a["w"])
     for relu, bias in ((True, b), (False, None)):
         ref = oracle.conv_fast(oracle.ConvParams(**a), x, w, bias, relu)

@@ -20,20 +20,21 @@ def hgc():
     return binding
 
 
-# (name, layer): 2 MB of x and of y per chunk at least
+# (name, layer, chunks): 2 MB of x and of y per chunk at least
 CASES = [
-    ("3x3, five images in chunks of two and a last one of one", params_dict(5, 32, 149, 151, 32, 3, 3, 1, 1)),
-    ("1x1 read in place, chunks of one", params_dict(3, 128, 96, 96, 128, 1, 1)),
-    ("depthwise, four chunks", params_dict(10, 24, 160, 160, 24, 3, 3, 1, 1, 1, 1, 1, 1, 24)),
-    ("grouped, generic kernel", params_dict(4, 63, 131, 127, 63, 3, 3, 1, 1, 1, 1, 1, 1, 3)),
-    ("below two chunks: one piece", params_dict(3, 16, 100, 100, 16, 3, 3, 1, 1)),
+    ("3x3, five images in chunks of two and a last one of one", params_dict(5, 32, 149, 151, 32, 3, 3, 1, 1), 3),
+    ("1x1 read in place, chunks of one", params_dict(3, 128, 96, 96, 128, 1, 1), 3),
+    ("depthwise, four chunks", params_dict(10, 24, 160, 160, 24, 3, 3, 1, 1, 1, 1, 1, 1, 24), 4),
+    ("grouped, generic kernel", params_dict(4, 63, 131, 127, 63, 3, 3, 1, 1, 1, 1, 1, 1, 3), 2),
+    ("below two chunks: one piece", params_dict(3, 16, 100, 100, 16, 3, 3, 1, 1), 1),
 ]
 
 
-@pytest.mark.parametrize("name,a", CASES, ids=[c[0] for c in CASES])
-def test_host_forward_in_chunks(hgc, oracle, name, a):
+@pytest.mark.parametrize("name,a,chunks", CASES, ids=[c[0] for c in CASES])
+def test_host_forward_in_chunks(hgc, oracle, name, a, chunks):
     import torch
     d = hgc.ConvDesc(**a)
+    assert d.plan_info()["host_chunks"] == chunks
     d.ensure_workspace(host=True)
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
     shape = d.output_dims()
@@ -63,28 +64,29 @@ def test_host_forward_in_chunks(hgc, oracle, name, a):
     d.close()
 
 
-# (name, layer, flags): layers for which the planner, asked for a chunk's few images, would take the sums in
+# (name, layer, flags, chunks): layers for which the planner, asked for a chunk's few images, would take the sums in
 # another order than for the whole batch: other reduction blocks, tiles shared by CTAs or not
 SAME_BITS = [
-    ("blocks of 32 channels, a chunk alone would take 64", params_dict(4, 128, 112, 112, 128, 3, 3, 1, 1), ""),
-    ("the same, chunks of two and one", params_dict(5, 256, 56, 56, 256, 3, 3, 1, 1), ""),
-    ("a chunk alone would be split over clusters", params_dict(8, 512, 28, 28, 512, 3, 3, 1, 1), ""),
-    ("tiles shared by CTAs in the whole batch", params_dict(16, 256, 56, 56, 256, 3, 3, 1, 1), ""),
-    ("row pairs", params_dict(4, 64, 224, 224, 64, 3, 3, 1, 1), ""),
-    ("stem", params_dict(9, 3, 224, 224, 64, 7, 7, 3, 3, 2, 2), ""),
-    ("1x1 read in place", params_dict(8, 256, 56, 56, 512, 1, 1), ""),
-    ("CTA pairs", params_dict(6, 128, 56, 56, 256, 3, 3, 1, 1), "pairs"),
-    ("depthwise", params_dict(32, 32, 112, 112, 32, 3, 3, 1, 1, 1, 1, 1, 1, 32), ""),
-    ("depthwise channels-last", params_dict(32, 64, 112, 112, 64, 3, 3, 1, 1, 1, 1, 1, 1, 64), "nhwc"),
+    ("blocks of 32 channels, a chunk alone would take 64", params_dict(4, 128, 112, 112, 128, 3, 3, 1, 1), "", 4),
+    ("the same, chunks of two and one", params_dict(5, 256, 56, 56, 256, 3, 3, 1, 1), "", 3),
+    ("a chunk alone would be split over clusters", params_dict(8, 512, 28, 28, 512, 3, 3, 1, 1), "", 3),
+    ("tiles shared by CTAs in the whole batch", params_dict(16, 256, 56, 56, 256, 3, 3, 1, 1), "", 1),
+    ("row pairs", params_dict(4, 64, 224, 224, 64, 3, 3, 1, 1), "", 4),
+    ("stem", params_dict(33, 3, 224, 224, 64, 7, 7, 3, 3, 2, 2), "", 4),
+    ("1x1 read in place", params_dict(8, 256, 56, 56, 512, 1, 1), "", 4),
+    ("CTA pairs whose chunks would take other blocks", params_dict(6, 128, 56, 56, 256, 3, 3, 1, 1), "pairs", 1),
+    ("depthwise", params_dict(32, 32, 112, 112, 32, 3, 3, 1, 1, 1, 1, 1, 1, 32), "", 4),
+    ("depthwise channels-last", params_dict(32, 64, 112, 112, 64, 3, 3, 1, 1, 1, 1, 1, 1, 64), "nhwc", 4),
 ]
 
 
-@pytest.mark.parametrize("name,a,how", SAME_BITS, ids=[c[0] for c in SAME_BITS])
-def test_host_forward_gives_the_bits_of_the_device_forward(hgc, name, a, how):
+@pytest.mark.parametrize("name,a,how,chunks", SAME_BITS, ids=[c[0] for c in SAME_BITS])
+def test_host_forward_gives_the_bits_of_the_device_forward(hgc, name, a, how, chunks):
     import torch
     flags = {"": 0, "pairs": hgc.HGC_FLAG_CTA_PAIRS, "nhwc": hgc.HGC_FLAG_X_NHWC | hgc.HGC_FLAG_Y_NHWC}[how]
     g = torch.Generator(device="cuda").manual_seed(a["c"] * 100 + a["n"])
     d = hgc.ConvDesc(flags=flags, **a)
+    assert d.plan_info()["host_chunks"] == chunks, d.plan_info()
     d.ensure_workspace(host=True)
     n, k, p, q = d.output_dims()
     rand = lambda *s: (torch.rand(s, generator=g, device="cuda") * 2 - 1).half()   # noqa: E731

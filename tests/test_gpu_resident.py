@@ -40,7 +40,7 @@ def test_resident_weights(hgc, oracle, a, replicas):
     d = hgc.ConvDesc(**a)
     info = d.plan_info()
     d.close()
-    assert info["replicas"] == replicas and info["tiles"] > info["grid"], info
+    assert info["resident"] == 1 and info["replicas"] == replicas and info["tiles"] > info["grid"], info
     for relu, bias in ((True, b), (False, None)):
         ref = oracle.conv_fast(oracle.ConvParams(**a), x, w, bias, relu)
         got, _ = run_layer(hgc, a, x, w, bias, relu, register_weights=True)
