@@ -91,7 +91,9 @@ typedef struct hgc_conv_params {
  * takes this schedule only where its cost model expects a gain (long tiles, at least 2.5 per
  * CTA, a last wave that is mostly empty: VGG-16's 256-channel layers on 56x56 planes at batch
  * 16, 61 -> 56 us); with it, wherever the tiles do not fill whole waves.
- * HGC_FLAG_WHOLE_TILES: never (smaller workspace; ordinary launch).  Wins over the flag above.
+ * HGC_FLAG_WHOLE_TILES: never (smaller workspace; ordinary launch).  Wins over the flag above.  With
+ * it the reduction of a tile is not dealt out to a cluster of CTAs either, except in layers whose tiles
+ * would leave three quarters of the SMs idle (inner products, tiny planes).
  */
 #define HGC_FLAG_CTA_PAIRS 8
 #define HGC_FLAG_SHARED_TILES 16

@@ -136,7 +136,7 @@ int create_desc(hgc_conv_desc** out, const hgc_conv_params* p, int32_t want_kb, 
   g.no_fuse = (p->flags & HGC_FLAG_FUSED_LAYOUT) ? 0 : 1;
   g.no_gather = (p->flags & HGC_FLAG_GATHER_X) ? 0 : 1;
   g.want_kb = want_kb;
-  g.no_cluster = whole_sums ? 1 : 0;
+  g.no_cluster = whole_sums ? 1 : ((p->flags & HGC_FLAG_WHOLE_TILES) ? 2 : 0);
   if (whole_sums && g.no_split == 2) g.no_split = 1;
   const bool channels_last = g.x_nhwc || g.y_nhwc;
 

@@ -2622,7 +2622,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
       const int64_t tiles = (int64_t)((g.n + tn - 1) / tn) * ((g.p + th - 1) / th) * mg;
       for (int ks = 0; ks <= 3; ++ks) {
         // a slice keeps at least two channel blocks and a main loop of 24 MMAs
-        if (ks > 0 && (g.no_cluster || !can_split || (p.cblocks >> ks) < 2 || mpt / (1 << ks) < 24.0 || 4 * tiles > sms)) break;
+        if (ks > 0 && (g.no_cluster == 1 || !can_split || (p.cblocks >> ks) < 2 || mpt / (1 << ks) < 24.0 || 4 * tiles > sms)) break;
         const int64_t units = tiles << ks;
         const int64_t waves = (units + sms - 1) / sms;
         double cost = (double)waves * tile_clk((int64_t)tn * th * p.pitch, cols, ks) + finish_clk(ks) +

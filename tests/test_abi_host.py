@@ -322,3 +322,13 @@ def test_host_workspace_query_from_several_threads():
     for t in threads:
         t.join()
     assert not wrong, (len(wrong), wrong[0], want)
+
+
+def test_whole_tiles_flag_keeps_reductions_whole():
+    """HGC_FLAG_WHOLE_TILES: long reductions on few pixels are dealt out to clusters of CTAs without it and
+    stay whole with it; inner products are split either way."""
+    for args in ((1, 512, 28, 28, 512, 3, 3, 1, 1), (3, 224, 2, 106, 32, 7, 7, 3, 3), (16, 512, 14, 14, 512, 3, 3, 1, 1, 2, 2)):
+        flags = hgc.HGC_FLAG_X_NHWC | hgc.HGC_FLAG_Y_NHWC if len(args) > 9 else 0
+        assert hgc.ConvDesc(*args, flags=flags).plan_info()["k_slices"] > 1, args
+        assert hgc.ConvDesc(*args, flags=flags | hgc.HGC_FLAG_WHOLE_TILES).plan_info()["k_slices"] == 1, args
+    assert hgc.ConvDesc(1, 25088, 1, 1, 4096, 1, 1, flags=hgc.HGC_FLAG_WHOLE_TILES).plan_info()["k_slices"] > 1
