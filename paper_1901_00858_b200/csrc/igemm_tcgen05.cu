@@ -1203,6 +1203,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __shared__ __align__(8) uint64_t in_full[2 * kMaxDwTeams], in_empty[2 * kMaxDwTeams];  // depthwise input tiles (depthwise + pointwise blocks)
   __shared__ __align__(8) uint64_t slabs_full;  // row pairs: the weight slabs have arrived
   __shared__ __align__(8) uint64_t peers_done, parts_in;  // split reduction: the cluster's MMAs are complete; the parts have arrived
+  __shared__ __align__(8) uint64_t drain_bar;  // after giving up: the MMAs and commits that were issued are complete
   __shared__ __align__(8) uint64_t q_bar[4];  // whole-plane epilogue: meeting point of the two warps of a lane quarter
 
   // (through a shuffle: the compiler then knows that the roles' branches are taken by whole warps)
@@ -1241,6 +1242,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     mbar_init(smem_u32(&parts_in), a.ks_log2 > 2 ? 2 * EW : EW);
     mbar_init(smem_u32(&ho_bar), EW / 2);
     mbar_init(smem_u32(&pl_bar), EW / 2);
+    mbar_init(smem_u32(&drain_bar), 1);
     abort_flag = 0;
     produced_stages[0] = produced_stages[1] = -1;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -2209,9 +2211,23 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   }
 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  // A CTA that did its work has waited for its last accumulator.  One that gave up, or that found the status
+  // word raised after its producers and MMA issuer had started, has MMAs under way that write tensor memory
+  // and commits that arrive on barriers in shared memory: neither may go away before they are done.
+  if (warp == 1 && (!PAIR || rank == 0) && abort_flag) {
+    if (elect_one()) {  // (the lane that issued them)
+      const uint32_t bar = smem_u32(&drain_bar);
+      if constexpr (PAIR)
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+      else umma_commit(bar);
+      const uint64_t t0 = global_timer_ns();
+      while (!mbar_try_wait(bar, 0u) && global_timer_ns() - t0 < g_wait_limit_ns) {}
+    }
+    __syncwarp();
+  }
   // (a pair leaves together: the first CTA's MMAs read the partner's shared memory and write its tensor memory)
   if constexpr (PAIR) cluster_sync_all();
-  else __syncthreads();
   if constexpr (SPLIT) {
     // The CTAs of a split reduction write into one another's shared memory: one that has received
     // every part gets no more, and its own parts go to CTAs that cannot leave before they have them.
