@@ -412,7 +412,8 @@ int hgc_dwpw_forward(hgc_conv_desc* d, const void* x, const void* w_dw, const vo
  * hgc_debug_set_wait_limit_ns: the limit in nanoseconds for all later launches in this process
  * (0 restores the default); synchronous (it writes a device variable of the current device).
  * hgc_debug_drop_copies: index >= 0: in later launches the first CTA announces its index-th
- * copy (tensor-core path: ring stage; depthwise: tile) but never issues it, so the wait for it
+ * copy (tensor-core path: ring stage, or with index 2^20 the last of the weights that a row-pair layer keeps
+ * in shared memory; depthwise: tile) but never issues it, so the wait for it
  * runs out; -1 switches the hook off.  Nothing faults or traps: the kernel returns through the
  * path described above.  Errors: HGC_CUDA_ERROR.  Host-side state, not thread-safe.
  */

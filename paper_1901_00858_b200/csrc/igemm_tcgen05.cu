@@ -1182,6 +1182,7 @@ __device__ __noinline__ uint32_t epilogue_planes(uint32_t t_addr, uint32_t qstag
 
 constexpr int kLayoutWarps = 8;  // extra warps of the instantiations with the fused layout pass
 constexpr int kDwWarps = 8;      // extra warps of the depthwise + pointwise instantiations
+constexpr int kDropSlab = 1 << 20;  // test hook: as the index of a stage to drop, the last weight slab of a row-pair layer
 constexpr int kMaxDwTeams = 4;   // (and two input tiles per team)
 
 template <int KB, bool HALO, int EW, int EPI, bool SPLIT, bool PAIR = false, bool SHARED = false, bool FUSEL = false,
@@ -1195,7 +1196,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
-  __shared__ volatile int produced_stages[2];  // stages that each producer has announced, once it has left its loop
+  __shared__ volatile int produced_stages[2];  // stages that each producer has announced
   __shared__ __align__(8) uint64_t sk_bar;    // shared tiles: the partial sums of the unit's last tile are in its accumulator
   __shared__ __align__(8) uint64_t meet_bar;  // shared tiles: meeting point of all epilogue warps,
   __shared__ __align__(8) uint64_t ho_bar;    //   of the warps that hand accumulators over (the first of each lane quarter),
@@ -1244,7 +1245,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     mbar_init(smem_u32(&pl_bar), EW / 2);
     mbar_init(smem_u32(&drain_bar), 1);
     abort_flag = 0;
-    produced_stages[0] = produced_stages[1] = -1;
+    produced_stages[0] = produced_stages[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -1304,6 +1305,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       for (int i = 0; i < n_slabs; ++i) {
         // (kernel row a.R - 1 of w' is zero in its first 64 rows)
         const int r = i % a.R == 0 ? a.R - 1 : a.R - 1 - i % a.R, tap = i / a.R < a.S ? i / a.R : 0;
+        if (a.dbg_drop == kDropSlab && blockIdx.x == 0 && i == n_slabs - 1) break;  // (test hook, as below)
         tma_load_4d(ring_base + a.slab_off + (uint32_t)i * (64u * KB * 2u), &tmA, bar, 0, 0, r * a.S + tap, 0);
       }
     }
@@ -1410,43 +1412,6 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     }
     if (!weights) grid_launch_dependents();  // this CTA's last copy is under way: the next kernel may set itself up
     if (lane == 0) produced_stages[weights ? 1 : 0] = (int)issued;
-    if (PAIR && rank != 0) {
-      // (its copies are counted on the partner's barriers: after giving up it just waits a while)
-      if (abort_flag && lane == 0) {
-        const uint64_t t0 = global_timer_ns();
-        while (global_timer_ns() - t0 < 2000000ull) __nanosleep(1000);
-      }
-    } else if (abort_flag && lane == 0 && DWPW && !weights) {
-      const uint32_t bufs = 2u << a.dw_teams_log2;
-      for (uint32_t it = issued > bufs ? issued - bufs : 0; it < issued; ++it) {
-        const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(smem_u32(&in_full[it & (bufs - 1u)]), (it >> (1 + a.dw_teams_log2)) & 1u)) {
-          if (global_timer_ns() - t0 > g_wait_limit_ns) break;
-        }
-      }
-    } else if (abort_flag && lane == 0) {
-      // let the copies that were issued land before the CTA's shared memory goes away.  The other
-      // producer may have given up some stages earlier: its arrivals on those are made up for
-      // (otherwise their barriers would never complete).
-      const uint32_t first = issued > depth ? issued - depth : 0;
-      if (slabs && weights) {
-        const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(smem_u32(&slabs_full), 0u) && global_timer_ns() - t0 < g_wait_limit_ns) {}
-      }
-      if (!DWPW && !slabs) {
-        const uint64_t t0 = global_timer_ns();
-        int other;
-        while ((other = produced_stages[weights ? 0 : 1]) < 0 && global_timer_ns() - t0 < g_wait_limit_ns) __nanosleep(200);
-        for (uint32_t it = other > (int)first ? (uint32_t)other : first; other >= 0 && it < issued; ++it) mbar_arrive(smem_u32(&full_bar[it % depth]));
-      }
-      for (uint32_t it = first; it < issued; ++it) {
-        const uint32_t bar = smem_u32(&full_bar[it % depth]);
-        const uint64_t t0 = global_timer_ns();
-        while (!mbar_try_wait(bar, (it / depth) & 1u)) {
-          if (global_timer_ns() - t0 > g_wait_limit_ns) break;
-        }
-      }
-    }
     __syncwarp();
   } else if (warp == 1 && (!PAIR || rank == 0)) {
     // ---------------- MMA issuer (of a pair: the first CTA's, for both) ----------------
@@ -2213,8 +2178,35 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   // A CTA that did its work has waited for its last accumulator.  One that gave up, or that found the status
-  // word raised after its producers and MMA issuer had started, has MMAs under way that write tensor memory
-  // and commits that arrive on barriers in shared memory: neither may go away before they are done.
+  // word raised after its producers and MMA issuer had started, may have copies under way into its shared
+  // memory, MMAs that write tensor memory and commits that arrive on its barriers: nothing of it may go away
+  // before they are done.  (Only here is it known that no warp will raise abort_flag any more.)
+  if ((warp == 0 || warp == 2 + EW) && lane == 0 && abort_flag) {
+    const bool weights = warp != 0;
+    const uint32_t depth = (uint32_t)a.stages;
+    const uint32_t issued = (uint32_t)produced_stages[weights ? 1 : 0], other = (uint32_t)produced_stages[weights ? 0 : 1];
+    const bool slabs = EPI == 0 && a.slab_off != 0;
+    const uint64_t t0 = global_timer_ns();  // (one limit for all of them)
+    auto landed = [&](uint64_t* bar, uint32_t parity) {
+      while (!mbar_try_wait(smem_u32(bar), parity) && global_timer_ns() - t0 < g_wait_limit_ns) {}
+    };
+    if (PAIR && rank != 0) {
+      // (its copies are counted on the partner's barriers: it just waits a while)
+      while (global_timer_ns() - t0 < 2000000ull) __nanosleep(1000);
+    } else if (DWPW && !weights) {
+      const uint32_t bufs = 2u << a.dw_teams_log2;
+      for (uint32_t it = issued > bufs ? issued - bufs : 0; it < issued; ++it)
+        landed(&in_full[it & (bufs - 1u)], (it >> (1 + a.dw_teams_log2)) & 1u);
+    } else {
+      // The other producer may have given up some stages earlier: its arrivals on those are made up for
+      // (otherwise their barriers would never complete).
+      const uint32_t first = issued > depth ? issued - depth : 0;
+      if (slabs && weights) landed(&slabs_full, 0u);
+      if (!DWPW && !slabs)
+        for (uint32_t it = other > first ? other : first; it < issued; ++it) mbar_arrive(smem_u32(&full_bar[it % depth]));
+      for (uint32_t it = first; it < issued; ++it) landed(&full_bar[it % depth], (it / depth) & 1u);
+    }
+  }
   if (warp == 1 && (!PAIR || rank == 0) && abort_flag) {
     if (elect_one()) {  // (the lane that issued them)
       const uint32_t bar = smem_u32(&drain_bar);
