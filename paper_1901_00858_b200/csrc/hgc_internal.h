@@ -65,8 +65,9 @@ cudaError_t depthwise_nhwc_tma_set_wait_limit_ns(uint64_t ns);
 // half a block per SM: the preference would cost them blocks per SM (the general depthwise kernel on
 // 17 x 1024 x 167 x 167 1028 -> 1873 us, the tile transpose on 22 x 80 x 133 x 133 and its layer 115 -> 129),
 // and moving in early under the tensor-core kernel's split too (58 x 192 x 15 x 15 12.5 -> 16.8).
-constexpr int64_t kOverlapThreads = 148 * 512;
+constexpr int kOverlapThreads = 512;  // per SM
 constexpr unsigned kCopyKernelCarveout = 25;  // per cent
+int sm_count();  // SMs of the current device (148 if it cannot be queried)
 bool launch_overlap_enabled();
 void set_launch_overlap(bool on);
 
@@ -95,7 +96,7 @@ inline cudaError_t launch_kernel_attr(bool overlap, unsigned carveout, void (*ke
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                  Args... args) {
-  const bool small = (int64_t)grid.x * grid.y * grid.z * block.x <= kOverlapThreads;
+  const bool small = (int64_t)grid.x * grid.y * grid.z * block.x <= (int64_t)kOverlapThreads * sm_count();
   bool overlap = small || launch_overlap_enabled();
   if (!overlap) {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -107,7 +108,7 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_smem_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                       Args... args) {
-  const bool small = (int64_t)grid.x * grid.y * grid.z <= 74;
+  const bool small = (int64_t)grid.x * grid.y * grid.z * 2 <= sm_count();
   return launch_kernel_attr(small || launch_overlap_enabled(), 0, kernel, grid, block, smem, stream, args...);
 }
 // The persistent tensor-core kernel is always launched with the attribute: its set-up (barriers,
@@ -404,9 +405,6 @@ cudaError_t launch_igemm_weights(const ConvGeom& g, const IgemmPlan& p, const __
                                  cudaStream_t stream);
 cudaError_t launch_igemm_input(const ConvGeom& g, const IgemmPlan& p, const __half* x, __half* xp,
                                cudaStream_t stream);
-
-// number of SMs of the current device (148 if it cannot be queried)
-int sm_count();
 
 bool igemm_make_plan(const ConvGeom& g, IgemmPlan* out);
 bool igemm_encode_maps(const ConvGeom& g, IgemmPlan* p, void* ws);

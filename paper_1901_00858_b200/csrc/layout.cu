@@ -650,7 +650,7 @@ cudaError_t launch_nchw_to_nhwc8_bordered(const __half* src, __half* dst, int32_
     }
   }
   int64_t blocks = (total + 255) / 256;
-  if (blocks > 148 * 32) blocks = 148 * 32;
+  if (blocks > (int64_t)sm_count() * 32) blocks = (int64_t)sm_count() * 32;
   if (px_ch == 4)
     launch_kernel(nchw_to_nhwc8_bordered_kernel<4>, dim3((unsigned)blocks), dim3(256), 0, stream,
         reinterpret_cast<const uint16_t*>(src), reinterpret_cast<uint16_t*>(dst), c, h, w, pad_h, pad_w, hp, wp, total);
@@ -665,7 +665,7 @@ cudaError_t launch_weights_repack_window(const __half* src, __half* dst, int32_t
                                          int32_t kw_pix, cudaStream_t stream, int perm, int px_ch) {
   const int64_t total = (int64_t)k * r * kw_pix;
   int64_t blocks = (total + 255) / 256;
-  if (blocks > 148 * 16) blocks = 148 * 16;
+  if (blocks > (int64_t)sm_count() * 16) blocks = (int64_t)sm_count() * 16;
   if (px_ch == 4)
     launch_kernel(weights_repack_window_kernel<4>, dim3((unsigned)blocks), dim3(256), 0, stream,
         reinterpret_cast<const uint16_t*>(src), reinterpret_cast<uint16_t*>(dst), k, c, r, s, kw_pix, perm);
@@ -767,7 +767,7 @@ cudaError_t launch_weights_repack(const __half* src, __half* dst, int32_t k, int
   (void)group;  // groups are contiguous blocks of output channels: the permutation is per k
   const int64_t total = (int64_t)k * r * s * (c_pad / 8);
   int64_t blocks = (total + 255) / 256;
-  if (blocks > 148 * 16) blocks = 148 * 16;
+  if (blocks > (int64_t)sm_count() * 16) blocks = (int64_t)sm_count() * 16;
   if (blocks < 1) blocks = 1;
   launch_kernel(weights_repack_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, 
       reinterpret_cast<const uint16_t*>(src), reinterpret_cast<uint16_t*>(dst), k, cg, r * s, c_pad, perm);
@@ -821,7 +821,7 @@ cudaError_t launch_weights_repack_patch(const __half* src, __half* dst, int32_t 
                                         int32_t kelems, cudaStream_t stream, int perm) {
   const int64_t total = (int64_t)k * kelems;
   int64_t blocks = (total + 255) / 256;
-  if (blocks > 148 * 16) blocks = 148 * 16;
+  if (blocks > (int64_t)sm_count() * 16) blocks = (int64_t)sm_count() * 16;
   if (blocks < 1) blocks = 1;
   launch_kernel(weights_repack_patch_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, 
       reinterpret_cast<const uint16_t*>(src), reinterpret_cast<uint16_t*>(dst), k, c, r, s, kelems, perm);
