@@ -180,7 +180,7 @@ int hgc_conv_forward_host(hgc_conv_desc* d, const void* x, const void* w, const 
  * way to obtain the scratch buffer that hgc_conv_set_workspace wants.
  *
  * What it does: runs the tensor-core path (HGC_PATH_IGEMM) of hgc_conv_forward with its scratch
- * (status word, re-laid-out weights, NHWC copy of x, fp32 partial sums of a split reduction) in a
+ * (status word, re-laid-out weights, NHWC copy of x) in a
  * 32 MiB array that is part of the library image: every device that loads the library holds
  * those 32 MiB until the process exits.  It takes the layer description directly; no descriptor
  * object, no workspace, no weight registration (the weights are re-laid-out on every call).

@@ -115,7 +115,7 @@ template <int L>
 __global__ void __launch_bounds__(kBnThreads)
 bn_group_kernel(const uint16_t* __restrict__ x, float2* __restrict__ stats, int n_img, int C, int64_t hw, int chunks, float shift) {
   grid_dependency_wait();
-  grid_launch_dependents();
+  grid_launch_dependents();  // (not before the wait: the second kernel loads x before its own)
   const int c = (int)blockIdx.y;
   const int G = n_img * chunks;
   constexpr int kSlots = kBnThreads / L;  // groups per block and step

@@ -49,7 +49,9 @@ cudaError_t depthwise_nhwc_tma_set_wait_limit_ns(uint64_t ns);
 // kernel before it in the stream is still draining; every kernel of this library therefore
 // executes grid_dependency_wait() before its first access to global memory (it returns when the
 // preceding kernel has completed and its writes are visible; a no-op for a kernel launched
-// without the attribute), so only launch latency and on-chip set-up overlap.
+// without the attribute), so only launch latency and on-chip set-up overlap.  One exception: the second
+// batch norm kernel loads x before it waits.  It may, because the first one lets it start only after its
+// own wait (grid_launch_dependents behind grid_dependency_wait): whatever wrote x has completed by then.
 // Which kernels: the tensor-core kernels always (below); the copy, depthwise and element-wise kernels
 // when the launch is not being captured or their grid is at most two blocks of 256 threads per SM (or
 // hgc_set_launch_overlap asks for all).  In a graph, launches follow one another closely without it.
@@ -391,7 +393,6 @@ struct IgemmPlan {
   uint32_t dw_in_bytes, dw_in_alloc;
   int32_t dw_teams_log2;   // depthwise warps form 1, 2 or 4 teams
   int32_t pair, ncols_sub, pair_fit;
-  double est_clk;  // the cost model's estimate for the launch, in SM clocks
   size_t ws_status_off, ws_w_off, ws_x_off, ws_sk_off, ws_total;
   bool maps_ready;
   alignas(64) CUtensorMap tmA;

@@ -810,7 +810,6 @@ struct IgemmArgs {
   int32_t tma_store;  // 1: the epilogue stages fp16 tiles in shared memory and stores them with TMA
   int32_t plane_store;  // 1, 2: whole-plane tiles leave as one bulk copy per 32-channel block (epilogue_planes: its mode)
   uint32_t plane_bytes; //    bytes of a lane quarter's staging tile
-  int32_t rem;        // (th*Q) % 64: width of the last staged pass of a full tile (0 = none)
   int32_t nbuf;       // staging tiles per epilogue warp (1 or 2)
   int32_t dup_log2;   // log2 of the number of copies of the layer's rows in a weight tile (0, 1, 2)
   uint32_t slab_off;  // row pairs with all weights in shared memory: where their 64-row slabs lie, bytes from the ring's start (0: none)
@@ -1696,13 +1695,13 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     // so here too the warps of all lane quarters share the pixels of those channels.
     // (of a cluster of eight the first four finish a quarter each)
     const int fin_log2 = SPLIT ? (a.ks_log2 < 2 ? a.ks_log2 : 2) : 0;
-    const int rep_q = SPLIT ? 4 >> fin_log2 : (EPI == 0 ? (a.rowpair ? 2 : (4 >> a.dup_log2)) : 4);  // lane quarters per replica
+    constexpr bool kOwnLoop = EPI == 0 && !SPLIT && !PAIR && !SHARED && !DWPW;  // (replicas and row pairs come in this form only)
+    const int rep_q = SPLIT ? 4 >> fin_log2 : (kOwnLoop ? (a.rowpair ? 2 : (4 >> a.dup_log2)) : 4);  // lane quarters per replica
     const int part = SPLIT ? (int)blockIdx.x & ((1 << a.ks_log2) - 1) : 0;
     const int cq = (part & ((1 << fin_log2) - 1)) * rep_q + (quarter & (rep_q - 1));  // the quarter's place among the channels
-    const bool split_px = SPLIT || (EPI == 0 && !a.rowpair);
+    const bool split_px = SPLIT || (kOwnLoop && !a.rowpair);
     const int half_eff = split_px ? (quarter / rep_q) * kPerQuarter + half : half;  // which of the warps that share the pixels
     const int per_eff = split_px ? (kPerQuarter << (SPLIT ? fin_log2 : a.dup_log2)) : kPerQuarter;
-    const int odd_row = (EPI == 0 && a.rowpair) ? (quarter >> 1) : 0;
     const int row = cq * 32 + ((EPI == 2 && a.y_tma) ? ((lane & 3) << 3) + (lane >> 2) : lane);
     uint16_t* yb = reinterpret_cast<uint16_t*>(y);
     const uint32_t stage_base = ring_base + (uint32_t)a.stages * a.stage_bytes + (SPLIT ? a.recv_bytes : 0u);
@@ -1711,7 +1710,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     // this warp's own staging tiles: 32 channel rows of 128 bytes each, 128-byte swizzled
     const uint32_t my_stage = stage_base + (uint32_t)ew * (uint32_t)a.nbuf * kWarpStageBytes;
     const uint32_t row_off = (uint32_t)lane * 128u + (((uint32_t)lane & 7u) << 4);
-    uint32_t unit_ctr = 0, stage_sel = 0;
+    uint32_t stage_sel = 0;
     uint32_t lt = 0;
     uint32_t meet_phase = 0, ho_phase = 0, pl_phase = 0, q_phase = 0;
     bool gave_up = false;  // (a meeting of the whole-plane epilogue ran out of time)
@@ -1732,7 +1731,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       fin_tile = (int)(g_end / a.ts);
       if (g_end > g_beg && g_end % a.ts != 0 && (int64_t)fin_tile * a.ts >= g_beg) fin_item = fin_tile - (int)(g_beg / a.ts);
     }
-    if constexpr (EPI == 0 && !SPLIT && !PAIR && !SHARED && !DWPW) {
+    if constexpr (kOwnLoop) {
       // The staged TMA-store epilogue on its own loop (see the general one below for what it does): in
       // layers of short main loops an epilogue warp has one or two units per tile, and the
       // general loop's bookkeeping was 700 of the 1800 clocks that a tile took it.
@@ -1742,6 +1741,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       int hr_first = 0, wc_first = e_first;  // (row, column) of the warp's first pixel in a tile
       while (!linear && wc_first >= a.Q) { wc_first -= a.Q; ++hr_first; }
       const int live_k = a.rowpair ? 64 : a.kg;
+      const int odd_row = a.rowpair ? (quarter >> 1) : 0;
       const bool one_channel_tile = a.mtiles * a.group == 1;
       const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
       int grp = 0, m0 = 0;
@@ -1883,7 +1883,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     [[maybe_unused]] next_channel_tile:
       const int m0 = m0_item + ci * 128;
       const int kin = m0 + row;
-      const bool kvalid = kin < (a.rowpair ? 64 : a.kg);
+      const bool kvalid = kin < a.kg;
       const int k = grp * a.kg + (kvalid ? kin : 0);
       // (fetched again only when the channel changes: a load from global memory at the head of
       //  every tile's epilogue costs several hundred clocks, a third of a short tile's epilogue)
@@ -1902,7 +1902,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
       const uint32_t t_tile = tmem_base + buf * 256u + (uint32_t)(DWPW ? ci * a.acc_stride : 0) + ((uint32_t)(quarter * 32) << 16);
-      const bool quarter_live = m0 + cq * 32 < (a.rowpair ? 64 : a.kg);  // any real output channel in this warp's lanes?
+      const bool quarter_live = m0 + cq * 32 < a.kg;  // any real output channel in this warp's lanes?
       // the barrier the accumulator is handed back on (of a pair: the first CTA's)
       const uint32_t acc_empty_bar = PAIR ? cluster_addr(smem_u32(&acc_empty[buf]), 0) : smem_u32(&acc_empty[buf]);
 
@@ -2000,11 +2000,11 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           const bool last_row_tile = p0 + a.th >= a.P;
           // (row, column) of the unit's first pixel, kept up to date without divisions
           const bool linear = a.pitch == a.Q;  // no junk columns: accumulator columns are consecutive pixels
-          // pixels per unit: 64, or 32 where the replicas would otherwise leave warps without a unit
+          // pixels per unit: 64, or 32 where the CTAs of a cluster share them
           const int upx = a.fine_units ? a.fine_units : kPassElems;
           int hr = 0, wc = half_eff * upx;
           while (!linear && wc >= a.Q) { wc -= a.Q; ++hr; }
-          for (int e_lo = half_eff * upx; e_lo < e_valid; e_lo += per_eff * upx, ++unit_ctr) {
+          for (int e_lo = half_eff * upx; e_lo < e_valid; e_lo += per_eff * upx) {
             const int e_hi = e_lo + upx < e_valid ? e_lo + upx : e_valid;
             const uint32_t sbuf = my_stage + stage_sel * kWarpStageBytes;
             stage_sel = a.nbuf == 2 ? stage_sel ^ 1u : 0u;
@@ -2052,9 +2052,9 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (leader) {
-              // past P*Q the store is clipped (row pairs: the next row of y belongs to other warps)
-              const bool full_box = !a.fine_units && ((e_hi - e_lo == kPassElems) || (last_row_tile && !a.rowpair));
-              tma_store_4d(full_box ? &tmY : &tmYr, sbuf, (a.rowpair ? 2 * p0 + odd_row : p0) * a.Q + e_lo, m0 + cq * 32, grp, n0);
+              // past P*Q the store is clipped
+              const bool full_box = !a.fine_units && (e_hi - e_lo == kPassElems || last_row_tile);
+              tma_store_4d(full_box ? &tmY : &tmYr, sbuf, p0 * a.Q + e_lo, m0 + cq * 32, grp, n0);
               asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
             // first pixel of this warp's next unit
@@ -2538,6 +2538,10 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   // estimated clocks of one tile.
   const int sms = sm_count();
   const int junk = p.pitch - g.q;
+  // The cost model of whole tiles.  Its constants were fitted to an earlier form of the kernel, which issued
+  // copies and MMAs under `lane == 0`; those of stage_clk below are the present kernel's.  They stay because
+  // they rank the tile shapes, and with them 32- or 64-channel blocks and the sharing of tiles, as the
+  // measured tables have them: other constants would change the order of the sums.
   // An MMA step (128 channels x ncols pixels x 16 reduction elements) is bounded by
   //   the tensor pipe:     ncols / 2 clocks,
   //   L2 -> shared memory  (about 30 bytes per clock and SM, measured): its 4 KB slice of the
@@ -2595,8 +2599,9 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     *cost_out = (main_loop > epi ? main_loop : epi) + 300.0 * (tiles_per_cta > 1.0 ? tiles_per_cta : 1.0) + hand_over;
   };
   // Layers whose tiles leave three quarters of the SMs idle (inner products, tiny planes) share the
-  // reduction of a tile between 2, 4 or 8 CTAs.  (What the exchange was estimated at when it
-  // went through global memory; it decides the slices, and with them the order of the sums.)
+  // reduction of a tile between 2, 4 or 8 CTAs.  This is no measurement of the present exchange but
+  // what it was estimated at when it went through global memory and a second kernel: it decides the slices,
+  // and with them the order of the sums, and is kept for that.
   auto finish_clk = [&](int ks) {
     if (ks == 0) return 0.0;
     const double elems = (double)g.n * g.k * g.p * g.q;
@@ -2738,7 +2743,6 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     if (best_tn > 1) best_tn = (best_tn + 1) / 2;
     else best_th = (best_th + 1) / 2;
   }
-  p.est_clk = best;
   // CTA pairs (tcgen05 cta_group::2) for layers with more than 128 output channels per group: a
   // tile is 256 channels x two pixel sub-tiles of at most 128 accumulator columns each.  Every
   // CTA then reads 128 weight rows and HALF of the activation tile from its own shared memory per
@@ -2793,7 +2797,6 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     }
     if (pth == 0) return false;
     p.pair = 1;
-    p.est_clk = best_pair;
     best_th = pth;
     best_tn = ptn;
     best_shared = pshared;
@@ -3328,7 +3331,6 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   a.tma_store = p.tma_store;
   a.plane_store = p.plane_store;
   a.plane_bytes = p.plane_bytes;
-  a.rem = p.rem;
   a.nbuf = p.nbuf;
   a.dup_log2 = p.dup_log2;
   a.fine_units = p.fine_units;

@@ -87,8 +87,7 @@ extern "C" int hgc_conv_forward_static(const hgc_conv_params* p, const void* x, 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the array keeps whatever the previous call left: the header (status word, hand-over flags)
   // must start at zero; the re-layout kernels rewrite every byte of the weight and input copies
-  // that the tensor-core kernel reads, padding included, and a reduction slice writes every
-  // partial sum before the second pass reads it
+  // that the tensor-core kernel reads, padding included
   if (hgc::kCheckedBuild) {
     hgc::DebugRanges r{};
     hgc::debug_add_range(&r, x, (size_t)g.n * g.c * g.h * g.w * 2);
