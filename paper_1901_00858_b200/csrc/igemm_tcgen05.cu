@@ -1184,6 +1184,48 @@ constexpr int kDwWarps = 8;      // extra warps of the depthwise + pointwise ins
 constexpr int kDropSlab = 1 << 20;  // test hook: as the index of a stage to drop, the last weight slab of a row-pair layer
 constexpr int kMaxDwTeams = 4;   // (and two input tiles per team)
 
+// A CTA that did its work has waited for its last accumulator.  One that gave up, or that found the status
+// word raised after its producers and MMA issuer had started, may have copies under way into its shared
+// memory, MMAs that write tensor memory and commits that arrive on its barriers: nothing of it may go away
+// before they are done.  Called by all warps behind the CTA's last barrier; out of line, because the code at
+// the end of every launch should stay short (14 block kernels 155 us with it inline, 152 without).
+template <bool PAIR, bool DWPW>
+__device__ __noinline__ void wait_for_work_under_way(int warp, int epi_warps, uint32_t rank, uint32_t depth, bool slabs, uint32_t in_log2,
+                                                     uint32_t full_bar, uint32_t in_full, uint32_t slabs_full, uint32_t drain_bar,
+                                                     uint32_t produced_x, uint32_t produced_w) {
+  const uint64_t t0 = global_timer_ns();  // (one limit for all of a warp's waits)
+  auto landed = [&](uint32_t bar, uint32_t parity) {
+    while (!mbar_try_wait(bar, parity) && global_timer_ns() - t0 < g_wait_limit_ns) {}
+  };
+  if (warp == 1 && (!PAIR || rank == 0) && elect_one()) {  // (the lane that issued them)
+    if constexpr (PAIR)
+      asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(drain_bar) : "memory");
+    else umma_commit(drain_bar);
+    landed(drain_bar, 0u);
+  }
+  if ((warp == 0 || warp == 2 + epi_warps) && elect_one()) {
+    const bool weights = warp != 0;
+    const uint32_t issued = weights ? produced_w : produced_x, other = weights ? produced_x : produced_w;
+    if (PAIR && rank != 0) {
+      // (its copies are counted on the partner's barriers: it just waits a while)
+      while (global_timer_ns() - t0 < 2000000ull) __nanosleep(1000);
+    } else if (DWPW && !weights) {
+      const uint32_t bufs = 1u << in_log2;  // (input tiles)
+      for (uint32_t it = issued > bufs ? issued - bufs : 0; it < issued; ++it)
+        landed(in_full + 8u * (it & (bufs - 1u)), (it >> in_log2) & 1u);
+    } else {
+      // The other producer may have given up some stages earlier: its arrivals on those are made up for
+      // (otherwise their barriers would never complete).
+      const uint32_t first = issued > depth ? issued - depth : 0;
+      if (slabs && weights) landed(slabs_full, 0u);
+      if (!DWPW && !slabs)
+        for (uint32_t it = other > first ? other : first; it < issued; ++it) mbar_arrive(full_bar + 8u * (it % depth));
+      for (uint32_t it = first; it < issued; ++it) landed(full_bar + 8u * (it % depth), (it / depth) & 1u);
+    }
+  }
+  __syncwarp();
+}
+
 template <int KB, bool HALO, int EW, int EPI, bool SPLIT, bool PAIR = false, bool SHARED = false, bool FUSEL = false,
           bool DWPW = false>
 __global__ void __launch_bounds__(96 + 32 * EW + (FUSEL ? 32 * kLayoutWarps : 0) + (DWPW ? 32 * kDwWarps : 0), 1)
@@ -2177,47 +2219,11 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  // A CTA that did its work has waited for its last accumulator.  One that gave up, or that found the status
-  // word raised after its producers and MMA issuer had started, may have copies under way into its shared
-  // memory, MMAs that write tensor memory and commits that arrive on its barriers: nothing of it may go away
-  // before they are done.  (Only here is it known that no warp will raise abort_flag any more.)
-  if ((warp == 0 || warp == 2 + EW) && lane == 0 && abort_flag) {
-    const bool weights = warp != 0;
-    const uint32_t depth = (uint32_t)a.stages;
-    const uint32_t issued = (uint32_t)produced_stages[weights ? 1 : 0], other = (uint32_t)produced_stages[weights ? 0 : 1];
-    const bool slabs = EPI == 0 && a.slab_off != 0;
-    const uint64_t t0 = global_timer_ns();  // (one limit for all of them)
-    auto landed = [&](uint64_t* bar, uint32_t parity) {
-      while (!mbar_try_wait(smem_u32(bar), parity) && global_timer_ns() - t0 < g_wait_limit_ns) {}
-    };
-    if (PAIR && rank != 0) {
-      // (its copies are counted on the partner's barriers: it just waits a while)
-      while (global_timer_ns() - t0 < 2000000ull) __nanosleep(1000);
-    } else if (DWPW && !weights) {
-      const uint32_t bufs = 2u << a.dw_teams_log2;
-      for (uint32_t it = issued > bufs ? issued - bufs : 0; it < issued; ++it)
-        landed(&in_full[it & (bufs - 1u)], (it >> (1 + a.dw_teams_log2)) & 1u);
-    } else {
-      // The other producer may have given up some stages earlier: its arrivals on those are made up for
-      // (otherwise their barriers would never complete).
-      const uint32_t first = issued > depth ? issued - depth : 0;
-      if (slabs && weights) landed(&slabs_full, 0u);
-      if (!DWPW && !slabs)
-        for (uint32_t it = other > first ? other : first; it < issued; ++it) mbar_arrive(smem_u32(&full_bar[it % depth]));
-      for (uint32_t it = first; it < issued; ++it) landed(&full_bar[it % depth], (it / depth) & 1u);
-    }
-  }
-  if (warp == 1 && (!PAIR || rank == 0) && abort_flag) {
-    if (elect_one()) {  // (the lane that issued them)
-      const uint32_t bar = smem_u32(&drain_bar);
-      if constexpr (PAIR)
-        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-      else umma_commit(bar);
-      const uint64_t t0 = global_timer_ns();
-      while (!mbar_try_wait(bar, 0u) && global_timer_ns() - t0 < g_wait_limit_ns) {}
-    }
-    __syncwarp();
-  }
+  const bool gave_up_cta = abort_flag != 0;  // (final only here: no warp raises it any more)
+  if (gave_up_cta)
+    wait_for_work_under_way<PAIR, DWPW>(warp, EW, rank, (uint32_t)a.stages, EPI == 0 && a.slab_off != 0, 1u + (uint32_t)a.dw_teams_log2,
+                                        smem_u32(full_bar), smem_u32(in_full), smem_u32(&slabs_full), smem_u32(&drain_bar),
+                                        (uint32_t)produced_stages[0], (uint32_t)produced_stages[1]);
   // (a pair leaves together: the first CTA's MMAs read the partner's shared memory and write its tensor memory)
   if constexpr (PAIR) cluster_sync_all();
   if constexpr (SPLIT) {
@@ -2225,13 +2231,13 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     // every part gets no more, and its own parts go to CTAs that cannot leave before they have them.
     // After giving up that need not hold: then it stays until the others have given up or left.
     if (!met) cluster_wait();
-    if (abort_flag) cluster_sync_all();
+    if (gave_up_cta) cluster_sync_all();
   }
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
   }
-  if (threadIdx.x == 0 && abort_flag && status != nullptr) atomicExch(status, (int)HGC_DEVICE_TIMEOUT);
+  if (threadIdx.x == 0 && gave_up_cta && status != nullptr) atomicExch(status, (int)HGC_DEVICE_TIMEOUT);
   if constexpr (FUSEL) {
     // the CTA that finishes last lowers the segment counters for the next launch
     __shared__ int last_cta;
