@@ -446,8 +446,9 @@ int hgc_debug_shrink_ranges(int64_t bytes);
  * the stream is still draining, and waits, before it touches global memory, until that kernel
  * has completed; so its set-up overlaps the tail of the kernel before it, and where one
  * tensor-core kernel follows another its CTAs start as the previous kernel's leave.  Results are
- * the same either way.  Measured on B200, steps replayed as CUDA graphs: ResNet-50 channels-last
- * 1.065 -> 1.018 ms, MobileNet channels-last 0.332 -> 0.321 ms, NCHW steps unchanged.
+ * the same either way.  Measured on B200 when it was introduced, steps replayed as CUDA graphs: ResNet-50
+ * channels-last 1.065 -> 1.018 ms, MobileNet channels-last 0.332 -> 0.321 ms (0.878 and 0.292 by now), NCHW steps
+ * unchanged.
  * So are the other kernels of eager launches, and in captured graphs those of a small grid (at most two
  * blocks of 256 threads per SM).
  * With enabled != 0 the others are launched that way in graphs too (off by default: a captured step

@@ -78,8 +78,8 @@ inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // chunks, the copy out of one beside the copy in of the next.  A chunk moves at least 2 MB each
 // way and there are at most four: a copy costs the link about 3 us, and callers that spread their
 // layers over several streams have the overlap already and pay for chunks only (VGG-16 at batch 16 on
-// eight streams: 8.9 ms a pass without chunks, 8.9 with four of 3 MB, 9.5 with eight of 1 MB; on one
-// stream 14.6, 11.9 and 11.8).
+// eight streams: 8.5 to 9.0 ms a pass without chunks, 8.85 with at most four of 2 MB and more, 9.5 with eight of
+// 1 MB; on one stream 14.3, 12.0 and 11.8).
 constexpr int kMaxHostChunks = 4;
 constexpr size_t kHostChunkBytes = 2 << 20;
 
