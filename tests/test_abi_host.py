@@ -332,3 +332,14 @@ def test_whole_tiles_flag_keeps_reductions_whole():
         assert hgc.ConvDesc(*args, flags=flags).plan_info()["k_slices"] > 1, args
         assert hgc.ConvDesc(*args, flags=flags | hgc.HGC_FLAG_WHOLE_TILES).plan_info()["k_slices"] == 1, args
     assert hgc.ConvDesc(1, 25088, 1, 1, 4096, 1, 1, flags=hgc.HGC_FLAG_WHOLE_TILES).plan_info()["k_slices"] > 1
+
+
+def test_weights_stay_in_the_ring_only_where_every_lap_needs_the_same():
+    """plan_info resident: a whole number of tiles' stages in the ring and one channel tile per CTA."""
+    def info(*args):
+        return hgc.ConvDesc(*args).plan_info()
+    assert info(22, 64, 56, 56, 64, 3, 3, 1, 1)["resident"] == 1
+    assert info(16, 256, 56, 56, 256, 3, 3, 1, 1)["resident"] == 0     # shared tiles
+    assert info(64, 64, 56, 56, 384, 1, 1)["resident"] == 0            # three channel tiles, 148 CTAs
+    assert info(16, 512, 28, 28, 512, 3, 3, 1, 1)["resident"] == 0     # a tile's stages do not fit the ring
+    assert info(16, 64, 224, 224, 64, 3, 3, 1, 1)["resident"] == 0     # row pairs: slabs instead
