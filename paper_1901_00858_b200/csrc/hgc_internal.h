@@ -24,6 +24,7 @@ struct ConvGeom {
   int32_t no_pair;         // 1: never pair CTAs on 256-channel tiles
   int32_t no_fuse;         // 1: the layout pass stays a kernel of its own
   int32_t no_gather;       // 1: 1x1 layers on small planes keep the separate layout pass (never gathered by the kernel's own warps)
+  int32_t no_dup;          // 1: the weight rows are laid out once, whatever their number (IgemmPlan::dup_log2)
   // The order in which the sums are taken (chunks of images of one layer keep the whole layer's, see same_sums):
   int32_t want_kb;         // channels per reduction block: 32 or 64, or 0 = the planner's choice
   int32_t no_cluster;      // 1: no tile's reduction is dealt out to a cluster of CTAs; 2: only those of layers that leave most SMs idle

@@ -2925,7 +2925,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     const bool resident_ok = ts_est == 1;  // (a layer of one channel tile: its weights are fetched once, see below)
     const int px = p.th * g.q, copies_log2 = g.kg == 64 ? 1 : 2;
     if (!p.y_nhwc && p.tma_store && g.group == 1 && best_ks == 0 && !best_shared && !want_pair && g.dw_stride == 0 && !g.rowpair &&
-        !p.gather && g.no_fuse && (g.kg == 64 || g.kg == 32) && mpt <= (resident_ok ? 16.0 : 8.0) && px >= 96) {
+        !p.gather && g.no_fuse && !g.no_dup && (g.kg == 64 || g.kg == 32) && mpt <= (resident_ok ? 16.0 : 8.0) && px >= 96) {
       // (measured: VGG conv1_1 47.5 -> 41.1 us, 1x1 layers 32 -> 64 and 64 -> 64 channels 7 % faster,
       //  MobileNet's 32-channel stem 30.0 -> 26.6; with a longer reduction the doubled weight traffic costs
       //  more than the epilogue gains, ResNet-50's stem 76 -> 97, unless the weights stay resident: 60)

@@ -81,6 +81,11 @@ extern "C" int hgc_conv_forward_static(const hgc_conv_params* p, const void* x, 
   if (misaligned(x) || misaligned(w) || misaligned(y) || (bias != nullptr && misaligned(bias))) return HGC_BAD_ALIGNMENT;
   hgc::IgemmPlan plan{};  // on the stack: no host heap either
   if (!hgc::igemm_make_plan(g, &plan)) return HGC_UNSUPPORTED;  // only the tensor-core path has this variant
+  if (plan.ws_total > kStaticScratchBytes) {  // (copies of the weight rows are not worth a refusal)
+    g.no_dup = 1;
+    plan = hgc::IgemmPlan{};
+    if (!hgc::igemm_make_plan(g, &plan)) return HGC_UNSUPPORTED;
+  }
   if (plan.ws_total > kStaticScratchBytes) return HGC_NO_WORKSPACE;  // layer needs more than the fixed 32 MiB
   char* ws = static_cast<char*>(scratch_for_current_device());
   if (ws == nullptr) return HGC_CUDA_ERROR;

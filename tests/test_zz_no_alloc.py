@@ -58,7 +58,7 @@ MODES = [
     ("stem 3->16 3x3 stride 2 (expanded copy)", params_dict(2, 3, 21, 25, 16, 3, 3, 1, 1, 2, 2)),
     ("stem 7x7 stride 2 (windows of 4-channel pixels)", params_dict(1, 3, 30, 34, 24, 7, 7, 3, 3, 2, 2)),
     ("1x1 64->64 on 8x8 (x read in place)", params_dict(2, 64, 8, 8, 64, 1, 1)),
-    ("inner product 4096->130 (split reduction: partial sums in the array)", params_dict(4, 4096, 1, 1, 130, 1, 1)),
+    ("inner product 4096->130 (split reduction)", params_dict(4, 4096, 1, 1, 130, 1, 1)),
     ("1x1 5x5 c4096 k96 (split reduction on a small plane)", params_dict(3, 4096, 5, 5, 96, 1, 1)),
     ("grouped 5x5", params_dict(1, 96, 13, 13, 64, 5, 5, 2, 2, 1, 1, 1, 1, 2)),
 ]
@@ -75,6 +75,17 @@ def test_static_scratch_after_a_larger_call(hgc, oracle, name, args):
         got = _static_forward(hgc, a, x, w, b, True, free_must_not_change=a is not BIG)
         check_close(got, ref, what=f"static scratch vs oracle: {name} {a}")
         assert np.array_equal(got.view(np.uint16), want.view(np.uint16)), name   # same kernels, same plan: same bits
+
+
+def test_static_scratch_takes_layers_that_fit_without_replicated_weights(hgc, oracle):
+    """Four copies of this layer's weight rows would need 1 KiB more than the array has: one copy fits."""
+    a = params_dict(341, 128, 4, 96, 32, 1, 1, 0, 0, 2, 2)
+    d = hgc.ConvDesc(**a)
+    assert d.plan_info()["replicas"] == 4 and d.workspace_bytes() == (32 << 20) + 1024
+    d.close()
+    rng = np.random.default_rng(78)
+    x, w, b = workloads.random_layer_tensors(rng, a["n"], a["c"], a["h"], a["w"], a["k"], 1, 1, 1)
+    check_close(_static_forward(hgc, a, x, w, b, True), oracle.conv_fast(oracle.ConvParams(**a), x, w, b, True), what="one copy")
 
 
 def test_static_scratch_rejects_what_it_cannot_hold(hgc):
