@@ -64,8 +64,8 @@ cudaError_t depthwise_nhwc_tma_set_wait_limit_ns(uint64_t ns);
 // batch 64 1111 / 1115 / 1144 / 1075, VGG-16 at batch 16 628 / 629 / 636 / 620, at batch 1 188 / 188 / 184 / 183;
 // as graphs MobileNet 272 / 271 / 294 / 281, ResNet-50 1036 / 1040 / 1112 / 1042.  (All shared memory or
 // none: 3 to 6 % slower.)
-// Kernels that work in shared memory themselves keep the default split and overlap only with grids of
-// half a block per SM: the preference would cost them blocks per SM (the general depthwise kernel on
+// Kernels that work in shared memory themselves (the bordered stem copy where its grid does not fit at once)
+// keep the default split and overlap only with grids of half a block per SM: the preference would cost them blocks per SM (the general depthwise kernel on
 // 17 x 1024 x 167 x 167 1028 -> 1873 us, the tile transpose on 22 x 80 x 133 x 133 and its layer 115 -> 129),
 // and moving in early under the tensor-core kernel's split too (58 x 192 x 15 x 15 12.5 -> 16.8).
 constexpr int kOverlapThreads = 512;  // per SM

@@ -2355,8 +2355,8 @@ static inline ConvGeom effective_geom(const ConvGeom& g, const IgemmPlan& p) {
 
 bool igemm_make_plan(const ConvGeom& g, IgemmPlan* out) {
   // Row pairs: stride-1 layers of exactly 64 output channels with at least two kernel rows and a
-  // wide, even output plane, NCHW output through the TMA-store epilogue (VGG-16 conv1_2: the
-  // kernel 77 -> ... us).  Narrow planes would need several row pairs per tile, whose rows of
+  // wide, even output plane, NCHW output through the TMA-store epilogue (VGG-16 conv1_2, 16 images: the
+  // kernel 77 -> 61 us).  Narrow planes would need several row pairs per tile, whose rows of
   // one parity are not contiguous in y: not built.
   if (!g.rowpair && g.group == 1 && g.kg == 64 && g.cg >= 16 && g.r >= 2 && g.stride_h == 1 && g.stride_w == 1 &&
       g.dil_h == 1 && g.dil_w == 1 && !g.y_nhwc && g.dw_stride == 0 && (g.p % 2) == 0 && (g.q % 8) == 0 && g.q >= 112 &&
