@@ -2747,7 +2747,8 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   // eight parts of a tile have to fit into a CTA's shared memory: at most 128 columns
   while (best_ks > 2 && (int64_t)best_tn * best_th * p.pitch - junk > 128) {
     if (best_tn > 1) best_tn = (best_tn + 1) / 2;
-    else best_th = (best_th + 1) / 2;
+    else if (best_th > 1) best_th = (best_th + 1) / 2;
+    else best_ks = 2;  // (rows of more than 128 columns: four parts, which may go into the ring)
   }
   // CTA pairs (tcgen05 cta_group::2) for layers with more than 128 output channels per group: a
   // tile is 256 channels x two pixel sub-tiles of at most 128 accumulator columns each.  Every

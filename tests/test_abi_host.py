@@ -3,6 +3,8 @@ the header declares, validates descriptors and infers integer shapes exactly lik
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -343,3 +345,13 @@ def test_weights_stay_in_the_ring_only_where_every_lap_needs_the_same():
     assert info(64, 64, 56, 56, 384, 1, 1)["resident"] == 0            # three channel tiles, 148 CTAs
     assert info(16, 512, 28, 28, 512, 3, 3, 1, 1)["resident"] == 0     # a tile's stages do not fit the ring
     assert info(16, 64, 224, 224, 64, 3, 3, 1, 1)["resident"] == 0     # row pairs: slabs instead
+
+
+def test_split_reductions_of_rows_wider_than_eight_parts_allow():
+    """Eight parts of a tile fit into a CTA's shared memory up to 128 columns; one row of more than that has
+    to be planned with fewer slices (the search for a smaller tile did not end)."""
+    code = ("from paper_1901_00858_b200 import binding as hgc\n"
+            "for a in ((1, 1008, 4, 232, 298, 3, 1, 1, 0), (1, 1024, 2, 200, 32, 3, 1, 1, 0), (1, 1024, 1, 250, 128, 1, 3, 0, 1)):\n"
+            "    i = hgc.ConvDesc(*a).plan_info()\n"
+            "    assert i['path'] == hgc.HGC_PATH_IGEMM and (i['k_slices'] < 8 or i['ncols'] <= 128), (a, i)\n")
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=60, cwd=ROOT)
