@@ -357,6 +357,10 @@ int forward_impl(hgc_conv_desc* d, const void* x, const void* w, const void* bia
       hgc::IgemmPlan& ip = d->igemm;
       __half* wp = reinterpret_cast<__half*>(ws + ip.ws_w_off);
       __half* xp = reinterpret_cast<__half*>(ws + ip.ws_x_off);
+      if (hgc::stem_small_supported(g)) {  // (registered weights are kept as they are)
+        err = hgc::launch_stem_small(g, xh, d->registered_w == w ? wp : wh, bh, yh, relu, stream);
+        break;
+      }
       if (d->registered_w != w) {  // weights not prepared in advance: re-lay them out now
         err = hgc::launch_igemm_weights(g, ip, wh, wp, stream);
         if (err != cudaSuccess) break;
@@ -436,7 +440,7 @@ int forward_host_chunks(hgc_conv_desc* d, const HostStaging& h, const ChunkStagi
     if (c == 0 || (last && d->host_sub[1] != nullptr)) sub->registered_w = nullptr;  // new weights on every call
     rc = forward_impl(sub, xd, wd, bd, yd, relu, lane.compute);
     if (rc != HGC_OK) break;
-    sub->registered_w = wd;  // (laid out for the following chunks)
+    if (!hgc::stem_small_supported(sub->geom)) sub->registered_w = wd;  // (laid out for the following chunks)
     ok = cudaEventRecord(lane.y_done[c], lane.compute) == cudaSuccess && cudaStreamWaitEvent(lane.out, lane.y_done[c], 0) == cudaSuccess &&
          cudaMemcpyAsync(y + first * y_image, yd, images * y_image, cudaMemcpyDeviceToHost, lane.out) == cudaSuccess;
   }
@@ -601,8 +605,10 @@ int hgc_conv_set_weights(hgc_conv_desc* d, const void* w, void* stream) {
   if (d->path == HGC_PATH_IGEMM) {
     const hgc::ConvGeom& g = d->geom;
     __half* wp = reinterpret_cast<__half*>(static_cast<char*>(d->ws) + d->igemm.ws_w_off);
-    const cudaError_t err = hgc::launch_igemm_weights(g, d->igemm, static_cast<const __half*>(w), wp,
-                                                      static_cast<cudaStream_t>(stream));
+    const cudaError_t err =
+        hgc::stem_small_supported(g)
+            ? cudaMemcpyAsync(wp, w, (size_t)g.k * g.cg * g.r * g.s * 2, cudaMemcpyDeviceToDevice, static_cast<cudaStream_t>(stream))
+            : hgc::launch_igemm_weights(g, d->igemm, static_cast<const __half*>(w), wp, static_cast<cudaStream_t>(stream));
     if (err != cudaSuccess) return HGC_CUDA_ERROR;
   }
   d->registered_w = w;

@@ -296,6 +296,11 @@ void direct_debug_read(DebugViolation* v);
 cudaError_t launch_direct_conv(const ConvGeom& g, const __half* x, const __half* w,
                                const __half* bias, __half* y, int relu, cudaStream_t stream);
 
+// image stems of little work in one launch (the tensor-core path's layers: it takes a copy of x first)
+bool stem_small_supported(const ConvGeom& g);
+cudaError_t launch_stem_small(const ConvGeom& g, const __half* x, const __half* w, const __half* bias, __half* y, int relu,
+                              cudaStream_t stream);
+
 bool depthwise3x3_supported(const ConvGeom& g);
 cudaError_t launch_depthwise3x3(const ConvGeom& g, const __half* x, const __half* w,
                                 const __half* bias, __half* y, int relu, cudaStream_t stream);

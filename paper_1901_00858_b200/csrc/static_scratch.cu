@@ -108,6 +108,9 @@ extern "C" int hgc_conv_forward_static(const hgc_conv_params* p, const void* x, 
   const __half* wh = static_cast<const __half*>(w);
   __half* wp = reinterpret_cast<__half*>(ws + plan.ws_w_off);
   __half* xp = reinterpret_cast<__half*>(ws + plan.ws_x_off);
+  if (hgc::stem_small_supported(g))
+    return hgc::launch_stem_small(g, xh, wh, static_cast<const __half*>(bias), static_cast<__half*>(y), relu, st) == cudaSuccess ? HGC_OK
+                                                                                                                         : HGC_CUDA_ERROR;
   if (hgc::launch_igemm_weights(g, plan, wh, wp, st) != cudaSuccess) return HGC_CUDA_ERROR;
   if (hgc::launch_igemm_input(g, plan, xh, xp, st) != cudaSuccess) return HGC_CUDA_ERROR;
   if (hgc::launch_igemm(g, plan, ws, xh, static_cast<const __half*>(bias), static_cast<__half*>(y), relu, st) !=
