@@ -554,7 +554,7 @@ int hgc_conv_plan_info(const hgc_conv_desc* d, int32_t* info, int32_t count) {
     v[12] = p.ks_log2 > 0 ? 0 : ((p.pair && p.pair_fit > 0 && p.pair_fit < p.grid) ? p.pair_fit : p.grid);
     v[13] = p.sk_split;
     v[14] = p.pair;
-    v[15] = p.fuse_layout;
+    v[15] = p.fuse_layout ? 1 : (p.trans ? 2 : 0);
     v[16] = p.rowpair;
     v[17] = 1 << p.dup_log2;
     v[18] = p.plane_store ? 2 : (p.tma_store ? 1 : 0);

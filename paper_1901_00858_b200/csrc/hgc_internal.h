@@ -380,6 +380,11 @@ struct IgemmPlan {
   int32_t rowpair;
   // 1x1 layers whose rows make no tile of a multiple of 8 pixels: planes taken as rows of 8
   int32_t flat;
+  // x (NCHW) turned channels-last inside the kernel, no copy of it in memory: IgemmArgs::xt_*
+  int32_t ring_stages;
+  int32_t epi_tiles;
+  int32_t trans, xt_rows_in, xt_blocks, xt_slots, xt_dump;
+  uint32_t xt_bytes, xt_total;
   int32_t dup_log2;  // log2 of the number of copies of the layer's weight rows in w' and in a weight tile (0, 1, 2)
   size_t smem_bytes;
   int32_t ks_log2;  // log2 of the number of reduction slices a tile is split into (0 = none)

@@ -13,6 +13,8 @@
 //         (q0*stride - pad + s*dil, p0*stride - pad + r*dil) may lie outside the image: TMA
 //         zero-fills, which IS the zero padding).  At stride 1 the S taps of a kernel row share one
 //         tile: tap s starts s*dil pixel rows further in (a descriptor start offset);
+//       - tiles that extra warps of the kernel turn channels-last themselves, from blocks of x (NCHW) that the copy
+//         engine brings into shared memory: stride-1 layers on planes of a multiple of 8 pixels, no copy in memory;
 //       - x itself for 1x1 layers (3-D map (pixel, channel, image), boxes of 64 pixels x kb
 //         channels): pixel-major ("MN-major") tiles, no copy of x at all;
 //       - for few-channel stems, overlapping windows of a zero-bordered 8-channel copy, or an
@@ -862,6 +864,16 @@ struct IgemmArgs {
   int32_t dw_in_h, dw_in_w;
   uint32_t dw_in_bytes, dw_in_alloc;
   int32_t dw_teams_log2;  // log2 of the teams that the depthwise warps form: team t computes every stage s with s % teams == t
+  // x[N][C][H*W] turned channels-last inside the kernel (TRANS instantiations): a channel block of a tile is
+  // its th + (R-1)*dil input rows, fetched as blocks of 64 pixels x 32 channels into xt_slots staging slots
+  // and transposed into one of xt_bufs tiles [row][pitch][KB] that all R*S taps read
+  int32_t xt_w, xt_rows_in;       // pixels per row of x; input rows of a tile
+  uint32_t xt_magic;              // ceil(2^32 / xt_w): row of a pixel by a multiplication
+  int32_t xt_blocks, xt_slots, xt_bufs;
+  int32_t xt_dump;                // row of a transposed tile that nothing reads: pixels outside its input rows
+  uint32_t xt_bytes;              // bytes of a transposed tile
+  int32_t epi_tiles;              // epilogue warps that have staging tiles
+  uint32_t xt_total;              // bytes of the transposed tiles and the slots (behind the ring)
   int32_t dbg_drop;     // test hook: stage of the first CTA whose copies are left out (-1: none)
   int32_t ts;           // ring stages per tile: cblocks * R * (S / taps)
   // CTA pairs (clusters of two, tcgen05 cta_group::2): a tile is 256 output channels x two pixel
@@ -1181,6 +1193,9 @@ __device__ __noinline__ uint32_t epilogue_planes(uint32_t t_addr, uint32_t qstag
 
 constexpr int kLayoutWarps = 8;  // extra warps of the instantiations with the fused layout pass
 constexpr int kDwWarps = 8;      // extra warps of the depthwise + pointwise instantiations
+constexpr int kXtWarps = 4;      // extra warps of the instantiations that turn x channels-last themselves
+constexpr int kXtSlots = 8, kXtBufs = 2;  // staging slots at most, and transposed tiles
+constexpr uint32_t kXtSlotBytes = 64u * 32u * 2u;  // a block of 64 pixels x 32 channels
 constexpr int kDropSlab = 1 << 20;  // test hook: as the index of a stage to drop, the last weight slab of a row-pair layer
 constexpr int kMaxDwTeams = 4;   // (and two input tiles per team)
 
@@ -1189,8 +1204,10 @@ constexpr int kMaxDwTeams = 4;   // (and two input tiles per team)
 // memory, MMAs that write tensor memory and commits that arrive on its barriers: nothing of it may go away
 // before they are done.  Called by all warps behind the CTA's last barrier; out of line, because the code at
 // the end of every launch should stay short (14 block kernels 155 us with it inline, 152 without).
-template <bool PAIR, bool DWPW>
-__device__ __noinline__ void wait_for_work_under_way(int warp, int epi_warps, uint32_t rank, uint32_t depth, bool slabs, uint32_t in_log2,
+// `in_bufs`: where the activation producer's copies go to buffers of their own (IN_BUFS: blocks' input tiles,
+// blocks of x), their number.
+template <bool PAIR, bool IN_BUFS>
+__device__ __noinline__ void wait_for_work_under_way(int warp, int epi_warps, uint32_t rank, uint32_t depth, bool slabs, uint32_t in_bufs,
                                                      uint32_t full_bar, uint32_t in_full, uint32_t slabs_full, uint32_t drain_bar,
                                                      uint32_t produced_x, uint32_t produced_w) {
   const uint64_t t0 = global_timer_ns();  // (one limit for all of a warp's waits)
@@ -1209,16 +1226,15 @@ __device__ __noinline__ void wait_for_work_under_way(int warp, int epi_warps, ui
     if (PAIR && rank != 0) {
       // (its copies are counted on the partner's barriers: it just waits a while)
       while (global_timer_ns() - t0 < 2000000ull) __nanosleep(1000);
-    } else if (DWPW && !weights) {
-      const uint32_t bufs = 1u << in_log2;  // (input tiles)
-      for (uint32_t it = issued > bufs ? issued - bufs : 0; it < issued; ++it)
-        landed(in_full + 8u * (it & (bufs - 1u)), (it >> in_log2) & 1u);
+    } else if (IN_BUFS && !weights) {
+      for (uint32_t it = issued > in_bufs ? issued - in_bufs : 0; it < issued; ++it)
+        landed(in_full + 8u * (it % in_bufs), (it / in_bufs) & 1u);
     } else {
       // The other producer may have given up some stages earlier: its arrivals on those are made up for
       // (otherwise their barriers would never complete).
       const uint32_t first = issued > depth ? issued - depth : 0;
       if (slabs && weights) landed(slabs_full, 0u);
-      if (!DWPW && !slabs)
+      if (!IN_BUFS && !slabs)
         for (uint32_t it = other > first ? other : first; it < issued; ++it) mbar_arrive(full_bar + 8u * (it % depth));
       for (uint32_t it = first; it < issued; ++it) landed(full_bar + 8u * (it % depth), (it / depth) & 1u);
     }
@@ -1226,9 +1242,106 @@ __device__ __noinline__ void wait_for_work_under_way(int warp, int epi_warps, ui
   __syncwarp();
 }
 
+// Turns a tile's blocks of x (64 pixels x 32 channels, a channel's pixels in a row of 128 bytes, 16-byte chunks
+// swizzled by the row) into the K-major tile that the MMAs read ([input row][pitch][KB], swizzled likewise).  A
+// matrix load with transposition takes four 8 x 8 pieces of 8 pixels x 32 channels, one matrix store
+// writes them as 16-byte rows of 8 channels of a pixel; both are free of bank conflicts, and every lane
+// of a store has an address of its own, so that rows of any length end up at the tile's pitch.  A block is
+// one warp's: 8 loads, then 8 stores, while the other warps do the next blocks.  Shared-memory
+// traffic is three times the block's bytes (copy in, read, write), one ninth of it per tap of a 3x3 layer.
+// The columns left and right of the rows are the zero padding: no block writes them, so they are
+// cleared once.  Rows above and below the plane arrive as zeros.
+// What it costs: a block is about 250 clocks of addresses, 250 of matrix loads and stores and, once per tile of 32 or
+// 64 channels, 300 of the proxy fence, all beside the MMAs of the tile before (512->512 3x3 on 28x28: 106 clocks per MMA
+// of 208 columns, which is the tensor pipe's rate); a launch's first tile waits about 4500 clocks for it.
+template <int KB, bool SPLIT, bool SHARED>
+__device__ __forceinline__ void transpose_blocks(const IgemmArgs& a, int tw, uint32_t tiles, uint32_t in_full, uint32_t in_empty,
+                                                 uint32_t xb_full, uint32_t xb_empty, volatile int* abort_flag) {
+  constexpr uint32_t row_bytes = (uint32_t)KB * 2u;
+  const int lane = threadIdx.x & 31;
+  const uint32_t slots = tiles + (uint32_t)a.xt_bufs * a.xt_bytes;
+  const int pad = a.pitch - a.xt_w;  // columns of padding per row, left (pad_w) and right
+  for (int i = tw * 32 + lane; i < a.xt_bufs * a.xt_rows_in * pad * (KB / 8); i += kXtWarps * 32) {
+    const int chunk = i % (KB / 8), t = i / (KB / 8);
+    const int c = t % pad, row = t / pad;  // (rows of all tiles, one after the other)
+    const int tile = row / a.xt_rows_in;
+    const int pos = (row - tile * a.xt_rows_in) * a.pitch + (c < a.pad_w ? c : a.xt_w + c);
+    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(tiles + (uint32_t)tile * a.xt_bytes + (uint32_t)pos * row_bytes + (uint32_t)chunk * 16u),
+                 "r"(0)
+                 : "memory");
+  }
+  __syncwarp();
+  // matrix m = lane / 8 of a load or store: channels 8m .. 8m + 7 of 32; row lane % 8: a channel of the load, a pixel of the store
+  const uint32_t octet = (uint32_t)lane >> 3, sub = (uint32_t)lane & 7u;
+  const int px_in = a.xt_rows_in * a.xt_w;  // pixels of the tile's input rows
+  const int per_block = a.R * (a.S / a.taps);
+  // The warps take the blocks in turn, and a slot's blocks are always the same warp's: their number (8, 4 or
+  // 2) is a multiple of the number of warps that take part.  A warp that waits for a slot's next block has therefore
+  // seen the one before, which the parity of the wait does not tell from the one after.
+  const uint32_t turn = (uint32_t)(a.xt_slots < kXtWarps ? a.xt_slots : kXtWarps) - 1u;
+  uint32_t block = 0;
+  Ring ring, xb;
+  typename WorkIterOf<SPLIT, SHARED>::type it;
+  for (it.init(a); it.valid(a); it.next(a)) {
+    int s0, s1;
+    it.stage_range(a, s0, s1);
+    const int first = (it.ph * a.th - a.pad_h) * a.xt_w;
+    const int skew = (first & 7) - (int)sub;  // the blocks begin (first & 7) pixels before the input rows
+    const int cb1 = (s1 + per_block - 1) / per_block;
+    for (int cb = s0 / per_block; cb < cb1; ++cb) {
+      if (!mbar_wait_warp(xb_empty + 8u * xb.idx, xb.phase ^ 1u, abort_flag)) return;
+      const uint32_t tile = tiles + xb.idx * a.xt_bytes;
+      for (int j = 0; j < a.xt_blocks * (KB / 32); ++j, ++block) {
+        // (a vote: the compiler then knows that the whole warp takes the branch; elsewhere every matrix load and
+        // store would have its own convergence check)
+        if (__all_sync(0xffffffffu, (int)(block & turn) == tw)) {
+          const uint32_t src = slots + ring.idx * kXtSlotBytes + (uint32_t)lane * 128u;
+          const uint32_t half = (uint32_t)(j % (KB / 32)) << 6;  // (the upper 32 channels of a row of 64)
+          const int px0 = 64 * (j / (KB / 32)) - skew;           // this lane's pixel of the first store, counted from the first input row
+          uint32_t dst[8], v[8][4];
+#pragma unroll
+          for (int chunk = 0; chunk < 8; ++chunk) {
+            const int px = px0 + 8 * chunk;
+            int pos = a.xt_dump;
+            if (px >= 0 && px < px_in) {
+              const int row = (int)__umulhi((uint32_t)px, a.xt_magic);
+              pos = row * a.pitch + a.pad_w + (px - row * a.xt_w);
+            }
+            const uint32_t sw = KB == 64 ? ((uint32_t)pos & 7u) : (((uint32_t)pos >> 1) & 3u);
+            dst[chunk] = (tile + (uint32_t)pos * row_bytes + ((octet ^ sw) << 4)) ^ half;
+          }
+          // (the matrix loads and stores take their addresses from all lanes: the wait ends for the warp as one)
+          if (!mbar_wait_warp(in_full + 8u * ring.idx, ring.phase, abort_flag)) return;
+          __syncwarp();
+          // (all loads before the first store: a store waits for its load, and none of them for the one after)
+#pragma unroll
+          for (int chunk = 0; chunk < 8; ++chunk)
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(v[chunk][0]), "=r"(v[chunk][1]), "=r"(v[chunk][2]), "=r"(v[chunk][3])
+                         : "r"(src + (((uint32_t)chunk ^ sub) << 4))
+                         : "memory");
+#pragma unroll
+          for (int chunk = 0; chunk < 8; ++chunk)
+            asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(dst[chunk]), "r"(v[chunk][0]), "r"(v[chunk][1]),
+                         "r"(v[chunk][2]), "r"(v[chunk][3])
+                         : "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(in_empty + 8u * ring.idx);
+        }
+        ring.advance((uint32_t)a.xt_slots);
+      }
+      // the tensor core reads the tile through the async proxy
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(xb_full + 8u * xb.idx);
+      xb.advance((uint32_t)a.xt_bufs);
+    }
+  }
+}
+
 template <int KB, bool HALO, int EW, int EPI, bool SPLIT, bool PAIR = false, bool SHARED = false, bool FUSEL = false,
-          bool DWPW = false>
-__global__ void __launch_bounds__(96 + 32 * EW + (FUSEL ? 32 * kLayoutWarps : 0) + (DWPW ? 32 * kDwWarps : 0), 1)
+          bool DWPW = false, bool TRANS = false>
+__global__ void __launch_bounds__(96 + 32 * EW + (FUSEL ? 32 * kLayoutWarps : 0) + (DWPW ? 32 * kDwWarps : 0) + (TRANS ? 32 * kXtWarps : 0), 1)
 igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
              const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmYr,
              const IgemmArgs a, const __half* __restrict__ bias, __half* __restrict__ y, int* status) {
@@ -1242,7 +1355,9 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __shared__ __align__(8) uint64_t meet_bar;  // shared tiles: meeting point of all epilogue warps,
   __shared__ __align__(8) uint64_t ho_bar;    //   of the warps that hand accumulators over (the first of each lane quarter),
   __shared__ __align__(8) uint64_t pl_bar;    //   of the warps that fetch partial sums (the second of each lane quarter)
-  __shared__ __align__(8) uint64_t in_full[2 * kMaxDwTeams], in_empty[2 * kMaxDwTeams];  // depthwise input tiles (depthwise + pointwise blocks)
+  // depthwise input tiles (depthwise + pointwise blocks), or the staging slots of blocks of x (TRANS)
+  __shared__ __align__(8) uint64_t in_full[kXtSlots], in_empty[kXtSlots];
+  __shared__ __align__(8) uint64_t xb_full[kXtBufs], xb_empty[kXtBufs];  // transposed tiles (TRANS)
   __shared__ __align__(8) uint64_t slabs_full;  // row pairs: the weight slabs have arrived
   __shared__ __align__(8) uint64_t peers_done, parts_in;  // split reduction: the cluster's MMAs are complete; the parts have arrived
   __shared__ __align__(8) uint64_t drain_bar;  // after giving up: the MMAs and commits that were issued are complete
@@ -1265,16 +1380,20 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.stages; ++s) {
       // (one announcement per producer; blocks: the weights' + one arrival per depthwise / gathering warp)
-      mbar_init(smem_u32(&full_bar[s]), DWPW ? 1 + (kDwWarps >> a.dw_teams_log2) : (a.slab_off != 0 ? 1 : 2));
+      mbar_init(smem_u32(&full_bar[s]), DWPW ? 1 + (kDwWarps >> a.dw_teams_log2) : (TRANS || a.slab_off != 0 ? 1 : 2));
       mbar_init(smem_u32(&empty_bar[s]), 1);
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(smem_u32(&acc_full[s]), 1);
       mbar_init(smem_u32(&acc_empty[s]), PAIR ? 2 * EW : EW);  // one arrival per epilogue warp (of both CTAs)
     }
-    for (int b = 0; b < 2 * kMaxDwTeams; ++b) {
+    for (int b = 0; b < kXtSlots; ++b) {
       mbar_init(smem_u32(&in_full[b]), 1);
-      mbar_init(smem_u32(&in_empty[b]), kDwWarps >> a.dw_teams_log2);
+      mbar_init(smem_u32(&in_empty[b]), TRANS ? 1 : kDwWarps >> a.dw_teams_log2);
+    }
+    for (int b = 0; b < kXtBufs; ++b) {
+      mbar_init(smem_u32(&xb_full[b]), kXtWarps);
+      mbar_init(smem_u32(&xb_empty[b]), 1);
     }
     mbar_init(smem_u32(&sk_bar), PAIR ? EW : EW / 2);  // one arrival per fetching warp (of both CTAs)
     for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&q_bar[q]), EW / 4);
@@ -1350,6 +1469,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         tma_load_4d(ring_base + a.slab_off + (uint32_t)i * (64u * KB * 2u), &tmA, bar, 0, 0, r * a.S + tap, 0);
       }
     }
+    [[maybe_unused]] Ring in_ring;
     for (it.init(a); it.valid(a) && ok && !(DWPW && a.gather && !weights) && !(slabs && weights); it.next(a)) {
       int grp, m0;
       it.channel_tile(a, grp, m0);
@@ -1362,6 +1482,33 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       const int h_base = p0 * a.stride_h - a.pad_h;
       int s0, s1;
       it.stage_range(a, s0, s1);
+      if constexpr (TRANS) {
+        if (!weights) {
+          // blocks of 64 pixels x 32 channels of x itself, from the last multiple of 8 pixels before the tile's
+          // first input row on; rows outside the plane are the copies' out-of-bounds fill
+          const int px0 = (h_base * a.xt_w) & ~7;
+          const int cb1 = (s1 + stages_per_block - 1) / stages_per_block;
+          for (int cb = s0 / stages_per_block; cb < cb1 && ok; ++cb) {
+            for (int j = 0; j < a.xt_blocks * (KB / 32); ++j) {
+              if (!mbar_wait(smem_u32(&in_empty[in_ring.idx]), in_ring.phase ^ 1u, &abort_flag, 64)) {
+                ok = false;
+                break;
+              }
+              if (leader) {
+                const uint32_t bar = smem_u32(&in_full[in_ring.idx]);
+                mbar_expect_tx(bar, kXtSlotBytes);
+                if (!(a.dbg_drop >= 0 && blockIdx.x == 0 && issued == (uint32_t)a.dbg_drop))  // (test hook, as below)
+                  tma_load_3d(ring_base + (uint32_t)a.stages * a.stage_bytes + (uint32_t)a.xt_bufs * a.xt_bytes + in_ring.idx * kXtSlotBytes,
+                              &tmB, bar, px0 + 64 * (j / (KB / 32)), grp * a.cg + cb * KB + j % (KB / 32) * 32, n0);
+              }
+              __syncwarp();
+              in_ring.advance((uint32_t)a.xt_slots);
+              ++issued;
+            }
+          }
+          continue;
+        }
+      }
       if constexpr (FUSEL) {
         // the tile reads input rows h_base .. h_base + (th-1)*stride + (R-1)*dil of tn images
         if (!weights && !layout_wait(a.lay_flags, a.N, a.lay_hw / a.lay_w, a.lay_w, a.lay_seg_units * (32 / a.lay_ch) * a.lay_px,
@@ -1472,6 +1619,9 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     bool ready = mbar_test_warp(smem_u32(&full_bar[0]), 0u);
     const bool slabs = EPI == 0 && a.slab_off != 0;
     const uint32_t a_tap = (slabs ? (uint32_t)a.R * (64u * KB * 2u) : a.a_bytes) >> 4;
+    [[maybe_unused]] Ring xt_ring;  // TRANS: transposed tiles, one per channel block
+    [[maybe_unused]] const int xt_groups = a.S / a.taps, xt_spb = a.R * xt_groups;
+    [[maybe_unused]] const uint32_t xt_base = ring_base + depth * a.stage_bytes;
     bool ok_slabs = true;
     if (slabs) ok_slabs = mbar_wait_warp(smem_u32(&slabs_full), 0u, &abort_flag);
     typename WorkIterOf<SPLIT, SHARED>::type it;
@@ -1497,7 +1647,20 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           acc = 1;
         }
       }
+      // TRANS: the stage's kernel row and tap group within its channel block
+      [[maybe_unused]] int xt_st = 0, xt_r = 0, xt_sg = 0;
+      if (TRANS && SHARED) {  // (elsewhere an item starts with a channel block)
+        xt_st = s0 % xt_spb;
+        xt_r = xt_st / xt_groups;
+        xt_sg = xt_st - xt_r * xt_groups;
+      }
       for (int gi = 0; gi < groups_per_tile; ++gi) {
+        if constexpr (TRANS) {
+          if ((gi == 0 || xt_st == 0) && !mbar_wait_warp(smem_u32(&xb_full[xt_ring.idx]), xt_ring.phase, &abort_flag)) {
+            ok = false;
+            break;
+          }
+        }
         if (!ready && !mbar_wait_warp(smem_u32(&full_bar[ring.idx]), ring.phase, &abort_flag)) {
           ok = false;
           break;
@@ -1506,6 +1669,20 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         const uint32_t sbase = ring_base + ring.idx * a.stage_bytes;
         const uint32_t e_bar = smem_u32(&empty_bar[ring.idx]);
         uint32_t b_lo = b_fix | ((sbase & 0x3FFFFu) >> 4);
+        [[maybe_unused]] uint32_t xt_bar = 0;
+        if constexpr (TRANS) {
+          const uint32_t tile = xt_base + xt_ring.idx * a.xt_bytes + (uint32_t)(xt_r * a.dil_h * a.pitch) * row_bytes + (uint32_t)xt_sg * tap_step;
+          b_lo = b_fix | ((tile & 0x3FFFFu) >> 4);
+          if (++xt_sg == xt_groups) {
+            xt_sg = 0;
+            ++xt_r;
+          }
+          if (++xt_st == xt_spb) xt_st = xt_r = 0;
+          if (xt_st == 0 || gi == groups_per_tile - 1) {  // the item's last stage on this transposed tile
+            xt_bar = smem_u32(&xb_empty[xt_ring.idx]);
+            xt_ring.advance((uint32_t)a.xt_bufs);
+          }
+        }
         // (row pairs: one stage per kernel row, its weight tiles in the slabs)
         const uint32_t abase = slabs ? ring_base + a.slab_off + (uint32_t)(a.R - 1 - gi) * (64u * KB * 2u) : sbase + a.b_alloc;
         uint32_t a_lo = a_fix | ((abase & 0x3FFFFu) >> 4);
@@ -1527,6 +1704,9 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           }
           if constexpr (PAIR) umma_commit_pair(e_bar);
           else umma_commit(e_bar);
+          if constexpr (TRANS) {
+            if (xt_bar != 0) umma_commit(xt_bar);
+          }
         }
         __syncwarp();
         acc = 1;
@@ -1701,6 +1881,11 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         ring.advance(depth);
       }
     }
+  } else if (TRANS && warp >= 3 + EW) {
+    // ---------------- x -> channels-last (warps past the producers') ----------------
+    if constexpr (TRANS)
+      transpose_blocks<KB, SPLIT, SHARED>(a, warp - 3 - EW, ring_base + (uint32_t)a.stages * a.stage_bytes, smem_u32(in_full),
+                                          smem_u32(in_empty), smem_u32(xb_full), smem_u32(xb_empty), &abort_flag);
   } else if (FUSEL && warp >= 3 + EW) {
     // ---------------- fused layout pass (warps past the epilogue's) ----------------
     const int64_t gw = (int64_t)blockIdx.x * kLayoutWarps + (warp - 3 - EW);
@@ -1746,11 +1931,12 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     const int per_eff = split_px ? (kPerQuarter << (SPLIT ? fin_log2 : a.dup_log2)) : kPerQuarter;
     const int row = cq * 32 + ((EPI == 2 && a.y_tma) ? ((lane & 3) << 3) + (lane >> 2) : lane);
     uint16_t* yb = reinterpret_cast<uint16_t*>(y);
-    const uint32_t stage_base = ring_base + (uint32_t)a.stages * a.stage_bytes + (SPLIT ? a.recv_bytes : 0u);
+    const uint32_t stage_base = ring_base + (uint32_t)a.stages * a.stage_bytes + (TRANS ? a.xt_total : 0u) + (SPLIT ? a.recv_bytes : 0u);
     const bool relu = a.relu != 0;
     const bool leader = elect_one();  // issues this warp's bulk stores and waits for them (their groups are per thread)
     // this warp's own staging tiles: 32 channel rows of 128 bytes each, 128-byte swizzled
-    const uint32_t my_stage = stage_base + (uint32_t)ew * (uint32_t)a.nbuf * kWarpStageBytes;
+    // (TRANS, at most 64 channels: the warps of two quarters store, and have one each)
+    const uint32_t my_stage = stage_base + (uint32_t)(TRANS && a.epi_tiles < EW ? half * 2 + (quarter & 1) : ew) * (uint32_t)a.nbuf * kWarpStageBytes;
     const uint32_t row_off = (uint32_t)lane * 128u + (((uint32_t)lane & 7u) << 4);
     uint32_t stage_sel = 0;
     uint32_t lt = 0;
@@ -1994,7 +2180,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         const uint32_t col_bytes = (uint32_t)(128 * 4) >> fin_log2;
         const uint32_t part_bytes = (uint32_t)a.ncols * col_bytes;
         // (reads of whole vectors may run up to 31 columns past the last part: into the staging tiles)
-        const uint32_t recv_base = ring_base + (a.recv_bytes != 0 ? (uint32_t)a.stages * a.stage_bytes : 0u);
+        const uint32_t recv_base = ring_base + (a.recv_bytes != 0 ? (uint32_t)a.stages * a.stage_bytes + (TRANS ? a.xt_total : 0u) : 0u);
         cluster_wait();
         met = true;
         if (a.recv_bytes == 0) {
@@ -2221,9 +2407,10 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __syncthreads();
   const bool gave_up_cta = abort_flag != 0;  // (final only here: no warp raises it any more)
   if (gave_up_cta)
-    wait_for_work_under_way<PAIR, DWPW>(warp, EW, rank, (uint32_t)a.stages, EPI == 0 && a.slab_off != 0, 1u + (uint32_t)a.dw_teams_log2,
-                                        smem_u32(full_bar), smem_u32(in_full), smem_u32(&slabs_full), smem_u32(&drain_bar),
-                                        (uint32_t)produced_stages[0], (uint32_t)produced_stages[1]);
+    wait_for_work_under_way<PAIR, DWPW || TRANS>(warp, EW, rank, (uint32_t)a.stages, EPI == 0 && a.slab_off != 0,
+                                                 TRANS ? (uint32_t)a.xt_slots : 2u << a.dw_teams_log2, smem_u32(full_bar),
+                                                 smem_u32(in_full), smem_u32(&slabs_full), smem_u32(&drain_bar),
+                                                 (uint32_t)produced_stages[0], (uint32_t)produced_stages[1]);
   // (a pair leaves together: the first CTA's MMAs read the partner's shared memory and write its tensor memory)
   if constexpr (PAIR) cluster_sync_all();
   if constexpr (SPLIT) {
@@ -2381,7 +2568,14 @@ bool igemm_make_plan(const ConvGeom& g, IgemmPlan* out) {
     // stages fit as well (small pixel tiles: 14x14 and 7x7 planes) they are faster, because the
     // copies then move 128-byte rows (measured: VGG conv5 27.7 -> 22.9 us)
     IgemmPlan wide{};
-    if (make_plan_impl(gs, &wide, false, 64, true) && wide.kb == 64 && wide.stages >= 3) single = wide;
+    if (make_plan_impl(gs, &wide, false, 64, true) && wide.kb == 64 && wide.ring_stages >= 3) single = wide;
+  }
+  if (ok_single && single.kb == 64 && !single.trans && g.cg > 32 && g.want_kb == 0) {
+    // blocks of 32 channels where the kernel can turn x channels-last itself with those only (tiles of wide
+    // rows: two transposed tiles of 64 channels leave no room for the weights), and the pass over x is saved
+    // (64->128 on 112x112, 16 images 36.5 -> 29.9 us, one image 11.0 -> 8.5; 5x5 64->96 on 80x80 37.3 -> 31.1)
+    IgemmPlan narrow{};
+    if (make_plan_impl(gs, &narrow, false, 32, false) && narrow.trans) single = narrow;
   }
   if (!g.no_pair && g.kg > 128) {
     IgemmPlan pair{};
@@ -2966,6 +3160,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
       p.plane_bytes = (uint32_t)round_up_sz((size_t)(32 * pq * 2), 128) * (uint32_t)p.plane_store;
     }
   }
+  p.epi_tiles = p.epi_warps;
   const size_t stage_buf_bytes = p.plane_store ? (size_t)4 * p.plane_bytes : (size_t)p.epi_warps * kWarpStageBytes;
   // rings: B two or three deep, A with what is left (each A stage feeds kb/16 MMAs).  227 KB per
   // CTA minus alignment slack, static barriers and the two epilogue staging buffers.
@@ -3044,6 +3239,47 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
       p.ncols = (p.tn * p.th * g.q + 15) / 16 * 16;
     }
   }
+  // x turned channels-last by the kernel itself (IgemmArgs::xt_*): stride-1 layers of several taps whose planes
+  // the copy engine can address (a multiple of 8 pixels), tiles of one image, wherever two transposed tiles, the slots
+  // and two stages of weights fit.  Against the separate pass it was the faster form on every layer measured (us,
+  // pass included): 16 images 128->128 on 112x112 64.7 -> 51.4, 128->256 on 56x56 34.0 -> 30.6, 256->256 55.6 -> 51.3,
+  // 512->512 on 28x28 51.2 -> 49.9; 64 images 64->64 on 56x56 33.1 -> 27.1, 128->128 on 28x28 24.1 -> 18.3; one image 256->256 on
+  // 56x56 14.1 -> 12.0.  1x1 layers have less to hide it behind, and read such planes in place.
+  p.trans = 0;
+  p.xt_total = 0;
+  p.ring_stages = p.stages;  // (what the choice of the block's width goes by, see igemm_make_plan)
+  if (p.halo && !p.nchw && !p.x_nhwc && !p.y_nhwc && !p.window && !p.patch && !p.pair && !g.rowpair && g.dw_stride == 0 && g.no_fuse &&
+      !p.gather && p.kb >= 32 && p.tn == 1 && g.r * g.s > 1 && ((int64_t)g.h * g.w) % 8 == 0 && (g.group == 1 || g.cg % p.kb == 0) &&
+      p.epi_warps == kEpilogueWarps && p.dup_log2 == 0 && g.w > 1) {
+    const int rows_in = p.th + (g.r - 1) * g.dil_h;
+    const int skew = g.w % 8 == 0 ? 0 : 7;
+    size_t reach = (size_t)p.ncols + (size_t)(g.r - 1) * g.dil_h * p.pitch + (size_t)(g.s - 1) * g.dil_w;
+    if (reach < (size_t)rows_in * p.pitch) reach = (size_t)rows_in * p.pitch;
+    const size_t tile = round_up_sz((reach + 1) * p.kb * 2u, 1024);
+    const size_t recv_own = p.recv ? split_bytes(p.ncols, best_ks) : 0;  // (the parts of a split reduction stay where they were)
+    // A ring stage holds the weight tiles of a kernel row, three of them if they fit, else two.  (One tap per stage
+    // is a hand-shake per four MMAs; 16 KB of slots in place of 32 do not hide the latency of the copies.)
+    // Layers of at most 64 output channels need staging tiles for the warps of two lane quarters only.
+    const int32_t trans_epi = p.tma_store && g.kg <= 64 && best_ks == 0 && !best_shared ? kEpilogueWarps / 2 : kEpilogueWarps;
+    const size_t trans_budget = budget_all - (size_t)trans_epi * kWarpStageBytes;
+    const size_t st = (size_t)g.s * p.a_bytes;
+    const size_t xt = kXtBufs * tile + kXtSlots * (size_t)kXtSlotBytes;
+    int stages = xt + recv_own < trans_budget ? (int)((trans_budget - xt - recv_own) / st) : 0;
+    if (stages > kMaxStages) stages = kMaxStages;
+    if (stages >= 2 && (best_ks == 0 || p.recv || xt + stages * st >= split_bytes(p.ncols, best_ks))) {
+      p.trans = 1;
+      p.stages = stages;
+      p.b_alloc = 0;
+      p.stage_bytes = (uint32_t)st;
+      p.epi_tiles = trans_epi;
+      p.xt_rows_in = rows_in;
+      p.xt_blocks = (rows_in * g.w + skew + 63) / 64;
+      p.xt_slots = kXtSlots;
+      p.xt_dump = (int32_t)reach;
+      p.xt_bytes = (uint32_t)tile;
+      p.xt_total = (uint32_t)xt;
+    }
+  }
   // Resident weights: where every tile of a CTA has the same channel tile (the grid is a multiple of
   // their number) and the ring holds a whole number of tiles' stages, a stage finds the weights it
   // needs in place after the first lap; only activations are fetched from then on.  The ring is
@@ -3060,8 +3296,9 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     }
   }
   // a second staging tile per epilogue warp (its store overlaps the next unit) if memory is left
-  p.nbuf = (!p.plane_store && !p.recv && p.slabs == 0 && (size_t)p.stages * p.stage_bytes + 2u * stage_buf_bytes <= budget_all) ? 2 : 1;
-  p.smem_bytes = (size_t)p.stages * p.stage_bytes + (size_t)p.nbuf * stage_buf_bytes + (size_t)p.slabs + (p.dw_in_alloc << (1 + p.dw_teams_log2)) + 1024 +
+  const size_t epi_bytes = p.trans ? (size_t)p.epi_tiles * kWarpStageBytes : stage_buf_bytes;
+  p.nbuf = (!p.plane_store && !p.recv && p.slabs == 0 && (size_t)p.stages * p.stage_bytes + p.xt_total + 2u * epi_bytes <= budget_all) ? 2 : 1;
+  p.smem_bytes = (size_t)p.stages * p.stage_bytes + p.xt_total + (size_t)p.nbuf * epi_bytes + (size_t)p.slabs + (p.dw_in_alloc << (1 + p.dw_teams_log2)) + 1024 +
                  (p.recv ? split_bytes(p.ncols, best_ks) : 0u);
   // more than half of an SM's shared memory: at most one CTA per SM, so that the kernel can take
   // all 512 TMEM columns without ever waiting for another CTA to free them
@@ -3176,7 +3413,7 @@ bool igemm_encode_maps(const ConvGeom& g_layer, IgemmPlan* p, void* ws) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return false;
   }
-  if (p->nchw) {
+  if (p->nchw || p->trans) {
     // the activation map is over the caller's x and is encoded when x is known (igemm_encode_x_map)
   } else if (p->patch) {
     // x''[N][P][Q][kelems] as (element, -, output column, output row, image)
@@ -3226,15 +3463,15 @@ bool igemm_encode_maps(const ConvGeom& g_layer, IgemmPlan* p, void* ws) {
   return true;
 }
 
-// 1x1 layers that read x directly: x[N][C][H*W] seen as (pixel, channel, image), 64 pixels x kb
-// channels per box, 128-byte swizzle (pixel-major operand tiles).
+// Layers that read x directly: x[N][C][H*W] seen as (pixel, channel, image), 64 pixels x kb (32)
+// channels per box, 128-byte swizzle (pixel-major operand tiles of 1x1 layers, blocks to be transposed).
 bool igemm_encode_x_map(const ConvGeom& g, IgemmPlan* p, const void* x) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
   if (enc == nullptr) return false;
   const cuuint64_t hw = (cuuint64_t)g.h * g.w;
   cuuint64_t dims[3] = {hw, (cuuint64_t)g.c, (cuuint64_t)g.n};
   cuuint64_t strides[2] = {hw * 2, hw * 2 * (cuuint64_t)g.c};
-  cuuint32_t box[3] = {64, (cuuint32_t)p->kb, 1};
+  cuuint32_t box[3] = {64, p->trans ? 32u : (cuuint32_t)p->kb, 1};
   cuuint32_t es[3] = {1, 1, 1};
   if (enc(&p->tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(x), dims, strides, box, es,
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -3286,7 +3523,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   if (!p.maps_ready) return cudaErrorInvalidValue;
   if (dw != nullptr && (!p.x_nhwc || p.pair || p.sk_split || p.ks_log2 > 0 || p.fuse_layout || p.kb < 32))
     return cudaErrorInvalidValue;
-  if (p.nchw && !p.gather && p.x_mapped != x && !igemm_encode_x_map(g, &p, x)) return cudaErrorInvalidValue;
+  if (((p.nchw && !p.gather) || p.trans) && p.x_mapped != x && !igemm_encode_x_map(g, &p, x)) return cudaErrorInvalidValue;
   if (dw != nullptr && p.x_mapped != x) {  // the block's input tiles come from x (channels-last) with their border
     if (p.dw_in_bytes == 0 || !encode_dw_input_map(*dw, g.n, &p)) return cudaErrorInvalidValue;
     p.x_mapped = x;
@@ -3372,6 +3609,12 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   a.lay_hw = g.h * g.w; a.lay_w = g.w;
   a.lay_units_p = p.lay_units_p; a.lay_units_c = p.lay_units_c;
   a.lay_seg_units = p.lay_seg_units; a.lay_segs = p.lay_segs;
+  a.xt_w = g.w;
+  a.xt_rows_in = p.xt_rows_in;
+  a.xt_magic = (uint32_t)((0x100000000ull + (uint64_t)g.w - 1) / (uint64_t)g.w);
+  a.xt_blocks = p.xt_blocks; a.xt_slots = p.xt_slots; a.xt_bufs = kXtBufs;
+  a.epi_tiles = p.epi_tiles;
+  a.xt_dump = p.xt_dump; a.xt_bytes = p.xt_bytes; a.xt_total = p.xt_total;
   a.ts = p.ts;
   a.pair = p.pair;
   a.ncols_sub = p.ncols_sub;
@@ -3482,7 +3725,35 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
     else if (!p.tma_store) HGC_LAUNCH_PAIR_EPI(KBV, HALOV, 1);     \
     else HGC_LAUNCH_PAIR_EPI(KBV, HALOV, 0);                       \
   } while (0)
-  if (dw != nullptr || p.gather) {
+  // x turned channels-last by the kernel: its own instantiations (8 epilogue + 4 transposing warps)
+#define HGC_LAUNCH_TRANS_EPI(KBV, EPIV)                                                                    \
+  do {                                                                                                     \
+    const dim3 xt_block(96 + 32 * 8 + 32 * kXtWarps);                                                      \
+    if (p.ks_log2 > 0) {                                                                                   \
+      err = allow_dynamic_smem<igemm_kernel<KBV, true, 8, EPIV, true, false, false, false, false, true>>(); \
+      if (err == cudaSuccess)                                                                              \
+        err = launch_kernel_cluster(1u << p.ks_log2, igemm_kernel<KBV, true, 8, EPIV, true, false, false, false, false, true>, grid, \
+                                    xt_block, p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, status); \
+    } else if (p.sk_split) {                                                                               \
+      err = allow_dynamic_smem<igemm_kernel<KBV, true, 8, EPIV, false, false, true, false, false, true>>(); \
+      if (err == cudaSuccess)                                                                              \
+        err = launch_kernel_coop(true, igemm_kernel<KBV, true, 8, EPIV, false, false, true, false, false, true>, grid, \
+                                 xt_block, p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, status); \
+    } else {                                                                                               \
+      err = allow_dynamic_smem<igemm_kernel<KBV, true, 8, EPIV, false, false, false, false, false, true>>(); \
+      if (err == cudaSuccess)                                                                              \
+        err = launch_kernel_overlapped(igemm_kernel<KBV, true, 8, EPIV, false, false, false, false, false, true>, grid, \
+                                       xt_block, p.smem_bytes, stream, p.tmA, p.tmB, p.tmY, p.tmYr, a, bias, y, status); \
+    }                                                                                                      \
+  } while (0)
+#define HGC_LAUNCH_TRANS(KBV)                        \
+  do {                                               \
+    if (p.tma_store) HGC_LAUNCH_TRANS_EPI(KBV, 0);   \
+    else HGC_LAUNCH_TRANS_EPI(KBV, 1);               \
+  } while (0)
+  if (p.trans) {
+    if (p.kb == 64) HGC_LAUNCH_TRANS(64); else HGC_LAUNCH_TRANS(32);
+  } else if (dw != nullptr || p.gather) {
     if (p.kb == 64) HGC_LAUNCH_DWPW(64); else HGC_LAUNCH_DWPW(32);
   } else if (p.pair) {
     if (p.kb == 64) {
@@ -3537,6 +3808,8 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
 #undef HGC_LAUNCH_FUSED
 #undef HGC_LAUNCH_DWPW_EPI
 #undef HGC_LAUNCH_DWPW
+#undef HGC_LAUNCH_TRANS_EPI
+#undef HGC_LAUNCH_TRANS
   if (err != cudaSuccess) return err;
   count_launch();
   return cudaGetLastError();
