@@ -2316,11 +2316,15 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     const uint32_t sbuf = my_stage + stage_sel * kWarpStageBytes;
                     stage_sel = a.nbuf == 2 ? stage_sel ^ 1u : 0u;
                     bool first = true;
+                    // (without junk columns the rows of a unit are consecutive columns: one run, not nrows short ones;
+                    //  with the rows dealt out evenly 442 -> 433 us for ResNet-50's layers, channels-last, 16 images)
+                    const bool one_run = a.pitch == a.Q;
+                    const int runs = one_run ? 1 : nrows, run_px = one_run ? nrows * ncol : ncol;
 #pragma unroll 1
-                    for (int r = 0; r < nrows; ++r) {
+                    for (int r = 0; r < runs; ++r) {
 #pragma unroll 1
                       for (int g = 0; g < 2; ++g) {
-                        const int rem = ncol - g * 32;
+                        const int rem = run_px - g * 32;
                         if (rem <= 0) break;
                         const uint32_t tcol = (uint32_t)((img * a.th + hr0 + r) * a.pitch + wc0 + g * 32);
                         uint32_t v[32];
@@ -3104,11 +3108,17 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     p.tma_store = (g.kg % 32) == 0 ? 1 : 0;
     p.y_perm = p.tma_store;
     p.y_rpu = (g.q > 32 || best_ks > 0) ? 1 : (kPassElems / g.q < p.th ? kPassElems / g.q : p.th);  // (split tiles: more warps share them)
-    p.y_full_w = g.q > kPassElems ? kPassElems : p.y_rpu * g.q;
-    p.rem = g.q > kPassElems ? g.q % kPassElems : (p.th % p.y_rpu) * g.q;
     p.epi_warps = kEpilogueWarps;
     if (p.tma_store && mpt * 130.0 < 600.0 + 10.0 * p.ncols && p.tn * p.th * ((g.q + kPassElems - 1) / kPassElems) > 2)
       p.epi_warps = kEpilogueWarpsWide;
+    // One tile per CTA: no next tile's MMAs hide the epilogue, so it is dealt out evenly to the warps of a lane
+    // quarter (256->256 3x3 on 14x14, 16 images 9.84 -> 9.62 us; four warps per quarter gain nothing more).
+    if (p.tma_store && total <= sms && best_ks == 0 && !best_shared && !want_pair && g.dw_stride == 0 && !p.gather) {
+      const int even = (p.tn * p.th + p.epi_warps / 4 - 1) / (p.epi_warps / 4);
+      if (p.y_rpu > even) p.y_rpu = even;
+    }
+    p.y_full_w = g.q > kPassElems ? kPassElems : p.y_rpu * g.q;
+    p.rem = g.q > kPassElems ? g.q % kPassElems : (p.th % p.y_rpu) * g.q;
   }
   p.sk_split = best_shared;
   p.grid = best_grid;
