@@ -563,7 +563,7 @@ __device__ __forceinline__ void issue_mmas(uint32_t d_tmem, uint32_t a_lo, uint3
 
 // Where an epilogue reads its fp32 sums: the accumulator in tensor memory (lane = output channel), or,
 // for a tile whose reduction a cluster of CTAs shared (SPLIT), the parts that the CTAs put into this
-// one's shared memory as [part][column][lanes], added to the bias in the order of the parts.
+// one's shared memory as [part][pair of columns][lanes][2], added to the bias in the order of the parts.
 struct AccSource {
   uint32_t addr;        // tensor-memory address of column 0, or shared-memory address of this lane's column 0
   uint32_t col_bytes;   // SPLIT: bytes from column to column and from part to part, and the number of parts
@@ -581,10 +581,17 @@ __device__ __forceinline__ void acc_load(const AccSource& s, uint32_t col, uint3
 #pragma unroll
     for (int j = 0; j < N; ++j) f[j] = s.first;
     for (int p = 0; p < s.parts; ++p) {
-      const uint32_t src = s.addr + (uint32_t)p * s.part_bytes + col * s.col_bytes;
+      const uint32_t src = s.addr + (uint32_t)p * s.part_bytes + (col >> 1) * (2u * s.col_bytes);
       float t[N];  // (all of a part's loads are under way before the first sum waits for one)
+      if ((col & 1u) == 0) {
 #pragma unroll
-      for (int j = 0; j < N; ++j) asm volatile("ld.shared.f32 %0, [%1];" : "=f"(t[j]) : "r"(src + (uint32_t)j * s.col_bytes));
+        for (int j = 0; j < N; j += 2)
+          asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(t[j]), "=f"(t[j + 1]) : "r"(src + (uint32_t)j * s.col_bytes));
+      } else {
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+          asm volatile("ld.shared.f32 %0, [%1];" : "=f"(t[j]) : "r"(src + (uint32_t)((j + 1) / 2) * (2u * s.col_bytes) + (j % 2 == 0 ? 4u : 0u)));
+      }
 #pragma unroll
       for (int j = 0; j < N; ++j) f[j] += t[j];
     }
@@ -2171,8 +2178,9 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       AccSource acc_src{t_tile + (uint32_t)(sub * a.ncols_sub), 0u, 0u, 0, 0.f};
       if constexpr (SPLIT) {
         // Every CTA of the cluster has the sums of its ring stages for all 128 channels in its tensor
-        // memory and sends every CTA those of the channels that one finishes, as [part][column][lanes],
-        // 128 bytes per column and warp; the receiver adds the parts in order.  They go behind the
+        // memory and sends every CTA those of the channels that one finishes, as [part][pair of columns]
+        // [lanes][2], 256 bytes per pair and warp (single columns, twice the stores and loads: the VGG-16 classifier at batch 64
+        // 63.7 us, 62.4 in pairs); the receiver adds the parts in order.  They go behind the
         // ring where the plan found room (three ring stages are left), else into the ring
         // once all MMAs of the cluster are complete.  The transfer runs at about 27 bytes per clock and
         // SM, 1.2 us for 128 columns over four CTAs; waiting for the partners first costs 0.7 us.
@@ -2193,16 +2201,16 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         }
         const uint32_t dest = (uint32_t)(quarter / rep_q);
         const uint32_t dst = cluster_addr(recv_base, dest) + (uint32_t)part * part_bytes +
-                             (uint32_t)((quarter & (rep_q - 1)) * 32 + lane) * 4u;
+                             (uint32_t)((quarter & (rep_q - 1)) * 32 + lane) * 8u;
         if (m0 + quarter * 32 < a.kg) {
           for (int c = half * 32; c < a.ncols; c += kPerQuarter * 32) {
             uint32_t v[32];
             tmem_ld32(t_tile + (uint32_t)c, v);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
+            for (int j = 0; j < 32; j += 2)
               if (c + j < a.ncols)
-                asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(dst + (uint32_t)(c + j) * col_bytes), "r"(v[j]) : "memory");
+                asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(dst + (uint32_t)(c + j) * col_bytes), "r"(v[j]), "r"(v[j + 1]) : "memory");
           }
         }
         __syncwarp();
@@ -2212,7 +2220,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           gave_up = true;
           break;
         }
-        acc_src = AccSource{recv_base + (uint32_t)((quarter & (rep_q - 1)) * 32 + lane) * 4u, col_bytes, part_bytes, 1 << a.ks_log2, bv};
+        acc_src = AccSource{recv_base + (uint32_t)((quarter & (rep_q - 1)) * 32 + lane) * 8u, col_bytes, part_bytes, 1 << a.ks_log2, bv};
         bv = 0.f;  // (the sum begins with the bias; one tile per CTA here)
       }
       if constexpr (EPI == 0) {
