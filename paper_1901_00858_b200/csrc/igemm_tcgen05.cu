@@ -1394,11 +1394,12 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       mbar_init(smem_u32(&acc_full[s]), 1);
       mbar_init(smem_u32(&acc_empty[s]), PAIR ? 2 * EW : EW);  // one arrival per epilogue warp (of both CTAs)
     }
-    for (int b = 0; b < kXtSlots; ++b) {
+    // (an instantiation initialises the barriers that it uses: one after the other they take a launch's time)
+    for (int b = 0; b < (DWPW || TRANS ? kXtSlots : 0); ++b) {
       mbar_init(smem_u32(&in_full[b]), 1);
       mbar_init(smem_u32(&in_empty[b]), TRANS ? 1 : kDwWarps >> a.dw_teams_log2);
     }
-    for (int b = 0; b < kXtBufs; ++b) {
+    for (int b = 0; b < (TRANS ? kXtBufs : 0); ++b) {
       mbar_init(smem_u32(&xb_full[b]), kXtWarps);
       mbar_init(smem_u32(&xb_empty[b]), 1);
     }
