@@ -228,7 +228,8 @@ int hgc_conv_path(const hgc_conv_desc* d, int32_t* path);
  * as pixel-major tiles; channels-last x, which includes every input with a 1x1 plane), 2 = a
  * zero-bordered 8-channel NHWC copy read through
  * overlapping windows (few input channels), 3 = an expanded copy holding, per output pixel, the
- * values under the kernel (few input channels, strided), 4 = x itself, gathered by extra warps of
+ * values under the kernel (few input channels, strided; 2 and 3: layers of few products and a small
+ * input tile run as one CUDA-core launch instead and make no copy), 4 = x itself, gathered by extra warps of
  * the kernel (1x1 layers on small planes, see HGC_FLAG_GATHER_X), [11] the number of CTAs that share
  * the reduction of one tile (1, or 2 / 4 / 8 for layers with very few tiles, e.g. inner products:
  * a cluster whose CTAs send one another their fp32 sums and add them in a fixed order), [12] the
