@@ -103,9 +103,9 @@ HostStaging host_staging(const hgc_conv_desc* d) {
   return s;
 }
 
-// hgc_conv_desc_create; want_kb and whole_sums (no tile's reduction shared by CTAs) fix the order of the
-// sums, 0 and false leave it to the planner.
-int create_desc(hgc_conv_desc** out, const hgc_conv_params* p, int32_t want_kb, bool whole_sums) {
+// hgc_conv_desc_create; want_kb, whole_sums (no tile's reduction shared by CTAs) and no_small_stem fix the order
+// of the sums, 0 and false leave it to the planner.
+int create_desc(hgc_conv_desc** out, const hgc_conv_params* p, int32_t want_kb, bool whole_sums, bool no_small_stem) {
   if (p->n < 1 || p->c < 1 || p->h < 1 || p->w < 1 || p->k < 1 || p->r < 1 || p->s < 1)
     return HGC_INVALID_ARG;
   if (p->group < 1 || p->stride_h < 1 || p->stride_w < 1 || p->dil_h < 1 || p->dil_w < 1)
@@ -136,6 +136,7 @@ int create_desc(hgc_conv_desc** out, const hgc_conv_params* p, int32_t want_kb, 
   g.no_fuse = (p->flags & HGC_FLAG_FUSED_LAYOUT) ? 0 : 1;
   g.no_gather = (p->flags & HGC_FLAG_GATHER_X) ? 0 : 1;
   g.want_kb = want_kb;
+  g.no_small_stem = no_small_stem ? 1 : 0;
   g.no_cluster = whole_sums ? 1 : ((p->flags & HGC_FLAG_WHOLE_TILES) ? 2 : 0);
   if (whole_sums && g.no_split == 2) g.no_split = 1;
   const bool channels_last = g.x_nhwc || g.y_nhwc;
@@ -171,7 +172,8 @@ bool same_sums(const hgc_conv_desc* a, const hgc_conv_desc* b) {
   if (a->path != HGC_PATH_IGEMM) return true;
   const hgc::IgemmPlan &p = a->igemm, &q = b->igemm;
   return p.kb == q.kb && p.ks_log2 == q.ks_log2 && p.sk_split == 0 && q.sk_split == 0 && p.pair == q.pair &&
-         p.rowpair == q.rowpair && p.window == q.window && p.patch == q.patch;
+         p.rowpair == q.rowpair && p.window == q.window && p.patch == q.patch &&
+         hgc::stem_small_supported(a->geom) == hgc::stem_small_supported(b->geom);
 }
 
 // The layer of descriptor d for n images with the order of its sums kept; NULL where that cannot be had.
@@ -180,7 +182,9 @@ hgc_conv_desc* chunk_desc(const hgc_conv_desc* d, int32_t n) {
   p.n = n;
   hgc_conv_desc* sub = nullptr;
   const bool igemm = d->path == HGC_PATH_IGEMM;
-  if (create_desc(&sub, &p, igemm && d->igemm.kb >= 32 ? d->igemm.kb : 0, igemm && d->igemm.ks_log2 == 0) != HGC_OK) return nullptr;
+  if (create_desc(&sub, &p, igemm && d->igemm.kb >= 32 ? d->igemm.kb : 0, igemm && d->igemm.ks_log2 == 0,
+                  !hgc::stem_small_supported(d->geom)) != HGC_OK)
+    return nullptr;
   if (same_sums(d, sub)) return sub;
   hgc_conv_desc_destroy(sub);
   return nullptr;
@@ -460,7 +464,7 @@ extern "C" {
 int hgc_conv_desc_create(hgc_conv_desc** out, const hgc_conv_params* p) {
   if (out == nullptr) return HGC_INVALID_ARG;
   *out = nullptr;
-  return p == nullptr ? HGC_INVALID_ARG : create_desc(out, p, 0, false);
+  return p == nullptr ? HGC_INVALID_ARG : create_desc(out, p, 0, false, false);
 }
 
 int hgc_conv_desc_destroy(hgc_conv_desc* d) {

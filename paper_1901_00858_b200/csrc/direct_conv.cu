@@ -223,7 +223,7 @@ constexpr int64_t kStemProducts = 8 << 20;
 constexpr int64_t kStemLoads = 8 * kStemThreads;
 
 bool stem_small_supported(const ConvGeom& g) {
-  if (g.group != 1 || g.c > 8 || g.x_nhwc || g.y_nhwc) return false;
+  if (g.group != 1 || g.c > 8 || g.x_nhwc || g.y_nhwc || g.no_small_stem) return false;
   const int64_t pq = (int64_t)g.p * g.q;
   if ((int64_t)g.c * g.r * g.s > 512 || (int64_t)g.n * pq * g.k * g.c * g.r * g.s > kStemProducts) return false;
   const StemTile t = stem_tile(g);

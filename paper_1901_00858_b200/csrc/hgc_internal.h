@@ -27,6 +27,7 @@ struct ConvGeom {
   int32_t no_dup;          // 1: the weight rows are laid out once, whatever their number (IgemmPlan::dup_log2)
   // The order in which the sums are taken (chunks of images of one layer keep the whole layer's, see same_sums):
   int32_t want_kb;         // channels per reduction block: 32 or 64, or 0 = the planner's choice
+  int32_t no_small_stem;   // 1: not the one-launch form of image stems, however little work it is (chunks of a larger layer)
   int32_t no_cluster;      // 1: no tile's reduction is dealt out to a cluster of CTAs; 2: only those of layers that leave most SMs idle
   int32_t dw_stride;       // > 0: the pointwise layer of a depthwise + pointwise block; the depthwise layer's stride
   int32_t rowpair;         // planner-internal: this is the re-stated form of a 64-channel layer (IgemmPlan::rowpair)

@@ -73,6 +73,11 @@ SAME_BITS = [
     ("tiles shared by CTAs in the whole batch", params_dict(16, 256, 56, 56, 256, 3, 3, 1, 1), "", 1),
     ("row pairs", params_dict(4, 64, 224, 224, 64, 3, 3, 1, 1), "", 4),
     ("stem", params_dict(33, 3, 224, 224, 64, 7, 7, 3, 3, 2, 2), "", 4),
+    ("stem whose chunks are of little work (1x3)", params_dict(64, 2, 128, 128, 2, 1, 3, 0, 1), "", 2),
+    ("the same, 1x7", params_dict(128, 1, 128, 128, 1, 1, 7, 0, 3), "", 2),
+    ("the same, 2x2", params_dict(128, 1, 192, 192, 1, 2, 2), "", 4),
+    ("the same, 1x1, last chunk smaller", params_dict(200, 3, 128, 128, 1, 1, 1), "", 3),
+    ("the same, 1x1", params_dict(400, 3, 96, 96, 2, 1, 1), "", 4),
     ("1x1 read in place", params_dict(8, 256, 56, 56, 512, 1, 1), "", 4),
     ("CTA pairs whose chunks would take other blocks", params_dict(6, 128, 56, 56, 256, 3, 3, 1, 1), "pairs", 1),
     ("depthwise", params_dict(32, 32, 112, 112, 32, 3, 3, 1, 1, 1, 1, 1, 1, 32), "", 4),
