@@ -27,6 +27,7 @@ struct ConvGeom {
   int32_t no_dup;          // 1: the weight rows are laid out once, whatever their number (IgemmPlan::dup_log2)
   // The order in which the sums are taken (chunks of images of one layer keep the whole layer's, see same_sums):
   int32_t want_kb;         // channels per reduction block: 32 or 64, or 0 = the planner's choice
+  int32_t want_trans;      // 1: x turned channels-last inside the kernel wherever that is possible
   int32_t no_small_stem;   // 1: not the one-launch form of image stems, however little work it is (chunks of a larger layer)
   int32_t no_cluster;      // 1: no tile's reduction is dealt out to a cluster of CTAs; 2: only those of layers that leave most SMs idle
   int32_t dw_stride;       // > 0: the pointwise layer of a depthwise + pointwise block; the depthwise layer's stride
@@ -383,6 +384,7 @@ struct IgemmPlan {
   int32_t flat;
   // x (NCHW) turned channels-last inside the kernel, no copy of it in memory: IgemmArgs::xt_*
   int32_t ring_stages;
+  double est_clk;  // estimated clocks, a pass over x included (layers that could save it; 0: not one of them)
   int32_t epi_tiles;
   int32_t trans, xt_rows_in, xt_blocks, xt_slots, xt_dump;
   uint32_t xt_bytes, xt_total;

@@ -2584,11 +2584,17 @@ bool igemm_make_plan(const ConvGeom& g, IgemmPlan* out) {
     if (make_plan_impl(gs, &wide, false, 64, true) && wide.kb == 64 && wide.ring_stages >= 3) single = wide;
   }
   if (ok_single && single.kb == 64 && !single.trans && g.cg > 32 && g.want_kb == 0) {
-    // blocks of 32 channels where the kernel can turn x channels-last itself with those only (tiles of wide
-    // rows: two transposed tiles of 64 channels leave no room for the weights), and the pass over x is saved
-    // (64->128 on 112x112, 16 images 36.5 -> 29.9 us, one image 11.0 -> 8.5; 5x5 64->96 on 80x80 37.3 -> 31.1)
+    // Blocks of 32 channels where the kernel can turn x channels-last itself with those only (tiles of wide
+    // rows: two transposed tiles of 64 channels leave no room for the weights), the pass over x is saved and the
+    // estimate is below the one of the wide plan, which may deal a reduction out to a cluster or keep its weights
+    // in the ring where the narrow one cannot (64->128 on 112x112, 16 images 36.5 -> 29.9 us, one image 11.0 -> 8.5;
+    // 5x5 64->96 on 80x80 37.3 -> 31.1; but 1 x 986 -> 19, 3x1 on 20x20, eight slices 12.4, whole 28.9).  Tiles are not shared
+    // where the wide plan does not share them: layers that do have no chunks of host calls.
+    ConvGeom gn = gs;
+    gn.want_trans = 1;
+    if (gn.no_split == 2 && !single.sk_split) gn.no_split = 1;
     IgemmPlan narrow{};
-    if (make_plan_impl(gs, &narrow, false, 32, false) && narrow.trans) single = narrow;
+    if (make_plan_impl(gn, &narrow, false, 32, false) && narrow.trans && narrow.est_clk < single.est_clk) single = narrow;
   }
   if (!g.no_pair && g.kg > 128) {
     IgemmPlan pair{};
@@ -3258,25 +3264,73 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
       p.ncols = (p.tn * p.th * g.q + 15) / 16 * 16;
     }
   }
-  // x turned channels-last by the kernel itself (IgemmArgs::xt_*): stride-1 layers of several taps whose planes
-  // the copy engine can address (a multiple of 8 pixels), tiles of one image, wherever two transposed tiles, the slots
-  // and two stages of weights fit.  Against the separate pass it was the faster form on every layer measured (us,
-  // pass included): 16 images 128->128 on 112x112 64.7 -> 51.4, 128->256 on 56x56 34.0 -> 30.6, 256->256 55.6 -> 51.3,
-  // 512->512 on 28x28 51.2 -> 49.9; 64 images 64->64 on 56x56 33.1 -> 27.1, 128->128 on 28x28 24.1 -> 18.3; one image 256->256 on
-  // 56x56 14.1 -> 12.0.  1x1 layers have less to hide it behind, and read such planes in place.
+  // x turned channels-last by the kernel itself (IgemmArgs::xt_*) in place of the separate pass: stride-1 layers of
+  // several taps whose planes the copy engine can address (a multiple of 8 pixels), tiles of one image, where two
+  // transposed tiles, the slots and two stages of weights fit.  1x1 layers have less to hide it behind, and read
+  // such planes in place.
   p.trans = 0;
   p.xt_total = 0;
   p.ring_stages = p.stages;  // (what the choice of the block's width goes by, see igemm_make_plan)
-  if (p.halo && !p.nchw && !p.x_nhwc && !p.y_nhwc && !p.window && !p.patch && !p.pair && !g.rowpair && g.dw_stride == 0 && g.no_fuse &&
-      !p.gather && p.kb >= 32 && p.tn == 1 && g.r * g.s > 1 && ((int64_t)g.h * g.w) % 8 == 0 && (g.group == 1 || g.cg % p.kb == 0) &&
-      p.epi_warps == kEpilogueWarps && p.dup_log2 == 0 && g.w > 1) {
+  // Resident weights: where every tile of a CTA has the same channel tile (the grid is a multiple of
+  // their number) and the ring holds a whole number of tiles' stages, a stage finds the weights it
+  // needs in place after the first lap; only activations are fetched from then on.  The ring is
+  // cut to such a number when at least three stages are left.  (ResNet-50's 7x7 stem fetched 28 KB of
+  // weights for every output row of 13 KB.)
+  auto resident_stages = [&](int stages) {
+    const int64_t mgn = (int64_t)p.mtiles * g.group;
+    const int ts = p.cblocks * p.eff_r * (p.eff_s / p.taps), st = stages / ts * ts;
+    return !p.pair && !p.sk_split && best_ks == 0 && p.slabs == 0 && p.grid % mgn == 0 && p.total_tiles > p.grid && st > 0 &&
+                   (st == stages || st >= 3)
+               ? st
+               : 0;
+  };
+  // Estimated clocks of the layer, behind a pass over x or (xt_blocks > 0) with x transposed in the kernel, xt_blocks
+  // blocks of 64 pixels x 32 channels per tile and 32 channels.  A channel block is bounded by its MMAs, by about
+  // 300 clocks per stage and 60 per MMA for the issuing warp, or by its bytes (pixels of x' that do not start on
+  // 32-byte sectors take 1.9 times the time); the transposing warps take about 270 clocks per block of theirs, 800 for a
+  // tile at least, and do it again for every tile, the channel tiles of the same pixels included.  The
+  // pass takes 2 us and its bytes.  Fitted to 1892 random layers (1x2 to 5x5, 1x7 and 7x1, 17 to 1100 channels in and
+  // 8 to 2048 out, planes of 4 to 224) timed in both forms.  Against the faster of the two, the one that is chosen here is
+  // 0.3 % slower on average and more than 10 % in 24 layers; the transposed form wherever it fits 3.1 % and
+  // more than 10 % in 173 (16 x 512 -> 1024, 1x3 on 28x28 63.1 us, behind the pass 49.0; 4 x 512 -> 512, 3x1 on 56x56
+  // 38.0 and 27.6; the wide layers that it is for keep it: 16 images 128->128 3x3 on 112x112 64.7 -> 51.4, 128->256 on 56x56
+  // 34.0 -> 30.6, 512->512 on 28x28 51.2 -> 49.9, 64 images 64->64 on 56x56 33.1 -> 27.1).
+  auto form_clk = [&](int stages, int xt_blocks) {
+    const double mmas = (double)p.eff_r * p.eff_s * (p.kb / 16.0), cols = (double)p.ncols;  // MMAs per channel block
+    const int spb = p.eff_r * (p.eff_s / p.taps);                                           // ring stages per channel block
+    double t_mma = cols / 2.0;
+    if (32.0 + cols / 4.0 > t_mma) t_mma = 32.0 + cols / 4.0;
+    if (t_mma < 48.0) t_mma = 48.0;
+    const double weights = resident_stages(stages) ? 0.0 : p.eff_r * p.eff_s * p.kb * 2.0 * p.a_rows;
+    const double act = xt_blocks > 0 ? xt_blocks * 64.0 * p.kb * 2.0 : cols * p.kb * 2.0 * spb * (p.c_pad % 16 != 0 ? 1.9 : 1.0);
+    double block = mmas * t_mma;
+    if (spb * 300.0 + mmas * 60.0 > block) block = spb * 300.0 + mmas * 60.0;
+    if ((weights + act) / 78.0 > block) block = (weights + act) / 78.0;
+    if (xt_blocks > 0) {
+      const double blocks = xt_blocks * (p.kb / 32.0);
+      const double t = 270.0 * blocks > 800.0 ? 270.0 * blocks : 800.0;
+      if (t > block) block = t;
+    }
+    const double epi = 1.5 * epilogue_clk(p.ncols), main_loop = (double)((p.cblocks + (1 << best_ks) - 1) >> best_ks) * block;
+    const double tile = main_loop > epi ? main_loop : epi;
+    double clk = epi;
+    if (best_ks > 0) clk = main_loop + epi / (1 << best_ks) + 5000.0 + 512.0 * cols * (1.0 - 1.0 / (1 << best_ks)) / 27.0;
+    else if (best_shared) clk += (double)p.total_tiles / sms * tile + 10000.0;
+    else clk += (double)((p.total_tiles + sms - 1) / sms) * tile;
+    return xt_blocks > 0 ? clk : clk + 3800.0 + (double)g.n * g.c * g.h * g.w * 4.0 / 3600.0;
+  };
+  p.est_clk = 0.0;
+  if (g.stride_h == 1 && g.stride_w == 1 && !p.nchw && !p.x_nhwc && !p.y_nhwc && !p.window && !p.patch && !p.pair && !g.rowpair &&
+      g.dw_stride == 0 && g.no_fuse && !p.gather && p.kb >= 32 && g.r * g.s > 1 && ((int64_t)g.h * g.w) % 8 == 0)
+    p.est_clk = form_clk(p.stages, 0);
+  if (p.est_clk > 0.0 && p.halo && p.tn == 1 && (g.group == 1 || g.cg % p.kb == 0) && p.epi_warps == kEpilogueWarps && p.dup_log2 == 0 && g.w > 1) {
     const int rows_in = p.th + (g.r - 1) * g.dil_h;
     const int skew = g.w % 8 == 0 ? 0 : 7;
     size_t reach = (size_t)p.ncols + (size_t)(g.r - 1) * g.dil_h * p.pitch + (size_t)(g.s - 1) * g.dil_w;
     if (reach < (size_t)rows_in * p.pitch) reach = (size_t)rows_in * p.pitch;
     const size_t tile = round_up_sz((reach + 1) * p.kb * 2u, 1024);
     const size_t recv_own = p.recv ? split_bytes(p.ncols, best_ks) : 0;  // (the parts of a split reduction stay where they were)
-    // A ring stage holds the weight tiles of a kernel row, three of them if they fit, else two.  (One tap per stage
+    // A ring stage holds the weight tiles of a kernel row; as many stages as fit.  (One tap per stage
     // is a hand-shake per four MMAs; 16 KB of slots in place of 32 do not hide the latency of the copies.)
     // Layers of at most 64 output channels need staging tiles for the warps of two lane quarters only.
     const int32_t trans_epi = p.tma_store && g.kg <= 64 && best_ks == 0 && !best_shared ? kEpilogueWarps / 2 : kEpilogueWarps;
@@ -3285,34 +3339,27 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
     const size_t xt = kXtBufs * tile + kXtSlots * (size_t)kXtSlotBytes;
     int stages = xt + recv_own < trans_budget ? (int)((trans_budget - xt - recv_own) / st) : 0;
     if (stages > kMaxStages) stages = kMaxStages;
-    if (stages >= 2 && (best_ks == 0 || p.recv || xt + stages * st >= split_bytes(p.ncols, best_ks))) {
+    const int xt_blocks = (rows_in * g.w + skew + 63) / 64;
+    const double clk = form_clk(stages, xt_blocks);
+    if (stages >= 2 && (best_ks == 0 || p.recv || xt + stages * st >= split_bytes(p.ncols, best_ks)) && (g.want_trans || clk < p.est_clk)) {
       p.trans = 1;
+      p.est_clk = clk;
       p.stages = stages;
       p.b_alloc = 0;
       p.stage_bytes = (uint32_t)st;
       p.epi_tiles = trans_epi;
       p.xt_rows_in = rows_in;
-      p.xt_blocks = (rows_in * g.w + skew + 63) / 64;
+      p.xt_blocks = xt_blocks;
       p.xt_slots = kXtSlots;
       p.xt_dump = (int32_t)reach;
       p.xt_bytes = (uint32_t)tile;
       p.xt_total = (uint32_t)xt;
     }
   }
-  // Resident weights: where every tile of a CTA has the same channel tile (the grid is a multiple of
-  // their number) and the ring holds a whole number of tiles' stages, a stage finds the weights it
-  // needs in place after the first lap; only activations are fetched from then on.  The ring is
-  // cut to such a number when at least three stages are left.  (ResNet-50's 7x7 stem fetched 28 KB of
-  // weights for every output row of 13 KB.)
   p.resident = 0;
-  {
-    const int64_t mgn = (int64_t)p.mtiles * g.group;
-    const int ts = p.cblocks * p.eff_r * (p.eff_s / p.taps), st = p.stages / ts * ts;
-    if (!p.pair && !p.sk_split && best_ks == 0 && p.slabs == 0 && p.grid % mgn == 0 && p.total_tiles > p.grid && st > 0 &&
-        (st == p.stages || st >= 3)) {
-      p.resident = 1;
-      p.stages = st;
-    }
+  if (const int st = resident_stages(p.stages); st > 0) {
+    p.resident = 1;
+    p.stages = st;
   }
   // a second staging tile per epilogue warp (its store overlaps the next unit) if memory is left
   const size_t epi_bytes = p.trans ? (size_t)p.epi_tiles * kWarpStageBytes : stage_buf_bytes;

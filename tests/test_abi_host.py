@@ -355,3 +355,26 @@ def test_split_reductions_of_rows_wider_than_eight_parts_allow():
             "    i = hgc.ConvDesc(*a).plan_info()\n"
             "    assert i['path'] == hgc.HGC_PATH_IGEMM and (i['k_slices'] < 8 or i['ncols'] <= 128), (a, i)\n")
     subprocess.run([sys.executable, "-c", code], check=True, timeout=60, cwd=ROOT)
+
+
+# Stride-1 layers of several taps whose x the kernel can turn channels-last itself: (layer, channel blocks of, CTAs that
+# share a reduction, chunks of a host call, who makes x channels-last)
+@pytest.mark.parametrize("args,kb,slices,chunks,fused", [
+    ((1, 986, 20, 20, 19, 3, 1, 1, 0), 64, 8, 1, 0),       # blocks of 32 would give up the cluster's shared reduction
+    ((3, 1008, 24, 24, 240, 3, 1, 1, 0), 64, 8, 1, 0),
+    ((10, 1024, 8, 8, 192, 3, 1, 1, 0), 64, 8, 1, 0),
+    ((2, 452, 8, 151, 34, 3, 3, 1, 1), 64, 4, 1, 0),
+    ((15, 272, 68, 124, 64, 3, 3, 1, 1), 32, 1, 4, 2),     # blocks of 32, but no tiles shared by CTAs, which go in one piece
+    ((9, 256, 104, 118, 32, 3, 3, 1, 1), 32, 1, 3, 2),
+    ((38, 112, 72, 70, 16, 5, 5, 2, 2), 32, 1, 2, 2),
+    ((16, 512, 28, 28, 1024, 1, 3, 0, 1), 32, 1, 1, 0),    # x would be turned again for each of eight channel tiles
+    ((4, 512, 56, 56, 512, 3, 1, 1, 0), 64, 1, 4, 0),
+    ((4, 512, 56, 56, 1024, 2, 2, 0, 0), 64, 1, 1, 0),
+    ((16, 64, 28, 28, 1024, 1, 3, 0, 1), 64, 1, 1, 2),     # one channel block: the tile's stores take longer
+    ((4, 64, 56, 56, 128, 2, 2, 0, 0), 64, 1, 1, 2),
+    ((16, 64, 112, 112, 128, 3, 3, 1, 1), 32, 1, 4, 2),
+    ((16, 512, 28, 28, 512, 3, 3, 1, 1), 32, 1, 4, 2),
+])
+def test_transposed_tiles_are_chosen_by_their_cost(args, kb, slices, chunks, fused):
+    info = hgc.ConvDesc(*args).plan_info()
+    assert (info["kb"], info["k_slices"], info["host_chunks"], info["fused_layout"]) == (kb, slices, chunks, fused), info
