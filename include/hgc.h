@@ -47,7 +47,8 @@ typedef enum hgc_status {
 typedef enum hgc_path {
   HGC_PATH_DIRECT = 0,     /* direct convolution on CUDA cores, any valid layer */
   HGC_PATH_DEPTHWISE = 1,  /* 3x3 depthwise (group == C == K) stencil on CUDA cores */
-  HGC_PATH_IGEMM = 2       /* implicit GEMM on tcgen05 tensor cores with TMEM accumulators */
+  HGC_PATH_IGEMM = 2       /* implicit GEMM on tcgen05 tensor cores with TMEM accumulators (image stems of
+                              few products: one CUDA-core launch, see hgc_conv_plan_info [10] = 5) */
 } hgc_path;
 
 /* Layer description.  Scalars are plain host integers (Section 3.2: scalars stay in host
@@ -180,7 +181,7 @@ int hgc_conv_forward_host(hgc_conv_desc* d, const void* x, const void* w, const 
  * way to obtain the scratch buffer that hgc_conv_set_workspace wants.
  *
  * What it does: runs the tensor-core path (HGC_PATH_IGEMM) of hgc_conv_forward with its scratch
- * (status word, re-laid-out weights, NHWC copy of x) in a
+ * (status word, re-laid-out weights, NHWC copy of x; the one-launch image stems need none of it) in a
  * 32 MiB array that is part of the library image: every device that loads the library holds
  * those 32 MiB until the process exits.  It takes the layer description directly; no descriptor
  * object, no workspace, no weight registration (the weights are re-laid-out on every call).
@@ -228,9 +229,10 @@ int hgc_conv_path(const hgc_conv_desc* d, int32_t* path);
  * as pixel-major tiles; channels-last x, which includes every input with a 1x1 plane), 2 = a
  * zero-bordered 8-channel NHWC copy read through
  * overlapping windows (few input channels), 3 = an expanded copy holding, per output pixel, the
- * values under the kernel (few input channels, strided; 2 and 3: layers of few products and a small
- * input tile run as one CUDA-core launch instead and make no copy), 4 = x itself, gathered by extra warps of
- * the kernel (1x1 layers on small planes, see HGC_FLAG_GATHER_X), [11] the number of CTAs that share
+ * values under the kernel (few input channels, strided), 4 = x itself, gathered by extra warps of
+ * the kernel (1x1 layers on small planes, see HGC_FLAG_GATHER_X), 5 = x itself, read by the one CUDA-core
+ * launch that image stems of few products and a small input tile run as (it has none of the tiles that
+ * the other values describe: they are zero), [11] the number of CTAs that share
  * the reduction of one tile (1, or 2 / 4 / 8 for layers with very few tiles, e.g. inner products:
  * a cluster whose CTAs send one another their fp32 sums and add them in a fixed order), [12] the
  * number of CTAs of the launch when the ring stages of all tiles are dealt out as contiguous

@@ -549,7 +549,9 @@ int hgc_conv_plan_info(const hgc_conv_desc* d, int32_t* info, int32_t count) {
   if (d == nullptr || info == nullptr || count < 1) return HGC_INVALID_ARG;
   constexpr int kValues = 25;
   int32_t v[kValues] = {d->path};
-  if (d->path == HGC_PATH_IGEMM) {
+  if (d->path == HGC_PATH_IGEMM && hgc::stem_small_supported(d->geom)) {
+    v[10] = 5;  // (none of the plan's tiles: the one launch has its own)
+  } else if (d->path == HGC_PATH_IGEMM) {
     const hgc::IgemmPlan& p = d->igemm;
     v[1] = p.kb; v[2] = p.halo; v[3] = p.tn; v[4] = p.th; v[5] = p.pitch; v[6] = p.ncols;
     v[7] = p.total_tiles; v[8] = p.stages; v[9] = p.taps;

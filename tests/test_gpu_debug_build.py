@@ -35,7 +35,8 @@ CHILD = textwrap.dedent(r'''
         ("1x1 7x7", params_dict(9, 512, 7, 7, 130, 1, 1), 0),
         ("row pairs", params_dict(2, 16, 10, 112, 64, 3, 3, 1, 1), 0),
         ("replicated rows", params_dict(2, 32, 112, 112, 64, 1, 1), 0),
-        ("stem windows", params_dict(2, 3, 32, 40, 16, 3, 3, 1, 1), 0),
+        ("stem windows", params_dict(16, 3, 32, 40, 16, 3, 3, 1, 1), 0),
+        ("stem in one launch", params_dict(2, 3, 29, 37, 19, 3, 3, 1, 1), 0),
         ("stem patches", params_dict(2, 3, 64, 48, 32, 3, 3, 1, 1, 2, 2), 0),
         ("split reduction", params_dict(3, 4096, 5, 5, 96, 1, 1), 0),
         ("shared tiles", params_dict(2, 256, 24, 24, 256, 3, 3, 1, 1), hgc.HGC_FLAG_SHARED_TILES),
@@ -55,10 +56,14 @@ CHILD = textwrap.dedent(r'''
         ("direct (odd groups)", params_dict(2, 15, 9, 11, 10, 3, 2, 1, 0, 1, 1, 1, 1, 5), 0),
         ("direct (forced)", params_dict(2, 32, 12, 12, 48, 3, 3, 1, 1), hgc.HGC_FLAG_FORCE_DIRECT),
     ]
+    SOURCES = {"1x1 in place": 1, "stem windows": 2, "stem patches": 3, "x gathered by the kernel's warps": 4, "stem in one launch": 5}
+    assert SOURCES.keys() <= {c[0] for c in cases}
     for name, a, flags in cases:
         rng = np.random.default_rng(zlib.crc32(name.encode()))
         x, w, b = workloads.random_layer_tensors(rng, a["n"], a["c"], a["h"], a["w"], a["k"], a["r"], a["s"], a["group"])
         ref = oracle.conv_fast(oracle.ConvParams(**a), x, w, b, True)
+        if name in SOURCES:
+            assert hgc.ConvDesc(flags=flags, **a).plan_info()["x_source"] == SOURCES[name], name
         got, path = run_layer(hgc, a, x, w, b, True, flags=flags)
         check_close(got, ref, what=name)
         v = hgc.debug_violations()

@@ -13,7 +13,7 @@ from gpu_util import check_close, params_dict, run_layer
 
 pytestmark = pytest.mark.gpu
 
-X_NHWC_COPY, X_DIRECT, X_WINDOWS, X_PATCHES = 0, 1, 2, 3
+X_NHWC_COPY, X_DIRECT, X_WINDOWS, X_PATCHES, X_ONE_LAUNCH = 0, 1, 2, 3, 5
 
 
 @pytest.fixture(scope="module")
@@ -46,7 +46,7 @@ CASES = [
     ("1x1 5x5 c4096 k96: reduction split over several CTAs, ragged channel tile", params_dict(3, 4096, 5, 5, 96, 1, 1), X_NHWC_COPY),
     ("1x1 7x7 c2048 k200: reduction split, one-row tiles", params_dict(2, 2048, 7, 7, 200, 1, 1), X_NHWC_COPY),
     ("1x1 3x5 c4096 k64: reduction split, several images per tile", params_dict(4, 4096, 3, 5, 64, 1, 1), X_NHWC_COPY),
-    ("stem 3x3 c3 stride 1 (windows)", params_dict(2, 3, 32, 40, 16, 3, 3, 1, 1), X_WINDOWS),
+    ("stem 3x3 c3 stride 1 (windows)", params_dict(16, 3, 32, 40, 16, 3, 3, 1, 1), X_WINDOWS),
     ("stem 7x7 c3 stride 2 (windows)", params_dict(2, 3, 64, 64, 64, 7, 7, 3, 3, 2, 2), X_WINDOWS),
     ("stem 11x11 c3 stride 4 (windows)", params_dict(1, 3, 67, 67, 96, 11, 11, 0, 0, 4, 4), X_WINDOWS),
     ("stem 7x7 c3 stride 2, 224 wide (dense rows of 4-channel pixels, two rows per tile)",
@@ -54,18 +54,19 @@ CASES = [
     ("stem 5x5 c4 stride 2 (dense rows of 4-channel pixels)", params_dict(2, 4, 37, 45, 40, 5, 5, 2, 2, 2, 2), X_WINDOWS),
     ("stem 7x7 c3 stride 1 along H, 2 along W", params_dict(2, 3, 30, 50, 24, 7, 7, 3, 3, 1, 2), X_WINDOWS),
     ("stem 7x7 c1 stride 1 along H, 2 along W (49 values under the kernel: patches)",
-     params_dict(2, 1, 30, 50, 24, 7, 7, 3, 3, 1, 2), X_PATCHES),
+     params_dict(10, 1, 30, 50, 24, 7, 7, 3, 3, 1, 2), X_PATCHES),
     ("stem 9x9 c3 stride 2 (64-element windows)", params_dict(1, 3, 41, 41, 32, 9, 9, 4, 4, 2, 2), X_WINDOWS),
     ("stem 5x5 c5 stride 2 (8-channel pixels: one request per window)", params_dict(2, 5, 33, 33, 16, 5, 5, 2, 2, 2, 2), X_WINDOWS),
     ("stem 5x5 c3 stride 1 (dense rows, shared kernel rows)", params_dict(2, 3, 30, 70, 48, 5, 5, 2, 2), X_WINDOWS),
     ("stem 3x3 c8 stride 1, 250 wide (dense rows at the column limit)", params_dict(1, 8, 9, 250, 16, 3, 3, 1, 1), X_WINDOWS),
     ("stem 3x3 c3 stride 1, 256 wide (rows too wide for the dense form)", params_dict(1, 3, 6, 256, 16, 3, 3, 1, 1), X_WINDOWS),
     ("stem 3x3 c3 stride 2 (patches)", params_dict(2, 3, 64, 48, 32, 3, 3, 1, 1, 2, 2), X_PATCHES),
-    ("stem 3x3 c1 stride 2 (patches)", params_dict(3, 1, 33, 31, 24, 3, 3, 1, 1, 2, 2), X_PATCHES),
+    ("stem 3x3 c1 stride 2 (patches)", params_dict(36, 1, 33, 31, 96, 3, 3, 1, 1, 2, 2), X_PATCHES),
     ("stem 3x3 c4 stride 2, 44 wide (patches from aligned words)", params_dict(2, 4, 30, 44, 16, 3, 3, 1, 1, 2, 2), X_PATCHES),
-    ("stem 3x3 c1 stride 2 x 1, 70 wide, pad 2 x 1 (patches from aligned words)", params_dict(3, 1, 21, 70, 24, 3, 3, 2, 1, 1, 2), X_PATCHES),
+    ("stem 3x3 c1 stride 2 x 1, 70 wide, pad 2 x 1 (patches from aligned words)", params_dict(49, 1, 21, 70, 24, 3, 3, 2, 1, 1, 2), X_PATCHES),
     ("stem 3x3 c4 stride 2 dilated (patches)", params_dict(2, 4, 30, 30, 20, 3, 3, 2, 2, 2, 2, 2, 2), X_PATCHES),
     ("stem 5x5 c2 stride 3 (patches, generic expansion)", params_dict(2, 2, 29, 35, 20, 5, 5, 2, 2, 3, 3), X_PATCHES),
+    ("stem 3x3 c3 stride 1, few products (one launch)", params_dict(2, 3, 32, 40, 16, 3, 3, 1, 1), X_ONE_LAUNCH),
     ("stem 1x1 c8 stride 2 (patches)", params_dict(2, 8, 18, 18, 16, 1, 1, 0, 0, 2, 2), X_PATCHES),
     # 64 output channels: odd output rows in the upper accumulator lanes (row pairs) ...
     ("row pairs 3x3 c16 112 wide", params_dict(2, 16, 10, 112, 64, 3, 3, 1, 1), X_NHWC_COPY),

@@ -50,6 +50,8 @@ def test_small_stem(hgc, oracle, a, launches):
         check_close(got, ref, what=str(a))
         assert max_ulp_error(got, ref) <= 1, a
     d = hgc.ConvDesc(**a)
+    info = d.plan_info()
+    assert (info["x_source"] == 5) == (launches == 1) and (info["tiles"] == 0) == (launches == 1), info
     d.ensure_workspace()
     xd, wd = (torch.from_numpy(t.view(np.int16)).cuda().view(torch.float16) for t in (x, w))
     d.set_weights(wd)

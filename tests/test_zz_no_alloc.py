@@ -54,7 +54,8 @@ def _static_forward(hgc, args, x, w, b, relu, free_must_not_change=False):
 BIG = params_dict(3, 48, 40, 44, 72, 3, 3, 1, 1)
 MODES = [
     ("NHWC copy, 3x3", params_dict(2, 32, 9, 9, 40, 3, 3, 1, 1, 2, 2)),
-    ("stem 3->16 3x3 stride 1 (bordered copy, dense rows)", params_dict(2, 3, 20, 24, 16, 3, 3, 1, 1)),
+    ("stem 3->16 3x3 stride 1 (bordered copy, dense rows)", params_dict(41, 3, 20, 24, 16, 3, 3, 1, 1)),
+    ("stem 3->16 3x3 stride 1, few products (one launch)", params_dict(2, 3, 20, 24, 16, 3, 3, 1, 1)),
     ("stem 3->16 3x3 stride 2 (expanded copy)", params_dict(2, 3, 21, 25, 16, 3, 3, 1, 1, 2, 2)),
     ("stem 7x7 stride 2 (windows of 4-channel pixels)", params_dict(1, 3, 30, 34, 24, 7, 7, 3, 3, 2, 2)),
     ("1x1 64->64 on 8x8 (x read in place)", params_dict(2, 64, 8, 8, 64, 1, 1)),
@@ -66,6 +67,8 @@ MODES = [
 
 @pytest.mark.parametrize("name,args", MODES, ids=[m[0] for m in MODES])
 def test_static_scratch_after_a_larger_call(hgc, oracle, name, args):
+    for words, source in (("bordered copy", 2), ("expanded copy", 3), ("windows", 2), ("one launch", 5)):
+        assert words not in name or hgc.ConvDesc(**args).plan_info()["x_source"] == source, name
     rng = np.random.default_rng(77)
     for a in (BIG, args, args):          # the mode under test runs twice in a row after the large layer
         x, w, b = workloads.random_layer_tensors(rng, a["n"], a["c"], a["h"], a["w"], a["k"], a["r"], a["s"], a["group"])
