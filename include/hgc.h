@@ -202,7 +202,8 @@ int hgc_conv_forward_host(hgc_conv_desc* d, const void* x, const void* w, const 
  * Limits and errors: HGC_UNSUPPORTED if the layer is not one the tensor-core path takes (fewer
  * than 9 channels per group unless it is an image stem, very wide rows ...: use hgc_conv_forward)
  * or if p->flags asks for channels-last tensors or the direct path; HGC_NO_WORKSPACE if the layer
- * needs more than the 32 MiB (1 KiB + K*R*S*c_w*2 + N*H*W*c_pad*2 bytes, channels rounded up);
+ * needs more than the 32 MiB (1 KiB + K*R*S*c_w*2 + N*H*W*c_pad*2 bytes, channels rounded up; the last
+ * term only where a copy of x is made);
  * HGC_INVALID_ARG / HGC_BAD_ALIGNMENT as for hgc_conv_forward;
  * HGC_CUDA_ERROR.  A device-side timeout cannot be read back through this entry point.
  *

@@ -3381,7 +3381,7 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
   p.ws_status_off = 0;
   p.ws_w_off = kWsHeaderBytes;
   p.ws_x_off = p.ws_w_off + round_up_sz(((size_t)g.k << p.dup_log2) * p.eff_r * p.eff_s * p.cw * 2, 256);
-  p.ws_total = p.ws_x_off + ((p.nchw || p.x_nhwc) ? 0
+  p.ws_total = p.ws_x_off + ((p.nchw || p.x_nhwc || p.trans) ? 0
                                     : round_up_sz(p.patch    ? (size_t)g.n * g.p * g.q * p.cw * 2
                                                   : p.window ? (size_t)g.n * p.hp * p.wp * p.px_ch * 2 + 256
                                                            : (size_t)g.n * g.h * g.w * p.c_pad * 2, 256));

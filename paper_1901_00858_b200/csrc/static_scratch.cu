@@ -102,15 +102,19 @@ extern "C" int hgc_conv_forward_static(const hgc_conv_params* p, const void* x, 
     hgc::debug_add_range(&r, ws, plan.ws_total);
     hgc::debug_set_call_ranges(r, st);
   }
+  // image stems of few products: one launch without scratch.  (The array has been looked up all the same: a small
+  // layer's call is what a caller warms this entry point up with.)
+  if (hgc::stem_small_supported(g)) {
+    const cudaError_t err = hgc::launch_stem_small(g, static_cast<const __half*>(x), static_cast<const __half*>(w),
+                                                   static_cast<const __half*>(bias), static_cast<__half*>(y), relu, st);
+    return err == cudaSuccess ? HGC_OK : HGC_CUDA_ERROR;
+  }
   if (cudaMemsetAsync(ws + plan.ws_status_off, 0, hgc::kWsHeaderBytes, st) != cudaSuccess) return HGC_CUDA_ERROR;
   if (!hgc::igemm_encode_maps(g, &plan, ws)) return HGC_CUDA_ERROR;
   const __half* xh = static_cast<const __half*>(x);
   const __half* wh = static_cast<const __half*>(w);
   __half* wp = reinterpret_cast<__half*>(ws + plan.ws_w_off);
   __half* xp = reinterpret_cast<__half*>(ws + plan.ws_x_off);
-  if (hgc::stem_small_supported(g))
-    return hgc::launch_stem_small(g, xh, wh, static_cast<const __half*>(bias), static_cast<__half*>(y), relu, st) == cudaSuccess ? HGC_OK
-                                                                                                                         : HGC_CUDA_ERROR;
   if (hgc::launch_igemm_weights(g, plan, wh, wp, st) != cudaSuccess) return HGC_CUDA_ERROR;
   if (hgc::launch_igemm_input(g, plan, xh, xp, st) != cudaSuccess) return HGC_CUDA_ERROR;
   if (hgc::launch_igemm(g, plan, ws, xh, static_cast<const __half*>(bias), static_cast<__half*>(y), relu, st) !=

@@ -378,3 +378,11 @@ def test_split_reductions_of_rows_wider_than_eight_parts_allow():
 def test_transposed_tiles_are_chosen_by_their_cost(args, kb, slices, chunks, fused):
     info = hgc.ConvDesc(*args).plan_info()
     assert (info["kb"], info["k_slices"], info["host_chunks"], info["fused_layout"]) == (kb, slices, chunks, fused), info
+
+
+@pytest.mark.parametrize("args", [(16, 128, 112, 112, 128, 3, 3, 1, 1), (64, 64, 56, 56, 64, 3, 3, 1, 1), (1, 512, 28, 28, 512, 3, 3, 1, 1)])
+def test_no_workspace_for_a_copy_of_x_that_is_not_made(args):
+    d = hgc.ConvDesc(*args)
+    info = d.plan_info()
+    assert info["fused_layout"] == 2 and info["shared_tiles"] == 0
+    assert d.workspace_bytes() == 1024 + args[4] * args[1] * 9 * 2    # header and weights

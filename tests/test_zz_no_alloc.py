@@ -91,6 +91,24 @@ def test_static_scratch_takes_layers_that_fit_without_replicated_weights(hgc, or
     check_close(_static_forward(hgc, a, x, w, b, True), oracle.conv_fast(oracle.ConvParams(**a), x, w, b, True), what="one copy")
 
 
+def test_static_scratch_needs_no_room_for_a_copy_of_x_that_is_not_made(hgc):
+    """An NHWC copy of this layer's x would need 38 MB; the kernel turns x channels-last itself."""
+    import torch
+    a = params_dict(12, 128, 112, 112, 24, 3, 3, 1, 1)
+    d = hgc.ConvDesc(**a)
+    assert d.plan_info()["fused_layout"] == 2 and d.plan_info()["shared_tiles"] == 0
+    d.ensure_workspace()
+    g = torch.Generator(device="cuda").manual_seed(79)
+    x = torch.rand((12, 128, 112, 112), generator=g, device="cuda").half()
+    w, b = (torch.randn(s, generator=g, device="cuda").half() * 0.05 for s in ((24, 128, 3, 3), (24,)))
+    y, z = (torch.full((12, 24, 112, 112), float("nan"), dtype=torch.float16, device="cuda") for _ in range(2))
+    hgc.conv_forward(d, x, w, b, y, True)
+    hgc.conv_forward_static(_params(hgc, a), x, w, b, z, True)
+    torch.cuda.synchronize()
+    assert torch.equal(y.view(torch.int16), z.view(torch.int16)) and float(y.float().max()) > 0
+    d.close()
+
+
 def test_static_scratch_rejects_what_it_cannot_hold(hgc):
     import torch
     dummy = torch.zeros(64, dtype=torch.float16, device="cuda")
