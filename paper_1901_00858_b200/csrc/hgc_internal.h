@@ -386,7 +386,7 @@ struct IgemmPlan {
   int32_t ring_stages;
   double est_clk;  // estimated clocks, a pass over x included (layers that could save it; 0: not one of them)
   int32_t epi_tiles;
-  int32_t trans, xt_rows_in, xt_blocks, xt_slots, xt_dump;
+  int32_t trans, xt_rows_in, xt_blocks, xt_dump;
   uint32_t xt_bytes, xt_total;
   int32_t dup_log2;  // log2 of the number of copies of the layer's weight rows in w' and in a weight tile (0, 1, 2)
   size_t smem_bytes;

@@ -566,8 +566,8 @@ __device__ __forceinline__ void issue_mmas(uint32_t d_tmem, uint32_t a_lo, uint3
 // one's shared memory as [part][pair of columns][lanes][2], added to the bias in the order of the parts.
 struct AccSource {
   uint32_t addr;        // tensor-memory address of column 0, or shared-memory address of this lane's column 0
-  uint32_t col_bytes;   // SPLIT: bytes from column to column and from part to part, and the number of parts
-  uint32_t part_bytes;
+  uint32_t col_bytes;   // SPLIT: a column's bytes in a part (half the distance between pairs of columns), a part's bytes
+  uint32_t part_bytes;  //   and their number
   int parts;
   float first;          // SPLIT: what the sum begins with (the bias)
 };
@@ -871,16 +871,6 @@ struct IgemmArgs {
   int32_t dw_in_h, dw_in_w;
   uint32_t dw_in_bytes, dw_in_alloc;
   int32_t dw_teams_log2;  // log2 of the teams that the depthwise warps form: team t computes every stage s with s % teams == t
-  // x[N][C][H*W] turned channels-last inside the kernel (TRANS instantiations): a channel block of a tile is
-  // its th + (R-1)*dil input rows, fetched as blocks of 64 pixels x 32 channels into xt_slots staging slots
-  // and transposed into one of xt_bufs tiles [row][pitch][KB] that all R*S taps read
-  int32_t xt_w, xt_rows_in;       // pixels per row of x; input rows of a tile
-  uint32_t xt_magic;              // ceil(2^32 / xt_w): row of a pixel by a multiplication
-  int32_t xt_blocks, xt_slots, xt_bufs;
-  int32_t xt_dump;                // row of a transposed tile that nothing reads: pixels outside its input rows
-  uint32_t xt_bytes;              // bytes of a transposed tile
-  int32_t epi_tiles;              // epilogue warps that have staging tiles
-  uint32_t xt_total;              // bytes of the transposed tiles and the slots (behind the ring)
   int32_t dbg_drop;     // test hook: stage of the first CTA whose copies are left out (-1: none)
   int32_t ts;           // ring stages per tile: cblocks * R * (S / taps)
   // CTA pairs (clusters of two, tcgen05 cta_group::2): a tile is 256 output channels x two pixel
@@ -893,6 +883,16 @@ struct IgemmArgs {
   int32_t sk_cols32;    // accumulator columns handed over, in units of 32
   float* sk_part;
   int* sk_flags;
+  // x[N][C][H*W] turned channels-last inside the kernel (TRANS instantiations): a channel block of a tile is
+  // its th + (R-1)*dil input rows, fetched as blocks of 64 pixels x 32 channels into kXtSlots staging slots
+  // and transposed into one of kXtBufs tiles [row][pitch][KB] that all R*S taps read
+  int32_t xt_w, xt_rows_in;       // pixels per row of x; input rows of a tile
+  uint32_t xt_magic;              // ceil(2^32 / xt_w): row of a pixel by a multiplication
+  int32_t xt_blocks;
+  int32_t xt_dump;                // row of a transposed tile that nothing reads: pixels outside its input rows
+  uint32_t xt_bytes;              // bytes of a transposed tile
+  int32_t epi_tiles;              // epilogue warps that have staging tiles
+  uint32_t xt_total;              // bytes of the transposed tiles and the slots (behind the ring)
 };
 
 // The tiles of one CTA: blockIdx.x, blockIdx.x + gridDim.x, ...  Tile t = (pixel tile px, channel
@@ -1201,7 +1201,7 @@ __device__ __noinline__ uint32_t epilogue_planes(uint32_t t_addr, uint32_t qstag
 constexpr int kLayoutWarps = 8;  // extra warps of the instantiations with the fused layout pass
 constexpr int kDwWarps = 8;      // extra warps of the depthwise + pointwise instantiations
 constexpr int kXtWarps = 4;      // extra warps of the instantiations that turn x channels-last themselves
-constexpr int kXtSlots = 8, kXtBufs = 2;  // staging slots at most, and transposed tiles
+constexpr int kXtSlots = 8, kXtBufs = 2;  // staging slots and transposed tiles
 constexpr uint32_t kXtSlotBytes = 64u * 32u * 2u;  // a block of 64 pixels x 32 channels
 constexpr int kDropSlab = 1 << 20;  // test hook: as the index of a stage to drop, the last weight slab of a row-pair layer
 constexpr int kMaxDwTeams = 4;   // (and two input tiles per team)
@@ -1258,17 +1258,19 @@ __device__ __noinline__ void wait_for_work_under_way(int warp, int epi_warps, ui
 // traffic is three times the block's bytes (copy in, read, write), one ninth of it per tap of a 3x3 layer.
 // The columns left and right of the rows are the zero padding: no block writes them, so they are
 // cleared once.  Rows above and below the plane arrive as zeros.
-// What it costs: a block is about 250 clocks of addresses, 250 of matrix loads and stores and, once per tile of 32 or
-// 64 channels, 300 of the proxy fence, all beside the MMAs of the tile before (512->512 3x3 on 28x28: 106 clocks per MMA
-// of 208 columns, which is the tensor pipe's rate); a launch's first tile waits about 4500 clocks for it.
+// What it costs (clock counters): a block is about 260 clocks of addresses, 260 of matrix loads and stores and, once per
+// tile of 32 or 64 channels, of the proxy fence (512->512 3x3 on 28x28 300, 128->128 on 112x112 150), all beside the MMAs of
+// the tile before (the former layer: 106 clocks per MMA of 208 columns, which is the tensor pipe's rate).  A launch's first
+// tile waits about 4500 clocks for it (the latter: 5800).  Layers of few MMAs per block are bound by it, at about
+// 270 clocks of the CTA per block, more than the four warps' own work: the planner's estimate goes by that.
 template <int KB, bool SPLIT, bool SHARED>
 __device__ __forceinline__ void transpose_blocks(const IgemmArgs& a, int tw, uint32_t tiles, uint32_t in_full, uint32_t in_empty,
                                                  uint32_t xb_full, uint32_t xb_empty, volatile int* abort_flag) {
   constexpr uint32_t row_bytes = (uint32_t)KB * 2u;
   const int lane = threadIdx.x & 31;
-  const uint32_t slots = tiles + (uint32_t)a.xt_bufs * a.xt_bytes;
+  const uint32_t slots = tiles + (uint32_t)kXtBufs * a.xt_bytes;
   const int pad = a.pitch - a.xt_w;  // columns of padding per row, left (pad_w) and right
-  for (int i = tw * 32 + lane; i < a.xt_bufs * a.xt_rows_in * pad * (KB / 8); i += kXtWarps * 32) {
+  for (int i = tw * 32 + lane; i < kXtBufs * a.xt_rows_in * pad * (KB / 8); i += kXtWarps * 32) {
     const int chunk = i % (KB / 8), t = i / (KB / 8);
     const int c = t % pad, row = t / pad;  // (rows of all tiles, one after the other)
     const int tile = row / a.xt_rows_in;
@@ -1282,10 +1284,9 @@ __device__ __forceinline__ void transpose_blocks(const IgemmArgs& a, int tw, uin
   const uint32_t octet = (uint32_t)lane >> 3, sub = (uint32_t)lane & 7u;
   const int px_in = a.xt_rows_in * a.xt_w;  // pixels of the tile's input rows
   const int per_block = a.R * (a.S / a.taps);
-  // The warps take the blocks in turn, and a slot's blocks are always the same warp's: their number (8, 4 or
-  // 2) is a multiple of the number of warps that take part.  A warp that waits for a slot's next block has therefore
-  // seen the one before, which the parity of the wait does not tell from the one after.
-  const uint32_t turn = (uint32_t)(a.xt_slots < kXtWarps ? a.xt_slots : kXtWarps) - 1u;
+  // The warps take the blocks in turn, and a slot's blocks are always the same warp's.  A warp that waits for a slot's
+  // next block has therefore seen the one before, which the parity of the wait does not tell from the one after.
+  static_assert((kXtWarps & (kXtWarps - 1)) == 0 && kXtSlots % kXtWarps == 0, "a slot belongs to one warp");
   uint32_t block = 0;
   Ring ring, xb;
   typename WorkIterOf<SPLIT, SHARED>::type it;
@@ -1301,7 +1302,7 @@ __device__ __forceinline__ void transpose_blocks(const IgemmArgs& a, int tw, uin
       for (int j = 0; j < a.xt_blocks * (KB / 32); ++j, ++block) {
         // (a vote: the compiler then knows that the whole warp takes the branch; elsewhere every matrix load and
         // store would have its own convergence check)
-        if (__all_sync(0xffffffffu, (int)(block & turn) == tw)) {
+        if (__all_sync(0xffffffffu, (int)(block & (kXtWarps - 1)) == tw)) {
           const uint32_t src = slots + ring.idx * kXtSlotBytes + (uint32_t)lane * 128u;
           const uint32_t half = (uint32_t)(j % (KB / 32)) << 6;  // (the upper 32 channels of a row of 64)
           const int px0 = 64 * (j / (KB / 32)) - skew;           // this lane's pixel of the first store, counted from the first input row
@@ -1335,13 +1336,13 @@ __device__ __forceinline__ void transpose_blocks(const IgemmArgs& a, int tw, uin
           __syncwarp();
           if (lane == 0) mbar_arrive(in_empty + 8u * ring.idx);
         }
-        ring.advance((uint32_t)a.xt_slots);
+        ring.advance((uint32_t)kXtSlots);
       }
       // the tensor core reads the tile through the async proxy
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(xb_full + 8u * xb.idx);
-      xb.advance((uint32_t)a.xt_bufs);
+      xb.advance((uint32_t)kXtBufs);
     }
   }
 }
@@ -1363,6 +1364,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __shared__ __align__(8) uint64_t ho_bar;    //   of the warps that hand accumulators over (the first of each lane quarter),
   __shared__ __align__(8) uint64_t pl_bar;    //   of the warps that fetch partial sums (the second of each lane quarter)
   // depthwise input tiles (depthwise + pointwise blocks), or the staging slots of blocks of x (TRANS)
+  static_assert(kXtSlots >= 2 * kMaxDwTeams, "the barriers serve both");
   __shared__ __align__(8) uint64_t in_full[kXtSlots], in_empty[kXtSlots];
   __shared__ __align__(8) uint64_t xb_full[kXtBufs], xb_empty[kXtBufs];  // transposed tiles (TRANS)
   __shared__ __align__(8) uint64_t slabs_full;  // row pairs: the weight slabs have arrived
@@ -1506,11 +1508,11 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 const uint32_t bar = smem_u32(&in_full[in_ring.idx]);
                 mbar_expect_tx(bar, kXtSlotBytes);
                 if (!(a.dbg_drop >= 0 && blockIdx.x == 0 && issued == (uint32_t)a.dbg_drop))  // (test hook, as below)
-                  tma_load_3d(ring_base + (uint32_t)a.stages * a.stage_bytes + (uint32_t)a.xt_bufs * a.xt_bytes + in_ring.idx * kXtSlotBytes,
+                  tma_load_3d(ring_base + (uint32_t)a.stages * a.stage_bytes + (uint32_t)kXtBufs * a.xt_bytes + in_ring.idx * kXtSlotBytes,
                               &tmB, bar, px0 + 64 * (j / (KB / 32)), grp * a.cg + cb * KB + j % (KB / 32) * 32, n0);
               }
               __syncwarp();
-              in_ring.advance((uint32_t)a.xt_slots);
+              in_ring.advance((uint32_t)kXtSlots);
               ++issued;
             }
           }
@@ -1688,7 +1690,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           if (++xt_st == xt_spb) xt_st = xt_r = 0;
           if (xt_st == 0 || gi == groups_per_tile - 1) {  // the item's last stage on this transposed tile
             xt_bar = smem_u32(&xb_empty[xt_ring.idx]);
-            xt_ring.advance((uint32_t)a.xt_bufs);
+            xt_ring.advance((uint32_t)kXtBufs);
           }
         }
         // (row pairs: one stage per kernel row, its weight tiles in the slabs)
@@ -2421,7 +2423,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   const bool gave_up_cta = abort_flag != 0;  // (final only here: no warp raises it any more)
   if (gave_up_cta)
     wait_for_work_under_way<PAIR, DWPW || TRANS>(warp, EW, rank, (uint32_t)a.stages, EPI == 0 && a.slab_off != 0,
-                                                 TRANS ? (uint32_t)a.xt_slots : 2u << a.dw_teams_log2, smem_u32(full_bar),
+                                                 TRANS ? (uint32_t)kXtSlots : 2u << a.dw_teams_log2, smem_u32(full_bar),
                                                  smem_u32(in_full), smem_u32(&slabs_full), smem_u32(&drain_bar),
                                                  (uint32_t)produced_stages[0], (uint32_t)produced_stages[1]);
   // (a pair leaves together: the first CTA's MMAs read the partner's shared memory and write its tensor memory)
@@ -3350,7 +3352,6 @@ bool make_plan_impl(const ConvGeom& g, IgemmPlan* out, bool want_pair, int kb_ma
       p.epi_tiles = trans_epi;
       p.xt_rows_in = rows_in;
       p.xt_blocks = xt_blocks;
-      p.xt_slots = kXtSlots;
       p.xt_dump = (int32_t)reach;
       p.xt_bytes = (uint32_t)tile;
       p.xt_total = (uint32_t)xt;
@@ -3678,7 +3679,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   a.xt_w = g.w;
   a.xt_rows_in = p.xt_rows_in;
   a.xt_magic = (uint32_t)((0x100000000ull + (uint64_t)g.w - 1) / (uint64_t)g.w);
-  a.xt_blocks = p.xt_blocks; a.xt_slots = p.xt_slots; a.xt_bufs = kXtBufs;
+  a.xt_blocks = p.xt_blocks;
   a.epi_tiles = p.epi_tiles;
   a.xt_dump = p.xt_dump; a.xt_bytes = p.xt_bytes; a.xt_total = p.xt_total;
   a.ts = p.ts;
