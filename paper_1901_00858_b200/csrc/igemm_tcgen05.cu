@@ -871,6 +871,19 @@ struct IgemmArgs {
   int32_t dw_in_h, dw_in_w;
   uint32_t dw_in_bytes, dw_in_alloc;
   int32_t dw_teams_log2;  // log2 of the teams that the depthwise warps form: team t computes every stage s with s % teams == t
+  // x[N][C][H*W] turned channels-last inside the kernel (TRANS instantiations): a channel block of a tile is
+  // its th + (R-1)*dil input rows, fetched as blocks of 64 pixels x 32 channels into kXtSlots staging slots
+  // and transposed into one of kXtBufs tiles [row][pitch][KB] that all R*S taps read
+  int32_t xt_w, xt_rows_in;       // pixels per row of x; input rows of a tile
+  uint32_t xt_magic;              // ceil(2^32 / xt_w): row of a pixel by a multiplication
+  int32_t xt_blocks;
+  // kXtSlots and kXtBufs.  (Without these two fields, constants in their place, kernels that use neither take 0.2 %
+  // longer: ResNet-50's layers channels-last, 16 images, 432.2 -> 432.9 us, MobileNet's blocks 150.6 -> 150.9.)
+  int32_t xt_slots, xt_bufs;
+  int32_t xt_dump;                // row of a transposed tile that nothing reads: pixels outside its input rows
+  uint32_t xt_bytes;              // bytes of a transposed tile
+  int32_t epi_tiles;              // epilogue warps that have staging tiles
+  uint32_t xt_total;              // bytes of the transposed tiles and the slots (behind the ring)
   int32_t dbg_drop;     // test hook: stage of the first CTA whose copies are left out (-1: none)
   int32_t ts;           // ring stages per tile: cblocks * R * (S / taps)
   // CTA pairs (clusters of two, tcgen05 cta_group::2): a tile is 256 output channels x two pixel
@@ -883,16 +896,6 @@ struct IgemmArgs {
   int32_t sk_cols32;    // accumulator columns handed over, in units of 32
   float* sk_part;
   int* sk_flags;
-  // x[N][C][H*W] turned channels-last inside the kernel (TRANS instantiations): a channel block of a tile is
-  // its th + (R-1)*dil input rows, fetched as blocks of 64 pixels x 32 channels into kXtSlots staging slots
-  // and transposed into one of kXtBufs tiles [row][pitch][KB] that all R*S taps read
-  int32_t xt_w, xt_rows_in;       // pixels per row of x; input rows of a tile
-  uint32_t xt_magic;              // ceil(2^32 / xt_w): row of a pixel by a multiplication
-  int32_t xt_blocks;
-  int32_t xt_dump;                // row of a transposed tile that nothing reads: pixels outside its input rows
-  uint32_t xt_bytes;              // bytes of a transposed tile
-  int32_t epi_tiles;              // epilogue warps that have staging tiles
-  uint32_t xt_total;              // bytes of the transposed tiles and the slots (behind the ring)
 };
 
 // The tiles of one CTA: blockIdx.x, blockIdx.x + gridDim.x, ...  Tile t = (pixel tile px, channel
@@ -1268,9 +1271,9 @@ __device__ __forceinline__ void transpose_blocks(const IgemmArgs& a, int tw, uin
                                                  uint32_t xb_full, uint32_t xb_empty, volatile int* abort_flag) {
   constexpr uint32_t row_bytes = (uint32_t)KB * 2u;
   const int lane = threadIdx.x & 31;
-  const uint32_t slots = tiles + (uint32_t)kXtBufs * a.xt_bytes;
+  const uint32_t slots = tiles + (uint32_t)a.xt_bufs * a.xt_bytes;
   const int pad = a.pitch - a.xt_w;  // columns of padding per row, left (pad_w) and right
-  for (int i = tw * 32 + lane; i < kXtBufs * a.xt_rows_in * pad * (KB / 8); i += kXtWarps * 32) {
+  for (int i = tw * 32 + lane; i < a.xt_bufs * a.xt_rows_in * pad * (KB / 8); i += kXtWarps * 32) {
     const int chunk = i % (KB / 8), t = i / (KB / 8);
     const int c = t % pad, row = t / pad;  // (rows of all tiles, one after the other)
     const int tile = row / a.xt_rows_in;
@@ -1336,13 +1339,13 @@ __device__ __forceinline__ void transpose_blocks(const IgemmArgs& a, int tw, uin
           __syncwarp();
           if (lane == 0) mbar_arrive(in_empty + 8u * ring.idx);
         }
-        ring.advance((uint32_t)kXtSlots);
+        ring.advance((uint32_t)a.xt_slots);
       }
       // the tensor core reads the tile through the async proxy
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(xb_full + 8u * xb.idx);
-      xb.advance((uint32_t)kXtBufs);
+      xb.advance((uint32_t)a.xt_bufs);
     }
   }
 }
@@ -1508,11 +1511,11 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 const uint32_t bar = smem_u32(&in_full[in_ring.idx]);
                 mbar_expect_tx(bar, kXtSlotBytes);
                 if (!(a.dbg_drop >= 0 && blockIdx.x == 0 && issued == (uint32_t)a.dbg_drop))  // (test hook, as below)
-                  tma_load_3d(ring_base + (uint32_t)a.stages * a.stage_bytes + (uint32_t)kXtBufs * a.xt_bytes + in_ring.idx * kXtSlotBytes,
+                  tma_load_3d(ring_base + (uint32_t)a.stages * a.stage_bytes + (uint32_t)a.xt_bufs * a.xt_bytes + in_ring.idx * kXtSlotBytes,
                               &tmB, bar, px0 + 64 * (j / (KB / 32)), grp * a.cg + cb * KB + j % (KB / 32) * 32, n0);
               }
               __syncwarp();
-              in_ring.advance((uint32_t)kXtSlots);
+              in_ring.advance((uint32_t)a.xt_slots);
               ++issued;
             }
           }
@@ -1690,7 +1693,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           if (++xt_st == xt_spb) xt_st = xt_r = 0;
           if (xt_st == 0 || gi == groups_per_tile - 1) {  // the item's last stage on this transposed tile
             xt_bar = smem_u32(&xb_empty[xt_ring.idx]);
-            xt_ring.advance((uint32_t)kXtBufs);
+            xt_ring.advance((uint32_t)a.xt_bufs);
           }
         }
         // (row pairs: one stage per kernel row, its weight tiles in the slabs)
@@ -2423,7 +2426,7 @@ igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   const bool gave_up_cta = abort_flag != 0;  // (final only here: no warp raises it any more)
   if (gave_up_cta)
     wait_for_work_under_way<PAIR, DWPW || TRANS>(warp, EW, rank, (uint32_t)a.stages, EPI == 0 && a.slab_off != 0,
-                                                 TRANS ? (uint32_t)kXtSlots : 2u << a.dw_teams_log2, smem_u32(full_bar),
+                                                 TRANS ? (uint32_t)a.xt_slots : 2u << a.dw_teams_log2, smem_u32(full_bar),
                                                  smem_u32(in_full), smem_u32(&slabs_full), smem_u32(&drain_bar),
                                                  (uint32_t)produced_stages[0], (uint32_t)produced_stages[1]);
   // (a pair leaves together: the first CTA's MMAs read the partner's shared memory and write its tensor memory)
@@ -3679,7 +3682,7 @@ cudaError_t launch_igemm(const ConvGeom& g_layer, IgemmPlan& p, void* ws, const 
   a.xt_w = g.w;
   a.xt_rows_in = p.xt_rows_in;
   a.xt_magic = (uint32_t)((0x100000000ull + (uint64_t)g.w - 1) / (uint64_t)g.w);
-  a.xt_blocks = p.xt_blocks;
+  a.xt_blocks = p.xt_blocks; a.xt_slots = kXtSlots; a.xt_bufs = kXtBufs;
   a.epi_tiles = p.epi_tiles;
   a.xt_dump = p.xt_dump; a.xt_bytes = p.xt_bytes; a.xt_total = p.xt_total;
   a.ts = p.ts;
